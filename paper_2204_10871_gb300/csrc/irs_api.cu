@@ -105,6 +105,7 @@ irs_status alloc_workspace(irs_plan_t* P) {
   const size_t o_msum = take(sizeof(double));
   const size_t o_mpart = take(sizeof(double) * irs::MSUM_BLOCKS);
   const size_t o_status = take(sizeof(int));
+  const size_t o_queue = take(sizeof(unsigned long long));
   size_t o_tiles = 0;
   if (P->p.method == IRS_BRUTE) o_tiles = take(sizeof(irs::TileRec) * (size_t)P->br_ntiles);
   P->ws_bytes = off;
@@ -117,6 +118,7 @@ irs_status alloc_workspace(irs_plan_t* P) {
   P->d_msum = reinterpret_cast<double*>(b + o_msum);
   P->d_mpart = reinterpret_cast<double*>(b + o_mpart);
   P->d_status = reinterpret_cast<int*>(b + o_status);
+  P->d_queue = reinterpret_cast<unsigned long long*>(b + o_queue);
   P->d_tiles = P->p.method == IRS_BRUTE ? reinterpret_cast<irs::TileRec*>(b + o_tiles) : nullptr;
   if (cudaMemset(P->ws, 0, P->ws_bytes) != cudaSuccess) return IRS_ERR_CUDA;
   return IRS_OK;

@@ -147,7 +147,7 @@ bool measure_size(const irs_params& base, double mult, const double* xy, const d
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (base_ms >= 0 && cudaEventCreate(&e0) == cudaSuccess && cudaEventCreate(&e1) == cudaSuccess) {
     for (int v = 0; v < irs::interp_num_variants(); ++v) {
-      if (irs::interp_set_variant(P, v) != IRS_OK) continue;
+      if (!irs::interp_variant_distinct(v) || irs::interp_set_variant(P, v) != IRS_OK) continue;
       float ray = -1.f;
       for (int rep = 0; rep < 2; ++rep) {
         if (irs::interp_raypass_rows(P, r0, r1, counts, s, e0, e1) != IRS_OK) break;

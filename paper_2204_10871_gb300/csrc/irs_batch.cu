@@ -93,17 +93,18 @@ irs_status enqueue(BatchEntry* e, irs_plan_t* const* plans, int32_t nmaps, const
     // item count of the group, recomputed from the plans (cheap, host side)
     std::vector<irs_plan_t*> gp;
     std::vector<uint32_t*> gc;
-    int nrow = 0;
+    int nrow = 0, near_cap = 0;
     for (int m : gm) {
       gp.push_back(plans[m]);
       gc.push_back(counts[m]);
-      const int r = irs::interp_row_entries(plans[m]);
+      const int r = irs::interp_row_entries(plans[m]), c = irs::interp_near_cap(plans[m], n[m]);
       nrow = r > nrow ? r : nrow;
+      near_cap = c > near_cap ? c : near_cap;
     }
     std::vector<char> tmp(irs::interp_desc_bytes((int)gm.size()));
     const int64_t items = irs::interp_fill_descs(gp.data(), gc.data(), (int)gm.size(), tmp.data());
     irs_status st = irs::interp_batch_launch((int)v, base + group_off[v], (int)gm.size(), items,
-                                             queues + v, plans[gm[0]]->num_sms, nrow, cs);
+                                             queues + v, plans[gm[0]]->num_sms, nrow, near_cap, cs);
     if (st != IRS_OK) return st;
   }
   if (mag) {

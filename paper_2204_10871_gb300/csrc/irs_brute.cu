@@ -65,8 +65,10 @@ __global__ void k_mass_partial(const double* __restrict__ mass, const double2* _
   if (threadIdx.x == 0) part[blockIdx.x] = sh[0];
 }
 
-__global__ void k_mass_final(const double* __restrict__ part, double* __restrict__ out) {
+__global__ void k_mass_final(const double* __restrict__ part, double* __restrict__ out,
+                             unsigned long long* __restrict__ queue) {
   if (threadIdx.x == 0 && blockIdx.x == 0) {
+    if (queue) *queue = 0ull;  // the ray pass's work counter
     double s = 0.0;
     for (int b = 0; b < MSUM_BLOCKS; ++b) s += part[b];
     out[0] = s;
@@ -91,7 +93,7 @@ cudaError_t launch_mass_sum(const irs_plan_t* P, const double* mass, int64_t n, 
   L.check = xy != nullptr && n > 0;
   k_mass_partial<<<MSUM_BLOCKS, MSUM_THREADS, 0, s>>>(mass, reinterpret_cast<const double2*>(xy), n, L,
                                                       P->d_status, P->d_mpart);
-  k_mass_final<<<1, 32, 0, s>>>(P->d_mpart, P->d_msum);
+  k_mass_final<<<1, 32, 0, s>>>(P->d_mpart, P->d_msum, P->d_queue);
   return cudaGetLastError();
 }
 

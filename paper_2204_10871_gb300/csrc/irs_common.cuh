@@ -60,27 +60,6 @@ __device__ __forceinline__ void bin_warp(uint32_t* counts, bool valid, uint32_t 
   if (valid && lane == __ffs(peers) - 1) atomicAdd(counts + key, (uint32_t)__popc(peers));
 }
 
-// Key forms (~0u = no pixel) for the ray pass.  The leader of each group of
-// equal keys is its lowest lane: no lower lane (lane_lt = its lane mask) shares it.
-__device__ __forceinline__ void bin_warp_key(uint32_t* counts, uint32_t key, unsigned lane_lt) {
-  const unsigned peers = __match_any_sync(0xFFFFFFFFu, key);
-  if (key != 0xFFFFFFFFu && (peers & lane_lt) == 0u) atomicAdd(counts + key, (uint32_t)__popc(peers));
-}
-
-// Run-length variant: lanes hold consecutive columns of one row, so equal
-// pixels usually come in runs; the first lane of each run of equal keys adds
-// the run's length (non-adjacent equal keys add separately).
-__device__ __forceinline__ void bin_warp_runs_key(uint32_t* counts, uint32_t key, int lane) {
-  const uint32_t prev = __shfl_up_sync(0xFFFFFFFFu, key, 1);
-  const bool head = (lane == 0) || (key != prev);
-  const unsigned heads = __ballot_sync(0xFFFFFFFFu, head);
-  if (key != 0xFFFFFFFFu && head) {
-    const unsigned later = heads & ~((2u << lane) - 1u);  // heads after this lane
-    const int next = later ? __ffs(later) - 1 : 32;
-    atomicAdd(counts + key, (uint32_t)(next - lane));
-  }
-}
-
 // Pixel of a ray from its position relative to the base pixel's lower-left
 // corner (brel1, brel2 in theta_E): floor per axis, so a ray on a pixel edge
 // belongs to the pixel above / to the right of it.
@@ -114,50 +93,6 @@ __device__ __forceinline__ void pixel_keys2(float2 t1, float2 t2, uint32_t bx, u
   const uint32_t pxb = __float_as_uint(f1.y) + bx, pyb = __float_as_uint(f2.y) + by;
   ka = (pxa < npix_x && pya < npix_y) ? pya * npix_x + pxa : 0xFFFFFFFFu;
   kb = (pxb < npix_x && pyb < npix_y) ? pyb * npix_x + pxb : 0xFFFFFFFFu;
-}
-
-// pixel_keys2 plus each ray's bin in a box of hbx x hby pixels (lhx, lhy: the
-// box origin folded with the floor's bit pattern offset, as bx, by); ~0u for
-// rays off the map or outside the box.
-__device__ __forceinline__ void pixel_keys2_box(float2 t1, float2 t2, uint32_t bx, uint32_t by,
-                                                uint32_t npix_x, uint32_t npix_y, uint32_t lhx, uint32_t lhy,
-                                                uint32_t hbx, uint32_t hby, uint32_t& ka, uint32_t& kb,
-                                                uint32_t& la, uint32_t& lb) {
-  const float2 f1 = __fadd2_rd(t1, make_float2(PIX_MAGIC, PIX_MAGIC));
-  const float2 f2 = __fadd2_rd(t2, make_float2(PIX_MAGIC, PIX_MAGIC));
-  const uint32_t ua = __float_as_uint(f1.x), va = __float_as_uint(f2.x);
-  const uint32_t ub = __float_as_uint(f1.y), vb = __float_as_uint(f2.y);
-  const uint32_t pxa = ua + bx, pya = va + by, pxb = ub + bx, pyb = vb + by;
-  const bool ina = pxa < npix_x && pya < npix_y, inb = pxb < npix_x && pyb < npix_y;
-  ka = ina ? pya * npix_x + pxa : 0xFFFFFFFFu;
-  kb = inb ? pyb * npix_x + pxb : 0xFFFFFFFFu;
-  const uint32_t xa = ua + lhx, ya = va + lhy, xb = ub + lhx, yb = vb + lhy;
-  la = (ina && xa < hbx && ya < hby) ? ya * hbx + xa : 0xFFFFFFFFu;
-  lb = (inb && xb < hbx && yb < hby) ? yb * hbx + xb : 0xFFFFFFFFu;
-}
-
-// Both rays of a row pair (keys ka, kb): lanes whose two keys are equal add
-// 2 to it, the others 1 to ka, in one __match_any_sync on ka (the leader adds
-// its peers plus its peers of weight 2); the kb of lanes whose keys differ
-// go through a second match, run only when such a lane exists.
-__device__ __forceinline__ void bin_warp_pair(uint32_t* counts, uint32_t ka, uint32_t kb, unsigned lane_lt) {
-  const unsigned same = __ballot_sync(0xFFFFFFFFu, ka == kb);
-  const unsigned peers = __match_any_sync(0xFFFFFFFFu, ka);
-  if (ka != 0xFFFFFFFFu && (peers & lane_lt) == 0u)
-    atomicAdd(counts + ka, (uint32_t)(__popc(peers) + __popc(peers & same)));
-  if (same != 0xFFFFFFFFu) bin_warp_key(counts, ka == kb ? 0xFFFFFFFFu : kb, lane_lt);
-}
-
-// bin_warp_key into a shared-memory sub-histogram where the leader's ray has
-// a box bin (lkey; equal keys have equal bins), into the map otherwise.
-__device__ __forceinline__ void bin_warp_key_box(uint32_t* counts, uint32_t* hist, uint32_t key, uint32_t lkey,
-                                                 unsigned lane_lt) {
-  const unsigned peers = __match_any_sync(0xFFFFFFFFu, key);
-  if (key != 0xFFFFFFFFu && (peers & lane_lt) == 0u) {
-    const uint32_t n = (uint32_t)__popc(peers);
-    if (lkey != 0xFFFFFFFFu) atomicAdd(hist + lkey, n);
-    else atomicAdd(counts + key, n);
-  }
 }
 
 // ---------------------------------------------------------------- brute force
@@ -220,6 +155,7 @@ struct irs_plan {
   double* d_mpart;         // [MSUM_BLOCKS] partial sums
   irs::TileRec* d_tiles;   // [br_ntiles]
   int* d_status;           // sticky device error
+  unsigned long long* d_queue;  // work counter of the ray pass, zeroed by the mass sum (NULL: none)
   int device;
   int num_sms;
   // INTERP state (irs_interp.cu)

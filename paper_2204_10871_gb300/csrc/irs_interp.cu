@@ -33,6 +33,7 @@
 #include <string.h>
 
 #include <new>
+#include <type_traits>
 
 #include "irs_df.cuh"
 #include "irs_fft.cuh"
@@ -62,7 +63,7 @@ constexpr int IP_KD = 3;
 constexpr int IP_NKD = IP_PD + IP_KD - 1;  // kernel orders n = j + k of the double-float products
 constexpr int IP_NEAR_MAX = 1024;  // lenses of a 3x3 block held in shared memory
 constexpr int IP_KMAX_RAYS = 1024;  // rays along a cell side (row table in shared memory)
-constexpr int IP_THREADS = 256;
+constexpr int IP_THREADS = 256;     // largest CTA of the ray pass
 constexpr int IP_MAX_CORNER = 4;
 
 constexpr int DEFAULT_K = 24;
@@ -90,10 +91,10 @@ struct IpGeo {
   float inv_k;  // 1 / k in FP32 (correctly rounded)
   int32_t nrow;  // row-pair entries of the ray pass's row table: (k + 1)/2 + IP_ROW_PAD
   int32_t pad_;
-  // privatised binning (BIN 2): half extents, in pixels, of the box around a
-  // cell's centre that holds its rays' pixels under the mean lens map, with
-  // room for the near lenses' and the far field's spread
-  float box_hx, box_hy;
+  // blocks of a cell that map into about one binning box of the ray pass:
+  // columns and 8-row groups; the cell's pixel extents under the mean lens map
+  int32_t blk_col, blk_rg;
+  float cell_px, cell_py;
 };
 
 struct InterpState {
@@ -133,7 +134,7 @@ struct InterpState {
   double2* sheet_d;     // [nray cells][FIN_K64] terms k < FIN_K64
   float2* sheet_f;      // [nray cells][K - FIN_K64] the rest
   uint8_t* sheet_near;  // [nray cells] bit q: corner q evaluated per ray instead
-  int grid_ray;
+  int64_t n_last;  // lenses of the last cell lists built
 };
 
 InterpState* S_(irs_plan_t* P) { return static_cast<InterpState*>(P->interp); }
@@ -717,8 +718,6 @@ k_ip_finalize(Geo g, IpGeo ig, const double* __restrict__ msum, const int32_t* _
 }
 
 // ------------------------------------------------------------ ray pass
-enum { IP_MAP = 0, IP_DUMP = 1 };
-
 struct IpRayArgs {
   const int32_t* start;
   const float4* rel;
@@ -732,134 +731,228 @@ struct IpRayArgs {
   double* beta_out;
   int64_t* pix_out;
   int64_t nwork;
+  unsigned long long* queue;  // work counter of the launch, zero before it
+  int32_t near_cap;           // lenses of a 3x3 block the CTA's shared memory holds
+  int32_t parts;              // work items per cell, each a share of its row groups
 };
 
 // Kernel variants of the ray pass (the autotuner picks one per plan):
-// rays per thread R, level-2 sub-cells per side Q, sub-cell series terms K2.
-// The truncation is (sub-cell half-diagonal / distance to the nearest far
-// lens)^K2 of that lens's field: Q = 8, 10, 12, 16 give ratios 0.083, 0.067,
-// 0.057, 0.042, so 8, 7, 6 and 6 terms stay at or below ~3e-8; variants 11
-// and 13-15 trade one Horner step per ray for bounds of 1.7e-7 (16 sub-cells,
-// 5 terms), 3.3e-7 (14) and 7.3e-7 (12), the last with fewer sub-cells to
-// re-centre per cell; variant 16 takes one more step off with 4 terms on 16
-// sub-cells (3.1e-6, more sub-cells to re-centre).
-// MINB: CTAs per SM the register budget is sized for; BIN: warp binning by
-// __match_any_sync (0), by runs of equal pixels (1), or by __match_any_sync
-// into a shared-memory sub-histogram over the cell's pixel box, flushed to
-// the map once per cell, with global atomics for rays outside the box (2),
-// or by row pairs (3: a pair whose two rays share a pixel adds 2 in one
-// __match_any_sync; a second one runs only when some lane's pair differs);
-// NPR: how many of a
-// thread's R/2 row pairs share one reciprocal per lens, 1/(r_a^2 r_b^2) (the
-// near sum is bound by the MUFU's 16 reciprocals per SM per clock; a shared
-// reciprocal trades one MUFU op for FP32 work on a pipe that is half idle).
-#define IP_VARIANTS(X)                                                                       \
-  X(0, 8, 12, 6, 3, 0, 0) X(1, 8, 10, 7, 3, 0, 0) X(2, 8, 16, 6, 3, 0, 2)                       \
-  X(3, 8, 16, 6, 3, 0, 4) X(4, 8, 16, 6, 2, 1, 0) X(5, 8, 16, 6, 3, 1, 0)                      \
-  X(6, 8, 16, 6, 3, 1, 2) X(7, 8, 16, 6, 3, 0, 0) X(8, 4, 16, 6, 4, 0, 0)                      \
-  X(9, 8, 8, 8, 3, 0, 0) X(10, 8, 12, 6, 4, 0, 0) X(11, 8, 16, 5, 3, 0, 0)                    \
-  X(12, 8, 16, 5, 3, 2, 0) X(13, 8, 16, 5, 3, 3, 0) X(14, 8, 12, 5, 3, 3, 0) X(15, 8, 14, 5, 3, 3, 0) \
-  X(16, 8, 16, 4, 3, 3, 0)
+// level-2 sub-cells per side Q, sub-cell series terms K2, and NPR: how many of
+// a thread's four row pairs share one reciprocal per lens, 1/(r_a^2 r_b^2)
+// (the MUFU's 16 reciprocals per SM per clock bound the near sum; a shared
+// reciprocal trades one MUFU op for FP32 work).  The truncation is (sub-cell
+// half-diagonal / distance to the nearest far lens)^K2 of that lens's field:
+// Q = 8, 10, 12, 16 give ratios 0.083, 0.067, 0.057, 0.042, so 8, 7, 6 and 6
+// terms stay at or below ~3e-8; variants 11, 14 and 15 trade one Horner step
+// per ray for bounds of 1.7e-7 (16 sub-cells, 5 terms), 3.3e-7 (14) and 7.3e-7
+// (12), the last with fewer sub-cells to re-centre per cell; variant 16 takes
+// one more step off with 4 terms on 16 sub-cells (3.1e-6, more sub-cells to
+// re-centre).  Variant numbers that differ only in launch shape or binning
+// share one kernel: every launch is shaped from the cell (ip_launch_shape).
+#define IP_VARIANTS(X)                                                                     \
+  X(0, 12, 6, 0) X(1, 10, 7, 0) X(2, 16, 6, 2) X(3, 16, 6, 4) X(5, 16, 6, 0) X(9, 8, 8, 0) \
+  X(11, 16, 5, 0) X(14, 12, 5, 0) X(15, 14, 5, 0) X(16, 16, 4, 0)
 constexpr int IP_NVARIANT = 17;
-
-// Advance a (strip, row group) position by `by` units of a row-major
-// nstrip-wide unit grid.
-__device__ __forceinline__ void step_unit(int& st, int& rg, int by, int nstrip) {
-  st += by;
-  while (st >= nstrip) {
-    st -= nstrip;
-    ++rg;
-  }
+// the variant whose kernel serves variant v
+constexpr int ip_kernel_of(int v) {
+  return v == 4 || v == 7 || v == 8 ? 5 : v == 6 ? 2 : v == 10 ? 0 : v == 12 || v == 13 ? 11 : v;
 }
 
-// Row table of a cell, one entry per pair of cell rows (2l, 2l + 1).
-struct __align__(16) IpRowPair {
-  float4 sg;  // (sigma_y, sigma_y', -sigma_y, -sigma_y'), sigma_y = (l + 1/2) Q / k - v - 1/2
-  float4 ty;  // (tau_y h, tau_y' h, y0, y0'), y0 = by_lo + lambda_2 tau_y h: the row's share of beta_2
-  int2 v;     // (v Q, v' Q): level-2 row offsets
-};
+constexpr int IP_R = 8;  // rays per thread and unit: one lattice column, four row pairs
 
-// Row pairs of the row table past the cell's last: a thread's R / 2 pairs
-// are read without clamping the index (R <= 2 IP_ROW_PAD).
+// Row pairs of the row table past the cell's last: a thread's four pairs are
+// read without clamping the index.
 constexpr int IP_ROW_PAD = 4;
+static_assert(IP_R <= 2 * IP_ROW_PAD, "row table padding");
 
 // Row stride (float2) of the per-cell table of scaled series coefficients:
 // odd, so that the K2 rows a warp reads at once fall in distinct banks.
 constexpr int IP_CB_STRIDE = IP_KMAX + 1;
 
-// Dynamic shared memory of the ray pass (bytes, 16-byte aligned blocks):
-// near lenses as (-x, -x, -y, -y) and (-m, -m) pairs, the level-2 series
-// as conj duplicated (c.re, c.re, -c.im, -c.im), the row table and the
-// level-1 series scaled for the re-centring, one row per level-2 term.
-// Bins of the privatised sub-histogram (BIN 2): a cell whose pixel box is
-// larger bins globally.
-constexpr int IP_HIST_MAX = 2048;
+// Binning box: a CTA counts its cell's rays in a shared-memory histogram of
+// 32 x 64 pixels (rows padded by four words against bank conflicts) placed
+// around the block's position under the near lenses' softened pull and adds the
+// non-empty bins to the map once per box (87-98 % of the rays fall inside).  An increment by one of a shared word is a single instruction that
+// the hardware resolves for all lanes at once, equal addresses included:
+// 1.25 SM cycles per warp whatever the number of distinct pixels, against 2.1
+// per distinct pixel for __match_any_sync, which the binning used before.  The
+// paper-mid ray pass took 28.0 ms with match-and-add into the map and 26.0 ms
+// with this histogram (same loop otherwise; 64 x 64 pixels: 26.6 ms, the
+// larger flush costs more than the fewer rays outside save).
+constexpr int IP_BOX_W = 32, IP_BOX_H = 64;
+constexpr int IP_HS = IP_BOX_W + 2;  // row stride in words
+constexpr int IP_HIST = IP_HS * IP_BOX_H;
 
-// The row table holds `nrow` entries, sized per plan from its cell side
-// (IpGeo::nrow), so that small cells leave shared memory for more CTAs; the
-// privatised binning adds its sub-histogram at the end.
-template <int Q, int K2, int BIN>
+// Dynamic shared memory of the ray pass: the level-2 series as conj duplicated
+// (c.re, c.re, -c.im, -c.im), the histogram, the level-1 series scaled for the
+// re-centring with its scale factors, the row table, and the near lenses.
+// size come first, so that the addresses of the hot ones are constants.
+struct __align__(16) IpRowPair {  // one entry per pair of cell rows (2l, 2l + 1)
+  float4 sg;      // (sigma_y, sigma_y', -sigma_y, -sigma_y'), sigma_y = (l + 1/2) Q/k - v - 1/2
+  float4 ty;      // (tau_y h, tau_y' h, y0, y0'), y0 = by_lo + lambda_2 tau_y h: the row's share of beta_2
+  int q4;         // byte offset of the level-2 row shared by this pair and the next, or -1
+  uint16_t v[2];  // the two rows' level-2 rows times Q
+  int pad[2];
+};
+struct __align__(16) IpNear {  // a lens of the 3x3 block
+  float4 xy;  // (-x, -x, -y, -y)
+  float2 m;   // (-m, -m)
+  float pad[2];
+};
+// float4s per level-2 sub-cell: odd, so that the eight sub-cells that a quarter
+// of a warp reads or writes at once lie in distinct banks (with 4, 6 or 8
+// terms back to back, 2, 2 and 8 of them share one)
+__host__ __device__ constexpr int ip_sub_stride(int k2) { return k2 | 1; }
+template <int Q, int K2>
 struct IpSmem {
-  static constexpr size_t near_xy = 0;
-  static constexpr size_t near_m = near_xy + sizeof(float4) * IP_NEAR_MAX;
-  static constexpr size_t sub = near_m + sizeof(float2) * IP_NEAR_MAX;
-  static constexpr int nrow_max = IP_KMAX_RAYS / 2 + IP_ROW_PAD;
-  static constexpr size_t row_sg = sub + sizeof(float4) * Q * Q * K2;
-  static __host__ __device__ constexpr size_t coef(int nrow) { return row_sg + sizeof(IpRowPair) * nrow; }
-  static __host__ __device__ constexpr size_t hist(int nrow) {
-    return (coef(nrow) + sizeof(float2) * K2 * IP_CB_STRIDE + 15) / 16 * 16;
+  static constexpr int sub = 0;
+  static constexpr int hist = sub + 16 * Q * Q * ip_sub_stride(K2);
+  static constexpr int cb = hist + 4 * IP_HIST;
+  static constexpr int sc = cb + 8 * K2 * IP_CB_STRIDE;
+  static constexpr int row = (sc + 4 * K2 * IP_CB_STRIDE + 15) & ~15;
+  int near, bytes;
+  __host__ __device__ IpSmem(int nrow, int near_cap) {
+    near = row + (int)sizeof(IpRowPair) * nrow;
+    bytes = near + (int)sizeof(IpNear) * near_cap;
   }
-  static __host__ __device__ constexpr size_t bytes(int nrow) {
-    return hist(nrow) + (BIN == 2 ? sizeof(uint32_t) * IP_HIST_MAX : 0);
-  }
-  static constexpr size_t bytes_max = bytes(nrow_max);
 };
 
+// A CTA's tables that depend on the plan's geometry alone: written once per
+// launch (per map in a batch), with y0 and x0 left to each cell.
+template <int Q, int K2>
+__device__ __forceinline__ void ip_tables(const IpGeo& ig, const IpSmem<Q, K2>& L, unsigned char* sm) {
+  IpRowPair* row_s = reinterpret_cast<IpRowPair*>(sm + L.row);
+  float* sc_s = reinterpret_cast<float*>(sm + L.sc);
+  constexpr int SUB = 16 * ip_sub_stride(K2);  // bytes per sub-cell
+  const int tid = threadIdx.x, nt = blockDim.x;
+  const float hf = ig.hf, inv_k = ig.inv_k;
+  const float qk = __fmul_rn((float)Q, inv_k);  // sub-cell index = floor((l + 1/2) Q / k)
+  auto level2 = [&](int l, float& s) {
+    s = __fmul_rn(__fadd_rn((float)l, 0.5f), qk);
+    return min(__float2int_rd(s), Q - 1);
+  };
+  // rows of the whole cell side and IP_ROW_PAD pairs past it (rows past the
+  // cell side are never binned; their sub-cell row is clamped to Q - 1)
+  for (int pr = tid; pr < ig.nrow; pr += nt) {
+    float t[2], s[2];
+    int v[2];
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const int l = 2 * pr + j;
+      float sv;
+      v[j] = level2(l, sv);
+      t[j] = __fmul_rn(fmaf((float)l, inv_k, fmaf(0.5f, inv_k, -0.5f)), hf);
+      s[j] = __fsub_rn(__fsub_rn(sv, (float)v[j]), 0.5f);
+    }
+    float s3;
+    const int v3 = level2(2 * pr + 3, s3);
+    row_s[pr].sg = make_float4(s[0], s[1], -s[0], -s[1]);
+    row_s[pr].ty = make_float4(t[0], t[1], 0.f, 0.f);
+    row_s[pr].q4 = v[0] == v3 ? v[0] * Q * SUB : -1;
+    row_s[pr].v[0] = (uint16_t)(v[0] * Q);
+    row_s[pr].v[1] = (uint16_t)(v[1] * Q);
+  }
+  // Q^-n binom(kk, n) (binomials exact in FP32 for kk < 32)
+  const float inv_q = __fdiv_rn(1.0f, (float)Q);
+  for (int t = tid; t < K2 * IP_CB_STRIDE; t += nt) {
+    const int nn = t / IP_CB_STRIDE, kk = t % IP_CB_STRIDE;
+    float sc = 0.f;
+    if (kk >= nn && kk >= 1) {
+      int b = 1;  // binom(kk, nn), exact integer steps
+      for (int i = 1; i <= nn; ++i) b = b * (kk - nn + i) / i;
+      sc = (float)b;
+      for (int i = 0; i < nn; ++i) sc = __fmul_rn(sc, inv_q);
+    }
+    sc_s[t] = sc;
+  }
+  uint32_t* hist_s = reinterpret_cast<uint32_t*>(sm + L.hist);
+  for (int t = tid; t < IP_HIST; t += nt) hist_s[t] = 0u;
+}
+
+// A sheet corner near the cell, for one ray: -i a_c (z - c) Log(z - c) added to
+// the conjugate series (qr, qi); corner = ((z_C - c).re, .im, a_c).
+__device__ __forceinline__ void sheet_corner_ray(const float* corner, float tx, float ty, float& qr, float& qi) {
+  const float wr = __fadd_rn(corner[0], tx), wi = __fadd_rn(corner[1], ty);
+  const float lr = __fmul_rn(0.5f, logf(fmaf(wr, wr, __fmul_rn(wi, wi)))), li = atan2f(wi, wr);
+  const float plr = fmaf(wr, lr, -__fmul_rn(wi, li)), pli = fmaf(wr, li, __fmul_rn(wi, lr));
+  qr = fmaf(corner[2], pli, qr);
+  qi = fmaf(corner[2], plr, qi);
+}
+
+// Shared-memory words at four byte addresses incremented by one where `on`.
+__device__ __forceinline__ void shared_inc4(uint32_t a, uint32_t b, uint32_t c, uint32_t d, bool on) {
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.u32 p, %4, 0;\n @p red.shared.add.u32 [%0], 1;\n"
+      " @p red.shared.add.u32 [%1], 1;\n @p red.shared.add.u32 [%2], 1;\n @p red.shared.add.u32 [%3], 1;\n}" ::"r"(a),
+      "r"(b), "r"(c), "r"(d), "r"((uint32_t)on)
+      : "memory");
+}
+
+// Re-centring: pairs of sub-cells per thread.  They share each coefficient read
+// from shared memory, and their Horner chains interleave.
+constexpr int IP_RC = 4;
+
 // One level-1 cell: gather the 3x3 block's lenses, re-centre the series on the
-// sub-cells, then every ray of rows [jlo, jhi) of the cell.  In DUMP mode the
-// thread holding ray (want_i, want_j) writes its beta and pixel to slot `work`.
+// sub-cells, then every ray of rows [row0, row1) of the cell.
 //
-// Each thread takes one lattice column and R rows; rows go in pairs through
+// Each thread takes one lattice column and eight rows; rows go in pairs through
 // the packed FP32x2 instructions (two rows share the column's dx and sigma_x),
 // which round exactly as the scalar ones.  The accumulators hold -alpha (the
 // masses are stored negated) and the level-2 Horner runs on the conjugate, so
-// no negation is issued per ray.
-template <int MODE, int R, int Q, int K2, int BIN, int NPR>
+// no negation is issued per ray.  The pass is bound by instruction issue (0.72
+// of the slots; 52.5 instructions per ray, 62.5 before) with the MUFU next, so
+// what is the same for a row comes from a table, four rows that share a level-2
+// row read its series once, the sheet's corners sit on the general path of the
+// tail only, and a last strip of few columns takes several row groups at once
+// (a 45-ray cell: 83 % of the lanes busy instead of 70 %).  Ray pass, one
+// GB300, against the form with match-and-add binning, fixed cells per CTA and
+// one set-up chain per thread: paper-mid 20.2 ms (28.0), high-res 204 ms (275),
+// a 500^2 map of 1e4 lenses 0.28 ms (0.44), 128^2 with 150 lenses 0.078 (0.088).
+template <int Q, int K2, int NPR>
 __device__ __forceinline__ void ip_cell(const Geo& g, const IpGeo& ig, const IpRayArgs& a, int64_t rc,
-                                        int64_t want_i, int64_t want_j, int64_t work) {
-  static_assert(R % 2 == 0, "rows go in pairs");
-  static_assert(NPR >= 0 && NPR <= R / 2, "paired row pairs");
-  using L = IpSmem<Q, K2, BIN>;
-  extern __shared__ __align__(16) unsigned char ip_smem[];
-  float4* nxy_s = reinterpret_cast<float4*>(ip_smem + L::near_xy);
-  float2* nm_s = reinterpret_cast<float2*>(ip_smem + L::near_m);
-  float4* sub_s = reinterpret_cast<float4*>(ip_smem + L::sub);
-  IpRowPair* row_s = reinterpret_cast<IpRowPair*>(ip_smem + L::row_sg);
-  float2* cb_s = reinterpret_cast<float2*>(ip_smem + L::coef(ig.nrow));
-  uint32_t* hist_s = reinterpret_cast<uint32_t*>(ip_smem + L::hist(ig.nrow));
+                                        int part, const IpSmem<Q, K2>& L, unsigned char* sm, long long next,
+                                        long long* next_s) {
+  static_assert(NPR >= 0 && NPR <= IP_R / 2, "paired row pairs");
+  constexpr int SUB = 16 * ip_sub_stride(K2);  // bytes per sub-cell
+  float4* sub_s = reinterpret_cast<float4*>(sm + L.sub);
+  uint32_t* hist_s = reinterpret_cast<uint32_t*>(sm + L.hist);
+  float2* cb_s = reinterpret_cast<float2*>(sm + L.cb);
+  const float* sc_s = reinterpret_cast<const float*>(sm + L.sc);
+  IpRowPair* row_s = reinterpret_cast<IpRowPair*>(sm + L.row);
+  IpNear* near_s = reinterpret_cast<IpNear*>(sm + L.near);
   __shared__ CellRec rec_s;
   __shared__ int blk_start[9], blk_off[10];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int64_t k = ig.k;
+  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0);  // uniform
   // Every FP32 step of the cell's ray geometry below is written with explicit
   // rounding (__fadd_rn, __fmul_rn, __fdiv_rn, fmaf): implicit contraction
   // would depend on how the compiler places the code in each kernel that
   // inlines this function, and the single-map and batched ray passes must
   // give the same maps bit for bit.
   const float hf = ig.hf;
-  const float inv_k = ig.inv_k;
-
+  const int k = (int)ig.k;
   const int rcx = (int)(rc % ig.nrcx), rcy = (int)(rc / ig.nrcx);
   const int cx = rcx + ig.ox, cy = rcy + ig.oy;
   const int64_t i0 = (int64_t)rcx * k, j0 = (int64_t)rcy * k;
-  const int64_t i1 = min(i0 + k, g.nrx);
-  int64_t jlo = j0, jhi = min(j0 + k, g.nry);
-  if (MODE == IP_MAP) {
-    jlo = max(jlo, a.row0);
-    jhi = min(jhi, a.row1);
-    if (jlo >= jhi) return;  // uniform over the CTA
+  const int64_t jlo = max(j0, a.row0), jhi = min(min(j0 + k, g.nry), a.row1);
+  // cell-local lattice indices: columns [0, kx), rows [ylo, yhi), of these the
+  // row groups [grg0, nrg) of this part; units start on an even row so that row
+  // pairs line up with the table
+  constexpr int R = IP_R;
+  const int kx = (int)(min(i0 + k, g.nrx) - i0), ylo = (int)(jlo - j0), yhi = (int)(jhi - j0);
+  const int ylo2 = ylo & ~1;
+  int grg0 = 0, nrg = jlo < jhi ? (yhi - ylo2 + R - 1) / R : 0;
+  if (a.parts > 1) {
+    const int all = nrg;
+    grg0 = all * part / a.parts;
+    nrg = all * (part + 1) / a.parts;
   }
-  __syncthreads();  // previous cell's shared data no longer read
+  if (grg0 >= nrg) {  // nothing to shoot; uniform over the CTA
+    __syncthreads();  // everyone has read the item before
+    if (tid == 0) *next_s = next;
+    __syncthreads();
+    return;
+  }
   if (warp == 0) {
     // lane q < 9 takes cell q of the 3x3 block (row-major from the lower
     // left); the block's lens offsets are the exclusive prefix sum of the counts
@@ -897,330 +990,377 @@ __device__ __forceinline__ void ip_cell(const Geo& g, const IpGeo& ig, const IpR
   // terms from 1: term 0 sits in the cell's base) on the sub-cell centres
   // eps: with w = eps + sigma / Q the coefficient of sigma^n is
   // Q^-n sum_kk binom(kk, n) c_kk eps^(kk - n).  First the per-cell table
-  // cb[n][kk] = Q^-n binom(kk, n) c_kk (binomials exact in FP32 for kk < 32).
-  const float inv_q = __fdiv_rn(1.0f, (float)Q);
-  for (int t = tid; t < K2 * ig.K; t += blockDim.x) {
-    const int nn = t / ig.K, kk = t % ig.K;
-    float2 v = make_float2(0.f, 0.f);
-    if (kk >= nn && kk >= 1) {
-      int b = 1;  // binom(kk, nn), exact integer steps
-      for (int i = 1; i <= nn; ++i) b = b * (kk - nn + i) / i;
-      float sc = (float)b;
-      for (int i = 0; i < nn; ++i) sc = __fmul_rn(sc, inv_q);
+  // cb[n][kk] = Q^-n binom(kk, n) c_kk.
+  for (int t = tid; t < K2 * IP_KMAX; t += nt) {
+    const int nn = t / IP_KMAX, kk = t % IP_KMAX;
+    if (kk < ig.K) {
       const float2 c = a.coef[rc * ig.K + kk];
-      v = make_float2(__fmul_rn(c.x, sc), __fmul_rn(c.y, sc));
+      const float sc = sc_s[nn * IP_CB_STRIDE + kk];
+      cb_s[nn * IP_CB_STRIDE + kk] =
+          kk >= 1 ? make_float2(__fmul_rn(c.x, sc), __fmul_rn(c.y, sc)) : make_float2(0.f, 0.f);
     }
-    cb_s[nn * IP_CB_STRIDE + kk] = v;
   }
   __syncthreads();
-  const int n_near = blk_off[9];
-  for (int t = tid; t < n_near; t += blockDim.x) {
+  const int n_near = __shfl_sync(0xFFFFFFFFu, blk_off[9], 0);
+  const bool near_fits = n_near <= a.near_cap;
+  // lens t of the block relative to the cell's centre
+  auto near_lens = [&](int t) {
     int q = 0;
-    while (q < 8 && t >= blk_off[q + 1]) ++q;
-    const float4 v = a.rel[blk_start[q] + (t - blk_off[q])];
-    const float ox = __fmul_rn((float)((q % 3) - 1), hf), oy = __fmul_rn((float)((q / 3) - 1), hf);
-    const float x = __fadd_rn(v.x, ox), y = __fadd_rn(v.y, oy);
-    nxy_s[t] = make_float4(-x, -x, -y, -y);
-    nm_s[t] = make_float2(-v.z, -v.z);
-  }
+#pragma unroll
+    for (int i = 1; i < 9; ++i) q += t >= blk_off[i] ? 1 : 0;
+    float4 v = a.rel[blk_start[q] + (t - blk_off[q])];
+    v.x = __fadd_rn(v.x, __fmul_rn((float)((q % 3) - 1), hf));
+    v.y = __fadd_rn(v.y, __fmul_rn((float)((q / 3) - 1), hf));
+    return v;
+  };
+  // this thread's first lens is in flight during the re-centring
+  float4 lens0 = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (near_fits && tid < n_near) lens0 = near_lens(tid);
   // then per (sub-cell, n) the polynomial sum_j cb[n][n + j] eps^j by Horner,
   // two sub-cells of one sub-cell row at a time (Q is even) through packed
-  // FP32x2 instructions: the same roundings as two scalar Horner chains
+  // FP32x2 instructions: the same roundings as two scalar Horner chains.  A
+  // thread runs IP_RC of these chains at once.
   static_assert(Q % 2 == 0, "sub-cells go in pairs along a row");
-  for (int t = tid; t < Q * Q * K2 / 2; t += blockDim.x) {
-    const int sp = t / K2, nn = t % K2;
-    const int sa = 2 * sp;  // sub-cells sa, sa + 1: same row, adjacent columns
-    const float er_a = __fmaf_rn(__fadd_rn((float)(sa % Q), 0.5f), inv_q, -0.5f);
-    const float er_b = __fmaf_rn(__fadd_rn((float)(sa % Q + 1), 0.5f), inv_q, -0.5f);
-    const float ei = __fmaf_rn(__fadd_rn((float)(sa / Q), 0.5f), inv_q, -0.5f);
-    const float2 ER = make_float2(er_a, er_b), EI = make_float2(ei, ei), NEI = make_float2(-ei, -ei);
+  constexpr int NPAIR = Q * Q / 2;
+  constexpr int NB = (NPAIR + IP_RC - 1) / IP_RC;  // batches of pairs per n
+  const float inv_q = __fdiv_rn(1.0f, (float)Q);
+  for (int t = tid; t < NB * K2; t += nt) {
+    const int nn = t / NB, b = t - nn * NB;
+    float2 ER[IP_RC], EI[IP_RC], NEI[IP_RC], SR[IP_RC], SI[IP_RC];
+#pragma unroll
+    for (int i = 0; i < IP_RC; ++i) {
+      const int sa = 2 * min(b + i * NB, NPAIR - 1);  // sub-cells sa, sa + 1: same row, adjacent columns
+      ER[i] = make_float2(__fmaf_rn(__fadd_rn((float)(sa % Q), 0.5f), inv_q, -0.5f),
+                          __fmaf_rn(__fadd_rn((float)(sa % Q + 1), 0.5f), inv_q, -0.5f));
+      const float ei = __fmaf_rn(__fadd_rn((float)(sa / Q), 0.5f), inv_q, -0.5f);
+      EI[i] = make_float2(ei, ei);
+      NEI[i] = make_float2(-ei, -ei);
+      SR[i] = SI[i] = make_float2(0.f, 0.f);
+    }
     const float2* cb = cb_s + nn * IP_CB_STRIDE;
-    float2 SR = make_float2(0.f, 0.f), SI = make_float2(0.f, 0.f);
 #pragma unroll 2
     for (int kk = ig.K - 1; kk >= nn; --kk) {
       const float2 c = cb[kk];
-      const float2 NR = __ffma2_rn(SR, ER, __ffma2_rn(SI, NEI, make_float2(c.x, c.x)));
-      SI = __ffma2_rn(SR, EI, __ffma2_rn(SI, ER, make_float2(c.y, c.y)));
-      SR = NR;
-    }
-    sub_s[sa * K2 + nn] = make_float4(SR.x, SR.x, -SI.x, -SI.x);
-    sub_s[(sa + 1) * K2 + nn] = make_float4(SR.y, SR.y, -SI.y, -SI.y);
-  }
-  // row table: t_y = tau_y h, sigma_y = (l + 1/2) Q / k - v - 1/2, v Q, rows of
-  // the whole cell side in pairs and R / 2 pairs past it (rows past the cell
-  // side are never binned; their sub-cell row is clamped to Q - 1)
-  static_assert(R <= 2 * IP_ROW_PAD, "row table padding");
-  const int npair_cell = (int)((k + 1) >> 1) + R / 2;
-  for (int pr = tid; pr < npair_cell; pr += blockDim.x) {
-    float tyv[2], sg[2], y0[2];
-    int vq[2];
 #pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      const int l = 2 * pr + j;
-      const float sv = __fmul_rn(__fadd_rn((float)l, 0.5f), __fmul_rn((float)Q, inv_k));
-      const int v = min(__float2int_rd(sv), Q - 1);
-      tyv[j] = __fmul_rn(fmaf((float)l, inv_k, fmaf(0.5f, inv_k, -0.5f)), hf);
-      y0[j] = __fmaf_rn(g.lam_s2, tyv[j], rec_s.by_lo);
-      sg[j] = __fsub_rn(__fsub_rn(sv, (float)v), 0.5f);
-      vq[j] = v * Q;
+      for (int i = 0; i < IP_RC; ++i) {
+        const float2 NR = __ffma2_rn(SR[i], ER[i], __ffma2_rn(SI[i], NEI[i], make_float2(c.x, c.x)));
+        SI[i] = __ffma2_rn(SR[i], EI[i], __ffma2_rn(SI[i], ER[i], make_float2(c.y, c.y)));
+        SR[i] = NR;
+      }
     }
-    row_s[pr].sg = make_float4(sg[0], sg[1], -sg[0], -sg[1]);
-    row_s[pr].ty = make_float4(tyv[0], tyv[1], y0[0], y0[1]);
-    row_s[pr].v = make_int2(vq[0], vq[1]);
+#pragma unroll
+    for (int i = 0; i < IP_RC; ++i) {
+      const int sp = b + i * NB;
+      if (NPAIR % IP_RC == 0 || sp < NPAIR) {
+        sub_s[(2 * sp) * ip_sub_stride(K2) + nn] = make_float4(SR[i].x, SR[i].x, -SI[i].x, -SI[i].x);
+        sub_s[(2 * sp + 1) * ip_sub_stride(K2) + nn] = make_float4(SR[i].y, SR[i].y, -SI[i].y, -SI[i].y);
+      }
+    }
   }
-  // privatised binning: the cell's pixel box [hx0, hx0 + hbx) x [hy0, hy0 + hby)
-  // around the centre's pixel offset (relative to the base pixel; no box when
-  // it exceeds the sub-histogram) and its bins cleared; lhx, lhy turn a ray's
-  // floor bit pattern into its box column and row
-  int32_t hx0 = 0, hy0 = 0, hbx = 0, hby = 0;
-  uint32_t lhx = 0, lhy = 0;
-  if (BIN == 2 && MODE == IP_MAP) {
-    const float cx_pix = __fmul_rn(rec_s.bx_hi, g.inv_sx), cy_pix = __fmul_rn(rec_s.by_hi, g.inv_sy);
-    hx0 = __float2int_rd(__fsub_rn(cx_pix, ig.box_hx));
-    hy0 = __float2int_rd(__fsub_rn(cy_pix, ig.box_hy));
-    hbx = __float2int_rd(__fadd_rn(cx_pix, ig.box_hx)) - hx0 + 1;
-    hby = __float2int_rd(__fadd_rn(cy_pix, ig.box_hy)) - hy0 + 1;
-    if (hbx * hby > IP_HIST_MAX) hbx = hby = 0;
-    lhx = (uint32_t)0u - PIX_MAGIC_BITS - (uint32_t)hx0;
-    lhy = (uint32_t)0u - PIX_MAGIC_BITS - (uint32_t)hy0;
-    for (int t = tid; t < hbx * hby; t += blockDim.x) hist_s[t] = 0u;
+  // the rows' shares of beta
+  for (int pr = tid; pr < ig.nrow; pr += nt) {
+    float4 t = row_s[pr].ty;
+    t.z = __fmaf_rn(g.lam_s2, t.x, rec_s.by_lo);
+    t.w = __fmaf_rn(g.lam_s2, t.y, rec_s.by_lo);
+    row_s[pr].ty = t;
+  }
+  if (near_fits) {
+    if (tid < n_near) {
+      near_s[tid].xy = make_float4(-lens0.x, -lens0.x, -lens0.y, -lens0.y);
+      near_s[tid].m = make_float2(-lens0.z, -lens0.z);
+    }
+    for (int t = tid + nt; t < n_near; t += nt) {
+      const float4 v = near_lens(t);
+      near_s[t].xy = make_float4(-v.x, -v.x, -v.y, -v.y);
+      near_s[t].m = make_float2(-v.z, -v.z);
+    }
   }
   __syncthreads();
 
   // base pixel of this cell for the 32-bit pixel test, folded with the
   // floor's bit pattern offset (pixel_keys2)
   const int32_t rix = rec_s.ix, riy = rec_s.iy;
-  const uint32_t rbx = (uint32_t)rix - PIX_MAGIC_BITS, rby = (uint32_t)riy - PIX_MAGIC_BITS;
   // the cell centre's beta (hi parts) in pixel units
   const float bxs = __fmul_rn(rec_s.bx_hi, g.inv_sx), bys = __fmul_rn(rec_s.by_hi, g.inv_sy);
-
-  const int n_corner = rec_s.n_corner;
-  const unsigned lane_lt = (1u << lane) - 1u;
-  // cell-local 32-bit lattice indices: columns [0, kx), rows [ylo, yhi); units
-  // start on an even row so that row pairs line up with the table
-  const int kx = (int)(i1 - i0), ylo = (int)(jlo - j0), yhi = (int)(jhi - j0);
-  const int ylo2 = ylo & ~1;
-  const float c_tau = fmaf(0.5f, inv_k, -0.5f);  // tau = (l + 1/2)/k - 1/2
-  const float qk = __fmul_rn((float)Q, inv_k);   // sub-cell index = floor((l + 1/2) Q / k)
+  const float2 BXS = make_float2(bxs, bxs), BYS = make_float2(bys, bys);
+  const float2 ISX = make_float2(g.inv_sx, g.inv_sx), ISY = make_float2(g.inv_sy, g.inv_sy);
+  const int n_corner = __shfl_sync(0xFFFFFFFFu, rec_s.n_corner, 0);
+  const int corner = n_corner ? -1 : 0;  // cells with sheet corners take the general path of the tail
   const float fnan = __int_as_float(0x7fffffff);
-  // work units (32-column strip x R-row group), dealt round-robin to warps
-  const int nwarps = blockDim.x / 32;
-  const int nstrip = (kx + 31) / 32;
-  const int nrg = (yhi - ylo2 + R - 1) / R;
-  const int nunit = nstrip * nrg;
-  // (strip, row group) of the warp's first unit, then stepped by nwarps units
-  // at a time: no integer division per unit
-  int st = warp % nstrip, rg = warp / nstrip;
-  for (int unit = warp; unit < nunit; unit += nwarps, step_unit(st, rg, nwarps, nstrip)) {
-    const int cl = st * 32 + lane;
-    const int rl0 = ylo2 + rg * R;
-    const int p0 = rl0 >> 1;
-    const float su = __fmul_rn(__fadd_rn((float)cl, 0.5f), qk);
-    const int u = min(__float2int_rd(su), Q - 1);
-    const float sgr = __fsub_rn(__fsub_rn(su, (float)u), 0.5f);
-    // rays outside the cell's columns get a NaN x, rays outside its rows a NaN
-    // y accumulator: both reach beta whatever the near sum does and fail the
-    // pixel test
-    const float tx = cl < kx ? __fmul_rn(fmaf((float)cl, inv_k, c_tau), hf) : fnan;
-    const float x0 = __fmaf_rn(g.lam_s1, tx, rec_s.bx_lo);  // the column's share of beta_1
-    const float2 TX = make_float2(tx, tx), SGR = make_float2(sgr, sgr), X0 = make_float2(x0, x0);
-    float2 TY[R / 2], NAX[R / 2], NAY[R / 2];
-#pragma unroll
-    for (int i = 0; i < R / 2; ++i) {
-      const float4 t = row_s[p0 + i].ty;
-      TY[i] = make_float2(t.x, t.y);
-      NAX[i] = make_float2(0.f, 0.f);
-      NAY[i] = make_float2(0.f, 0.f);
-    }
-    if (rl0 < ylo || rl0 + R > yhi) {  // a group at the band's edge (uniform over the warp)
-#pragma unroll
-      for (int i = 0; i < R / 2; ++i) {
-        const int ra = rl0 + 2 * i;
-        NAY[i] = make_float2(ra >= ylo && ra < yhi ? 0.f : fnan, ra + 1 < yhi ? 0.f : fnan);
-      }
-    }
-#pragma unroll 2
-    for (int q = 0; q < n_near; ++q) {
-      const float4 Lq = nxy_s[q];
-      const float2 NM = nm_s[q];
-      const float2 DX = __fadd2_rn(TX, make_float2(Lq.x, Lq.y));
-      const float2 DX2 = __fmul2_rn(DX, DX);
-      const float2 NLY = make_float2(Lq.z, Lq.w);
-#pragma unroll
-      for (int i = 0; i < R / 2; ++i) {
-        const float2 DY = __fadd2_rn(TY[i], NLY);
-        const float2 R2 = __ffma2_rn(DY, DY, DX2);
-        float2 W;
-        if (i < NPR) {  // -m/r_a^2 = -m r_b^2 / (r_a^2 r_b^2), and the same for b
-          const float mi = NM.x * rcp_approx(R2.x * R2.y);
-          W = __fmul2_rn(make_float2(R2.y, R2.x), make_float2(mi, mi));
-        } else {
-          W = __fmul2_rn(NM, make_float2(rcp_approx(R2.x), rcp_approx(R2.y)));
-        }
-        NAX[i] = __ffma2_rn(W, DX, NAX[i]);
-        NAY[i] = __ffma2_rn(W, DY, NAY[i]);
-      }
-    }
-    // tail in groups of HP row pairs: level-2 series (conj, in sigma), sheet
-    // corners, beta and pixel keys, binning; the chains of a group interleave
-    constexpr int HP = R / 2 < 2 ? R / 2 : 2;
-#pragma unroll
-    for (int h = 0; h < R / 2; h += HP) {
-      float2 QR[HP], QI[HP];
+  const float ulp0 = __uint_as_float(1u);  // the smallest denormal, 2^-149
+  const float2 ULP = make_float2(ulp0, ulp0);
+  const float hist_f = __uint_as_float((uint32_t)__cvta_generic_to_shared(hist_s));
+  const float c_tau = fmaf(0.5f, ig.inv_k, -0.5f);  // tau = (l + 1/2)/k - 1/2
+  const float qk = __fmul_rn((float)Q, ig.inv_k);   // sub-cell index = floor((l + 1/2) Q / k)
+  // blocks of the cell that map into about one box each; nearly always the
+  // whole cell
+  for (int g0 = grg0; g0 < nrg; g0 += ig.blk_rg) {
+    for (int c0 = 0; c0 < kx; c0 += ig.blk_col) {
+      const int w = min(ig.blk_col, kx - c0), ng = min(ig.blk_rg, nrg - g0);
+      // box origin: the block centre's beta under the mean lens map plus the
+      // near lenses' pull on it (softened), the same in every warp
+      int box_x, box_y;
       {
-        float4 SG[HP];  // (sigma_y, -sigma_y) of the pair
-        int va[HP];
-        bool aligned = true;  // no pair straddles a sub-cell row: uniform over the warp
-#pragma unroll
-        for (int i = 0; i < HP; ++i) {
-          SG[i] = row_s[p0 + h + i].sg;
-          const int2 v = row_s[p0 + h + i].v;
-          va[i] = (v.x + u) * K2;
-          aligned = aligned && (v.x == v.y);
-        }
-        if (aligned) {
-#pragma unroll
-          for (int i = 0; i < HP; ++i) {
-            const float4 dl = sub_s[va[i] + K2 - 1];
-            QR[i] = make_float2(dl.x, dl.y);
-            QI[i] = make_float2(dl.z, dl.w);
+        const float fx = w == k ? 0.f : ((float)c0 + 0.5f * (float)w) * ig.inv_k - 0.5f;
+        const float fy = ng * R >= k ? 0.f : ((float)(ylo2 + g0 * R) + 0.5f * (float)(ng * R)) * ig.inv_k - 0.5f;
+        float sx = 0.f, sy = 0.f;
+        const float eps = 0.15f * hf * hf;
+        if (near_fits)
+          for (int t = lane; t < n_near; t += 32) {
+            const float4 v = near_s[t].xy;
+            const float x = fx * hf + v.x, y = fy * hf + v.z;
+            const float wgt = near_s[t].m.x / (x * x + y * y + eps);
+            sx += wgt * x;
+            sy += wgt * y;
           }
 #pragma unroll
-          for (int nn = K2 - 2; nn >= 0; --nn) {
+        for (int d = 16; d; d >>= 1) {
+          sx += __shfl_xor_sync(0xFFFFFFFFu, sx, d);
+          sy += __shfl_xor_sync(0xFFFFFFFFu, sy, d);
+        }
+        const float ox = (rec_s.bx_hi + sx) * g.inv_sx + fx * ig.cell_px - 0.5f * IP_BOX_W;
+        const float oy = (rec_s.by_hi + sy) * g.inv_sy + fy * ig.cell_py - 0.5f * IP_BOX_H;
+        box_x = (int)fminf(fmaxf(ox, -1048576.f), 1048576.f);
+        box_y = (int)fminf(fmaxf(oy, -1048576.f), 1048576.f);
+      }
+      // A ray's bin: floor(T) - box in units of the smallest denormal, whose
+      // bit pattern is that integer when it is not negative.  One packed
+      // multiply-add rounded toward -inf does both rays of a pair exactly; a
+      // negative, infinite or NaN value has a pattern above every bin.  Two
+      // more give the shared-memory addresses of the bins (their sums stay
+      // below 2^23 units, hence exact).
+      float mgx = -(float)box_x * ulp0, mgy = -(float)box_y * ulp0;
+      asm volatile("" : "+f"(mgx), "+f"(mgy));  // kept, not converted again for every group
+      const float2 MGX = make_float2(mgx, mgx), MGY = make_float2(mgy, mgy);
+      const float2 HA = make_float2(hist_f, hist_f);
+
+      // strips of 32 columns, walked down their row groups by the warps in
+      // turn; in a last strip of w <= 16 columns the lanes take 32 / w row
+      // groups at once
+      int ru = warp;
+      for (int cs = 0; cs < w; cs += 32) {
+        const int ws = min(32, w - cs), par = 32 / ws, nru = (ng + par - 1) / par;
+        if (ru >= nru) {
+          ru -= nru;
+          continue;
+        }
+        const int sub = lane / ws, c = c0 + cs + lane - sub * ws;
+        const bool lane_on = sub < par;
+        const float su = __fmul_rn(__fadd_rn((float)c, 0.5f), qk);
+        const int u = min(__float2int_rd(su), Q - 1);
+        const float sgx = __fsub_rn(__fsub_rn(su, (float)u), 0.5f);
+        const float tx = __fmul_rn(fmaf((float)c, ig.inv_k, c_tau), hf);
+        const float x0 = __fmaf_rn(g.lam_s1, tx, rec_s.bx_lo);  // the column's share of beta_1
+        const float2 TX = make_float2(tx, tx), X0 = make_float2(x0, x0), SGR = make_float2(sgx, sgx);
+        const char* sub_u = reinterpret_cast<const char*>(sub_s) + u * SUB;
+#pragma unroll 1
+        for (; ru < nru; ru += nt >> 5) {
+        const int rg = ru * par + sub;
+        const bool live = lane_on && rg < ng;
+        const int rl0 = ylo2 + (g0 + min(rg, ng - 1)) * R;
+        const IpRowPair* rows = row_s + (rl0 >> 1);
+        float2 TY[R / 2], NAX[R / 2], NAY[R / 2];
 #pragma unroll
-            for (int i = 0; i < HP; ++i) {
-              const float4 dn = sub_s[va[i] + nn];
-              const float2 sgi = make_float2(SG[i].x, SG[i].y), nsgi = make_float2(SG[i].z, SG[i].w);
-              const float2 t1 = __ffma2_rn(QI[i], sgi, make_float2(dn.x, dn.y));
-              const float2 t2 = __ffma2_rn(QI[i], SGR, make_float2(dn.z, dn.w));
-              const float2 nr = __ffma2_rn(QR[i], SGR, t1);
-              QI[i] = __ffma2_rn(QR[i], nsgi, t2);
-              QR[i] = nr;
+        for (int i = 0; i < R / 2; ++i) TY[i] = *reinterpret_cast<const float2*>(&rows[i].ty);
+        // FIRST: the accumulators start from this lens (0 + w d is w d)
+        auto near_step = [&](auto first, float2 NLX, float2 NLY, float2 NM) {
+          const float2 DX = __fadd2_rn(TX, NLX);
+          const float2 DX2 = __fmul2_rn(DX, DX);
+#pragma unroll
+          for (int i = 0; i < R / 2; ++i) {
+            const float2 DY = __fadd2_rn(TY[i], NLY);
+            const float2 R2 = __ffma2_rn(DY, DY, DX2);
+            float2 W;
+            if (i < NPR) {  // -m/r_a^2 = -m r_b^2 / (r_a^2 r_b^2), and the same for b
+              const float mi = NM.x * rcp_approx(R2.x * R2.y);
+              W = __fmul2_rn(make_float2(R2.y, R2.x), make_float2(mi, mi));
+            } else {
+              W = __fmul2_rn(NM, make_float2(rcp_approx(R2.x), rcp_approx(R2.y)));
+            }
+            NAX[i] = first ? __fmul2_rn(W, DX) : __ffma2_rn(W, DX, NAX[i]);
+            NAY[i] = first ? __fmul2_rn(W, DY) : __ffma2_rn(W, DY, NAY[i]);
+          }
+        };
+        if (n_near == 0 || !near_fits) {
+#pragma unroll
+          for (int i = 0; i < R / 2; ++i) NAX[i] = NAY[i] = make_float2(0.f, 0.f);
+        }
+        if (near_fits) {
+          if (n_near > 0)
+            near_step(std::true_type{}, make_float2(near_s[0].xy.x, near_s[0].xy.y),
+                      make_float2(near_s[0].xy.z, near_s[0].xy.w), near_s[0].m);
+#pragma unroll 2
+          for (int q = 1; q < n_near; ++q) {
+            const float4 v = near_s[q].xy;
+            near_step(std::false_type{}, make_float2(v.x, v.y), make_float2(v.z, v.w), near_s[q].m);
+          }
+        } else {  // more lenses than the shared buffer holds: straight from memory
+#pragma unroll 1
+          for (int q = 0; q < n_near; ++q) {
+            const float4 v = near_lens(q);
+            near_step(std::false_type{}, make_float2(-v.x, -v.x), make_float2(-v.y, -v.y), make_float2(-v.z, -v.z));
+          }
+        }
+        // a group at the band's edge, the first or the last: rays outside its
+        // rows get a NaN, which reaches beta and fails the pixel test
+        if (ru == 0 || ru == nru - 1) {
+#pragma unroll
+          for (int i = 0; i < R / 2; ++i) {
+            const int ra = rl0 + 2 * i;
+            NAY[i].x = ra >= ylo && ra < yhi ? NAY[i].x : fnan;
+            NAY[i].y = ra + 1 < yhi ? NAY[i].y : fnan;
+          }
+        }
+        // tail in groups of two row pairs: level-2 series (conj, in sigma),
+        // sheet corners, beta and its bin; the chains of a group interleave
+#pragma unroll
+        for (int h = 0; h < R / 2; h += 2) {
+          float2 QR[2], QI[2];
+          const float4 sga = rows[h].sg, sgb = rows[h + 1].sg;
+          const float2 SG[2] = {make_float2(sga.x, sga.y), make_float2(sgb.x, sgb.y)};
+          const float2 NSG[2] = {make_float2(sga.z, sga.w), make_float2(sgb.z, sgb.w)};
+          const int q4 = rows[h].q4 | corner;
+          if (__all_sync(0xFFFFFFFFu, q4 >= 0)) {  // four rows of one level-2 row
+            const float4* sp = reinterpret_cast<const float4*>(sub_u + q4);
+            const float4 dl = sp[K2 - 1];
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+              QR[i] = make_float2(dl.x, dl.y);
+              QI[i] = make_float2(dl.z, dl.w);
+            }
+#pragma unroll
+            for (int nn = K2 - 2; nn >= 0; --nn) {
+              const float4 dn = sp[nn];
+#pragma unroll
+              for (int i = 0; i < 2; ++i) {
+                const float2 t1 = __ffma2_rn(QI[i], SG[i], make_float2(dn.x, dn.y));
+                const float2 t2 = __ffma2_rn(QI[i], SGR, make_float2(dn.z, dn.w));
+                const float2 nr = __ffma2_rn(QR[i], SGR, t1);
+                QI[i] = __ffma2_rn(QR[i], NSG[i], t2);
+                QR[i] = nr;
+              }
+            }
+          } else {
+            const float4 *ea[2], *eb[2];
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+              ea[i] = reinterpret_cast<const float4*>(sub_u + rows[h + i].v[0] * SUB);
+              eb[i] = reinterpret_cast<const float4*>(sub_u + rows[h + i].v[1] * SUB);
+              QR[i] = make_float2(ea[i][K2 - 1].x, eb[i][K2 - 1].x);
+              QI[i] = make_float2(ea[i][K2 - 1].z, eb[i][K2 - 1].z);
+            }
+#pragma unroll
+            for (int nn = K2 - 2; nn >= 0; --nn) {
+#pragma unroll
+              for (int i = 0; i < 2; ++i) {
+                const float4 xa = ea[i][nn], xb = eb[i][nn];
+                const float2 t1 = __ffma2_rn(QI[i], SG[i], make_float2(xa.x, xb.x));
+                const float2 t2 = __ffma2_rn(QI[i], SGR, make_float2(xa.z, xb.z));
+                const float2 nr = __ffma2_rn(QR[i], SGR, t1);
+                QI[i] = __ffma2_rn(QR[i], NSG[i], t2);
+                QR[i] = nr;
+              }
+            }
+            if (n_corner) {  // corners of the sheet near this cell, per ray (uniform over the CTA)
+#pragma unroll
+              for (int i = 0; i < 2; ++i) {
+                float qr[2] = {QR[i].x, QR[i].y}, qi[2] = {QI[i].x, QI[i].y};
+                const float4 t = rows[h + i].ty;
+                const float tyr[2] = {t.x, t.y};
+#pragma unroll
+                for (int j = 0; j < 2; ++j)
+                  for (int c = 0; c < n_corner; ++c) sheet_corner_ray(rec_s.corner[c], tx, tyr[j], qr[j], qi[j]);
+                QR[i] = make_float2(qr[0], qr[1]);
+                QI[i] = make_float2(qi[0], qi[1]);
+              }
             }
           }
-        } else {
-          int vb[HP];
+          // beta relative to the base pixel, (by_hi, by_hi) + ((x0, y0) + L_local -
+          // alpha_near), in pixel units
+          float2 T1[2], T2[2], U[2], V[2];
 #pragma unroll
-          for (int i = 0; i < HP; ++i) vb[i] = (row_s[p0 + h + i].v.y + u) * K2;
-#pragma unroll
-          for (int i = 0; i < HP; ++i) {
-            const float4 ea = sub_s[va[i] + K2 - 1], eb = sub_s[vb[i] + K2 - 1];
-            QR[i] = make_float2(ea.x, eb.x);
-            QI[i] = make_float2(ea.z, eb.z);
+          for (int i = 0; i < 2; ++i) {
+            const float2 y0 = *(reinterpret_cast<const float2*>(&rows[h + i].ty) + 1);
+            const float2 SX = __fadd2_rn(X0, __fadd2_rn(NAX[h + i], QR[i]));
+            const float2 SY = __fadd2_rn(y0, __fadd2_rn(NAY[h + i], QI[i]));
+            T1[i] = __ffma2_rn(SX, ISX, BXS);
+            T2[i] = __ffma2_rn(SY, ISY, BYS);
+            U[i] = __ffma2_rd(T1[i], ULP, MGX);
+            V[i] = __ffma2_rd(T2[i], ULP, MGY);
           }
+          const uint32_t ux = __float_as_uint(U[0].x) | __float_as_uint(U[0].y) | __float_as_uint(U[1].x) |
+                              __float_as_uint(U[1].y);
+          const uint32_t uy = __float_as_uint(V[0].x) | __float_as_uint(V[0].y) | __float_as_uint(V[1].x) |
+                              __float_as_uint(V[1].y);
+          if (!__any_sync(0xFFFFFFFFu, live && (ux >= (uint32_t)IP_BOX_W || uy >= (uint32_t)IP_BOX_H))) {
+            uint32_t ad[4];
 #pragma unroll
-          for (int nn = K2 - 2; nn >= 0; --nn) {
+            for (int i = 0; i < 2; ++i) {
+              const float2 A = __ffma2_rn(V[i], make_float2(4.f * IP_HS, 4.f * IP_HS),
+                                          __ffma2_rn(U[i], make_float2(4.f, 4.f), HA));
+              ad[2 * i] = __float_as_uint(A.x);
+              ad[2 * i + 1] = __float_as_uint(A.y);
+            }
+            shared_inc4(ad[0], ad[1], ad[2], ad[3], live);
+          } else if (live) {  // some ray of the warp outside the box: each on its own
 #pragma unroll
-            for (int i = 0; i < HP; ++i) {
-              const float4 ea = sub_s[va[i] + nn], eb = sub_s[vb[i] + nn];
-              const float2 sgi = make_float2(SG[i].x, SG[i].y), nsgi = make_float2(SG[i].z, SG[i].w);
-              const float2 t1 = __ffma2_rn(QI[i], sgi, make_float2(ea.x, eb.x));
-              const float2 t2 = __ffma2_rn(QI[i], SGR, make_float2(ea.z, eb.z));
-              const float2 nr = __ffma2_rn(QR[i], SGR, t1);
-              QI[i] = __ffma2_rn(QR[i], nsgi, t2);
-              QR[i] = nr;
+            for (int i = 0; i < 2; ++i) {
+              uint32_t key[2];
+              pixel_keys2(T1[i], T2[i], (uint32_t)rix - PIX_MAGIC_BITS, (uint32_t)riy - PIX_MAGIC_BITS,
+                          (uint32_t)g.npix_x, (uint32_t)g.npix_y, key[0], key[1]);
+#pragma unroll
+              for (int j = 0; j < 2; ++j) {
+                const uint32_t u = __float_as_uint(j ? U[i].y : U[i].x), v = __float_as_uint(j ? V[i].y : V[i].x);
+                if (u < (uint32_t)IP_BOX_W && v < (uint32_t)IP_BOX_H)
+                  atomicAdd(hist_s + v * IP_HS + u, 1u);
+                else if (key[j] != 0xFFFFFFFFu)
+                  atomicAdd(a.counts + key[j], 1u);
+              }
             }
           }
         }
       }
-      if (n_corner) {  // corners of the sheet near this cell, per ray (uniform over the CTA)
-#pragma unroll
-        for (int i = 0; i < HP; ++i) {
-          float qr[2] = {QR[i].x, QR[i].y}, qi[2] = {QI[i].x, QI[i].y};
-          const float4 t = row_s[p0 + h + i].ty;
-          const float tyr[2] = {t.x, t.y};
-#pragma unroll
-          for (int j = 0; j < 2; ++j) {
-            for (int c = 0; c < n_corner; ++c) {
-              const float wr = __fadd_rn(rec_s.corner[c][0], tx), wi = __fadd_rn(rec_s.corner[c][1], tyr[j]);
-              const float lr = __fmul_rn(0.5f, logf(fmaf(wr, wr, __fmul_rn(wi, wi)))), li = atan2f(wi, wr);
-              const float plr = fmaf(wr, lr, -__fmul_rn(wi, li)), pli = fmaf(wr, li, __fmul_rn(wi, lr));
-              qr[j] = fmaf(rec_s.corner[c][2], pli, qr[j]);
-              qi[j] = fmaf(rec_s.corner[c][2], plr, qi[j]);
-            }
-          }
-          QR[i] = make_float2(qr[0], qr[1]);
-          QI[i] = make_float2(qi[0], qi[1]);
-        }
+        ru -= nru;
       }
-      // beta relative to the base pixel, (by_hi, by_hi) + ((x0, y0) + L_local -
-      // alpha_near), in pixel units, then the pixel key of every ray (~0
-      // where none)
-      uint32_t key[2 * HP], lkey[2 * HP];
-#pragma unroll
-      for (int i = 0; i < HP; ++i) {
-        const float4 t = row_s[p0 + h + i].ty;
-        const float2 y0 = make_float2(t.z, t.w);
-        const float2 SX = __fadd2_rn(X0, __fadd2_rn(NAX[h + i], QR[i]));
-        const float2 SY = __fadd2_rn(y0, __fadd2_rn(NAY[h + i], QI[i]));
-        const float2 T1 = __ffma2_rn(SX, make_float2(g.inv_sx, g.inv_sx), make_float2(bxs, bxs));
-        const float2 T2 = __ffma2_rn(SY, make_float2(g.inv_sy, g.inv_sy), make_float2(bys, bys));
-        if (BIN == 2 && MODE == IP_MAP)
-          pixel_keys2_box(T1, T2, rbx, rby, (uint32_t)g.npix_x, (uint32_t)g.npix_y, lhx, lhy, (uint32_t)hbx,
-                          (uint32_t)hby, key[2 * i], key[2 * i + 1], lkey[2 * i], lkey[2 * i + 1]);
-        else
-          pixel_keys2(T1, T2, rbx, rby, (uint32_t)g.npix_x, (uint32_t)g.npix_y, key[2 * i], key[2 * i + 1]);
-        if (MODE == IP_DUMP) {
-#pragma unroll
-          for (int j = 0; j < 2; ++j) {
-            if (i0 + cl == want_i && j0 + rl0 + 2 * (h + i) + j == want_j) {
-              const double b1 = (double)rec_s.bx_hi + (double)(j ? SX.y : SX.x);
-              const double b2 = (double)rec_s.by_hi + (double)(j ? SY.y : SY.x);
-              a.beta_out[2 * work] = (g.src_x0 + (double)rix * g.sx) + b1;
-              a.beta_out[2 * work + 1] = (g.src_y0 + (double)riy * g.sy) + b2;
-              if (a.pix_out) a.pix_out[work] = key[2 * i + j] != 0xFFFFFFFFu ? (int64_t)key[2 * i + j] : -1;
-            }
+      // flush the box, four bins of a row at a time, and leave it zero; bins
+      // off the map are dropped
+      if (tid == 0) *next_s = next;  // the counter's answer has arrived by now
+      __syncthreads();
+      const int ox = rix + box_x, oy = riy + box_y;
+      for (int t = tid; t < IP_HIST / 2; t += nt) {
+        const uint2 v = reinterpret_cast<const uint2*>(hist_s)[t];
+        if (v.x | v.y) {
+          reinterpret_cast<uint2*>(hist_s)[t] = make_uint2(0u, 0u);
+          const int y = t / (IP_HS / 2), x = 2 * (t - y * (IP_HS / 2));
+          const uint32_t px = (uint32_t)(ox + x), py = (uint32_t)(oy + y), nx = (uint32_t)g.npix_x;
+          if (py < (uint32_t)g.npix_y) {
+            uint32_t* c = a.counts + ((int64_t)py * g.npix_x + (ox + x));
+            if (v.x && px < nx) atomicAdd(c, v.x);
+            if (v.y && px + 1u < nx) atomicAdd(c + 1, v.y);
           }
         }
       }
-      if (MODE == IP_MAP) {
-#pragma unroll
-        if (BIN == 3) {
-#pragma unroll
-          for (int i = 0; i < HP; ++i) bin_warp_pair(a.counts, key[2 * i], key[2 * i + 1], lane_lt);
-        } else {
-#pragma unroll
-          for (int r = 0; r < 2 * HP; ++r) {
-            if (BIN == 2) bin_warp_key_box(a.counts, hist_s, key[r], lkey[r], lane_lt);
-            else if (BIN == 1) bin_warp_runs_key(a.counts, key[r], lane);
-            else bin_warp_key(a.counts, key[r], lane_lt);
-          }
-        }
-      }
-    }
-  }
-  if (BIN == 2 && MODE == IP_MAP && hbx > 0) {
-    // flush the cell's sub-histogram: one global add per non-empty bin (bins
-    // off the map never receive a ray: only on-map keys reach the box)
-    __syncthreads();
-    for (int t = tid; t < hbx * hby; t += blockDim.x) {
-      const uint32_t v = hist_s[t];
-      if (v) {
-        const int by = t / hbx, bx = t - by * hbx;
-        atomicAdd(a.counts + (int64_t)(riy + hy0 + by) * g.npix_x + (rix + hx0 + bx), v);
-      }
+      if (g0 + ng < nrg || c0 + w < kx) __syncthreads();  // another block of this cell
     }
   }
 }
 
-// One map: persistent grid over its ray cells (MAP) or requested rays (DUMP).
-template <int MODE, int R, int Q, int K2, int MINB, int BIN, int NPR>
-__global__ void __launch_bounds__(IP_THREADS, MINB) k_ip_ray(Geo g, IpGeo ig, IpRayArgs a) {
-  for (int64_t work = blockIdx.x; work < a.nwork; work += gridDim.x) {
-    if (MODE == IP_MAP) {
-      ip_cell<IP_MAP, R, Q, K2, BIN, NPR>(g, ig, a, a.rc_base + work, -1, -1, work);
-    } else {
-      const int64_t f = a.idx[work];
-      if (f < 0 || f >= g.nrx * g.nry) {  // not a lattice ray: report it, touch nothing else
-        if (threadIdx.x == 0) {
-          a.beta_out[2 * work] = a.beta_out[2 * work + 1] = nan("");
-          if (a.pix_out) a.pix_out[work] = -1;
-        }
-        continue;
-      }
-      const int64_t wi = f % g.nrx, wj = f / g.nrx;
-      ip_cell<IP_DUMP, R, Q, K2, BIN, NPR>(g, ig, a, (wj / ig.k) * ig.nrcx + wi / ig.k, wi, wj, work);
-    }
+// One map: a persistent grid over its ray cells.  CTAs take cells from a
+// counter: with a fixed share each, the CTAs that the SM's scheduler favours
+// ran out early and left it with 5.3 of 6 warps per scheduler on average.
+template <int Q, int K2, int NPR>
+__global__ void __launch_bounds__(IP_THREADS, 3) k_ip_ray(Geo g, IpGeo ig, IpRayArgs a) {
+  extern __shared__ __align__(16) unsigned char ip_smem[];
+  __shared__ long long next_s;
+  const IpSmem<Q, K2> L(ig.nrow, a.near_cap);
+  ip_tables<Q, K2>(ig, L, ip_smem);
+  __syncthreads();
+  long long next = 0;
+  for (long long work = blockIdx.x; work < a.nwork * a.parts; work = next_s) {
+    if (threadIdx.x == 0) next = (long long)gridDim.x + (long long)atomicAdd(a.queue, 1ull);
+    const unsigned cell = a.parts == 1 ? (unsigned)work : (unsigned)work / (unsigned)a.parts;
+    ip_cell<Q, K2, NPR>(g, ig, a, a.rc_base + cell, (int)((unsigned)work - cell * (unsigned)a.parts), L, ip_smem, next,
+                        &next_s);
   }
 }
 
@@ -1233,103 +1373,242 @@ struct MapDesc {
   int64_t item0;  // index of the map's first item in the concatenated list
 };
 
-template <int R, int Q, int K2, int MINB, int BIN, int NPR>
-__global__ void __launch_bounds__(IP_THREADS, MINB)
+template <int Q, int K2, int NPR>
+__global__ void __launch_bounds__(IP_THREADS, 3)
 k_ip_ray_batch(const MapDesc* __restrict__ maps, int nmaps, int64_t nitems,
-               unsigned long long* __restrict__ queue) {
+               unsigned long long* __restrict__ queue, int near_cap) {
+  extern __shared__ __align__(16) unsigned char ip_smem[];
   __shared__ MapDesc md;
-  __shared__ long long item_s;
-  __shared__ int map_s;
-  if (threadIdx.x == 0) map_s = -1;
-  for (;;) {
-    __syncthreads();  // everyone is done with md / item_s
-    if (threadIdx.x == 0) {
-      const long long it = (long long)atomicAdd(queue, 1ull);
-      item_s = it;
-      if (it < nitems) {
+  __shared__ long long next_s, end_s;  // end_s: one past the loaded map's last item
+  long long next = 0, end = -1;
+  for (long long it = blockIdx.x; it < nitems; it = next_s) {
+    if (it >= end) {  // items of one map are contiguous: reload on change only
+      __syncthreads();  // everyone is done with md and the tables
+      if (threadIdx.x == 0) {
         int lo = 0, hi = nmaps - 1;  // last map with item0 <= it
         while (lo < hi) {
           const int mid = (lo + hi + 1) >> 1;
           if (maps[mid].item0 <= it) lo = mid; else hi = mid - 1;
         }
-        if (lo != map_s) {  // items of one map are contiguous: copy on change only
-          md = maps[lo];
-          map_s = lo;
-        }
+        md = maps[lo];
+        md.a.near_cap = near_cap;
+        end_s = lo + 1 < nmaps ? maps[lo + 1].item0 : nitems;
       }
+      __syncthreads();
+      end = end_s;
+      ip_tables<Q, K2>(md.ig, IpSmem<Q, K2>(md.ig.nrow, near_cap), ip_smem);
+      __syncthreads();
     }
-    __syncthreads();
-    const long long it = item_s;
-    if (it >= nitems) break;
-    ip_cell<IP_MAP, R, Q, K2, BIN, NPR>(md.g, md.ig, md.a, md.a.rc_base + (it - md.item0), -1, -1, it);
+    if (threadIdx.x == 0) next = (long long)gridDim.x + (long long)atomicAdd(queue, 1ull);
+    const IpSmem<Q, K2> L(md.ig.nrow, near_cap);
+    ip_cell<Q, K2, NPR>(md.g, md.ig, md.a, md.a.rc_base + (it - md.item0), 0, L, ip_smem, next, &next_s);
+  }
+}
+
+// Chosen rays (irs_shoot_rays): one thread per ray, the arithmetic of ip_cell
+// for that ray alone -- the same operations in the same order and roundings,
+// so the beta written is the one the map's ray pass bins.  A thread re-centres
+// only its ray's level-2 series and walks its 3x3 block in memory; the form
+// before gave each ray a whole cell's pass (all k^2 rays of it).
+template <int Q, int K2, int NPR>
+__global__ void __launch_bounds__(128) k_ip_dump(Geo g, IpGeo ig, IpRayArgs a) {
+  const int64_t work = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (work >= a.nwork) return;
+  const int64_t f = a.idx[work];
+  if (f < 0 || f >= g.nrx * g.nry) {  // not a lattice ray: report it, touch nothing else
+    a.beta_out[2 * work] = a.beta_out[2 * work + 1] = nan("");
+    if (a.pix_out) a.pix_out[work] = -1;
+    return;
+  }
+  const int64_t wi = f % g.nrx, wj = f / g.nrx;
+  const int rcx = (int)(wi / ig.k), rcy = (int)(wj / ig.k);
+  const int c = (int)(wi - rcx * ig.k), l = (int)(wj - rcy * ig.k);
+  const int64_t rc = (int64_t)rcy * ig.nrcx + rcx;
+  const CellRec& rec = a.recs[rc];
+  const float hf = ig.hf, inv_k = ig.inv_k, qk = __fmul_rn((float)Q, inv_k);
+  auto tau_h = [&](int i) { return __fmul_rn(fmaf((float)i, inv_k, fmaf(0.5f, inv_k, -0.5f)), hf); };
+  const float tx = tau_h(c), ty = tau_h(l);
+  // the row that shares this row's reciprocal, where the variant pairs them:
+  // pairs (2p, 2p + 1) with p mod 4 < NPR
+  const bool paired = ((l >> 1) & (IP_R / 2 - 1)) < NPR;
+  const float typ = tau_h(l ^ 1);
+  float nax = 0.f, nay = 0.f;
+  int left = IP_NEAR_MAX;
+  for (int q = 0; q < 9; ++q) {
+    const int x = rcx + ig.ox + (q % 3) - 1, y = rcy + ig.oy + (q / 3) - 1;
+    if (x < 0 || x >= ig.ncx || y < 0 || y >= ig.ncy) continue;
+    const int64_t s = (int64_t)y * ig.ncx + x;
+    const int b = a.start[s];
+    int e = a.start[s + 1];
+    if (e - b > left) {
+      atomicCAS(a.status, 0, (int)IRS_ERR_OVERFLOW);  // the first error stays
+      e = b + left;
+    }
+    left -= e - b;
+    const float ox = __fmul_rn((float)((q % 3) - 1), hf), oy = __fmul_rn((float)((q / 3) - 1), hf);
+    for (int p = b; p < e; ++p) {
+      const float4 v = a.rel[p];
+      const float dx = __fadd_rn(tx, -__fadd_rn(v.x, ox)), ly = -__fadd_rn(v.y, oy);
+      const float dx2 = __fmul_rn(dx, dx), dy = __fadd_rn(ty, ly);
+      const float r2 = __fmaf_rn(dy, dy, dx2);
+      float wgt;
+      if (NPR > 0 && paired) {
+        const float dyp = __fadd_rn(typ, ly), r2p = __fmaf_rn(dyp, dyp, dx2);
+        wgt = __fmul_rn(r2p, __fmul_rn(-v.z, rcp_approx(__fmul_rn(r2, r2p))));
+      } else {
+        wgt = __fmul_rn(-v.z, rcp_approx(r2));
+      }
+      nax = __fmaf_rn(wgt, dx, nax);
+      nay = __fmaf_rn(wgt, dy, nay);
+    }
+  }
+  // the level-2 series of the ray's sub-cell, then its Horner on the conjugate
+  const float inv_q = __fdiv_rn(1.0f, (float)Q);
+  auto level2 = [&](int i, float& sig) {
+    const float s = __fmul_rn(__fadd_rn((float)i, 0.5f), qk);
+    const int v = min(__float2int_rd(s), Q - 1);
+    sig = __fsub_rn(__fsub_rn(s, (float)v), 0.5f);
+    return v;
+  };
+  float sgx, sgy;
+  const int u = level2(c, sgx), v = level2(l, sgy);
+  const float er = __fmaf_rn(__fadd_rn((float)u, 0.5f), inv_q, -0.5f);
+  const float ei = __fmaf_rn(__fadd_rn((float)v, 0.5f), inv_q, -0.5f);
+  const float2* coef = a.coef + rc * ig.K;
+  float qr = 0.f, qi = 0.f;
+#pragma unroll 1
+  for (int nn = K2 - 1; nn >= 0; --nn) {
+    float sr = 0.f, si = 0.f;
+    for (int kk = ig.K - 1; kk >= nn; --kk) {
+      float2 cc = make_float2(0.f, 0.f);
+      if (kk >= 1) {
+        int b = 1;
+        for (int i = 1; i <= nn; ++i) b = b * (kk - nn + i) / i;
+        float sc = (float)b;
+        for (int i = 0; i < nn; ++i) sc = __fmul_rn(sc, inv_q);
+        cc = make_float2(__fmul_rn(coef[kk].x, sc), __fmul_rn(coef[kk].y, sc));
+      }
+      const float nr = __fmaf_rn(sr, er, __fmaf_rn(si, -ei, cc.x));
+      si = __fmaf_rn(sr, ei, __fmaf_rn(si, er, cc.y));
+      sr = nr;
+    }
+    if (nn == K2 - 1) {
+      qr = sr;
+      qi = -si;
+    } else {
+      const float nr = __fmaf_rn(qr, sgx, __fmaf_rn(qi, sgy, sr));
+      qi = __fmaf_rn(qr, -sgy, __fmaf_rn(qi, sgx, -si));
+      qr = nr;
+    }
+  }
+  for (int n = 0; n < rec.n_corner; ++n) sheet_corner_ray(rec.corner[n], tx, ty, qr, qi);
+  const float x0 = __fmaf_rn(g.lam_s1, tx, rec.bx_lo), y0 = __fmaf_rn(g.lam_s2, ty, rec.by_lo);
+  const float sx = __fadd_rn(x0, __fadd_rn(nax, qr)), sy = __fadd_rn(y0, __fadd_rn(nay, qi));
+  a.beta_out[2 * work] = (g.src_x0 + (double)rec.ix * g.sx) + ((double)rec.bx_hi + (double)sx);
+  a.beta_out[2 * work + 1] = (g.src_y0 + (double)rec.iy * g.sy) + ((double)rec.by_hi + (double)sy);
+  if (a.pix_out) {
+    const float t1 = __fmaf_rn(sx, g.inv_sx, __fmul_rn(rec.bx_hi, g.inv_sx));
+    const float t2 = __fmaf_rn(sy, g.inv_sy, __fmul_rn(rec.by_hi, g.inv_sy));
+    uint32_t ka, kb;
+    pixel_keys2(make_float2(t1, t1), make_float2(t2, t2), (uint32_t)rec.ix - PIX_MAGIC_BITS,
+                (uint32_t)rec.iy - PIX_MAGIC_BITS, (uint32_t)g.npix_x, (uint32_t)g.npix_y, ka, kb);
+    a.pix_out[work] = ka != 0xFFFFFFFFu ? (int64_t)ka : -1;
   }
 }
 
 // Dynamic shared memory above the 48 KB default: set once per instantiation,
 // before any launch or graph capture that uses it.
-#define IP_DECL_ATTR(V, R, Q, K2, MINB, BIN, NPR)                                                           \
-  case V: {                                                                                            \
-    const int b = (int)IpSmem<Q, K2, BIN>::bytes_max;                                                      \
-    e = cudaFuncSetAttribute(k_ip_ray<IP_MAP, R, Q, K2, MINB, BIN, NPR>,                                   \
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, b);                         \
-    if (e == cudaSuccess)                                                                              \
-      e = cudaFuncSetAttribute(k_ip_ray<IP_DUMP, R, Q, K2, MINB, BIN, NPR>,                                \
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, b);                       \
-    if (e == cudaSuccess)                                                                              \
-      e = cudaFuncSetAttribute(k_ip_ray_batch<R, Q, K2, MINB, BIN, NPR>,                                   \
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, b);                       \
-    break;                                                                                             \
-  }
+#define IP_DECL_ATTR(V, Q, K2, NPR)                                                                          \
+  case V:                                                                                                    \
+    e = cudaFuncSetAttribute(k_ip_ray<Q, K2, NPR>, cudaFuncAttributeMaxDynamicSharedMemorySize, IP_SMEM_MAX); \
+    if (e == cudaSuccess)                                                                                    \
+      e = cudaFuncSetAttribute(k_ip_ray_batch<Q, K2, NPR>, cudaFuncAttributeMaxDynamicSharedMemorySize,      \
+                               IP_SMEM_MAX);                                                                 \
+    break;
+constexpr int IP_SMEM_MAX = 160 * 1024;
 cudaError_t ip_ray_attributes(int variant) {
   cudaError_t e = cudaErrorInvalidValue;
-  switch (variant) { IP_VARIANTS(IP_DECL_ATTR) default: break; }
+  switch (ip_kernel_of(variant)) { IP_VARIANTS(IP_DECL_ATTR) default: break; }
   return e;
 }
 
-#define IP_DECL_OCC(V, R, Q, K2, MINB, BIN, NPR)                                                       \
-  case V:                                                                                         \
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_ip_ray<IP_MAP, R, Q, K2, MINB, BIN, NPR>, \
-                                                  IP_THREADS, IpSmem<Q, K2, BIN>::bytes(nrow));        \
-    break;
-// CTAs per SM of a variant whose row table has `nrow` entries
-int ip_ray_occupancy(int variant, int nrow) {
-  int per_sm = 0;
-  switch (variant) { IP_VARIANTS(IP_DECL_OCC) default: break; }
-  return per_sm > 0 ? per_sm : 1;
-}
-
-#define IP_DECL_BYTES(V, R, Q, K2, MINB, BIN, NPR) \
-  case V:                                          \
-    return IpSmem<Q, K2, BIN>::bytes(nrow);
-size_t ip_ray_smem(int variant, int nrow) {
-  switch (variant) { IP_VARIANTS(IP_DECL_BYTES) default: break; }
+#define IP_DECL_BYTES(V, Q, K2, NPR) \
+  case V:                            \
+    return IpSmem<Q, K2>(nrow, near_cap).bytes;
+int ip_ray_smem(int variant, int nrow, int near_cap) {
+  switch (ip_kernel_of(variant)) { IP_VARIANTS(IP_DECL_BYTES) default: break; }
   return 0;
 }
 
-#define IP_DECL_LAUNCH(V, R, Q, K2, MINB, BIN, NPR)                                                           \
-  case V:                                                                                                \
-    if (mode == IP_MAP)                                                                                  \
-      k_ip_ray<IP_MAP, R, Q, K2, MINB, BIN, NPR><<<(unsigned)grid, IP_THREADS, IpSmem<Q, K2, BIN>::bytes(ig.nrow), \
-                                                   s>>>(g, ig, a);                                           \
-    else                                                                                                 \
-      k_ip_ray<IP_DUMP, R, Q, K2, MINB, BIN, NPR><<<(unsigned)grid, IP_THREADS, IpSmem<Q, K2, BIN>::bytes(ig.nrow), \
-                                                    s>>>(g,                                                  \
-                                                                                                 ig, a); \
+// Launch shape of the ray pass: the register budget (80 per thread) holds 24
+// warps per SM, as six CTAs of 128 threads where their shared memory fits and
+// three of 256 otherwise.  Six small CTAs hide each other's per-cell set-up
+// better: 204 against 217 ms at the high-res map (224-ray cells).
+struct IpShape {
+  int threads, grid, smem;
+};
+IpShape ip_launch_shape(int variant, int nrow, int near_cap, int num_sms) {
+  constexpr int SM_BYTES = 228 * 1024, CTA_RESERVED = 1024, STATIC = 256;
+  const int b = ip_ray_smem(variant, nrow, near_cap);
+  int best = 0;
+  IpShape s{};
+  for (int threads : {128, 256}) {
+    const int fit = SM_BYTES / (b + CTA_RESERVED + STATIC), regs = 24 * 32 / threads;
+    const int per_sm = fit < regs ? (fit < 1 ? 1 : fit) : regs;
+    if (per_sm * threads > best) {
+      best = per_sm * threads;
+      s.threads = threads;
+      s.grid = num_sms * per_sm;
+      s.smem = b;
+    }
+  }
+  return s;
+}
+
+// Lenses of a 3x3 block kept in shared memory: the mean of n lenses over the
+// cell grid and six deviations; fuller blocks read theirs from memory.
+int ip_near_cap(const IpGeo& ig, int64_t n) {
+  const double mean = 9.0 * (double)n / ((double)ig.ncx * (double)ig.ncy);
+  double cap = mean + 6.0 * sqrt(mean) + 8.0;
+  if (cap > (double)n) cap = (double)n;
+  int c = cap >= (double)IP_NEAR_MAX ? IP_NEAR_MAX : (int)ceil(cap);
+  c = (c + 15) & ~15;
+  return c < 16 ? 16 : c;
+}
+
+#define IP_DECL_LAUNCH(V, Q, K2, NPR)                                                             \
+  case V:                                                                                         \
+    k_ip_ray<Q, K2, NPR><<<(unsigned)grid, sh.threads, sh.smem, s>>>(g, ig, a);                     \
     break;
-cudaError_t launch_ip_ray(int variant, int mode, int64_t grid, cudaStream_t s, const Geo& g,
-                          const IpGeo& ig, const IpRayArgs& a) {
-  switch (variant) { IP_VARIANTS(IP_DECL_LAUNCH) default: return cudaErrorInvalidValue; }
+// A map of few cells is cut into more work items, each a share of a cell's row
+// groups (with the cell's set-up of its own), until every CTA slot has two.
+cudaError_t launch_ip_ray(int num_sms, cudaStream_t s, const Geo& g, const IpGeo& ig, IpRayArgs a) {
+  if (a.nwork <= 0) return cudaSuccess;
+  const IpShape sh = ip_launch_shape(ig.variant, ig.nrow, a.near_cap, num_sms);
+  const int64_t want = (2 * (int64_t)sh.grid + a.nwork - 1) / a.nwork, most = (ig.k + 4 * IP_R - 1) / (4 * IP_R);
+  a.parts = (int32_t)(want < most ? want : most);
+  const int64_t items = a.nwork * a.parts, grid = items < sh.grid ? items : sh.grid;
+  switch (ip_kernel_of(ig.variant)) { IP_VARIANTS(IP_DECL_LAUNCH) default: return cudaErrorInvalidValue; }
   return cudaGetLastError();
 }
 
-#define IP_DECL_BATCH(V, R, Q, K2, MINB, BIN, NPR)                                                       \
-  case V:                                                                                           \
-    k_ip_ray_batch<R, Q, K2, MINB, BIN, NPR><<<(unsigned)grid, IP_THREADS, IpSmem<Q, K2, BIN>::bytes(nrow), s>>>( \
-        maps, nmaps, nitems, queue);                                                                \
+#define IP_DECL_DUMP(V, Q, K2, NPR)                                                    \
+  case V:                                                                              \
+    k_ip_dump<Q, K2, NPR><<<(unsigned)((a.nwork + 127) / 128), 128, 0, s>>>(g, ig, a); \
     break;
-cudaError_t launch_ip_ray_batch(int variant, int64_t grid, cudaStream_t s, const MapDesc* maps,
-                                int nmaps, int64_t nitems, unsigned long long* queue, int nrow) {
-  switch (variant) { IP_VARIANTS(IP_DECL_BATCH) default: return cudaErrorInvalidValue; }
+cudaError_t launch_ip_dump(cudaStream_t s, const Geo& g, const IpGeo& ig, const IpRayArgs& a) {
+  switch (ip_kernel_of(ig.variant)) { IP_VARIANTS(IP_DECL_DUMP) default: return cudaErrorInvalidValue; }
+  return cudaGetLastError();
+}
+
+#define IP_DECL_BATCH(V, Q, K2, NPR)                                                                            \
+  case V:                                                                                                       \
+    k_ip_ray_batch<Q, K2, NPR><<<(unsigned)grid, sh.threads, sh.smem, s>>>(maps, nmaps, nitems, queue, near_cap); \
+    break;
+cudaError_t launch_ip_ray_batch(int variant, const IpShape& sh, cudaStream_t s, const MapDesc* maps, int nmaps,
+                                int64_t nitems, unsigned long long* queue, int near_cap) {
+  const int64_t grid = nitems < sh.grid ? nitems : sh.grid;
+  switch (ip_kernel_of(variant)) { IP_VARIANTS(IP_DECL_BATCH) default: return cudaErrorInvalidValue; }
   return cudaGetLastError();
 }
 
@@ -1394,6 +1673,7 @@ irs_status build_cells_and_far(irs_plan_t* P, const double* xy, const double* ma
     if (st != IRS_OK) return st;
   }
   const double2* xy2 = reinterpret_cast<const double2*>(xy);
+  S->n_last = n;
   IP_TRY(cudaMemsetAsync(S->cell_count, 0, sizeof(int32_t) * ncells, s));
   if (n > 0) k_ip_count<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(ig, xy2, n, S->lens_cell, S->cell_count);
   const int64_t nb = (ncells + SCAN_B - 1) / SCAN_B;
@@ -1458,6 +1738,8 @@ IpRayArgs ray_args(irs_plan_t* P) {
   a.recs = S->recs;
   a.coef = S->coef;
   a.status = P->d_status;
+  a.queue = P->d_queue;
+  a.near_cap = ip_near_cap(S->ig, S->n_last);
   return a;
 }
 
@@ -1486,11 +1768,14 @@ irs_status interp_plan(irs_plan_t* P) {
   ig.k = k;
   ig.nrow = (int32_t)((k + 1) / 2) + IP_ROW_PAD;
   ig.h = (double)k * g.dx3;
-  // a cell of side h maps to |1 - kappa -+ gamma| h under the mean lens map
-  // (declared kappa_*); half of that in pixels, grown by half for the far
-  // field's and the near lenses' spread, plus two pixels
-  ig.box_hx = (float)(0.75 * fabs(P->lambda1) * ig.h / g.sx + 2.0);
-  ig.box_hy = (float)(0.75 * fabs(P->lambda2) * ig.h / g.sy + 2.0);
+  // under the mean lens map (declared kappa_*) a cell covers (1 - kappa -+
+  // gamma) h; a block of it is kept to three quarters of a binning box
+  ig.cell_px = (float)(P->lambda1 * ig.h / g.sx);
+  ig.cell_py = (float)(P->lambda2 * ig.h / g.sy);
+  const double bc = 0.75 * IP_BOX_W * (double)k / fabs((double)ig.cell_px);
+  const double br = 0.75 * IP_BOX_H * (double)k / fabs((double)ig.cell_py);
+  ig.blk_col = bc >= (double)k ? (int32_t)k : (bc < 64.0 ? 32 : (int32_t)bc & ~31);
+  ig.blk_rg = br >= (double)k ? (int32_t)k : (br < 16.0 ? 1 : (int32_t)(br / IP_R));
   ig.hf = (float)ig.h;
   ig.inv_k = 1.0f / (float)k;
   ig.nrcx = (int32_t)((g.nrx + k - 1) / k);
@@ -1600,7 +1885,6 @@ irs_status interp_plan(irs_plan_t* P) {
   }
   if (cudaDeviceSynchronize() != cudaSuccess) return IRS_ERR_CUDA;
   if (ip_ray_attributes(ig.variant) != cudaSuccess) return IRS_ERR_CUDA;
-  S->grid_ray = P->num_sms * ip_ray_occupancy(ig.variant, ig.nrow);
   if (p.method == IRS_MLP) {
     if (p.plane != IRS_PLANE_RECT) return IRS_ERR_UNSUPPORTED;
     irs_status st2 = mlp_plan(P, ig.gx0, ig.gy0, ig.h, ig.ncx, ig.ncy, ig.nrcx, ig.nrcy, ig.ox, ig.oy, 1 << 20);
@@ -1647,8 +1931,7 @@ irs_status interp_run(irs_plan_t* P, const double* xy, const double* mass, int64
     a.row1 = row1;
     a.rc_base = rc0;
     a.nwork = rc1 - rc0;
-    const int64_t grid = (rc1 - rc0) < S->grid_ray ? (rc1 - rc0) : S->grid_ray;
-    if (launch_ip_ray(S->ig.variant, IP_MAP, grid, s, P->g, S->ig, a) != cudaSuccess) return IRS_ERR_CUDA;
+    if (launch_ip_ray(P->num_sms, s, P->g, S->ig, a) != cudaSuccess) return IRS_ERR_CUDA;
   }
   mark(P, EV_RAY1, s);
   return IRS_OK;
@@ -1660,7 +1943,6 @@ irs_status interp_set_variant(irs_plan_t* P, int variant) {
   if (ip_ray_attributes(variant) != cudaSuccess) return IRS_ERR_CUDA;
   S->ig.variant = variant;
   P->p.kernel_variant = variant;
-  S->grid_ray = P->num_sms * ip_ray_occupancy(variant, S->ig.nrow);
   return IRS_OK;
 }
 
@@ -1676,9 +1958,9 @@ irs_status interp_raypass_rows(irs_plan_t* P, int64_t row0, int64_t row1, uint32
   a.row1 = row1;
   a.rc_base = rc0;
   a.nwork = rc1 - rc0;
-  const int64_t grid = (rc1 - rc0) < S->grid_ray ? (rc1 - rc0) : S->grid_ray;
+  if (cudaMemsetAsync(P->d_queue, 0, sizeof(unsigned long long), s) != cudaSuccess) return IRS_ERR_CUDA;
   if (cudaEventRecord(e0, s) != cudaSuccess) return IRS_ERR_CUDA;
-  if (launch_ip_ray(S->ig.variant, IP_MAP, grid, s, P->g, S->ig, a) != cudaSuccess) return IRS_ERR_CUDA;
+  if (launch_ip_ray(P->num_sms, s, P->g, S->ig, a) != cudaSuccess) return IRS_ERR_CUDA;
   if (cudaEventRecord(e1, s) != cudaSuccess) return IRS_ERR_CUDA;
   return IRS_OK;
 }
@@ -1694,9 +1976,7 @@ irs_status interp_shoot_rays(irs_plan_t* P, const double* xy, const double* mass
   a.beta_out = beta;
   a.pix_out = pix;
   a.nwork = nidx;
-  const int64_t grid = nidx < S->grid_ray ? nidx : S->grid_ray;
-  return launch_ip_ray(S->ig.variant, IP_DUMP, grid, s, P->g, S->ig, a) == cudaSuccess ? IRS_OK
-                                                                                     : IRS_ERR_CUDA;
+  return launch_ip_dump(s, P->g, S->ig, a) == cudaSuccess ? IRS_OK : IRS_ERR_CUDA;
 }
 
 irs_status interp_ensure_capacity(irs_plan_t* P, int64_t n) {
@@ -1713,7 +1993,9 @@ irs_status interp_prepare(irs_plan_t* P, const double* xy, const double* mass, i
 
 int interp_variant(const irs_plan_t* P) { return S_(P)->ig.variant; }
 int interp_row_entries(const irs_plan_t* P) { return S_(P)->ig.nrow; }
+int interp_near_cap(const irs_plan_t* P, int64_t n) { return ip_near_cap(S_(P)->ig, n); }
 int interp_num_variants() { return IP_NVARIANT; }
+bool interp_variant_distinct(int variant) { return ip_kernel_of(variant) == variant; }
 
 size_t interp_desc_bytes(int nmaps) { return sizeof(MapDesc) * (size_t)(nmaps > 0 ? nmaps : 1); }
 
@@ -1731,6 +2013,7 @@ int64_t interp_fill_descs(irs_plan_t* const* plans, uint32_t* const* counts, int
     d[k].a.row1 = plans[k]->g.nry;
     d[k].a.rc_base = 0;
     d[k].a.nwork = (int64_t)S->ig.nrcx * S->ig.nrcy;
+    d[k].a.parts = 1;
     d[k].item0 = items;
     items += d[k].a.nwork;
   }
@@ -1738,13 +2021,12 @@ int64_t interp_fill_descs(irs_plan_t* const* plans, uint32_t* const* counts, int
 }
 
 irs_status interp_batch_launch(int variant, const void* dev_descs, int nmaps, int64_t nitems,
-                               unsigned long long* queue, int num_sms, int nrow, cudaStream_t s) {
+                               unsigned long long* queue, int num_sms, int nrow, int near_cap, cudaStream_t s) {
   if (nmaps <= 0 || nitems <= 0) return IRS_OK;
-  int64_t grid = (int64_t)num_sms * ip_ray_occupancy(variant, nrow);
-  if (grid > nitems) grid = nitems;
+  const IpShape sh = ip_launch_shape(variant, nrow, near_cap, num_sms);
   if (cudaMemsetAsync(queue, 0, sizeof(unsigned long long), s) != cudaSuccess) return IRS_ERR_CUDA;
-  return launch_ip_ray_batch(variant, grid, s, static_cast<const MapDesc*>(dev_descs), nmaps, nitems,
-                             queue, nrow) == cudaSuccess
+  return launch_ip_ray_batch(variant, sh, s, static_cast<const MapDesc*>(dev_descs), nmaps, nitems, queue,
+                             near_cap) == cudaSuccess
              ? IRS_OK
              : IRS_ERR_CUDA;
 }

@@ -1,0 +1,72 @@
+"""The interpolated ray pass against the chosen-ray path, ray by ray: both run
+the same arithmetic, so the pixels that irs_shoot_rays reports for every ray of
+the lattice must add up to the count map exactly, whatever route the ray pass
+takes for a cell -- last strips of few columns, cells cut into several work
+items or several binning boxes, rays outside the box, row bands that start and
+end inside a row group, blocks of more lenses than the shared buffer holds.
+Both sides are integers from identical roundings: the tolerance is zero."""
+import numpy as np
+import pytest
+
+from paper_2204_10871_gb300 import irs
+from gpu_common import lenses_for, params_pair, require_gpu, to_dev
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+# (kappa_*, kappa_s, gamma, source region, pixels, rays/px, lenses, plane, options)
+ROUTES = {
+    "one row of cells per part": ((0.3, 0.0, 0.3, (-2.5, 2.5, -2.5, 2.5), 64, 4.0), 40, 0, {}),
+    "strips of 1 to 31 columns": ((0.3, 0.1, 0.25, (-2, 3, -2.5, 2.1), (101, 93), 4.0), 900, 0, {"cell_mult": 0.7}),
+    "four rays per cell side": ((0.4, 0.0, 0.1, (-1, 1, -1, 1), 40, 1.0), 20000, 0, {"kernel_variant": 16}),
+    "several boxes per cell": ((0.3, 0.0, 0.2, (-3, 3, -3, 3), (600, 580), 1.0), 150, 0, {"kernel_variant": 14}),
+    "every ray its own pixel": ((0.2, 0.0, -0.2, (-1, 1, -1, 1), (700, 900), 0.25), 60, 0, {"kernel_variant": 1}),
+    "shared reciprocals": ((0.3, 0.0, 0.3, (-2, 2, -2, 2), 64, 9.0), 200, 0, {"kernel_variant": 2}),
+    "circle off the origin": ((0.35, 0.1, 0.25, (-1.5, 2.5, -2.7, 1.3), (61, 67), 6.0), 700, 1, {"kernel_variant": 9}),
+    "no lenses": ((0.2, 0.1, 0.2, (-1.5, 1.5, -1.5, 1.5), 48, 10.25), 0, 0, {"n_star": 60}),
+}
+
+
+def _counts_of(pix, shape):
+    pix = pix[pix >= 0]
+    return np.bincount(pix, minlength=shape[0] * shape[1]).reshape(shape)
+
+
+def _check(torch, pl, plan, dxy, dm):
+    info = plan.info
+    counts, _ = plan.make_map(dxy, dm)
+    _, pix = plan.shoot_rays(dxy, dm, torch.arange(int(info.n_rays), device="cuda"))
+    plan.sync()
+    pix = pix.cpu().numpy()
+    shape = (pl.npix_y, pl.npix_x)
+    assert np.array_equal(counts.cpu().numpy().astype(np.int64), _counts_of(pix, shape))
+    nrx, nry = int(info.n_rays_x), int(info.n_rays_y)
+    for r0, r1 in ((1, 2), (nry // 3, nry // 3 + 13), (nry - 9, nry)):
+        counts.zero_()
+        irs.irs_make_map_rows(plan.handle, dxy, dm, r0, r1, counts)
+        plan.sync()
+        assert np.array_equal(counts.cpu().numpy().astype(np.int64), _counts_of(pix[r0 * nrx:r1 * nrx], shape)), (r0, r1)
+
+
+@pytest.mark.parametrize("route", sorted(ROUTES))
+def test_map_equals_its_rays(route):
+    torch = require_gpu()
+    args, n, plane, kw = ROUTES[route]
+    po, pl = params_pair(*args, plane=plane, method=irs.IRS_INTERP, **{"n_star": n, **kw})
+    qo = oracle.size(po)
+    xy, m = lenses_for(qo, n, shape="uniform", seed=7, kappa_star=args[0], plane=plane)
+    with irs.Plan(pl) as plan:
+        _check(torch, pl, plan, *to_dev(torch, xy, m))
+
+
+def test_a_block_fuller_than_the_shared_buffer():
+    """600 lenses within 0.05 theta_E of each other: their block's lenses are
+    read from memory, every other block's from the shared buffer."""
+    torch = require_gpu()
+    args = (0.3, 0.0, 0.3, (-2.0, 2.0, -2.0, 2.0), 48, 9.0)
+    po, pl = params_pair(*args, method=irs.IRS_INTERP, n_star=900)
+    qo = oracle.size(po)
+    xy, m = lenses_for(qo, 900, shape="equal", seed=3, kappa_star=args[0])
+    xy[:600] = 0.02 + np.random.default_rng(1).uniform(-0.025, 0.025, (600, 2))
+    with irs.Plan(pl) as plan:
+        _check(torch, pl, plan, *to_dev(torch, xy, m))
