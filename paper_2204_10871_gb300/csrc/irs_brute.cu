@@ -215,7 +215,34 @@ cudaError_t launch_brute_setup(const irs_plan_t* P, cudaStream_t s) {
 }
 
 // ------------------------------------------------------------ ray pass
-enum { MODE_MAP = 0, MODE_DUMP = 1 };
+// Source position of a ray relative to its tile's base pixel corner, from its
+// offset (tx, ty) to the tile centre and its lens sums: smooth terms, the
+// sheet's series, corners near the tile.  The rounding of every step is
+// explicit: the map's and the chosen-ray kernels must agree bit for bit.
+__device__ __forceinline__ void brute_beta(const Geo& g, const TileRec& rec, float tx, float ty, float axh, float axl,
+                                           float ayh, float ayl, float& b1, float& b2) {
+  // P(t) = sum_n T_n t^n by Horner, complex FP32
+  float pr = 0.f, pi = 0.f;
+#pragma unroll
+  for (int k = SHEET_TERMS - 1; k >= 0; --k) {
+    const float ar = __fadd_rn(rec.T[k][0], pr), ai = __fadd_rn(rec.T[k][1], pi);
+    pr = __fmaf_rn(ar, tx, -__fmul_rn(ai, ty));
+    pi = __fmaf_rn(ar, ty, __fmul_rn(ai, tx));
+  }
+  for (int c = 0; c < rec.n_near; ++c) {
+    const float wr = __fadd_rn(rec.near[c][0], tx), wi = __fadd_rn(rec.near[c][1], ty);
+    const float lr = __fmul_rn(0.5f, logf(__fmaf_rn(wr, wr, __fmul_rn(wi, wi)))), li = atan2f(wi, wr);
+    const float plr = __fmaf_rn(wr, lr, -__fmul_rn(wi, li)), pli = __fmaf_rn(wi, lr, __fmul_rn(wr, li));  // w Log w
+    pr = __fmaf_rn(rec.near[c][2], pli, pr);   // -i a_c (w Log w)
+    pi = __fmaf_rn(-rec.near[c][2], plr, pi);
+  }
+  float s1, e1, s2, e2;
+  two_sum(rec.cx_hi, -axh, s1, e1);
+  two_sum(rec.cy_hi, -ayh, s2, e2);
+  b1 = __fadd_rn(s1, __fadd_rn(__fsub_rn(__fadd_rn(e1, rec.cx_lo), axl), __fmaf_rn(g.lam_s1, tx, pr)));
+  b2 = __fadd_rn(s2, __fadd_rn(__fsub_rn(__fadd_rn(e2, rec.cy_lo), ayl), __fmaf_rn(g.lam_s2, ty, -pi)));
+}
+
 
 // Variants: R rows per thread (the tile stays 32 x 64: 64/R warps per CTA),
 // PAIRED rows per thread that share one reciprocal per two rows, QUAD groups
@@ -249,12 +276,11 @@ constexpr int BR_NVARIANT = 16;
 // distances stay inside the FP32 range with a wide margin ((1e4)^8 = 1e32).
 constexpr double BR_QUAD_MAX_DIAG = 1.0e4;
 
-template <int MODE, int R, int PAIRED, int QUAD, int PACK, int TPSM>
+template <int R, int PAIRED, int QUAD, int PACK, int TPSM>
 __global__ void __launch_bounds__(32 * (BR_TY / R), TPSM / (32 * (BR_TY / R)))
 k_brute(Geo g, const double2* __restrict__ xy, const double* __restrict__ mass, int64_t n,
         const TileRec* __restrict__ recs, int64_t ntx, int64_t nwork, int64_t row0, int64_t row1,
-        uint32_t* __restrict__ counts, const int64_t* __restrict__ idx,
-        double* __restrict__ beta_out, int64_t* __restrict__ pix_out) {
+        uint32_t* __restrict__ counts) {
   constexpr int NT = 32 * (BR_TY / R);
   static_assert(PAIRED % 2 == 0 && (!PACK || (R - PAIRED) % 2 == 0), "rows go in pairs");
   static_assert(QUAD == 0 || PACK, "quads are packed");
@@ -272,22 +298,7 @@ k_brute(Geo g, const double2* __restrict__ xy, const double* __restrict__ mass, 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
   for (int64_t work = blockIdx.x; work < nwork; work += gridDim.x) {
-    int64_t tile, want_i = -1, want_j = -1;
-    if (MODE == MODE_MAP) {
-      tile = (row0 / BR_TY) * ntx + work;  // tile rows covering [row0, row1)
-    } else {
-      const int64_t f = idx[work];
-      if (f < 0 || f >= g.nrx * g.nry) {  // not a lattice ray: report it, touch nothing else
-        if (tid == 0) {
-          beta_out[2 * work] = beta_out[2 * work + 1] = nan("");
-          if (pix_out) pix_out[work] = -1;
-        }
-        continue;
-      }
-      want_i = f % g.nrx;
-      want_j = f / g.nrx;
-      tile = (want_j / BR_TY) * ntx + want_i / BR_TX;
-    }
+    const int64_t tile = (row0 / BR_TY) * ntx + work;  // tile rows covering [row0, row1)
     const TileGeo tg = tile_geo(g, tile, ntx);
     const double zx = g.a1 + tg.ci * g.dx3, zy = g.b1 + tg.cj * g.dx3;
     const int64_t col = tg.i0 + lane;
@@ -434,40 +445,12 @@ k_brute(Geo g, const double2* __restrict__ xy, const double* __restrict__ mass, 
     for (int r = 0; r < R; ++r) {
       const int64_t row = tg.j0 + warp * R + r;
       const bool inside = (col < tg.i1) && (row < tg.j1) && (row >= row0) && (row < row1);
-      // P(t) = sum_n T_n t^n by Horner, complex FP32
-      float pr = 0.f, pi = 0.f;
-#pragma unroll
-      for (int k = SHEET_TERMS - 1; k >= 0; --k) {
-        const float ar = rec.T[k][0] + pr, ai = rec.T[k][1] + pi;
-        pr = ar * tx - ai * ty[r];
-        pi = ar * ty[r] + ai * tx;
-      }
-      for (int c = 0; c < rec.n_near; ++c) {
-        const float wr = rec.near[c][0] + tx, wi = rec.near[c][1] + ty[r];
-        const float lr = 0.5f * logf(wr * wr + wi * wi), li = atan2f(wi, wr);
-        const float plr = wr * lr - wi * li, pli = wr * li + wi * lr;  // w Log w
-        pr += rec.near[c][2] * pli;                                    // -i a_c (w Log w)
-        pi -= rec.near[c][2] * plr;
-      }
-      const float axh = acc_s[0][r][tid], axl = acc_s[1][r][tid];
-      const float ayh = acc_s[2][r][tid], ayl = acc_s[3][r][tid];
-      float s1, e1, s2, e2;
-      two_sum(rec.cx_hi, -axh, s1, e1);
-      two_sum(rec.cy_hi, -ayh, s2, e2);
-      const float b1 = s1 + (((e1 + rec.cx_lo) - axl) + (g.lam_s1 * tx + pr));
-      const float b2 = s2 + (((e2 + rec.cy_lo) - ayl) + (g.lam_s2 * ty[r] - pi));
+      float b1, b2;
+      brute_beta(g, rec, tx, ty[r], acc_s[0][r][tid], acc_s[1][r][tid], acc_s[2][r][tid], acc_s[3][r][tid], b1, b2);
       uint32_t key = 0;
       int64_t pix = -1;
       const bool ok = inside && pixel_from_rel(g, rec.ix, rec.iy, b1, b2, key, pix);
-      if (MODE == MODE_MAP) {
-        bin_warp(counts, ok, key);
-      } else {
-        if (col == want_i && row == want_j) {
-          beta_out[2 * work] = (g.src_x0 + (double)rec.ix * g.sx) + (double)b1;
-          beta_out[2 * work + 1] = (g.src_y0 + (double)rec.iy * g.sy) + (double)b2;
-          if (pix_out) pix_out[work] = pix;
-        }
-      }
+      bin_warp(counts, ok, key);
     }
   }
 }
@@ -475,7 +458,7 @@ k_brute(Geo g, const double2* __restrict__ xy, const double* __restrict__ mass, 
 #define BR_DECL_OCC(V, R, PAIRED, QUAD, PACK, TPSM)                                             \
   case V:                                                                                       \
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm,                                  \
-                                                      k_brute<MODE_MAP, R, PAIRED, QUAD, PACK, TPSM>, \
+                                                      k_brute<R, PAIRED, QUAD, PACK, TPSM>, \
                                                       32 * (BR_TY / R), 0) != cudaSuccess)      \
       per_sm = 1;                                                                               \
     break;
@@ -503,19 +486,17 @@ int brute_grid_size(int num_sms, int variant) {
   return num_sms * (per_sm < 1 ? 1 : per_sm);
 }
 
-#define BR_DECL_LAUNCH(V, R, PAIRED, QUAD, PACK, TPSM)                                         \
-  case V:                                                                                      \
-    if (mode == MODE_MAP)                                                                      \
-      k_brute<MODE_MAP, R, PAIRED, QUAD, PACK, TPSM><<<(unsigned)grid, 32 * (BR_TY / R), 0, s>>>( \
-          P->g, xy2, mass, n, P->d_tiles, P->br_ntx, nwork, row0, row1, counts, idx, beta, pix); \
-    else                                                                                       \
-      k_brute<MODE_DUMP, R, PAIRED, QUAD, PACK, TPSM><<<(unsigned)grid, 32 * (BR_TY / R), 0, s>>>( \
-          P->g, xy2, mass, n, P->d_tiles, P->br_ntx, nwork, row0, row1, counts, idx, beta, pix); \
+#define BR_DECL_LAUNCH(V, R, PAIRED, QUAD, PACK, TPSM)                                              \
+  case V:                                                                                           \
+    k_brute<R, PAIRED, QUAD, PACK, TPSM><<<(unsigned)grid, 32 * (BR_TY / R), 0, s>>>(               \
+        P->g, xy2, mass, n, P->d_tiles, P->br_ntx, nwork, row0, row1, counts);                      \
     break;
-static cudaError_t launch_brute(const irs_plan_t* P, int mode, int64_t grid, const double* xy,
-                                const double* mass, int64_t n, int64_t nwork, int64_t row0,
-                                int64_t row1, uint32_t* counts, const int64_t* idx, double* beta,
-                                int64_t* pix, cudaStream_t s) {
+cudaError_t launch_brute_map(const irs_plan_t* P, const double* xy, const double* mass, int64_t n,
+                             int64_t row0, int64_t row1, uint32_t* counts, cudaStream_t s) {
+  if (row1 <= row0) return cudaSuccess;
+  const int64_t tr0 = row0 / BR_TY, tr1 = (row1 + BR_TY - 1) / BR_TY;
+  const int64_t nwork = (tr1 - tr0) * P->br_ntx;
+  const int64_t grid = nwork < P->br_grid ? nwork : P->br_grid;
   const double2* xy2 = reinterpret_cast<const double2*>(xy);
   switch (P->p.kernel_variant) {
     BR_VARIANTS(BR_DECL_LAUNCH)
@@ -525,21 +506,234 @@ static cudaError_t launch_brute(const irs_plan_t* P, int mode, int64_t grid, con
   return cudaGetLastError();
 }
 
-cudaError_t launch_brute_map(const irs_plan_t* P, const double* xy, const double* mass, int64_t n,
-                             int64_t row0, int64_t row1, uint32_t* counts, cudaStream_t s) {
-  if (row1 <= row0) return cudaSuccess;
-  const int64_t tr0 = row0 / BR_TY, tr1 = (row1 + BR_TY - 1) / BR_TY;
-  const int64_t nwork = (tr1 - tr0) * P->br_ntx;
-  const int64_t grid = nwork < P->br_grid ? nwork : P->br_grid;
-  return launch_brute(P, MODE_MAP, grid, xy, mass, n, nwork, row0, row1, counts, nullptr, nullptr,
-                      nullptr, s);
+// ------------------------------------------------------------ chosen rays
+// irs_shoot_rays: each ray by itself, in the arithmetic of k_brute -- lens
+// positions relative to the ray's tile centre, FP32 sums of 256 lenses in
+// order folded by TwoSum, and the reciprocal shared with the rows that the
+// variant groups it with (their squared distances are computed for that
+// alone).  The sums of different stages of 256 lenses are independent, so a
+// CTA runs several stages of a ray at once and folds them in order.  The form
+// before shot the ray's whole tile, 2048 rays.
+//
+// Two layouts.  BY_TILE: a CTA serves the chosen rays of one tile (a share of
+// them), found by a scan over the indices, and converts each lens to the
+// tile's frame once for all of them.  Otherwise a CTA takes 32 rays wherever
+// they lie and every ray converts for itself, bound by the FP64 subtractions
+// (GB300 issues two a clock per SM).  The first is chosen from 8 rays per
+// tile on average: 5e4 rays of a 923^2 lattice with 1e4 lenses take
+// 0.91 ms by tile and 3.96 ms by ray, and took 209 ms before.
+constexpr int BD_THREADS = 256;
+constexpr int BD_STAGES = BD_THREADS / 32;  // stages at once where every ray converts for itself
+constexpr int BD_LIST = 256;                // rays of a tile served at once
+constexpr int BD_PARTS = 8;                 // CTAs per tile
+
+struct RowGroup {  // rows that share a ray's reciprocal
+  int kind;        // 0: none, 1: one row (a), 2: three rows; a the row two on, b and c the others
+  float ta, tb, tc;
+};
+
+struct BruteForm {  // the variant's row groups (BR_VARIANTS)
+  int R, paired, quad;
+};
+
+__device__ __forceinline__ RowGroup row_group(const BruteForm& f, const TileGeo& tg, double dx3, int64_t row) {
+  RowGroup q{0, 0.f, 0.f, 0.f};
+  const int64_t slab = tg.j0 + (row - tg.j0) / f.R * f.R;
+  const int r = (int)(row - slab);
+  auto ty = [&](int i) { return (float)(((double)(slab + i) + 0.5 - tg.cj) * dx3); };
+  if (r < f.paired) {
+    q.kind = 1;
+    q.ta = ty(r ^ 1);
+  } else if (r - f.paired < 4 * f.quad) {
+    const int b = f.paired + ((r - f.paired) & ~3), i = (r - f.paired) & 3;
+    q.kind = 2;
+    q.ta = ty(b + (i ^ 2));
+    q.tb = ty(b + (i ^ 1));
+    q.tc = ty(b + (i ^ 3));
+  }
+  return q;
+}
+
+// one lens (offset x, y to the tile centre, mass m) into a ray's stage sums
+__device__ __forceinline__ void ray_pair(float tx, float ty, const RowGroup& q, float x, float y, float m, float& px,
+                                         float& py) {
+  const float dx = __fsub_rn(tx, x), dx2 = __fmul_rn(dx, dx), dy = __fsub_rn(ty, y);
+  const float r2 = __fmaf_rn(dy, dy, dx2);
+  float w;
+  if (q.kind == 0) {
+    w = __fmul_rn(m, rcp_approx(r2));
+  } else {
+    const float da = __fsub_rn(q.ta, y), ra = __fmaf_rn(da, da, dx2);
+    if (q.kind == 1) {
+      w = __fmul_rn(ra, __fmul_rn(m, rcp_approx(__fmul_rn(r2, ra))));
+    } else {
+      const float db = __fsub_rn(q.tb, y), dc = __fsub_rn(q.tc, y);
+      const float own = __fmul_rn(r2, ra);
+      const float other = __fmul_rn(__fmaf_rn(db, db, dx2), __fmaf_rn(dc, dc, dx2));
+      w = __fmul_rn(__fmul_rn(__fmul_rn(m, rcp_approx(__fmul_rn(own, other))), other), ra);
+    }
+  }
+  px = __fmaf_rn(w, dx, px);
+  py = __fmaf_rn(w, dy, py);
+}
+
+__device__ __forceinline__ void fold(float& hi, float& lo, float p) {
+  float s, e;
+  two_sum(hi, p, s, e);
+  hi = s;
+  lo = __fadd_rn(lo, e);
+}
+
+__device__ __forceinline__ void write_ray(const Geo& g, const TileRec& rec, float tx, float ty, float axh, float axl,
+                                          float ayh, float ayl, int64_t slot, double* beta_out, int64_t* pix_out) {
+  float b1, b2;
+  brute_beta(g, rec, tx, ty, axh, axl, ayh, ayl, b1, b2);
+  beta_out[2 * slot] = (g.src_x0 + (double)rec.ix * g.sx) + (double)b1;
+  beta_out[2 * slot + 1] = (g.src_y0 + (double)rec.iy * g.sy) + (double)b2;
+  if (pix_out) {
+    uint32_t key = 0;
+    int64_t pix = -1;
+    pixel_from_rel(g, rec.ix, rec.iy, b1, b2, key, pix);
+    pix_out[slot] = pix;
+  }
+}
+
+template <bool BY_TILE>
+__global__ void __launch_bounds__(BD_THREADS)
+k_brute_rays(Geo g, BruteForm form, const double2* __restrict__ xy, const double* __restrict__ mass, int64_t n,
+             const TileRec* __restrict__ recs, int64_t ntx, const int64_t* __restrict__ idx, int64_t nidx,
+             double* __restrict__ beta_out, int64_t* __restrict__ pix_out) {
+  // a stage's lenses: by tile as FP32 offsets (x, y, m), else as given
+  __shared__ double2 pos_s[BY_TILE ? 1 : BD_STAGES * BR_LT];
+  __shared__ float m_s[BY_TILE ? 1 : BD_STAGES * BR_LT];
+  __shared__ float4 lens_s[BY_TILE ? BD_STAGES * BR_LT : 1];
+  __shared__ float2 part_s[BD_THREADS];
+  __shared__ int64_t list_s[BY_TILE ? BD_LIST : 1];
+  __shared__ int found_s, grouped_s;
+  const int tid = threadIdx.x;
+  const int64_t tile = BY_TILE ? (int64_t)blockIdx.x / BD_PARTS : 0;
+  const int64_t n_rays = g.nrx * g.nry;
+  int64_t scan = BY_TILE ? (int64_t)(blockIdx.x % BD_PARTS) * BD_THREADS : (int64_t)blockIdx.x * 32;
+  while (scan < nidx) {
+    // ---- the rays of this round: `live` of them, ray k's slot in the caller's arrays
+    int live;
+    if (BY_TILE) {
+      __syncthreads();
+      if (tid == 0) found_s = grouped_s = 0;
+      __syncthreads();
+      for (; scan < nidx; scan += (int64_t)BD_PARTS * BD_THREADS) {
+        const int64_t i = scan + tid;
+        bool mine = false, grouped = false;
+        if (i < nidx) {
+          const int64_t f = idx[i];
+          if (f < 0 || f >= n_rays) {
+            mine = tile == 0;  // not a lattice ray: reported by the first tile's CTAs
+          } else {
+            const bool small = n_rays < ((int64_t)1 << 32);
+            const int64_t j = small ? (int64_t)((uint32_t)f / (uint32_t)g.nrx) : f / g.nrx;
+            mine = (j / BR_TY) * ntx + (f - j * g.nrx) / BR_TX == tile;
+            grouped = (int)(j % BR_TY) % form.R < form.paired + 4 * form.quad;
+          }
+        }
+        const int have = found_s + grouped_s;  // read before the barrier: nobody adds until everyone has passed it
+        const int hits = __syncthreads_count(mine);
+        if (have + hits > BD_LIST) break;  // next round starts here (a scan step adds at most BD_THREADS)
+        // rays that share reciprocals from the list's end, so that few warps mix both kinds
+        if (mine) list_s[grouped ? BD_LIST - 1 - atomicAdd(&grouped_s, 1) : atomicAdd(&found_s, 1)] = i;
+        __syncthreads();
+      }
+      live = found_s + grouped_s;
+      if (live == 0) continue;
+    } else {
+      live = (int)min((int64_t)32, nidx - scan);
+    }
+    // thread (ray, stage group): rays fastest; S groups of `live` threads
+    const int S = BY_TILE ? min(BD_STAGES, BD_THREADS / live) : BD_STAGES;
+    const int ray = BY_TILE ? tid % live : tid % 32, grp = BY_TILE ? tid / live : tid / 32;
+    const bool on = ray < live && grp < S;
+    int64_t slot = 0, f = -1;
+    if (on) {
+      slot = BY_TILE ? list_s[ray < found_s ? ray : BD_LIST - live + ray] : scan + ray;
+      f = idx[slot];
+    }
+    const bool ok = f >= 0 && f < n_rays;
+    const int64_t col = ok ? f % g.nrx : 0, row = ok ? f / g.nrx : 0;
+    const int64_t mytile = (row / BR_TY) * ntx + col / BR_TX;
+    const TileGeo tg = tile_geo(g, BY_TILE ? tile : mytile, ntx);
+    const double zx = g.a1 + tg.ci * g.dx3, zy = g.b1 + tg.cj * g.dx3;
+    const float tx = (float)(((double)col + 0.5 - tg.ci) * g.dx3), ty = (float)(((double)row + 0.5 - tg.cj) * g.dx3);
+    const RowGroup q = ok ? row_group(form, tg, g.dx3, row) : RowGroup{0, 0.f, 0.f, 0.f};
+    float axh = 0.f, axl = 0.f, ayh = 0.f, ayl = 0.f;
+    for (int64_t base = 0; base < n; base += (int64_t)S * BR_LT) {
+      const int total = (int)min((int64_t)S * BR_LT, n - base);
+      __syncthreads();  // the stages and partial sums before are used up
+      for (int t = tid; t < total; t += BD_THREADS) {
+        const double2 p = xy[base + t];
+        if (BY_TILE) {
+          lens_s[t] = make_float4((float)(p.x - zx), (float)(p.y - zy), (float)mass[base + t], 0.f);
+        } else {
+          pos_s[t] = p;
+          m_s[t] = (float)mass[base + t];
+        }
+      }
+      __syncthreads();
+      float px = 0.f, py = 0.f;
+      if (on && ok) {
+        const int e = min((grp + 1) * BR_LT, total);
+#pragma unroll 4
+        for (int t = grp * BR_LT; t < e; ++t) {
+          if (BY_TILE) {
+            const float4 L = lens_s[t];
+            ray_pair(tx, ty, q, L.x, L.y, L.z, px, py);
+          } else {
+            const double2 p = pos_s[t];
+            ray_pair(tx, ty, q, (float)(p.x - zx), (float)(p.y - zy), m_s[t], px, py);
+          }
+        }
+      }
+      part_s[tid] = make_float2(px, py);
+      __syncthreads();
+      if (on && grp == 0) {  // fold the stages in order
+        const int ns = (total + BR_LT - 1) / BR_LT, step = BY_TILE ? live : 32;
+        for (int k = 0; k < ns; ++k) {
+          const float2 p = part_s[ray + k * step];
+          fold(axh, axl, p.x);
+          fold(ayh, ayl, p.y);
+        }
+      }
+    }
+    if (on && grp == 0) {
+      if (ok) {
+        write_ray(g, recs[mytile], tx, ty, axh, axl, ayh, ayl, slot, beta_out, pix_out);
+      } else {  // not a lattice ray: report it, touch nothing else
+        beta_out[2 * slot] = beta_out[2 * slot + 1] = nan("");
+        if (pix_out) pix_out[slot] = -1;
+      }
+    }
+    if (!BY_TILE) scan = nidx;  // one round of 32 rays
+  }
+}
+
+#define BR_DECL_FORM(V, R, PAIRED, QUAD, PACK, TPSM) \
+  case V:                                            \
+    return BruteForm{R, PAIRED, QUAD};
+static BruteForm brute_form(int variant) {
+  switch (variant) { BR_VARIANTS(BR_DECL_FORM) default: break; }
+  return BruteForm{16, 0, 0};
 }
 
 cudaError_t launch_brute_dump(const irs_plan_t* P, const double* xy, const double* mass, int64_t n,
                               const int64_t* idx, int64_t nidx, double* beta, int64_t* pix,
                               cudaStream_t s) {
-  const int64_t grid = nidx < P->br_grid ? nidx : P->br_grid;
-  return launch_brute(P, MODE_DUMP, grid, xy, mass, n, nidx, 0, P->g.nry, nullptr, idx, beta, pix, s);
+  const double2* xy2 = reinterpret_cast<const double2*>(xy);
+  const BruteForm form = brute_form(P->p.kernel_variant);
+  if (nidx >= 8 * P->br_ntiles && P->br_ntiles * BD_PARTS < ((int64_t)1 << 31))
+    k_brute_rays<true><<<(unsigned)(P->br_ntiles * BD_PARTS), BD_THREADS, 0, s>>>(
+        P->g, form, xy2, mass, n, P->d_tiles, P->br_ntx, idx, nidx, beta, pix);
+  else
+    k_brute_rays<false><<<(unsigned)((nidx + 31) / 32), BD_THREADS, 0, s>>>(P->g, form, xy2, mass, n, P->d_tiles,
+                                                                            P->br_ntx, idx, nidx, beta, pix);
+  return cudaGetLastError();
 }
 
 // ------------------------------------------------------------ magnification

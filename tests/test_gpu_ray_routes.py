@@ -70,3 +70,28 @@ def test_a_block_fuller_than_the_shared_buffer():
     xy[:600] = 0.02 + np.random.default_rng(1).uniform(-0.025, 0.025, (600, 2))
     with irs.Plan(pl) as plan:
         _check(torch, pl, plan, *to_dev(torch, xy, m))
+
+
+@pytest.mark.parametrize("variant,n", [(0, 700), (1, 40), (2, 257), (11, 256), (14, 9), (15, 513), (0, 0)])
+def test_brute_map_equals_its_rays(variant, n):
+    """The brute force: every ray of the lattice (served tile by tile) adds up
+    to the map, and a few rays asked for alone (each with its own lenses'
+    conversion) come out with the same beta and pixel, whatever rows share
+    their reciprocals."""
+    torch = require_gpu()
+    args = (0.3, 0.1, 0.25, (-2, 3, -2.5, 2.1), (37, 29), 4.0)
+    po, pl = params_pair(*args, method=irs.IRS_BRUTE, n_star=n, kernel_variant=variant)
+    qo = oracle.size(po)
+    xy, m = lenses_for(qo, n, shape="uniform", seed=5, kappa_star=args[0])
+    dxy, dm = to_dev(torch, xy, m)
+    with irs.Plan(pl) as plan:
+        counts, _ = plan.make_map(dxy, dm)
+        idx = torch.arange(int(plan.info.n_rays), device="cuda")
+        beta, pix = plan.shoot_rays(dxy, dm, idx)
+        some = torch.from_numpy(np.random.default_rng(2).integers(0, idx.numel(), 95)).cuda()
+        b1, p1 = plan.shoot_rays(dxy, dm, torch.cat([some, torch.tensor([-1, idx.numel()], device="cuda")]))
+        plan.sync()
+    shape = (pl.npix_y, pl.npix_x)
+    assert np.array_equal(counts.cpu().numpy().astype(np.int64), _counts_of(pix.cpu().numpy(), shape))
+    assert torch.equal(b1[:95], beta[some]) and torch.equal(p1[:95], pix[some])
+    assert torch.isnan(b1[95:]).all() and (p1[95:] == -1).all()
