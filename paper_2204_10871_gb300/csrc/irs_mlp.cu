@@ -35,9 +35,8 @@ namespace {
 
 constexpr int OFF_W1 = 0, OFF_B1 = 4096, OFF_W2 = 4160, OFF_B2 = 8256, OFF_W3 = 8320,
               OFF_B3 = 12416, OFF_W4 = 12480, OFF_B4 = 12992;
-constexpr int MLP_WARPS = 4;                 // warps per CTA, 16 samples each
-constexpr int MLP_CTA = MLP_WARPS * 32;
-constexpr int MLP_TILE = 16 * MLP_W;         // one [16][64] FP32 activation tile
+constexpr int MLP_WARPS = 4;    // warps per training CTA that carry 16 samples each
+constexpr int MLP_CTA = 2 * MLP_WARPS * 32;  // as many again help with the weights and their gradients
 constexpr int FF_THREADS = 256;
 
 struct MlpState {
@@ -269,202 +268,364 @@ __device__ __forceinline__ void mma_bf16(float c[4], uint32_t a0, uint32_t a1, u
       : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
-// acc[nt] (16 x 8 tiles) += A (16 x K) * B (K x 8 NT) on one warp; A(m, k) =
-// A[m ars + k acs] (0 for m >= mv or k >= kv), B(k, n) = B[k brs + n bcs]
-// (0 for k >= kv); operands rounded to BF16, products accumulated in FP32.
-// Fragment layouts of mma.m16n8k16: A rows gid / gid+8, cols 2 tig (+1, +8, +9);
-// B rows 2 tig (+1, +8, +9), col gid; C rows gid / gid+8, cols 2 tig (+1).
-template <int NT>
-__device__ __forceinline__ void warp_gemm(const float* A, int ars, int acs, int mv, const float* B, int brs,
-                                          int bcs, int K, int kv, float (*acc)[4]) {
-  const int lane = threadIdx.x & 31, gid = lane >> 2, tig = lane & 3;
-  auto a = [&](int m, int k) { return (m < mv && k < kv) ? A[m * ars + k * acs] : 0.f; };
-  auto b = [&](int k, int n) { return k < kv ? B[k * brs + n * bcs] : 0.f; };
-  for (int k0 = 0; k0 < K; k0 += 16) {
-    const int c0 = k0 + 2 * tig;
-    const uint32_t a0 = pack_bf16(a(gid, c0), a(gid, c0 + 1));
-    const uint32_t a1 = pack_bf16(a(gid + 8, c0), a(gid + 8, c0 + 1));
-    const uint32_t a2 = pack_bf16(a(gid, c0 + 8), a(gid, c0 + 9));
-    const uint32_t a3 = pack_bf16(a(gid + 8, c0 + 8), a(gid + 8, c0 + 9));
-#pragma unroll
-    for (int nt = 0; nt < NT; ++nt) {
-      const int n = nt * 8 + gid;
-      const uint32_t b0 = pack_bf16(b(c0, n), b(c0 + 1, n));
-      const uint32_t b1 = pack_bf16(b(c0 + 8, n), b(c0 + 9, n));
-      mma_bf16(acc[nt], a0, a1, a2, a3, b0, b1);
-    }
-  }
+// The network on one warp, 16 samples at a time, without leaving registers: the
+// C fragment of mma.m16n8k16 (rows gid, gid + 8; columns 2 tig, 2 tig + 1 of an
+// 8-column tile; gid = lane / 4, tig = lane % 4) of tiles 2k, 2k + 1 holds
+// exactly the elements of the next product's A fragment of k-step k.  The
+// weights sit in shared memory as BF16 B fragments, packed once per CTA (one
+// conflict-free 8-byte load per product).  Activations are rounded to BF16 where
+// they enter a product, and the k-steps of a product accumulate in order.
+// Before, each CTA of four warps kept FP32 weights and activations in shared
+// memory (one CTA per SM), and every operand was read with eight-way bank
+// conflicts and packed on each use: 3e5 points took 518 us, a training batch of
+// 4096 with its gradient 78 us; now 64 us and 23 us.  Both are bound by
+// instruction issue: the exact tanhf and sincosf are three quarters of it.
+__device__ __forceinline__ int mlp_woff(int l) { return l == 0 ? OFF_W1 : l == 1 ? OFF_W2 : OFF_W3; }
+__device__ __forceinline__ int mlp_boff(int l) { return l == 0 ? OFF_B1 : l == 1 ? OFF_B2 : OFF_B3; }
+
+struct MlpForwardS {
+  uint2 w[3][4][8][32];  // layer, k-step, column tile, lane: W[n][k] for out n = 8 nt + gid
+  uint2 head[4][32];
+  float b[3][MLP_W];
+  float b4[MLP_OUT];
+  float2 freq[MLP_NF];
+};
+
+// BF16 pair (W[row][k], W[row][k + 1]) of a row-major [out][64] matrix
+__device__ __forceinline__ uint32_t pack_row(const float* __restrict__ W, int row, int k) {
+  return pack_bf16(W[row * MLP_W + k], W[row * MLP_W + k + 1]);
 }
 
-// C-fragment element q of tile nt: row and column in the 16 x (8 NT) result.
-__device__ __forceinline__ int frag_row(int q) { return ((threadIdx.x & 31) >> 2) + (q >= 2 ? 8 : 0); }
-__device__ __forceinline__ int frag_col(int nt, int q) { return nt * 8 + 2 * ((threadIdx.x & 31) & 3) + (q & 1); }
-
-// Forward pass of 16 samples on one warp.  act: [4][16][64] (features, h1,
-// h2, h3); W: packed FP32 weights in shared memory.  y[q] = output element
-// (frag_row(q), frag_col(0, q)) of the 16 x 8 head.
-__device__ void mlp_forward_warp(const float* W, const float* freq, const float2* x16, int ns, float* act,
-                                 float y[4]) {
-  const int lane = threadIdx.x & 31;
-  float* F = act;
-  for (int e = lane; e < 16 * MLP_NF; e += 32) {
-    const int s = e / MLP_NF, j = e % MLP_NF;
-    float sv = 0.f, cv = 0.f;
-    if (s < ns) {
-      const float a = 3.14159265358979f * (freq[2 * j] * x16[s].x + freq[2 * j + 1] * x16[s].y);
-      sincosf(a, &sv, &cv);
-    }
-    F[s * MLP_W + j] = sv;
-    F[s * MLP_W + MLP_NF + j] = cv;
+__device__ __forceinline__ void mlp_pack_forward(MlpForwardS& S, const float* __restrict__ theta,
+                                                 const float* __restrict__ freq) {
+#pragma unroll 4
+  for (int t = threadIdx.x; t < 3 * 4 * 8 * 32 + 4 * 32; t += blockDim.x) {
+    const int lane = t & 31, gid = lane >> 2, tig = lane & 3, u = t >> 5;
+    const bool hd = u >= 96;
+    const int l = u >> 5, kt = hd ? u - 96 : (u >> 3) & 3, nt = hd ? 0 : u & 7;
+    const float* W = theta + (hd ? OFF_W4 : mlp_woff(l));
+    const int c = kt * 16 + 2 * tig, row = nt * 8 + gid;
+    const uint2 v = make_uint2(pack_row(W, row, c), pack_row(W, row, c + 8));
+    if (hd) S.head[kt][lane] = v;
+    else S.w[l][kt][nt][lane] = v;
   }
-  __syncwarp();
-  const int woff[3] = {OFF_W1, OFF_W2, OFF_W3}, boff[3] = {OFF_B1, OFF_B2, OFF_B3};
-  for (int l = 0; l < 3; ++l) {
-    const float* Hin = act + l * MLP_TILE;
-    float* Hout = act + (l + 1) * MLP_TILE;
-    float acc[8][4];
+  for (int t = threadIdx.x; t < 3 * MLP_W; t += blockDim.x) S.b[t / MLP_W][t % MLP_W] = theta[mlp_boff(t / MLP_W) + t % MLP_W];
+  for (int t = threadIdx.x; t < MLP_OUT; t += blockDim.x) S.b4[t] = theta[OFF_B4 + t];
+  for (int t = threadIdx.x; t < MLP_NF; t += blockDim.x) S.freq[t] = make_float2(freq[2 * t], freq[2 * t + 1]);
+}
+
+// [sin, cos](pi B x) of rows gid (xa) and gid + 8 (xb) as the first layer's A
+// fragments; rows that are off hold zeros
+__device__ __forceinline__ void mlp_features(const MlpForwardS& S, float2 xa, bool on_a, float2 xb, bool on_b,
+                                             uint32_t A[4][4]) {
+  const int tig = threadIdx.x & 3;
 #pragma unroll
-    for (int nt = 0; nt < 8; ++nt) acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.f;
-    warp_gemm<8>(Hin, MLP_W, 1, 16, W + woff[l], 1, MLP_W, MLP_W, MLP_W, acc);
+  for (int kt = 0; kt < 2; ++kt)
 #pragma unroll
-    for (int nt = 0; nt < 8; ++nt)
+    for (int half = 0; half < 2; ++half) {
+      float s[2][2], c[2][2];  // row, frequency
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int o = frag_col(nt, q);
-        Hout[frag_row(q) * MLP_W + o] = tanhf(acc[nt][q] + W[boff[l] + o]);
+      for (int e = 0; e < 2; ++e) {
+        const float2 f = S.freq[kt * 16 + half * 8 + 2 * tig + e];
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+          const float2 x = r ? xb : xa;
+          sincosf(__fmul_rn(3.14159265358979f, __fmaf_rn(f.x, x.x, __fmul_rn(f.y, x.y))), &s[r][e], &c[r][e]);
+          if (!(r ? on_b : on_a)) s[r][e] = c[r][e] = 0.f;
+        }
       }
-    __syncwarp();
-  }
-  float acc4[1][4] = {{0.f, 0.f, 0.f, 0.f}};
-  warp_gemm<1>(act + 3 * MLP_TILE, MLP_W, 1, 16, W + OFF_W4, 1, MLP_W, MLP_W, MLP_W, acc4);
-#pragma unroll
-  for (int q = 0; q < 4; ++q) y[q] = acc4[0][q] + W[OFF_B4 + frag_col(0, q)];
+      A[kt][2 * half] = pack_bf16(s[0][0], s[0][1]);
+      A[kt][2 * half + 1] = pack_bf16(s[1][0], s[1][1]);
+      A[kt + 2][2 * half] = pack_bf16(c[0][0], c[0][1]);
+      A[kt + 2][2 * half + 1] = pack_bf16(c[1][0], c[1][1]);
+    }
 }
 
-// Fused forward + backward of a batch; weight gradients accumulate in shared
-// memory per CTA, then once per CTA into `grad`.  Samples: idx[b] when given,
-// else a seeded draw per (step, slot).
+// acc = A (16 x 64) times a 64 x 64 matrix given as B fragments
+__device__ __forceinline__ void mlp_product(const uint32_t A[4][4], const uint2 (*w)[8][32], float acc[8][4]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int nt = 0; nt < 8; ++nt) acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.f;
+#pragma unroll
+  for (int kt = 0; kt < 4; ++kt)
+#pragma unroll
+    for (int nt = 0; nt < 8; ++nt) {
+      const uint2 b = w[kt][nt][lane];
+      mma_bf16(acc[nt], A[kt][0], A[kt][1], A[kt][2], A[kt][3], b.x, b.y);
+    }
+}
+
+// C fragments of a 16 x 64 result as the next product's A fragments
+__device__ __forceinline__ void mlp_as_operand(const float c[8][4], uint32_t A[4][4]) {
+#pragma unroll
+  for (int kt = 0; kt < 4; ++kt) {
+    A[kt][0] = pack_bf16(c[2 * kt][0], c[2 * kt][1]);
+    A[kt][1] = pack_bf16(c[2 * kt][2], c[2 * kt][3]);
+    A[kt][2] = pack_bf16(c[2 * kt + 1][0], c[2 * kt + 1][1]);
+    A[kt][3] = pack_bf16(c[2 * kt + 1][2], c[2 * kt + 1][3]);
+  }
+}
+
+// One hidden layer: h = tanh(A W^T + b)
+__device__ __forceinline__ void mlp_layer(const MlpForwardS& S, int l, const uint32_t A[4][4], float h[8][4]) {
+  const int tig = threadIdx.x & 3;
+  mlp_product(A, S.w[l], h);
+#pragma unroll
+  for (int nt = 0; nt < 8; ++nt) {
+    const float2 b = *reinterpret_cast<const float2*>(&S.b[l][nt * 8 + 2 * tig]);
+    h[nt][0] = tanhf(h[nt][0] + b.x);
+    h[nt][1] = tanhf(h[nt][1] + b.y);
+    h[nt][2] = tanhf(h[nt][2] + b.x);
+    h[nt][3] = tanhf(h[nt][3] + b.y);
+  }
+}
+
+// The linear head: y = outputs (gid, 2 tig), (gid, 2 tig + 1), (gid + 8, ...)
+__device__ __forceinline__ void mlp_head(const MlpForwardS& S, const uint32_t A[4][4], float y[4]) {
+  const int lane = threadIdx.x & 31, tig = lane & 3;
+  y[0] = y[1] = y[2] = y[3] = 0.f;
+#pragma unroll
+  for (int kt = 0; kt < 4; ++kt) {
+    const uint2 b = S.head[kt][lane];
+    mma_bf16(y, A[kt][0], A[kt][1], A[kt][2], A[kt][3], b.x, b.y);
+  }
+  y[0] += S.b4[2 * tig];
+  y[1] += S.b4[2 * tig + 1];
+  y[2] += S.b4[2 * tig];
+  y[3] += S.b4[2 * tig + 1];
+}
+
+// Training: a CTA takes 64 samples.  Four warps each run 16 of them through the
+// network and back with everything in registers but BF16 copies of the
+// activations and of dL/dz, which go to shared memory for the weight gradients:
+// those are products over the CTA's 64 samples, each of eight warps computing
+// 16 rows by 32 columns of every dW, added once per CTA into `grad`.  (Before, each warp
+// added its own 16 samples' dW into shared memory, 13,000 atomic additions a
+// warp.)
+constexpr int MLP_SAMPLES = 16 * MLP_WARPS;  // per CTA
+constexpr int MLP_ROW = MLP_W + 8;           // BF16 per sample row: rows shift four banks
+struct MlpTrainS {
+  MlpForwardS f;
+  uint2 back[2][4][8][32];  // W3, W2 as B fragments of dz W
+  uint32_t back4[8][32];    // W4 (8 rows; the other half of the k-step is zero)
+  __nv_bfloat16 h[4][MLP_SAMPLES][MLP_ROW];   // features, h1, h2, h3
+  __nv_bfloat16 dz[3][MLP_SAMPLES][MLP_ROW];  // dL/dz of layers 1..3
+  __nv_bfloat16 dy[MLP_SAMPLES][8];
+};
+
+__device__ __forceinline__ void ldmatrix_x4_t(uint32_t r[4], const void* p) {
+  const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(a));
+}
+__device__ __forceinline__ void ldmatrix_x2_t(uint32_t r[2], const void* p) {
+  const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
+  asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(a));
+}
+
+// a fragment pair (rows gid and gid + 8, columns 2 tig and 2 tig + 1 of tile nt)
+__device__ __forceinline__ void store_frag(__nv_bfloat16 (*m)[MLP_ROW], int row0, int nt, uint32_t lo, uint32_t hi) {
+  const int lane = threadIdx.x & 31, gid = lane >> 2, tig = lane & 3;
+  *reinterpret_cast<uint32_t*>(&m[row0 + gid][nt * 8 + 2 * tig]) = lo;
+  *reinterpret_cast<uint32_t*>(&m[row0 + gid + 8][nt * 8 + 2 * tig]) = hi;
+}
+
+// A fragments of a 16 x 64 operand, as rows of a shared matrix
+__device__ __forceinline__ void store_operand(__nv_bfloat16 (*m)[MLP_ROW], int row0, const uint32_t A[4][4]) {
+#pragma unroll
+  for (int kt = 0; kt < 4; ++kt) {
+    store_frag(m, row0, 2 * kt, A[kt][0], A[kt][1]);
+    store_frag(m, row0, 2 * kt + 1, A[kt][2], A[kt][3]);
+  }
+}
+
+// column sums of a 16 x 64 result over its 16 rows, added to g[0..63]
+__device__ __forceinline__ void add_columns(const float c[8][4], float* __restrict__ g) {
+  const int lane = threadIdx.x & 31, tig = lane & 3;
+#pragma unroll
+  for (int nt = 0; nt < 8; ++nt) {
+    float a = c[nt][0] + c[nt][2], b = c[nt][1] + c[nt][3];
+#pragma unroll
+    for (int d = 4; d < 32; d <<= 1) {
+      a += __shfl_xor_sync(0xFFFFFFFFu, a, d);
+      b += __shfl_xor_sync(0xFFFFFFFFu, b, d);
+    }
+    if (lane < 4) {
+      atomicAdd(g + nt * 8 + 2 * tig, a);
+      atomicAdd(g + nt * 8 + 2 * tig + 1, b);
+    }
+  }
+}
+
+// dz = dh (1 - h^2), its column sums into g
+__device__ __forceinline__ void through_tanh(float c[8][4], const float h[8][4], float* __restrict__ g) {
+#pragma unroll
+  for (int nt = 0; nt < 8; ++nt)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) c[nt][q] = __fmul_rn(c[nt][q], __fmaf_rn(-h[nt][q], h[nt][q], 1.f));
+  add_columns(c, g);
+}
+
+// One warp's 16 samples, forward and backward
+__device__ __forceinline__ void mlp_chain(MlpTrainS& S, const float2* __restrict__ xs, const float* __restrict__ ts,
+                                          int64_t n_samples, int64_t batch, uint64_t seed, int ordered,
+                                          float* __restrict__ grad, double* __restrict__ loss) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gid = lane >> 2, tig = lane & 3;
+  // this lane's rows of the warp's 16 samples: gid and gid + 8
+  const int row0 = warp * 16;
+  const int64_t b0 = (int64_t)blockIdx.x * MLP_SAMPLES + row0;
+  int64_t sid[2];
+  float2 x[2];
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    const int64_t b = b0 + gid + 8 * r;
+    sid[r] = b >= batch ? -1
+             : ordered  ? b
+                        : (int64_t)(splitmix64(seed ^ (uint64_t)b * 0x2545F4914F6CDD1Dull) % (uint64_t)n_samples);
+    x[r] = sid[r] >= 0 ? xs[sid[r]] : make_float2(0.f, 0.f);
+  }
+  float h1[8][4], h2[8][4], h3[8][4], y[4];
+  uint32_t A[4][4];
+  mlp_features(S.f, x[0], sid[0] >= 0, x[1], sid[1] >= 0, A);
+  store_operand(S.h[0], row0, A);
+  mlp_layer(S.f, 0, A, h1);
+  mlp_as_operand(h1, A);
+  store_operand(S.h[1], row0, A);
+  mlp_layer(S.f, 1, A, h2);
+  mlp_as_operand(h2, A);
+  store_operand(S.h[2], row0, A);
+  mlp_layer(S.f, 2, A, h3);
+  mlp_as_operand(h3, A);
+  store_operand(S.h[3], row0, A);
+  mlp_head(S.f, A, y);
+  // loss and dL/dy (mean over the whole batch and the 8 outputs)
+  const float scale = 2.0f / (float)(batch * MLP_OUT);
+  float lsum = 0.f;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int64_t s = sid[q >> 1];
+    float d = 0.f;
+    if (s >= 0) {
+      d = y[q] - ts[s * MLP_OUT + 2 * tig + (q & 1)];
+      lsum = __fmaf_rn(d, d, lsum);
+    }
+    y[q] = d * scale;
+  }
+  for (int off = 16; off; off >>= 1) lsum += __shfl_xor_sync(0xFFFFFFFFu, lsum, off);
+  if (lane == 0 && b0 < batch) atomicAdd(loss, (double)lsum);
+  const uint32_t dy0 = pack_bf16(y[0], y[1]), dy1 = pack_bf16(y[2], y[3]);
+  *reinterpret_cast<uint32_t*>(&S.dy[row0 + gid][2 * tig]) = dy0;
+  *reinterpret_cast<uint32_t*>(&S.dy[row0 + gid + 8][2 * tig]) = dy1;
+  {
+    float a = y[0] + y[2], b = y[1] + y[3];
+#pragma unroll
+    for (int d = 4; d < 32; d <<= 1) {
+      a += __shfl_xor_sync(0xFFFFFFFFu, a, d);
+      b += __shfl_xor_sync(0xFFFFFFFFu, b, d);
+    }
+    if (lane < 4) {
+      atomicAdd(grad + OFF_B4 + 2 * tig, a);
+      atomicAdd(grad + OFF_B4 + 2 * tig + 1, b);
+    }
+  }
+  float c[8][4];
+#pragma unroll
+  for (int nt = 0; nt < 8; ++nt) {
+    c[nt][0] = c[nt][1] = c[nt][2] = c[nt][3] = 0.f;
+    mma_bf16(c[nt], dy0, dy1, 0u, 0u, S.back4[nt][lane], 0u);
+  }
+  through_tanh(c, h3, grad + OFF_B3);
+  mlp_as_operand(c, A);
+  store_operand(S.dz[2], row0, A);
+  mlp_product(A, S.back[0], c);
+  through_tanh(c, h2, grad + OFF_B2);
+  mlp_as_operand(c, A);
+  store_operand(S.dz[1], row0, A);
+  mlp_product(A, S.back[1], c);
+  through_tanh(c, h1, grad + OFF_B1);
+  mlp_as_operand(c, A);
+  store_operand(S.dz[0], row0, A);
+}
+
+// Fused forward + backward of a batch.  Samples: in order when `ordered`, else a
+// seeded draw per (step, slot).
 __global__ void __launch_bounds__(MLP_CTA) k_mlp_train(const float* __restrict__ theta,
                                                        const float* __restrict__ freq,
                                                        const float2* __restrict__ xs,
                                                        const float* __restrict__ ts, int64_t n_samples,
                                                        int64_t batch, uint64_t seed, int ordered,
                                                        float* __restrict__ grad, double* __restrict__ loss) {
-  extern __shared__ float smem[];
-  float* W = smem;                          // MLP_NPARAM
-  float* G = W + MLP_NPARAM;                // MLP_NPARAM gradient accumulator
-  float* actall = G + MLP_NPARAM;           // warps x (4 + 1) tiles + dy
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  for (int k = tid; k < MLP_NPARAM; k += blockDim.x) {
-    W[k] = theta[k];
-    G[k] = 0.f;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  MlpTrainS& S = *reinterpret_cast<MlpTrainS*>(smem_raw);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, gid = lane >> 2, tig = lane & 3;
+  mlp_pack_forward(S.f, theta, freq);
+#pragma unroll 4
+  for (int t = tid; t < 2 * 4 * 8 * 32 + 8 * 32; t += MLP_CTA) {
+    const int ln = t & 31, g = ln >> 2, k = 2 * (ln & 3), u = t >> 5;
+    if (u < 64) {  // B(k, n) = W[k][n]
+      const float* W = theta + (u < 32 ? OFF_W3 : OFF_W2);
+      const int kt = (u >> 3) & 3, n = (u & 7) * 8 + g, c = kt * 16 + k;
+      S.back[u >> 5][kt][u & 7][ln] =
+          make_uint2(pack_bf16(W[c * MLP_W + n], W[(c + 1) * MLP_W + n]),
+                     pack_bf16(W[(c + 8) * MLP_W + n], W[(c + 9) * MLP_W + n]));
+    } else {
+      const int n = (u - 64) * 8 + g;
+      S.back4[u - 64][ln] = pack_bf16(theta[OFF_W4 + k * MLP_W + n], theta[OFF_W4 + (k + 1) * MLP_W + n]);
+    }
   }
   __syncthreads();
-  float* act = actall + warp * (5 * MLP_TILE + 16 * MLP_OUT);
-  float* DZ = act + 4 * MLP_TILE;
-  float* DY = DZ + MLP_TILE;
-  __shared__ float2 xw[MLP_WARPS][16];
-  __shared__ int64_t sid[MLP_WARPS][16];
-  const int64_t b0 = ((int64_t)blockIdx.x * MLP_WARPS + warp) * 16;
-  int ns = 0;
-  if (lane < 16) {
-    const int64_t b = b0 + lane;
-    int64_t s = -1;
-    if (b < batch)
-      s = ordered ? b : (int64_t)(splitmix64(seed ^ (uint64_t)b * 0x2545F4914F6CDD1Dull) % (uint64_t)n_samples);
-    sid[warp][lane] = s;
-    xw[warp][lane] = s >= 0 ? xs[s] : make_float2(0.f, 0.f);
-  }
-  __syncwarp();
-  for (int k = 0; k < 16; ++k) ns += sid[warp][k] >= 0 ? 1 : 0;
-  float y[4];
-  mlp_forward_warp(W, freq, xw[warp], ns, act, y);
-  // loss and dL/dy (mean over the whole batch and the 8 outputs)
-  const float scale = 2.0f / (float)(batch * MLP_OUT);
-  float lsum = 0.f;
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int s = frag_row(q), o = frag_col(0, q);
-    float d = 0.f;
-    if (s < ns) {
-      d = y[q] - ts[sid[warp][s] * MLP_OUT + o];
-      lsum += d * d;
-    }
-    DY[s * MLP_OUT + o] = d * scale;
-  }
-  for (int off = 16; off; off >>= 1) lsum += __shfl_xor_sync(0xFFFFFFFFu, lsum, off);
-  if (lane == 0 && ns > 0) atomicAdd(loss, (double)lsum);
-  __syncwarp();
-  float* H[4] = {act, act + MLP_TILE, act + 2 * MLP_TILE, act + 3 * MLP_TILE};
-  // head: dW4[o][i] = sum_s dy[s][o] h3[s][i]; db4; dh3 = dy W4
-  {
-    float acc[8][4];
-#pragma unroll
-    for (int nt = 0; nt < 8; ++nt) acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.f;
-    warp_gemm<8>(DY, 1, MLP_OUT, MLP_OUT, H[3], MLP_W, 1, 16, 16, acc);
-#pragma unroll
-    for (int nt = 0; nt < 8; ++nt)
-#pragma unroll
-      for (int q = 0; q < 2; ++q) atomicAdd(&G[OFF_W4 + frag_row(q) * MLP_W + frag_col(nt, q)], acc[nt][q]);
-    if (lane < MLP_OUT) {
-      float sb = 0.f;
-      for (int s = 0; s < 16; ++s) sb += DY[s * MLP_OUT + lane];
-      atomicAdd(&G[OFF_B4 + lane], sb);
-    }
-#pragma unroll
-    for (int nt = 0; nt < 8; ++nt) acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.f;
-    warp_gemm<8>(DY, MLP_OUT, 1, 16, W + OFF_W4, MLP_W, 1, 16, MLP_OUT, acc);
-    __syncwarp();
-#pragma unroll
-    for (int nt = 0; nt < 8; ++nt)
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int s = frag_row(q), i = frag_col(nt, q);
-        const float h = H[3][s * MLP_W + i];
-        DZ[s * MLP_W + i] = acc[nt][q] * (1.f - h * h);
-      }
-    __syncwarp();
-  }
-  const int woff[3] = {OFF_W1, OFF_W2, OFF_W3}, boff[3] = {OFF_B1, OFF_B2, OFF_B3};
-  for (int l = 2; l >= 0; --l) {
-    // dW_l[o][i] = sum_s dz[s][o] Hin[s][i] in four 16-row tiles of o; db_l
-    const float* Hin = H[l];
-    for (int mt = 0; mt < 4; ++mt) {
-      float acc[8][4];
-#pragma unroll
-      for (int nt = 0; nt < 8; ++nt) acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.f;
-      warp_gemm<8>(DZ + mt * 16, 1, MLP_W, 16, Hin, MLP_W, 1, 16, 16, acc);
-#pragma unroll
-      for (int nt = 0; nt < 8; ++nt)
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-          atomicAdd(&G[woff[l] + (mt * 16 + frag_row(q)) * MLP_W + frag_col(nt, q)], acc[nt][q]);
-    }
-    for (int o = lane; o < MLP_W; o += 32) {
-      float sb = 0.f;
-      for (int s = 0; s < 16; ++s) sb += DZ[s * MLP_W + o];
-      atomicAdd(&G[boff[l] + o], sb);
-    }
-    if (l == 0) break;
-    // dH_{l} = dz W_l, then dz_{l-1} = dH (1 - h^2)
-    float acc[8][4];
-#pragma unroll
-    for (int nt = 0; nt < 8; ++nt) acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.f;
-    warp_gemm<8>(DZ, MLP_W, 1, 16, W + woff[l], MLP_W, 1, MLP_W, MLP_W, acc);
-    __syncwarp();
-#pragma unroll
-    for (int nt = 0; nt < 8; ++nt)
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int s = frag_row(q), i = frag_col(nt, q);
-        const float h = Hin[s * MLP_W + i];
-        DZ[s * MLP_W + i] = acc[nt][q] * (1.f - h * h);
-      }
-    __syncwarp();
-  }
+  if (warp < MLP_WARPS) mlp_chain(S, xs, ts, n_samples, batch, seed, ordered, grad, loss);
   __syncthreads();
-  for (int k = tid; k < MLP_NPARAM; k += blockDim.x)
-    if (G[k] != 0.f) atomicAdd(&grad[k], G[k]);
+  // dW_l[o][i] = sum_s dz[s][o] h[s][i], 16 rows o and 32 columns i of this warp;
+  // the lane's row of an ldmatrix: sample (lane & 7), + 8 for the second k half
+  const int mrow = lane & 7, mk = (lane >> 4) & 1, mn = (lane >> 3) & 1;
+  const int o0 = (warp & 3) * 16, i0 = (warp >> 2) * 32;
+  float c[4][4];
+#pragma unroll 1
+  for (int l = 0; l < 3; ++l) {
+#pragma unroll
+    for (int nt = 0; nt < 4; ++nt) c[nt][0] = c[nt][1] = c[nt][2] = c[nt][3] = 0.f;
+#pragma unroll
+    for (int kt = 0; kt < MLP_SAMPLES / 16; ++kt) {
+      uint32_t a[4];  // (k, m), (k, m + 8), (k + 8, m), (k + 8, m + 8)
+      ldmatrix_x4_t(a, &S.dz[l][kt * 16 + 8 * mk + mrow][o0 + 8 * mn]);
+#pragma unroll
+      for (int nt = 0; nt < 4; nt += 2) {
+        uint32_t b[4];  // (k, n), (k + 8, n), (k, n + 8), (k + 8, n + 8)
+        ldmatrix_x4_t(b, &S.h[l][kt * 16 + 8 * mn + mrow][i0 + nt * 8 + 8 * mk]);
+        mma_bf16(c[nt], a[0], a[1], a[2], a[3], b[0], b[1]);
+        mma_bf16(c[nt + 1], a[0], a[1], a[2], a[3], b[2], b[3]);
+      }
+    }
+    float* g = grad + mlp_woff(l) + (o0 + gid) * MLP_W + i0 + 2 * tig;
+#pragma unroll
+    for (int nt = 0; nt < 4; ++nt) {
+      atomicAdd(g + nt * 8, c[nt][0]);
+      atomicAdd(g + nt * 8 + 1, c[nt][1]);
+      atomicAdd(g + nt * 8 + 8 * MLP_W, c[nt][2]);
+      atomicAdd(g + nt * 8 + 8 * MLP_W + 1, c[nt][3]);
+    }
+  }
+  // dW4: eight rows, one column tile a warp
+  c[0][0] = c[0][1] = c[0][2] = c[0][3] = 0.f;
+#pragma unroll
+  for (int kt = 0; kt < MLP_SAMPLES / 16; ++kt) {
+    uint32_t a[2], b[2];  // (k, m), (k + 8, m); (k, n), (k + 8, n)
+    ldmatrix_x2_t(a, &S.dy[kt * 16 + 8 * mn + mrow][0]);
+    ldmatrix_x2_t(b, &S.h[3][kt * 16 + 8 * mn + mrow][warp * 8]);
+    mma_bf16(c[0], a[0], 0u, a[1], 0u, b[0], b[1]);
+  }
+  float* g = grad + OFF_W4 + gid * MLP_W + warp * 8 + 2 * tig;
+  atomicAdd(g, c[0][0]);
+  atomicAdd(g + 1, c[0][1]);
+}
+
+// zero the gradient and the loss sum
+__global__ void k_mlp_zero(float* __restrict__ grad, double* __restrict__ loss) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k < MLP_NPARAM) grad[k] = 0.f;
+  if (k == 0) loss[0] = 0.0;
 }
 
 __global__ void k_adamw(float* __restrict__ theta, float* __restrict__ m, float* __restrict__ v,
@@ -481,30 +642,39 @@ __global__ void k_adamw(float* __restrict__ theta, float* __restrict__ m, float*
   g[k] = 0.f;
 }
 
-// Network output at arbitrary inputs (standardised units), 16 per warp.
-__global__ void __launch_bounds__(MLP_CTA) k_mlp_eval(const float* __restrict__ theta,
-                                                      const float* __restrict__ freq,
-                                                      const float2* __restrict__ x, int64_t n,
-                                                      float* __restrict__ y_out) {
-  extern __shared__ float smem[];
-  float* W = smem;
-  float* actall = W + MLP_NPARAM;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  for (int k = tid; k < MLP_NPARAM; k += blockDim.x) W[k] = theta[k];
+// Network output at arbitrary inputs (standardised units): a persistent grid,
+// 16 samples per warp and turn.
+constexpr int MLP_EVAL_THREADS = 256;
+__global__ void __launch_bounds__(MLP_EVAL_THREADS, 2) k_mlp_eval(const float* __restrict__ theta,
+                                                                  const float* __restrict__ freq,
+                                                                  const float2* __restrict__ x, int64_t n,
+                                                                  float* __restrict__ y_out) {
+  __shared__ MlpForwardS S;
+  mlp_pack_forward(S, theta, freq);
   __syncthreads();
-  float* act = actall + warp * 4 * MLP_TILE;
-  __shared__ float2 xw[MLP_WARPS][16];
-  const int64_t b0 = ((int64_t)blockIdx.x * MLP_WARPS + warp) * 16;
-  const int ns = (int)min((int64_t)16, n - b0);
-  if (ns <= 0) return;
-  if (lane < 16) xw[warp][lane] = lane < ns ? x[b0 + lane] : make_float2(0.f, 0.f);
-  __syncwarp();
-  float y[4];
-  mlp_forward_warp(W, freq, xw[warp], ns, act, y);
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int s = frag_row(q);
-    if (s < ns) y_out[(b0 + s) * MLP_OUT + frag_col(0, q)] = y[q];
+  const int lane = threadIdx.x & 31, gid = lane >> 2, tig = lane & 3;
+  const int64_t step = (int64_t)gridDim.x * (MLP_EVAL_THREADS / 32) * 16;
+  for (int64_t b0 = ((int64_t)blockIdx.x * (MLP_EVAL_THREADS / 32) + (threadIdx.x >> 5)) * 16; b0 < n; b0 += step) {
+    const int64_t ra = b0 + gid, rb = ra + 8;
+    const float2 zero = make_float2(0.f, 0.f), xa = ra < n ? x[ra] : zero, xb = rb < n ? x[rb] : zero;
+    uint32_t A[4][4];
+    mlp_features(S, xa, ra < n, xb, rb < n, A);
+#pragma unroll 1
+    for (int l = 0; l < 3; ++l) {
+      float h[8][4];
+      mlp_layer(S, l, A, h);
+      mlp_as_operand(h, A);
+    }
+    float y[4];
+    mlp_head(S, A, y);
+    if (ra < n) {
+      y_out[ra * MLP_OUT + 2 * tig] = y[0];
+      y_out[ra * MLP_OUT + 2 * tig + 1] = y[1];
+    }
+    if (rb < n) {
+      y_out[rb * MLP_OUT + 2 * tig] = y[2];
+      y_out[rb * MLP_OUT + 2 * tig + 1] = y[3];
+    }
   }
 }
 
@@ -527,10 +697,13 @@ __global__ void k_mlp_cell_outputs(const float* __restrict__ y, int64_t nrc, con
                                       y[rc * MLP_OUT + 2 * k + 1] * sd[2 * k + 1] + mean[2 * k + 1]);
 }
 
-size_t train_smem() {
-  return sizeof(float) * (2 * MLP_NPARAM + MLP_WARPS * (5 * MLP_TILE + 16 * MLP_OUT));
+// two CTAs per SM, fewer for few samples
+void launch_eval(const irs_plan_t* P, const float* theta, const float* freq, const float2* x, int64_t n, float* y,
+                 cudaStream_t s) {
+  constexpr int64_t per_cta = MLP_EVAL_THREADS / 32 * 16;
+  const int64_t need = (n + per_cta - 1) / per_cta, most = 2 * (int64_t)P->num_sms;
+  k_mlp_eval<<<(unsigned)(need < most ? need : most), MLP_EVAL_THREADS, 0, s>>>(theta, freq, x, n, y);
 }
-size_t eval_smem() { return sizeof(float) * (MLP_NPARAM + MLP_WARPS * 4 * MLP_TILE); }
 
 }  // namespace
 
@@ -605,10 +778,8 @@ irs_status mlp_plan(irs_plan_t* P, double gx0, double gy0, double h, int ncx, in
   if (!pts.empty() &&
       cudaMemcpy(M->corner_pts, pts.data(), sizeof(double2) * pts.size(), cudaMemcpyHostToDevice) != cudaSuccess)
     return IRS_ERR_CUDA;
-  if (cudaFuncSetAttribute(k_mlp_train, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)train_smem()) !=
-          cudaSuccess ||
-      cudaFuncSetAttribute(k_mlp_eval, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)eval_smem()) !=
-          cudaSuccess)
+  if (cudaFuncSetAttribute(k_mlp_train, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(MlpTrainS)) !=
+      cudaSuccess)
     return IRS_ERR_CUDA;
   return IRS_OK;
 }
@@ -641,8 +812,7 @@ irs_status mlp_prepare(irs_plan_t* P, const double* xy, const double* mass, int6
     cudaMemsetAsync(M->exact, 0, sizeof(double2) * MLP_KEXACT * M->ncorner, s);
   k_mlp_cell_inputs<<<(unsigned)((nrc + 255) / 256), 256, 0, s>>>(gx0, gy0, h, nrcx, ox, oy, nrc, M->cx, M->cy,
                                                                  M->half, scratch_x);
-  const int64_t blocks = (nrc + 16 * MLP_WARPS - 1) / (16 * MLP_WARPS);
-  k_mlp_eval<<<(unsigned)blocks, MLP_CTA, eval_smem(), s>>>(M->theta, M->freq, scratch_x, nrc, scratch_y);
+  launch_eval(P, M->theta, M->freq, scratch_x, nrc, scratch_y, s);
   k_mlp_cell_outputs<<<(unsigned)((nrc + 255) / 256), 256, 0, s>>>(scratch_y, nrc, M->out_mean, M->out_std, M->U);
   if (cudaGetLastError() != cudaSuccess) return IRS_ERR_CUDA;
   far->U = M->U;
@@ -678,10 +848,9 @@ irs_status mlp_grad(irs_plan_t* P, const float* x, const float* t, int64_t n, fl
   MlpState* M = M_(P);
   if (!M) return IRS_ERR_UNSUPPORTED;
   if (n <= 0 || !x || !t || !grad || !loss) return IRS_ERR_ARG;
-  if (cudaMemsetAsync(grad, 0, 4 * MLP_NPARAM, s) != cudaSuccess) return IRS_ERR_CUDA;
-  if (cudaMemsetAsync(loss, 0, 8, s) != cudaSuccess) return IRS_ERR_CUDA;
+  k_mlp_zero<<<(MLP_NPARAM + 255) / 256, 256, 0, s>>>(grad, loss);
   const int64_t blocks = (n + 16 * MLP_WARPS - 1) / (16 * MLP_WARPS);
-  k_mlp_train<<<(unsigned)blocks, MLP_CTA, train_smem(), s>>>(M->theta, M->freq, reinterpret_cast<const float2*>(x),
+  k_mlp_train<<<(unsigned)blocks, MLP_CTA, sizeof(MlpTrainS), s>>>(M->theta, M->freq, reinterpret_cast<const float2*>(x),
                                                               t, n, n, 0, 1, grad, loss);
   return cudaGetLastError() == cudaSuccess ? IRS_OK : IRS_ERR_CUDA;
 }
@@ -690,9 +859,7 @@ irs_status mlp_forward(irs_plan_t* P, const float* x, int64_t n, float* y, cudaS
   MlpState* M = M_(P);
   if (!M) return IRS_ERR_UNSUPPORTED;
   if (n <= 0) return IRS_OK;
-  const int64_t blocks = (n + 16 * MLP_WARPS - 1) / (16 * MLP_WARPS);
-  k_mlp_eval<<<(unsigned)blocks, MLP_CTA, eval_smem(), s>>>(M->theta, M->freq, reinterpret_cast<const float2*>(x),
-                                                           n, y);
+  launch_eval(P, M->theta, M->freq, reinterpret_cast<const float2*>(x), n, y, s);
   return cudaGetLastError() == cudaSuccess ? IRS_OK : IRS_ERR_CUDA;
 }
 
@@ -804,7 +971,7 @@ irs_status mlp_train(irs_plan_t* P, const double* xy, const double* mass, int64_
         const float warm = step < 100 ? (float)step / 100.f : 1.f;
         const float lr = lr0 * warm * 0.5f * (1.f + cosf(3.14159265f * (float)step / (float)steps));
         cudaMemsetAsync(M->loss, 0, 8, s);
-        k_mlp_train<<<(unsigned)blocks, MLP_CTA, train_smem(), s>>>(M->theta, M->freq, M->xs, M->ts, n_samples,
+        k_mlp_train<<<(unsigned)blocks, MLP_CTA, sizeof(MlpTrainS), s>>>(M->theta, M->freq, M->xs, M->ts, n_samples,
                                                                     batch, seed ^ (0xABCDull * step), 0,
                                                                     M->grad, M->loss);
         k_adamw<<<(MLP_NPARAM + 255) / 256, 256, 0, s>>>(M->theta, M->adam_m, M->adam_v, M->grad, lr, b1, b2,
@@ -828,7 +995,7 @@ irs_status mlp_train(irs_plan_t* P, const double* xy, const double* mass, int64_
       r.loss_first = nfirst ? lsum_first / nfirst : 0;
       r.loss_final = nlast ? lsum_last / nlast : 0;
       // held-out error in physical units
-      k_mlp_eval<<<(unsigned)((n_valid + 63) / 64), MLP_CTA, eval_smem(), s>>>(M->theta, M->freq, xv, n_valid, yv);
+      launch_eval(P, M->theta, M->freq, xv, n_valid, yv, s);
       hu.resize((size_t)MLP_OUT * n_valid);
       hy.resize((size_t)MLP_OUT * n_valid);
       if (cudaMemcpyAsync(hu.data(), u + MLP_OUT * n_samples, sizeof(double) * hu.size(), cudaMemcpyDeviceToHost,
