@@ -106,6 +106,7 @@ irs_status alloc_workspace(irs_plan_t* P) {
   const size_t o_mpart = take(sizeof(double) * irs::MSUM_BLOCKS);
   const size_t o_status = take(sizeof(int));
   const size_t o_queue = take(sizeof(unsigned long long));
+  const size_t o_mdone = take(sizeof(unsigned int));
   size_t o_tiles = 0;
   if (P->p.method == IRS_BRUTE) o_tiles = take(sizeof(irs::TileRec) * (size_t)P->br_ntiles);
   P->ws_bytes = off;
@@ -119,6 +120,7 @@ irs_status alloc_workspace(irs_plan_t* P) {
   P->d_mpart = reinterpret_cast<double*>(b + o_mpart);
   P->d_status = reinterpret_cast<int*>(b + o_status);
   P->d_queue = reinterpret_cast<unsigned long long*>(b + o_queue);
+  P->d_mdone = reinterpret_cast<unsigned int*>(b + o_mdone);
   P->d_tiles = P->p.method == IRS_BRUTE ? reinterpret_cast<irs::TileRec*>(b + o_tiles) : nullptr;
   if (cudaMemset(P->ws, 0, P->ws_bytes) != cudaSuccess) return IRS_ERR_CUDA;
   return IRS_OK;
@@ -144,18 +146,18 @@ irs_status run_map(irs_plan_t* P, const double* xy, const double* mass, int64_t 
   if (st != IRS_OK) return st;
   const size_t npix = (size_t)P->g.npix_x * P->g.npix_y;
   if (clear) IRS_TRY(cudaMemsetAsync(counts, 0, npix * sizeof(uint32_t), s));
-  P->launches = 2;  // mass sum
+  P->launches = 1;  // mass sum
   mark(P, irs::EV_START, s);
   IRS_TRY(irs::launch_mass_sum(P, mass, n, s, xy));
   if (P->p.method == IRS_BRUTE) {
-    IRS_TRY(irs::launch_brute_setup(P, s));
+    IRS_TRY(irs::launch_brute_setup(P, row0, row1, s));
     mark(P, irs::EV_PREP, s);
     mark(P, irs::EV_CELLS, s);
     mark(P, irs::EV_FIN, s);
     mark(P, irs::EV_FAR, s);
     mark(P, irs::EV_RAY0, s);
     IRS_TRY(irs::launch_brute_map(P, xy, mass, n, row0, row1, counts, s));
-    P->launches += row1 > row0 ? 2 : 1;
+    P->launches += row1 > row0 ? 2 : 0;
     mark(P, irs::EV_RAY1, s);
   } else {
     st = irs::interp_run(P, xy, mass, n, row0, row1, counts, s);
@@ -315,7 +317,7 @@ irs_status irs_shoot_rays(irs_plan_t* P, const double* xy, const double* mass, i
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   IRS_TRY(irs::launch_mass_sum(P, mass, n, s, xy));
   if (P->p.method == IRS_BRUTE) {
-    IRS_TRY(irs::launch_brute_setup(P, s));
+    IRS_TRY(irs::launch_brute_setup(P, 0, P->g.nry, s));
     IRS_TRY(irs::launch_brute_dump(P, xy, mass, n, ray_idx, n_idx, beta, pixel, s));
     return IRS_OK;
   }

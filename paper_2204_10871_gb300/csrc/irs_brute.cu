@@ -23,8 +23,8 @@
 namespace irs {
 
 // ------------------------------------------------------------ mass sum (FP64)
-// Deterministic two-pass sum of the masses: fixed strides per thread, fixed
-// reduction tree, fixed order of the block partials.  With lens positions
+// Deterministic sum of the masses: fixed strides per thread, fixed reduction
+// tree, fixed order of the block partials.  With lens positions
 // given, the same pass checks that every lens lies in the plan's lens region
 // (the rectangle that is both image and lens plane, Sec. 2.2, or the
 // circumscribed circle), with a margin of 1e-9 of the plane's extent for
@@ -45,12 +45,20 @@ __device__ __forceinline__ bool lens_inside(const LensRegion& L, double2 p) {
   return p.x >= L.x0 && p.x <= L.x1 && p.y >= L.y0 && p.y <= L.y1;
 }
 
-__global__ void k_mass_partial(const double* __restrict__ mass, const double2* __restrict__ xy, int64_t n,
-                               LensRegion region, int* __restrict__ status, double* __restrict__ part) {
+// One launch: the block that finishes last adds the partial sums, in block
+// order.  Blocks past the last lens would only add zeros and are not launched
+// (a map of few lenses took 8 us in a second launch of one thread that added
+// 128 of them); the stride between a thread's lenses is that of all
+// MSUM_BLOCKS either way, so the sum is the same bits.
+__global__ void k_mass_sum(const double* __restrict__ mass, const double2* __restrict__ xy, int64_t n,
+                           LensRegion region, int* __restrict__ status, double* __restrict__ part,
+                           unsigned int* __restrict__ done, double* __restrict__ out,
+                           unsigned long long* __restrict__ queue) {
   __shared__ double sh[MSUM_THREADS];
+  __shared__ bool last;
   double s = 0.0;
   bool outside = false;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  const int64_t stride = (int64_t)MSUM_BLOCKS * MSUM_THREADS;
   for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += stride) {
     s += mass[k];
     if (region.check) outside |= !lens_inside(region, xy[k]);
@@ -62,16 +70,22 @@ __global__ void k_mass_partial(const double* __restrict__ mass, const double2* _
     if ((int)threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
     __syncthreads();
   }
-  if (threadIdx.x == 0) part[blockIdx.x] = sh[0];
-}
-
-__global__ void k_mass_final(const double* __restrict__ part, double* __restrict__ out,
-                             unsigned long long* __restrict__ queue) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
+  if (threadIdx.x == 0) {
+    part[blockIdx.x] = sh[0];
+    __threadfence();
+    last = atomicAdd(done, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  if (threadIdx.x < gridDim.x) sh[threadIdx.x] = __ldcg(part + threadIdx.x);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double t = 0.0;
+    for (unsigned b = 0; b < gridDim.x; ++b) t += sh[b];
+    out[0] = t;
+    *done = 0u;               // for the next sum on this plan
     if (queue) *queue = 0ull;  // the ray pass's work counter
-    double s = 0.0;
-    for (int b = 0; b < MSUM_BLOCKS; ++b) s += part[b];
-    out[0] = s;
   }
 }
 
@@ -91,9 +105,11 @@ cudaError_t launch_mass_sum(const irs_plan_t* P, const double* mass, int64_t n, 
   L.r2 = (P->circle_r + tol) * (P->circle_r + tol);
   L.circle = g.plane == IRS_PLANE_CIRCLE;
   L.check = xy != nullptr && n > 0;
-  k_mass_partial<<<MSUM_BLOCKS, MSUM_THREADS, 0, s>>>(mass, reinterpret_cast<const double2*>(xy), n, L,
-                                                      P->d_status, P->d_mpart);
-  k_mass_final<<<1, 32, 0, s>>>(P->d_mpart, P->d_msum, P->d_queue);
+  static_assert(MSUM_BLOCKS <= MSUM_THREADS, "one partial sum per thread");
+  const int64_t need = (n + MSUM_THREADS - 1) / MSUM_THREADS;
+  const unsigned blocks = need < 1 ? 1u : need < MSUM_BLOCKS ? (unsigned)need : (unsigned)MSUM_BLOCKS;
+  k_mass_sum<<<blocks, MSUM_THREADS, 0, s>>>(mass, reinterpret_cast<const double2*>(xy), n, L, P->d_status, P->d_mpart,
+                                             P->d_mdone, P->d_msum, P->d_queue);
   return cudaGetLastError();
 }
 
@@ -124,22 +140,68 @@ __device__ __forceinline__ cd clog_p(cd a) {
 //              phi_c^(n) = -i a_c (-1)^n (n-2)! / (z-c)^(n-1)  (n >= 2).
 // Corners closer than 6 tile half-diagonals are left out of the series and
 // evaluated per ray instead (the series would converge slowly there).
-__global__ void k_brute_setup(Geo g, const double* __restrict__ msum, int64_t ntx, int64_t ntiles,
-                              TileRec* __restrict__ recs) {
-  const int64_t tile = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (tile >= ntiles) return;
+//
+// Bound by FP64 latency and issue (GB300 runs FP64 at 1/64 of FP32), so a CTA
+// of four warps takes 32 tiles: first one thread per (tile, corner) for the
+// logarithm, arctangent and powers, then one warp sums the corners of each
+// tile in order and adds the centre's terms.  With one thread per tile for all
+// of it 5,120 tiles and 224 tiles took 32 us each, now 20 and 16 us.
+constexpr int SETUP_TILES = 32;
+constexpr int SETUP_VALUES = 4 + 2 * (SHEET_TERMS - 1);  // Log w, w Log w, w^-1 ... w^-7
+
+__global__ void __launch_bounds__(4 * SETUP_TILES)
+k_brute_setup(Geo g, const double* __restrict__ msum, int64_t ntx, int64_t tile0, int64_t tile1,
+              TileRec* __restrict__ recs) {
+  __shared__ double val_s[4][SETUP_VALUES][SETUP_TILES];
+  __shared__ bool near_s[4][SETUP_TILES];
+  const int lt = threadIdx.x & 31;  // a warp per corner
+  const int64_t tile = min(tile0 + (int64_t)blockIdx.x * SETUP_TILES + lt, tile1 - 1);
   const TileGeo tg = tile_geo(g, tile, ntx);
+  const double zx = g.a1 + tg.ci * g.dx3, zy = g.b1 + tg.cj * g.dx3;
+  auto corner = [&](int c) { return cd{zx - ((c & 1) ? g.a2 : g.a1), zy - ((c & 2) ? g.b2 : g.b1)}; };
+  if (g.plane != IRS_PLANE_CIRCLE) {
+    const int c = threadIdx.x >> 5;
+    const cd w = corner(c);
+    // the exact test only where a cheap upper bound of the radius leaves it open
+    const double ub = 6.0 * fmax(0.5 * g.dx3 * (double)((tg.i1 - tg.i0) + (tg.j1 - tg.j0)), g.dx3);
+    bool near = fmax(fabs(w.re), fabs(w.im)) < ub;
+    if (near) {
+      const double half_diag = 0.5 * g.dx3 * hypot((double)(tg.i1 - tg.i0), (double)(tg.j1 - tg.j0));
+      near = hypot(w.re, w.im) < 6.0 * fmax(half_diag, g.dx3);
+    }
+    near_s[c][lt] = near;
+    if (!near) {
+      cd L = clog_p(w);
+      // branch continuous with the rectangle's interior (tile centres are
+      // inside it, so this only guards the two right-hand corners' cuts)
+      if (c == 3 && w.re < 0.0 && w.im > 0.0) L.im -= 2.0 * M_PI;
+      if (c == 1 && w.re < 0.0 && w.im < 0.0) L.im += 2.0 * M_PI;
+      const cd wl = cmul(w, L);
+      val_s[c][0][lt] = L.re;
+      val_s[c][1][lt] = L.im;
+      val_s[c][2][lt] = wl.re;
+      val_s[c][3][lt] = wl.im;
+      const cd inv = crecip(w);
+      cd pw = inv;
+#pragma unroll
+      for (int k = 0; k < SHEET_TERMS - 1; ++k) {
+        val_s[c][4 + 2 * k][lt] = pw.re;
+        val_s[c][5 + 2 * k][lt] = pw.im;
+        pw = cmul(pw, inv);
+      }
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x >= SETUP_TILES || tile0 + (int64_t)blockIdx.x * SETUP_TILES + lt >= tile1) return;
+
   const double ks = g.kstar_scale * msum[0];  // kappa_*^act = pi sum(m) / A of the lenses passed in
   const double kap = g.kappa_s + ks;
-  const double zx = g.a1 + tg.ci * g.dx3, zy = g.b1 + tg.cj * g.dx3;
-
   // base pixel from the mean lens map of the tile centre
   const double m1 = (1.0 - kap - g.gamma) * zx, m2 = (1.0 - kap + g.gamma) * zy;
   double fx = floor((m1 - g.src_x0) / g.sx), fy = floor((m2 - g.src_y0) / g.sy);
   fx = fmin(fmax(fx, -1.0e9), 1.0e9);
   fy = fmin(fmax(fy, -1.0e9), 1.0e9);
   const double base_x = g.src_x0 + fx * g.sx, base_y = g.src_y0 + fy * g.sy;
-
   TileRec r;
   r.ix = (int32_t)fx;
   r.iy = (int32_t)fy;
@@ -147,7 +209,6 @@ __global__ void k_brute_setup(Geo g, const double* __restrict__ msum, int64_t nt
   r.pad_ = 0;
   for (int k = 0; k < SHEET_TERMS; ++k) r.T[k][0] = r.T[k][1] = 0.f;
   for (int k = 0; k < MAX_NEAR; ++k) r.near[k][0] = r.near[k][1] = r.near[k][2] = r.near[k][3] = 0.f;
-
   double cre, cim;  // conj(beta) of the centre without the lens sum
   if (g.plane == IRS_PLANE_CIRCLE) {
     // Eq. (alpha) + k_* theta_c:  conj(beta) = (1-k_s) conj(z) - g z - k_* conj(z_c) - L
@@ -157,45 +218,36 @@ __global__ void k_brute_setup(Geo g, const double* __restrict__ msum, int64_t nt
     // Eq. (alpha1): conj(beta) = (1-k) conj(z) - g z - L + conj(alpha_sheet,+)
     cd T0 = {ks * (2.0 * zx - 2.0 * g.a2), 0.0};  // kappa_* (conj z + z - 2 a2)
     cd T[SHEET_TERMS];
+#pragma unroll
     for (int k = 0; k < SHEET_TERMS; ++k) T[k] = {0.0, 0.0};
     T[0].re = ks;  // derivative of kappa_* (z - 2 a2)
-    const double half_diag = 0.5 * g.dx3 * hypot((double)(tg.i1 - tg.i0), (double)(tg.j1 - tg.j0));
-    const double rho = 6.0 * fmax(half_diag, g.dx3);
-    const double cxs[4] = {g.a1, g.a2, g.a1, g.a2};
-    const double cys[4] = {g.b1, g.b1, g.b2, g.b2};
-    const double sgn[4] = {1.0, -1.0, -1.0, 1.0};
+#pragma unroll
     for (int c = 0; c < 4; ++c) {
-      const double ac = ks / M_PI * sgn[c];
-      const cd w = {zx - cxs[c], zy - cys[c]};
+      const double ac = ks / M_PI * ((c == 0 || c == 3) ? 1.0 : -1.0);
       if (ac == 0.0) continue;
-      if (hypot(w.re, w.im) < rho && r.n_near < MAX_NEAR) {
+      if (near_s[c][lt]) {
+        const cd w = corner(c);
         r.near[r.n_near][0] = (float)w.re;
         r.near[r.n_near][1] = (float)w.im;
         r.near[r.n_near][2] = (float)ac;
         r.n_near++;
         continue;
       }
-      cd L = clog_p(w);
-      // branch continuous with the rectangle's interior (tile centres are
-      // inside it, so this only guards the two right-hand corners' cuts)
-      if (c == 3 && w.re < 0.0 && w.im > 0.0) L.im -= 2.0 * M_PI;
-      if (c == 1 && w.re < 0.0 && w.im < 0.0) L.im += 2.0 * M_PI;
-      const cd wl = cmul(w, L);
-      T0.re += ac * wl.im;  // -i a_c (w L)
-      T0.im -= ac * wl.re;
-      T[0].re += ac * L.im;  // -i a_c (L + 1)
-      T[0].im -= ac * (L.re + 1.0);
-      const cd inv = crecip(w);
-      cd pw = inv;
+      auto v = [&](int k) { return val_s[c][k][lt]; };
+      T0.re += ac * v(3);  // -i a_c (w L)
+      T0.im -= ac * v(2);
+      T[0].re += ac * v(1);  // -i a_c (L + 1)
+      T[0].im -= ac * (v(0) + 1.0);
+#pragma unroll
       for (int n = 2; n <= SHEET_TERMS; ++n) {
         const double coef = ((n & 1) ? -1.0 : 1.0) / (double)(n * (n - 1));
-        T[n - 1].re += ac * coef * pw.im;
-        T[n - 1].im -= ac * coef * pw.re;
-        pw = cmul(pw, inv);
+        T[n - 1].re += ac * coef * v(2 * n + 1);
+        T[n - 1].im -= ac * coef * v(2 * n);
       }
     }
     cre = (1.0 - kap - g.gamma) * zx + T0.re;
     cim = -(1.0 - kap + g.gamma) * zy + T0.im;
+#pragma unroll
     for (int k = 0; k < SHEET_TERMS; ++k) {
       r.T[k][0] = (float)T[k].re;
       r.T[k][1] = (float)T[k].im;
@@ -206,43 +258,48 @@ __global__ void k_brute_setup(Geo g, const double* __restrict__ msum, int64_t nt
   recs[tile] = r;
 }
 
-cudaError_t launch_brute_setup(const irs_plan_t* P, cudaStream_t s) {
-  const int64_t nt = P->br_ntiles;
-  const int threads = 128;
-  const int64_t blocks = (nt + threads - 1) / threads;
-  k_brute_setup<<<(unsigned)blocks, threads, 0, s>>>(P->g, P->d_msum, P->br_ntx, nt, P->d_tiles);
+// Tile constants of the tile rows that cover lattice rows [row0, row1).
+cudaError_t launch_brute_setup(const irs_plan_t* P, int64_t row0, int64_t row1, cudaStream_t s) {
+  const int64_t t0 = row0 / BR_TY * P->br_ntx, t1 = (row1 + BR_TY - 1) / BR_TY * P->br_ntx;
+  if (t1 <= t0) return cudaSuccess;
+  const int64_t blocks = (t1 - t0 + SETUP_TILES - 1) / SETUP_TILES;
+  k_brute_setup<<<(unsigned)blocks, 4 * SETUP_TILES, 0, s>>>(P->g, P->d_msum, P->br_ntx, t0, t1, P->d_tiles);
   return cudaGetLastError();
 }
 
 // ------------------------------------------------------------ ray pass
 // Source position of a ray relative to its tile's base pixel corner, from its
-// offset (tx, ty) to the tile centre and its lens sums: smooth terms, the
-// sheet's series, corners near the tile.  The rounding of every step is
-// explicit: the map's and the chosen-ray kernels must agree bit for bit.
-__device__ __forceinline__ void brute_beta(const Geo& g, const TileRec& rec, float tx, float ty, float axh, float axl,
-                                           float ayh, float ayl, float& b1, float& b2) {
-  // P(t) = sum_n T_n t^n by Horner, complex FP32
-  float pr = 0.f, pi = 0.f;
-#pragma unroll
-  for (int k = SHEET_TERMS - 1; k >= 0; --k) {
-    const float ar = __fadd_rn(rec.T[k][0], pr), ai = __fadd_rn(rec.T[k][1], pi);
-    pr = __fmaf_rn(ar, tx, -__fmul_rn(ai, ty));
-    pi = __fmaf_rn(ar, ty, __fmul_rn(ai, tx));
-  }
-  for (int c = 0; c < rec.n_near; ++c) {
-    const float wr = __fadd_rn(rec.near[c][0], tx), wi = __fadd_rn(rec.near[c][1], ty);
-    const float lr = __fmul_rn(0.5f, logf(__fmaf_rn(wr, wr, __fmul_rn(wi, wi)))), li = atan2f(wi, wr);
-    const float plr = __fmaf_rn(wr, lr, -__fmul_rn(wi, li)), pli = __fmaf_rn(wi, lr, __fmul_rn(wr, li));  // w Log w
-    pr = __fmaf_rn(rec.near[c][2], pli, pr);   // -i a_c (w Log w)
-    pi = __fmaf_rn(-rec.near[c][2], plr, pi);
-  }
+// offset (tx, ty) to the tile centre and its lens sums: the sheet's series
+// P(t) = sum_n T_n t^n, corners near the tile, the smooth terms and the centre.
+// The rounding of every step is explicit: the map's and the chosen-ray kernels
+// must agree bit for bit.
+__device__ __forceinline__ void brute_corner(const float* near, float tx, float ty, float& pr, float& pi) {
+  const float wr = __fadd_rn(near[0], tx), wi = __fadd_rn(near[1], ty);
+  const float lr = __fmul_rn(0.5f, logf(__fmaf_rn(wr, wr, __fmul_rn(wi, wi)))), li = atan2f(wi, wr);
+  const float plr = __fmaf_rn(wr, lr, -__fmul_rn(wi, li)), pli = __fmaf_rn(wi, lr, __fmul_rn(wr, li));  // w Log w
+  pr = __fmaf_rn(near[2], pli, pr);  // -i a_c (w Log w)
+  pi = __fmaf_rn(-near[2], plr, pi);
+}
+__device__ __forceinline__ void brute_sum(const Geo& g, const TileRec& rec, float tx, float ty, float pr, float pi,
+                                          float axh, float axl, float ayh, float ayl, float& b1, float& b2) {
   float s1, e1, s2, e2;
   two_sum(rec.cx_hi, -axh, s1, e1);
   two_sum(rec.cy_hi, -ayh, s2, e2);
   b1 = __fadd_rn(s1, __fadd_rn(__fsub_rn(__fadd_rn(e1, rec.cx_lo), axl), __fmaf_rn(g.lam_s1, tx, pr)));
   b2 = __fadd_rn(s2, __fadd_rn(__fsub_rn(__fadd_rn(e2, rec.cy_lo), ayl), __fmaf_rn(g.lam_s2, ty, -pi)));
 }
-
+__device__ __forceinline__ void brute_beta(const Geo& g, const TileRec& rec, float tx, float ty, float axh, float axl,
+                                           float ayh, float ayl, float& b1, float& b2) {
+  float pr = 0.f, pi = 0.f;
+#pragma unroll
+  for (int k = SHEET_TERMS - 1; k >= 0; --k) {  // Horner, complex FP32
+    const float ar = __fadd_rn(rec.T[k][0], pr), ai = __fadd_rn(rec.T[k][1], pi);
+    pr = __fmaf_rn(ar, tx, -__fmul_rn(ai, ty));
+    pi = __fmaf_rn(ar, ty, __fmul_rn(ai, tx));
+  }
+  for (int c = 0; c < rec.n_near; ++c) brute_corner(rec.near[c], tx, ty, pr, pi);
+  brute_sum(g, rec, tx, ty, pr, pi, axh, axl, ayh, ayl, b1, b2);
+}
 
 // Variants: R rows per thread (the tile stays 32 x 64: 64/R warps per CTA),
 // PAIRED rows per thread that share one reciprocal per two rows, QUAD groups
@@ -294,6 +351,7 @@ k_brute(Geo g, const double2* __restrict__ xy, const double* __restrict__ mass, 
   __shared__ float4 lens_s[BR_LT];
   __shared__ float2 lensm_s[PACK ? BR_LT : 1];
   __shared__ float acc_s[4][R][NT];  // x hi, x lo, y hi, y lo
+  __shared__ float2 ty_s[BR_TY / 2];  // row offsets to the tile centre, in pairs
   __shared__ TileRec rec;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
@@ -304,18 +362,23 @@ k_brute(Geo g, const double2* __restrict__ xy, const double* __restrict__ mass, 
     const int64_t col = tg.i0 + lane;
     const float tx = (float)(((double)col + 0.5 - tg.ci) * g.dx3);
     const float2 TX2 = make_float2(tx, tx);
+    __syncthreads();  // previous tile's readers of rec / lens_s / ty_s are done
+    if (tid == 0) rec = recs[tile];
+    if (tid < BR_TY)
+      reinterpret_cast<float*>(ty_s)[tid] = (float)(((double)(tg.j0 + tid) + 0.5 - tg.cj) * g.dx3);
+    __syncthreads();
     float ty[R];
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-      ty[r] = (float)(((double)(tg.j0 + warp * R + r) + 0.5 - tg.cj) * g.dx3);
-      acc_s[0][r][tid] = acc_s[1][r][tid] = acc_s[2][r][tid] = acc_s[3][r][tid] = 0.f;
+    for (int r = 0; r < R; r += 2) {
+      const float2 t = ty_s[(warp * R + r) / 2];
+      ty[r] = t.x;
+      ty[r + 1] = t.y;
     }
+#pragma unroll
+    for (int r = 0; r < R; ++r) acc_s[0][r][tid] = acc_s[1][r][tid] = acc_s[2][r][tid] = acc_s[3][r][tid] = 0.f;
     float2 TYP[NPK > 0 ? NPK : 1];
 #pragma unroll
     for (int q = 0; q < NPK; ++q) TYP[q] = make_float2(ty[PAIRED + 2 * q], ty[PAIRED + 2 * q + 1]);
-
-    __syncthreads();  // previous tile's readers of rec / lens_s are done
-    if (tid == 0) rec = recs[tile];
 
     for (int64_t base = 0; base < n; base += BR_LT) {
       float4 v[BR_LT / NT];
@@ -438,19 +501,37 @@ k_brute(Geo g, const double2* __restrict__ xy, const double* __restrict__ mass, 
         acc_s[3][r][tid] += e;
       }
     }
-    __syncthreads();  // rec visible
-
-    // ---- per-ray: smooth terms, sheet series, near corners, pixel
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
+    // ---- per-ray: smooth terms, sheet series, near corners, pixel; two rows at
+    // a time through the packed instructions, the roundings of brute_beta
+    const bool colok = col < tg.i1;
+    const uint32_t npx = (uint32_t)g.npix_x, npy = (uint32_t)g.npix_y;
+#pragma unroll 1
+    for (int r = 0; r < R; r += 2) {
       const int64_t row = tg.j0 + warp * R + r;
-      const bool inside = (col < tg.i1) && (row < tg.j1) && (row >= row0) && (row < row1);
-      float b1, b2;
-      brute_beta(g, rec, tx, ty[r], acc_s[0][r][tid], acc_s[1][r][tid], acc_s[2][r][tid], acc_s[3][r][tid], b1, b2);
-      uint32_t key = 0;
-      int64_t pix = -1;
-      const bool ok = inside && pixel_from_rel(g, rec.ix, rec.iy, b1, b2, key, pix);
-      bin_warp(counts, ok, key);
+      const float2 TY = ty_s[(warp * R + r) / 2], NTY = make_float2(-TY.x, -TY.y);
+      float2 PR = make_float2(0.f, 0.f), PI = make_float2(0.f, 0.f);
+#pragma unroll
+      for (int k = SHEET_TERMS - 1; k >= 0; --k) {
+        const float2 AR = __fadd2_rn(make_float2(rec.T[k][0], rec.T[k][0]), PR);
+        const float2 AI = __fadd2_rn(make_float2(rec.T[k][1], rec.T[k][1]), PI);
+        PR = __ffma2_rn(AR, TX2, __fmul2_rn(AI, NTY));
+        PI = __ffma2_rn(AR, TY, __fmul2_rn(AI, TX2));
+      }
+      float p1[2] = {PR.x, PR.y}, p2[2] = {PI.x, PI.y};
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const float tyr = j ? TY.y : TY.x;
+        for (int c = 0; c < rec.n_near; ++c) brute_corner(rec.near[c], tx, tyr, p1[j], p2[j]);
+        float b1, b2;
+        brute_sum(g, rec, tx, tyr, p1[j], p2[j], acc_s[0][r + j][tid], acc_s[1][r + j][tid], acc_s[2][r + j][tid],
+                  acc_s[3][r + j][tid], b1, b2);
+        const bool inside = colok && row + j < tg.j1 && row + j >= row0 && row + j < row1;
+        // pixel_from_rel in 32 bits: base pixels are within 1e9 (k_brute_setup)
+        const float f1 = floorf(b1 * g.inv_sx), f2 = floorf(b2 * g.inv_sy);
+        const uint32_t px = (uint32_t)rec.ix + (uint32_t)(int)f1, py = (uint32_t)rec.iy + (uint32_t)(int)f2;
+        const bool ok = inside && fabsf(f1) < 1.0e9f && fabsf(f2) < 1.0e9f && px < npx && py < npy;
+        bin_warp(counts, ok, py * npx + px);
+      }
     }
   }
 }

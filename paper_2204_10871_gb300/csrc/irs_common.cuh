@@ -153,6 +153,7 @@ struct irs_plan {
   size_t ws_bytes;
   double* d_msum;          // [1] sum of masses
   double* d_mpart;         // [MSUM_BLOCKS] partial sums
+  unsigned int* d_mdone;   // blocks of the mass sum that have finished; zero between sums
   irs::TileRec* d_tiles;   // [br_ntiles]
   int* d_status;           // sticky device error
   unsigned long long* d_queue;  // work counter of the ray pass, zeroed by the mass sum (NULL: none)
@@ -183,7 +184,7 @@ constexpr int MSUM_THREADS = 256;
 // into d_status otherwise).
 cudaError_t launch_mass_sum(const irs_plan_t* P, const double* mass, int64_t n, cudaStream_t s,
                             const double* xy = nullptr);
-cudaError_t launch_brute_setup(const irs_plan_t* P, cudaStream_t s);
+cudaError_t launch_brute_setup(const irs_plan_t* P, int64_t row0, int64_t row1, cudaStream_t s);
 cudaError_t launch_brute_map(const irs_plan_t* P, const double* xy, const double* mass, int64_t n,
                              int64_t row0, int64_t row1, uint32_t* counts, cudaStream_t s);
 cudaError_t launch_brute_dump(const irs_plan_t* P, const double* xy, const double* mass, int64_t n,

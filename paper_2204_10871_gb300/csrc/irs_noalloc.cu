@@ -35,6 +35,7 @@ constexpr int64_t NOALLOC_MAX_TILES = 49152;
 constexpr size_t OFF_MSUM = 0;
 constexpr size_t OFF_MPART = 256;
 constexpr size_t OFF_STATUS = OFF_MPART + ((sizeof(double) * irs::MSUM_BLOCKS + 255) & ~(size_t)255);
+constexpr size_t OFF_MDONE = OFF_STATUS + 128;  // zero-initialised, left zero by every mass sum
 constexpr size_t OFF_TILES = OFF_STATUS + 256;
 constexpr size_t SCRATCH_BYTES = OFF_TILES + sizeof(irs::TileRec) * NOALLOC_MAX_TILES;
 
@@ -115,6 +116,7 @@ extern "C" irs_status irs_make_map_brute_noalloc(const irs_params* params, const
   P.d_mpart = reinterpret_cast<double*>(scratch + OFF_MPART);
   P.d_status = reinterpret_cast<int*>(scratch + OFF_STATUS);
   P.d_tiles = reinterpret_cast<irs::TileRec*>(scratch + OFF_TILES);
+  P.d_mdone = reinterpret_cast<unsigned int*>(scratch + OFF_MDONE);
 
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   // the partial sums and tile records are rewritten in full by every call;
@@ -123,7 +125,7 @@ extern "C" irs_status irs_make_map_brute_noalloc(const irs_params* params, const
   const size_t npix = (size_t)p.npix_x * p.npix_y;
   if (cudaMemsetAsync(counts, 0, npix * sizeof(uint32_t), s) != cudaSuccess) return IRS_ERR_CUDA;
   if (irs::launch_mass_sum(&P, mass, n, s) != cudaSuccess) return IRS_ERR_CUDA;
-  if (irs::launch_brute_setup(&P, s) != cudaSuccess) return IRS_ERR_CUDA;
+  if (irs::launch_brute_setup(&P, 0, P.g.nry, s) != cudaSuccess) return IRS_ERR_CUDA;
   if (irs::launch_brute_map(&P, lens_xy, mass, n, 0, P.g.nry, counts, s) != cudaSuccess)
     return IRS_ERR_CUDA;
   if (mag && irs::launch_magnify(&P, counts, mag, s) != cudaSuccess) return IRS_ERR_CUDA;
