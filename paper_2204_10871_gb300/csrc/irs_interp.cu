@@ -495,9 +495,255 @@ __global__ void k_ip_sheet_table(Geo g, IpGeo ig, double2* __restrict__ sheet_d,
   sheet_near[rc] = (uint8_t)near;
 }
 
+// Centre term and base pixel of a cell from its series' first terms: acc[0..2]
+// (FP64, before the sheet's share when `sheet`), written to the record and the
+// first coefficients.
+__device__ __forceinline__ void finish_cell(const Geo& g, const IpGeo& ig, double ks, double zx, double zy, int64_t rc,
+                                            cd* acc, bool sheet, const double2* __restrict__ sheet_d,
+                                            const uint8_t* __restrict__ sheet_near, CellRec* __restrict__ recs,
+                                            float2* __restrict__ coef) {
+  const double kap = g.kappa_s + ks, h = ig.h;
+  CellRec r;
+  r.n_corner = 0;
+  r.pad_ = 0;
+  for (int q = 0; q < IP_MAX_CORNER; ++q) r.corner[q][0] = r.corner[q][1] = r.corner[q][2] = r.corner[q][3] = 0.f;
+  cd B;
+  if (sheet && g.plane == IRS_PLANE_CIRCLE) {
+    B = {(1.0 - g.kappa_s - g.gamma) * zx - ks * g.cx, -(1.0 - g.kappa_s + g.gamma) * zy + ks * g.cy};
+  } else {
+    if (sheet) {
+      // sheet: g(z) = kappa_* (z - 2 a2) + sum_c -i a_c (z - c) Log(z - c); adds
+      // g_k h^k.  a_c = +-kappa_* / pi, so the corner sums are kappa_* times a
+      // per-plan table (k_ip_sheet_table); corners near the cell go to the rays.
+      acc[0].re += ks * (zx - 2.0 * g.a2);
+      acc[0].im += ks * zy;
+      acc[1].re += ks * h;
+      if (ks != 0.0) {
+        const unsigned near = sheet_near[rc];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          if (!((near >> q) & 1u)) continue;
+          r.corner[r.n_corner][0] = (float)(zx - sheet_corner_x(g, q));
+          r.corner[r.n_corner][1] = (float)(zy - sheet_corner_y(g, q));
+          r.corner[r.n_corner][2] = (float)(ks / M_PI * sheet_corner_sign(q));
+          r.n_corner++;
+        }
+#pragma unroll
+        for (int k = 0; k < FIN_K64; ++k) {
+          const double2 t = sheet_d[rc * FIN_K64 + k];
+          acc[k].re += ks * t.x;
+          acc[k].im += ks * t.y;
+        }
+      }
+    }
+    B = {(1.0 - g.kappa_s - g.gamma) * zx, -(1.0 - g.kappa_s + g.gamma) * zy};
+  }
+  B.re += acc[0].re;
+  B.im += acc[0].im;
+  const double m1 = (1.0 - kap - g.gamma) * zx, m2 = (1.0 - kap + g.gamma) * zy;
+  double fx = floor((m1 - g.src_x0) / g.sx), fy = floor((m2 - g.src_y0) / g.sy);
+  fx = fmin(fmax(fx, -1.0e9), 1.0e9);
+  fy = fmin(fmax(fy, -1.0e9), 1.0e9);
+  r.ix = (int32_t)fx;
+  r.iy = (int32_t)fy;
+  split_df(B.re - (g.src_x0 + fx * g.sx), r.bx_hi, r.bx_lo);
+  split_df(-B.im - (g.src_y0 + fy * g.sy), r.by_hi, r.by_lo);
+  recs[rc] = r;
+#pragma unroll
+  for (int k = 0; k < FIN_K64; ++k) coef[rc * ig.K + k] = make_float2((float)acc[k].re, (float)acc[k].im);
+}
+
 // Per ray cell of [rc0, rc1): window P2L, M2L result, sheet series, centre
-// term, base pixel.  NF: FP32 series terms computed (k = FIN_K64 ...
-// FIN_K64 + NF - 1; at least K - FIN_K64).
+// term, base pixel (series mode).  NF: FP32 series terms computed (k = FIN_K64
+// ... FIN_K64 + NF - 1; at least K - FIN_K64).
+//
+// A warp takes four cells at a time, eight lanes each.  A cell's window lenses,
+// which lie in a few contiguous ranges of the sorted lists, are dealt to its
+// lanes, each of which computes one lens's powers (double-float reciprocal,
+// first terms, FP32 terms) into shared memory; then the lanes change places
+// and each sums some (cell, term) components over the eight lenses, in list
+// order -- the sums come out as if one thread had walked the window.  One
+// thread per cell was bound by that walk where cells are few (40 lenses of
+// ~500 instructions in a row): 67 us for 250 cells, 83 us for 2.1e4, 355 us for
+// 3.0e5 (paper-mid); now 20, 39 and 333 us.
+constexpr int FG_WARPS = 4;                 // warps per CTA
+constexpr int FG_CELLS = 32;                // cells per CTA: the FP64 end runs on one full warp (fewer for few cells)
+constexpr int FG_LANES = 8;                 // lanes per cell
+constexpr int FG_WMAX = 16;                 // largest direct window
+constexpr int FG_RANGES = 2 * FG_WMAX + 4;  // list ranges of a window
+
+template <int NF>
+__global__ void __launch_bounds__(32 * FG_WARPS, 6)
+k_ip_finalize_group(Geo g, IpGeo ig, const double* __restrict__ msum, const int32_t* __restrict__ start,
+                    const float4* __restrict__ pos_df, const float2* __restrict__ m_df,
+                    const float4* __restrict__ conv_d, const float2* __restrict__ conv_f,
+                    const double2* __restrict__ sheet_d, const float2* __restrict__ sheet_f,
+                    const uint8_t* __restrict__ sheet_near, CellRec* __restrict__ recs, float2* __restrict__ coef,
+                    int64_t rc0, int64_t rc1, int cta_cells) {
+  constexpr int NV = 2 * NF + 4 * FIN_K64;  // values per lens
+  constexpr int NS = (4 * 2 * NF + 31) / 32;  // FP32 sums per lane
+  __shared__ float val_s[FG_WARPS][NV][33];
+  __shared__ int from_s[FG_WARPS][4][FG_RANGES], off_s[FG_WARPS][4][FG_RANGES + 1];
+  __shared__ float2 sum_s[FG_CELLS][2 * FIN_K64];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t base = rc0 + (int64_t)blockIdx.x * cta_cells;
+  const int64_t ncells = (int64_t)ig.ncx * ig.ncy;
+  const double h = ig.h, inv_h = 1.0 / h;
+  const double ks = g.kstar_scale * msum[0];
+  const float inv_hf = (float)inv_h, ksf = (float)ks;
+  const bool table = g.plane != IRS_PLANE_CIRCLE && ks != 0.0;
+  const int K = ig.K, nsf = K - FIN_K64, W = ig.W, nr = 2 * W + 4;
+  const float2 ih_df = df_from_double(inv_h);
+  for (int grp = warp; grp < cta_cells / 4; grp += FG_WARPS) {
+    if (base + 4 * grp >= rc1) break;  // uniform over the warp
+    // ---- this lane's cell and the list ranges of its window: rows dy = -W ... W
+    // of cells x - W ... x + W, the middle three without their near columns
+    const int ci = lane >> 3, sub = lane & 7;
+    const int64_t rc = base + 4 * grp + ci;
+    const bool cell_on = rc < rc1;
+    const int cx = (int)(rc % ig.nrcx) + ig.ox, cy = (int)(rc / ig.nrcx) + ig.oy;
+    int total = 0;
+    for (int r0 = 0; r0 < nr; r0 += FG_LANES) {
+      const int r = r0 + sub;
+      int from = 0, len = 0;
+      if (cell_on && r < nr) {
+        int dy, xa = cx - W, xb = cx + W;
+        if (r < W - 1) dy = r - W;
+        else if (r < W + 5) {
+          dy = (r - (W - 1)) / 2 - 1;
+          if ((r - (W - 1)) & 1) xa = cx + 2; else xb = cx - 2;
+        } else dy = r - (W + 5) + 2;
+        const int y = cy + dy;
+        xa = max(xa, 0);
+        xb = min(xb, ig.ncx - 1);
+        if (y >= 0 && y < ig.ncy && xa <= xb) {
+          from = start[(int64_t)y * ig.ncx + xa];
+          len = start[(int64_t)y * ig.ncx + xb + 1] - from;
+        }
+      }
+      int inc = len;
+#pragma unroll
+      for (int d = 1; d < FG_LANES; d <<= 1) {
+        const int v = __shfl_up_sync(0xFFFFFFFFu, inc, d, FG_LANES);
+        if (sub >= d) inc += v;
+      }
+      if (r < nr) {
+        from_s[warp][ci][r] = from;
+        off_s[warp][ci][r] = total + inc - len;
+      }
+      total += __shfl_sync(0xFFFFFFFFu, inc, FG_LANES - 1, FG_LANES);
+    }
+    if (sub == 0) off_s[warp][ci][nr] = total;
+    __syncwarp();
+    const double zx = ig.gx0 + (cx + 0.5) * h, zy = ig.gy0 + (cy + 0.5) * h;
+    const float2 zx_df = df_from_double(zx), zy_df = df_from_double(zy);
+    // ---- sums this lane keeps: FP32 component j of cell c for index lane + 32 i,
+    // and one double-float component of a cell for lanes < 24
+    float accf[NS];
+#pragma unroll
+    for (int i = 0; i < NS; ++i) accf[i] = 0.f;
+    float2 accd = make_float2(0.f, 0.f);
+    const int dc = lane / (2 * FIN_K64), dj = lane % (2 * FIN_K64);  // double-float sum: cell, component
+    int steps = (total + FG_LANES - 1) / FG_LANES;
+#pragma unroll
+    for (int d = FG_LANES; d < 32; d <<= 1) steps = max(steps, __shfl_xor_sync(0xFFFFFFFFu, steps, d));
+    int r = 0;
+    float4 next_q = make_float4(0.f, 0.f, 0.f, 0.f);  // the lane's next lens, loaded a step ahead
+    float2 next_m = make_float2(0.f, 0.f);
+    auto load = [&](int t) {
+      if (t >= total) return;
+      while (t >= off_s[warp][ci][r + 1]) ++r;
+      const int p = from_s[warp][ci][r] + (t - off_s[warp][ci][r]);
+      next_q = pos_df[p];
+      next_m = m_df[p];
+    };
+    load(sub);
+    for (int step = 0; step < steps; ++step) {
+      const int t = step * FG_LANES + sub;
+      const float4 q4 = next_q;
+      const float2 m2 = next_m;
+      load(t + FG_LANES);
+      if (t < total) {
+        const float2 dre = df_mul(df_sub(make_float2(q4.x, q4.y), zx_df), ih_df);
+        const float2 dim = df_mul(df_sub(make_float2(q4.z, q4.w), zy_df), ih_df);
+        const float4 inv = dfc_recip(dre, dim);
+        float4 pw = dfc_scale(inv, m2);  // + m d^-(k+1)
+#pragma unroll
+        for (int k = 0; k < FIN_K64; ++k) {
+          val_s[warp][4 * k][lane] = pw.x;
+          val_s[warp][4 * k + 1][lane] = pw.y;
+          val_s[warp][4 * k + 2][lane] = pw.z;
+          val_s[warp][4 * k + 3][lane] = pw.w;
+          pw = dfc_mul(pw, inv);
+        }
+        const float2 invf = make_float2(inv.x, inv.z);
+        float2 pf = make_float2(pw.x, pw.z);
+#pragma unroll
+        for (int k = 0; k < NF; ++k) {
+          val_s[warp][4 * FIN_K64 + 2 * k][lane] = pf.x;
+          val_s[warp][4 * FIN_K64 + 2 * k + 1][lane] = pf.y;
+          pf = cmulf(pf, invf);
+        }
+      } else {  // no lens: zeros leave every sum as it is
+#pragma unroll
+        for (int v = 0; v < NV; ++v) val_s[warp][v][lane] = 0.f;
+      }
+      __syncwarp();
+      if (lane < 4 * 2 * FIN_K64) {
+#pragma unroll
+        for (int i = 0; i < FG_LANES; ++i)
+          accd = df_add(accd, make_float2(val_s[warp][2 * dj][dc * FG_LANES + i], val_s[warp][2 * dj + 1][dc * FG_LANES + i]));
+      }
+#pragma unroll
+      for (int s = 0; s < NS; ++s) {
+        const int idx = lane + 32 * s, c = idx / (2 * NF), j = idx - c * (2 * NF);
+        if (4 * 2 * NF % 32 == 0 || c < 4) {
+          const float* v = &val_s[warp][4 * FIN_K64 + j][c * FG_LANES];
+#pragma unroll
+          for (int i = 0; i < FG_LANES; ++i) accf[s] += v[i];
+        }
+      }
+      __syncwarp();
+    }
+    if (lane < 4 * 2 * FIN_K64) sum_s[4 * grp + dc][dj] = accd;
+    // ---- terms k >= FIN_K64: M2L result, 1/h, sheet
+#pragma unroll
+    for (int s = 0; s < NS; ++s) {
+      const int idx = lane + 32 * s, c = idx / (2 * NF), j = idx - c * (2 * NF), k = FIN_K64 + (j >> 1);
+      const int64_t crc = base + 4 * grp + c;
+      if (c < 4 && crc < rc1 && k < K) {
+        float v = accf[s];
+        const int64_t cell = (int64_t)((int)(crc / ig.nrcx) + ig.oy) * ig.ncx + (int)(crc % ig.nrcx) + ig.ox;
+        if (k < IP_KF) v += reinterpret_cast<const float*>(conv_f + (int64_t)(k - IP_KD) * ncells + cell)[j & 1];
+        v *= inv_hf;
+        if (table) v = fmaf(ksf, reinterpret_cast<const float*>(sheet_f + crc * nsf + (k - FIN_K64))[j & 1], v);
+        reinterpret_cast<float*>(coef + crc * K + k)[j & 1] = v;
+      }
+    }
+  }
+  __syncthreads();
+  // ---- the FP64 end, one lane per cell
+  const int64_t rc = base + threadIdx.x;
+  if ((int)threadIdx.x >= cta_cells || rc >= rc1) return;
+  const int cx = (int)(rc % ig.nrcx) + ig.ox, cy = (int)(rc / ig.nrcx) + ig.oy;
+  const int64_t c = (int64_t)cy * ig.ncx + cx;
+  const double zx = ig.gx0 + (cx + 0.5) * h, zy = ig.gy0 + (cy + 0.5) * h;
+  cd acc[FIN_K64];
+#pragma unroll
+  for (int k = 0; k < FIN_K64; ++k) {
+    acc[k] = {df_to_double(sum_s[threadIdx.x][2 * k]), df_to_double(sum_s[threadIdx.x][2 * k + 1])};
+    static_assert(IP_KD == FIN_K64, "the M2L's double-float terms are the FP64 ones");
+    const float4 v = conv_d[(int64_t)k * ncells + c];
+    acc[k].re += df_to_double(dfc_re(v));
+    acc[k].im += df_to_double(dfc_im(v));
+    acc[k].re *= inv_h;
+    acc[k].im *= inv_h;
+  }
+  finish_cell(g, ig, ks, zx, zy, rc, acc, true, sheet_d, sheet_near, recs, coef);
+}
+
+// The same for learned far fields and for windows wider than FG_WMAX cells: one
+// thread per cell.
 template <int NF>
 __global__ void __launch_bounds__(64)
 k_ip_finalize(Geo g, IpGeo ig, const double* __restrict__ msum, const int32_t* __restrict__ start,
@@ -639,14 +885,7 @@ k_ip_finalize(Geo g, IpGeo ig, const double* __restrict__ msum, const int32_t* _
   }
 
   const double ks = g.kstar_scale * msum[0];
-  const double kap = g.kappa_s + ks;
-  CellRec r;
-  r.n_corner = 0;
-  r.pad_ = 0;
-  for (int q = 0; q < IP_MAX_CORNER; ++q) r.corner[q][0] = r.corner[q][1] = r.corner[q][2] = r.corner[q][3] = 0.f;
-  cd B;
   if (learned) {
-    const double ks0 = g.kstar_scale * msum[0];
 #pragma unroll
     for (int k = 0; k < MLP_KFF; ++k) {
       if (k >= K) break;
@@ -659,61 +898,24 @@ k_ip_finalize(Geo g, IpGeo ig, const double* __restrict__ msum, const int32_t* _
         accf[k - FIN_K64].y -= u.y;
       }
     }
-    acc[0].re -= ks0 * zx;  // kappa_* conj(z_C)
-    acc[0].im += ks0 * zy;
-    B = {(1.0 - g.kappa_s - g.gamma) * zx, -(1.0 - g.kappa_s + g.gamma) * zy};
-  } else if (g.plane == IRS_PLANE_CIRCLE) {
-    B = {(1.0 - g.kappa_s - g.gamma) * zx - ks * g.cx, -(1.0 - g.kappa_s + g.gamma) * zy + ks * g.cy};
-  } else {
-    // sheet: g(z) = kappa_* (z - 2 a2) + sum_c -i a_c (z - c) Log(z - c); adds
-    // g_k h^k.  a_c = +-kappa_* / pi, so the corner sums are kappa_* times a
-    // per-plan table (k_ip_sheet_table); corners near the cell go to the rays.
-    acc[0].re += ks * (zx - 2.0 * g.a2);
+    acc[0].re -= ks * zx;  // kappa_* conj(z_C)
     acc[0].im += ks * zy;
-    acc[1].re += ks * h;
-    if (ks != 0.0) {
-      const unsigned near = sheet_near[rc];
+  } else if (g.plane != IRS_PLANE_CIRCLE && ks != 0.0) {
+    const int nsf = K - FIN_K64;
+    const float ksf = (float)ks;
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        if (!((near >> q) & 1u)) continue;
-        r.corner[r.n_corner][0] = (float)(zx - sheet_corner_x(g, q));
-        r.corner[r.n_corner][1] = (float)(zy - sheet_corner_y(g, q));
-        r.corner[r.n_corner][2] = (float)(ks / M_PI * sheet_corner_sign(q));
-        r.n_corner++;
-      }
-#pragma unroll
-      for (int k = 0; k < FIN_K64; ++k) {
-        const double2 t = sheet_d[rc * FIN_K64 + k];
-        acc[k].re += ks * t.x;
-        acc[k].im += ks * t.y;
-      }
-      const int nsf = K - FIN_K64;
-      const float ksf = (float)ks;
-#pragma unroll
-      for (int k = 0; k < NF; ++k) {
-        if (k >= nsf) break;
-        const float2 t = sheet_f[rc * nsf + k];
-        accf[k].x = fmaf(ksf, t.x, accf[k].x);
-        accf[k].y = fmaf(ksf, t.y, accf[k].y);
-      }
+    for (int k = 0; k < NF; ++k) {
+      if (k >= nsf) break;
+      const float2 t = sheet_f[rc * nsf + k];
+      accf[k].x = fmaf(ksf, t.x, accf[k].x);
+      accf[k].y = fmaf(ksf, t.y, accf[k].y);
     }
-    B = {(1.0 - g.kappa_s - g.gamma) * zx, -(1.0 - g.kappa_s + g.gamma) * zy};
   }
-  B.re += acc[0].re;
-  B.im += acc[0].im;
-  const double m1 = (1.0 - kap - g.gamma) * zx, m2 = (1.0 - kap + g.gamma) * zy;
-  double fx = floor((m1 - g.src_x0) / g.sx), fy = floor((m2 - g.src_y0) / g.sy);
-  fx = fmin(fmax(fx, -1.0e9), 1.0e9);
-  fy = fmin(fmax(fy, -1.0e9), 1.0e9);
-  r.ix = (int32_t)fx;
-  r.iy = (int32_t)fy;
-  split_df(B.re - (g.src_x0 + fx * g.sx), r.bx_hi, r.bx_lo);
-  split_df(-B.im - (g.src_y0 + fy * g.sy), r.by_hi, r.by_lo);
-  recs[rc] = r;
+  finish_cell(g, ig, ks, zx, zy, rc, acc, !learned, sheet_d, sheet_near, recs, coef);
 #pragma unroll
-  for (int k = 0; k < FIN_K64 + NF; ++k) {
-    if (k >= K) break;
-    coef[rc * K + k] = k < FIN_K64 ? make_float2((float)acc[k].re, (float)acc[k].im) : accf[k - FIN_K64];
+  for (int k = 0; k < NF; ++k) {
+    if (FIN_K64 + k >= K) break;
+    coef[rc * K + FIN_K64 + k] = accf[k];
   }
 }
 
@@ -1714,16 +1916,20 @@ irs_status build_cells_and_far(irs_plan_t* P, const double* xy, const double* ma
   mark(P, EV_FIN, s);
   if (rc1 > rc0) {
     // the default K = 24 needs 21 FP32 terms; larger K the full FIN_K32
-    const unsigned nb = (unsigned)((rc1 - rc0 + 63) / 64);
-    if (ig.K - FIN_K64 <= 21)
-      k_ip_finalize<21><<<nb, 64, 0, s>>>(P->g, ig, P->d_msum, S->cell_start, S->lens_pos, S->lens_m,
-                                          S->lens_pdf, S->lens_mdf, S->conv_d, S->conv_f, far, S->sheet_d,
-                                          S->sheet_f, S->sheet_near, S->recs, S->coef, rc0, rc1);
-    else
-      k_ip_finalize<FIN_K32><<<nb, 64, 0, s>>>(P->g, ig, P->d_msum, S->cell_start, S->lens_pos, S->lens_m,
-                                               S->lens_pdf, S->lens_mdf, S->conv_d, S->conv_f, far,
-                                               S->sheet_d, S->sheet_f, S->sheet_near, S->recs, S->coef, rc0,
-                                               rc1);
+    const bool few = ig.K - FIN_K64 <= 21;
+    if (!far.active && ig.W <= FG_WMAX) {
+      const int cta_cells = rc1 - rc0 <= 4 * FG_CELLS * (int64_t)P->num_sms ? FG_CELLS / 2 : FG_CELLS;
+      const unsigned nb = (unsigned)((rc1 - rc0 + cta_cells - 1) / cta_cells);
+      auto* kern = few ? k_ip_finalize_group<21> : k_ip_finalize_group<FIN_K32>;
+      kern<<<nb, 32 * FG_WARPS, 0, s>>>(P->g, ig, P->d_msum, S->cell_start, S->lens_pdf, S->lens_mdf, S->conv_d,
+                                        S->conv_f, S->sheet_d, S->sheet_f, S->sheet_near, S->recs, S->coef, rc0, rc1, cta_cells);
+    } else {
+      const unsigned nb = (unsigned)((rc1 - rc0 + 63) / 64);
+      auto* kern = few ? k_ip_finalize<21> : k_ip_finalize<FIN_K32>;
+      kern<<<nb, 64, 0, s>>>(P->g, ig, P->d_msum, S->cell_start, S->lens_pos, S->lens_m, S->lens_pdf, S->lens_mdf,
+                             S->conv_d, S->conv_f, far, S->sheet_d, S->sheet_f, S->sheet_near, S->recs, S->coef, rc0,
+                             rc1);
+    }
   }
   IP_TRY(cudaGetLastError());
   mark(P, EV_FAR, s);
