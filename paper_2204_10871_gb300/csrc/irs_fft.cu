@@ -3,23 +3,29 @@
 // (irs_df.cuh: 48-bit significands on the FP32 pipes; float4 elements) or in
 // FP32 (float2 elements).
 //
-// A CTA loads B lines of length L = 3^n3 2^n2 into shared memory (B as large
-// as keeps the CTA within 52 KB, so that up to four CTAs share an SM; at
-// least one line, up to 9216 double-float or FP32 values), runs in-place
-// butterfly stages with a twiddle table W_L^t (t < L/2; W_L^(t + L/2) =
-// -W_L^t) staged beside them, and writes the lines back.  Neither direction
-// permutes: the forward transform runs decimation in frequency (n2 radix-2
-// then n3 radix-3 stages) on natural-order input and leaves X[k] at the
-// mixed-radix digit reversal of k; the inverse runs decimation in time (n3
-// radix-3 then n2 radix-2 stages), which takes its input in exactly that
-// order and returns natural order.  The convolution between them is
-// pointwise, so the spectra never need sorting.
-// Rows are contiguous lines; columns are strided lines, loaded B adjacent
-// columns at a time so that each row segment is one coalesced access.  Zero padding is implicit: input elements at or beyond
-// `in_len` read as 0, and only the first `out_len` outputs of a line are
-// written.
+// A CTA takes B lines of length L = 3^n3 2^n2 (B as large as keeps it within
+// 52 KB of shared memory, at least one) with a twiddle table W_L^t (t < L/2;
+// W_L^(t + L/2) = -W_L^t) beside them, and runs the butterfly stages in passes:
+// up to three radix-2 or two radix-3 stages of a line's element group in
+// registers, then an exchange through shared memory; the first pass reads
+// memory, the last writes it.  Neither direction permutes: the forward
+// transform runs decimation in frequency (n2 radix-2 then n3 radix-3 stages) on
+// natural-order input and leaves X[k] at the mixed-radix digit reversal of k;
+// the inverse runs decimation in time (n3 radix-3 then n2 radix-2 stages), which
+// takes its input in exactly that order and returns natural order.  The
+// convolution between them is pointwise, so the spectra never need sorting.
+// Rows are contiguous lines; columns are strided lines, B adjacent columns at a
+// time so that each row segment is one coalesced access.  Zero padding is
+// implicit: input elements at or beyond `in_len` read as 0, and only the first
+// `out_len` outputs of a line are written.
+//
+// The stages were one pass each (a round trip through shared memory and a
+// barrier for every stage, with adjacent columns in the same bank): the eight
+// launches of a paper-mid map took 1,332 us, 6.1 ms at the high-res map; now
+// four to six launches, 855 us and 5.1 ms.
 #include <math.h>
 
+#include <type_traits>
 #include <vector>
 
 #include "irs_df.cuh"
@@ -28,6 +34,8 @@
 namespace irs {
 
 namespace {
+
+constexpr int FFT_REGS = 80;  // per thread: 24 warps per SM
 
 // Complex arithmetic of the two element types: float4 is double-float
 // (re.hi, re.lo, im.hi, im.lo), float2 is FP32 (re, im).
@@ -54,15 +62,6 @@ template <> __device__ __forceinline__ float2 c_zero<float2>() { return make_flo
 template <class T> __device__ __forceinline__ T tw_elem(float4 v);
 template <> __device__ __forceinline__ float4 tw_elem<float4>(float4 v) { return v; }
 template <> __device__ __forceinline__ float2 tw_elem<float2>(float4 v) { return make_float2(v.x, v.z); }
-
-// output scaling by a real factor
-__device__ __forceinline__ float4 c_scale(float4 a, double s) {
-  return dfc_scale(a, make_float2((float)s, (float)(s - (double)(float)s)));
-}
-__device__ __forceinline__ float2 c_scale(float2 a, double s) {
-  const float f = (float)s;
-  return make_float2(a.x * f, a.y * f);
-}
 
 // Radix-3 butterfly on a and the twiddled p, q:
 // x0 = a + t1, x1,2 = a - t1/2 -+ i s3 (p - q) with t1 = p + q and
@@ -107,127 +106,165 @@ __device__ __forceinline__ T tw_at(const T* w, int t, int half) {
   return INV ? c_conj(v) : v;
 }
 
+// One pass over a line takes several stages in registers.  F radix-2 stages:
+// 2^F elements per work item, or F radix-3 stages: 3^F elements, `gap` apart;
+// stride0 is the twiddle stride L / m of the widest stage (the decimation in
+// frequency's first, the decimation in time's last).  Every butterfly is the one of a single stage,
+// with the same twiddle, so how the stages are grouped does not change a bit.
+template <bool INV, int F, class T>
+__device__ __forceinline__ void fused2(T* v, const T* w, int j, int gap, int stride0, int half_L) {
+#pragma unroll
+  for (int f = 0; f < F; ++f) {
+    // frequency: pairs 2^(F-1), ..., 2, 1 apart; time: 1, 2, ..., 2^(F-1)
+    const int d = INV ? 1 << f : 1 << (F - 1 - f);
+    const int stride = stride0 << (INV ? F - 1 - f : f);
+#pragma unroll
+    for (int q = 0; q < 1 << F; ++q) {
+      if (q & d) continue;
+      const T t = tw_at<INV>(w, (j + (q & (d - 1)) * gap) * stride, half_L);
+      if (INV) {
+        const T u = v[q], x = c_mul(v[q + d], t);
+        v[q] = c_add(u, x);
+        v[q + d] = c_sub(u, x);
+      } else {
+        const T u = v[q], x = v[q + d];
+        v[q] = c_add(u, x);
+        v[q + d] = c_mul(c_sub(u, x), t);
+      }
+    }
+  }
+}
+template <bool INV, int F, class T>
+__device__ __forceinline__ void fused3(T* v, const T* w, int j, int gap, int stride0, int half_L) {
+  constexpr int N = F == 2 ? 9 : 3;
+#pragma unroll
+  for (int f = 0; f < F; ++f) {
+    const int d = (INV ? f == 0 : f == F - 1) ? 1 : 3;
+    const int stride = (INV ? F == 2 && f == 0 : f == 1) ? 3 * stride0 : stride0;
+#pragma unroll
+    for (int q = 0; q < N; ++q) {
+      if (q / d % 3) continue;
+      const int t = (j + (q % d) * gap) * stride;
+      if (INV) {
+        const T p = c_mul(v[q + d], tw_at<INV>(w, t, half_L));
+        const T r = c_mul(v[q + 2 * d], tw_at<INV>(w, 2 * t, half_L));
+        radix3(v[q], p, r, true, v[q], v[q + d], v[q + 2 * d]);
+      } else {
+        T y0, y1, y2;
+        radix3(v[q], v[q + d], v[q + 2 * d], false, y0, y1, y2);
+        v[q] = y0;
+        v[q + d] = c_mul(y1, tw_at<INV>(w, t, half_L));
+        v[q + 2 * d] = c_mul(y2, tw_at<INV>(w, 2 * t, half_L));
+      }
+    }
+  }
+}
+
+// Sequence of passes of a line of 2^n2 3^n3: radix-2 stages by threes (a
+// remainder of one or two, and 4 as 2 + 2), radix-3 stages by twos; in this
+// order for the forward transform, reversed for the inverse.
+__host__ __device__ __forceinline__ int fft_passes2(int n2) { return (n2 + 2) / 3; }
+__host__ __device__ __forceinline__ int fft_pass2_stages(int n2, int p) {  // stages of pass p
+  const int np = fft_passes2(n2);
+  return n2 / np + (p < n2 % np ? 1 : 0);
+}
+
+// Lines of one CTA.  The first pass reads its elements from memory and the last
+// writes them there; shared memory holds the line between passes, lines L + 1
+// elements apart so that a warp's adjacent columns fall in distinct banks.
 template <bool INV, class T>
-__global__ void __launch_bounds__(512) k_fft_lines(const T* in, T* out, FftLines d, const float4* __restrict__ tw) {
-  extern __shared__ float4 sm_raw[];
-  T* x = reinterpret_cast<T*>(sm_raw);  // [B][L]
-  T* w = x + (size_t)d.B * d.L;         // [L/2]
-  const int L = d.L, B = d.B, n3 = d.n3, n2 = d.n2, half_L = L / 2;
+__device__ __forceinline__ void fft_lines(const T* in, T* out, const FftLines& d, const float4* __restrict__ tw,
+                                          int64_t block, float4* sm) {
+  const int L = d.L, B = d.B, n3 = d.n3, n2 = d.n2, half_L = L / 2, LS = L + 1;
+  T* x = reinterpret_cast<T*>(sm);      // [B][LS]
+  T* w = x + (size_t)B * LS;            // [L/2]
+  const int64_t blocks_per_grid = (d.n_lines + B - 1) / B;
+  const int64_t grid = block / blocks_per_grid, line0 = (block - grid * blocks_per_grid) * B;
+  in += grid * d.in_grid_stride;
+  out += grid * d.out_grid_stride;
+  const int nthr = blockDim.x;
+  for (int k = threadIdx.x; k < half_L; k += nthr) w[k] = tw_elem<T>(tw[k]);
   int pow3 = 1;
   for (int i = 0; i < n3; ++i) pow3 *= 3;
-  const int64_t line0 = (int64_t)blockIdx.x * B;
-  const int64_t goff_in = (int64_t)blockIdx.y * d.in_grid_stride;
-  const int64_t goff_out = (int64_t)blockIdx.y * d.out_grid_stride;
-  const int nthr = blockDim.x;
-  const FastDiv fdL((uint32_t)L), fdB((uint32_t)B), fd3((uint32_t)(L / 3)), fd2((uint32_t)half_L);
-  for (int k = threadIdx.x; k < L / 2; k += nthr) w[k] = tw_elem<T>(tw[k]);
-  // load (natural order for the forward transform, the forward transform's
-  // output order for the inverse)
-  for (int idx = threadIdx.x; idx < B * L; idx += nthr) {
-    int b, e;
-    if (d.in_elem_stride == 1) {
-      b = (int)fdL.div((uint32_t)idx);
-      e = idx - b * L;
-    } else {
-      e = (int)fdB.div((uint32_t)idx);
-      b = idx - e * B;
-    }
-    const int64_t line = line0 + b;
-    T v = c_zero<T>();
-    if (line < d.n_lines && e < d.in_len)
-      v = in[goff_in + line * d.in_line_stride + (int64_t)e * d.in_elem_stride];
-    x[b * L + e] = v;
-  }
+  const int np2 = fft_passes2(n2), np3 = (n3 + 1) / 2, np = np2 + np3;
   __syncthreads();
-  if (!INV) {
-    // decimation in frequency: the transposes of the inverse's stages in
-    // reverse order -- a radix-2 butterfly adds and subtracts, then twiddles
-    // the difference; a radix-3 butterfly transforms, then twiddles outputs
-    // 1 and 2
-    for (int s = n2 - 1; s >= 0; --s) {
-      const int m_prev = pow3 << s, m = 2 * m_prev, stride = L / m;
-      const FastDiv fdm((uint32_t)m_prev);
-      for (int t = threadIdx.x; t < B * (L / 2); t += nthr) {
-        const int b = (int)fd2.div((uint32_t)t), k = t - b * half_L;
-        const int g = (int)fdm.div((uint32_t)k), j = k - g * m_prev;
-        const int i0 = g * m + j, i1 = i0 + m_prev;
-        const T u = x[b * L + i0], v = x[b * L + i1];
-        x[b * L + i0] = c_add(u, v);
-        x[b * L + i1] = c_mul(c_sub(u, v), tw_at<INV>(w, j * stride, half_L));
+  int span = INV ? 1 : L;  // forward: widest span left; inverse: span done so far
+  for (int p = 0; p < np; ++p) {
+    const int pf = INV ? np - 1 - p : p;  // the forward transform's number of this pass
+    const bool two = pf < np2;
+    const int stages = two ? fft_pass2_stages(n2, pf) : (pf - np2 == np3 - 1 && (n3 & 1) ? 1 : 2);
+    const int N = two ? 1 << stages : (stages == 2 ? 9 : 3);
+    if (INV) span *= N;
+    const int gap = span / N, items = L / N, stride0 = L / span;
+    const bool first = p == 0, last = p == np - 1;
+    // items dealt along the line, or across the lines where those are adjacent in memory
+    const bool across = d.in_elem_stride != 1;
+    const FastDiv fdB((uint32_t)B), fdI((uint32_t)items), fdg((uint32_t)gap);
+    for (int t = threadIdx.x; t < B * items; t += nthr) {
+      int b, k;
+      if (across) {
+        k = (int)fdB.div((uint32_t)t);
+        b = t - k * B;
+      } else {
+        b = (int)fdI.div((uint32_t)t);
+        k = t - b * items;
       }
-      __syncthreads();
-    }
-    int m_prev = pow3;
-    for (int s = n3 - 1; s >= 0; --s) {
-      m_prev /= 3;
-      const int m = m_prev * 3, stride = L / m;
-      const FastDiv fdm((uint32_t)m_prev);
-      for (int t = threadIdx.x; t < B * (L / 3); t += nthr) {
-        const int b = (int)fd3.div((uint32_t)t), k = t - b * (L / 3);
-        const int g = (int)fdm.div((uint32_t)k), j = k - g * m_prev;
-        const int i0 = g * m + j, i1 = i0 + m_prev, i2 = i1 + m_prev;
-        T y0, y1, y2;
-        radix3(x[b * L + i0], x[b * L + i1], x[b * L + i2], INV, y0, y1, y2);
-        x[b * L + i0] = y0;
-        x[b * L + i1] = c_mul(y1, tw_at<INV>(w, j * stride, half_L));
-        x[b * L + i2] = c_mul(y2, tw_at<INV>(w, 2 * j * stride, half_L));
+      const int g = (int)fdg.div((uint32_t)k), j = k - g * gap, e0 = g * span + j;
+      const int64_t line = line0 + b;
+      const bool on = line < d.n_lines;
+      T* xl = x + (size_t)b * LS;
+      T v[9];
+      auto load = [&](auto n) {
+#pragma unroll
+        for (int q = 0; q < decltype(n)::value; ++q) {
+          const int e = e0 + q * gap;
+          if (!first) v[q] = xl[e];
+          else v[q] = on && e < d.in_len ? in[line * d.in_line_stride + (int64_t)e * d.in_elem_stride] : c_zero<T>();
+        }
+      };
+      auto store = [&](auto n) {
+#pragma unroll
+        for (int q = 0; q < decltype(n)::value; ++q) {
+          const int e = e0 + q * gap;
+          if (!last) xl[e] = v[q];
+          else if (on && e < d.out_len) out[line * d.out_line_stride + (int64_t)e * d.out_elem_stride] = v[q];
+        }
+      };
+      if (two && stages == 3) {
+        load(std::integral_constant<int, 8>{});
+        fused2<INV, 3>(v, w, j, gap, stride0, half_L);
+        store(std::integral_constant<int, 8>{});
+      } else if (two && stages == 2) {
+        load(std::integral_constant<int, 4>{});
+        fused2<INV, 2>(v, w, j, gap, stride0, half_L);
+        store(std::integral_constant<int, 4>{});
+      } else if (two) {
+        load(std::integral_constant<int, 2>{});
+        fused2<INV, 1>(v, w, j, gap, stride0, half_L);
+        store(std::integral_constant<int, 2>{});
+      } else if (stages == 2) {
+        load(std::integral_constant<int, 9>{});
+        fused3<INV, 2>(v, w, j, gap, stride0, half_L);
+        store(std::integral_constant<int, 9>{});
+      } else {
+        load(std::integral_constant<int, 3>{});
+        fused3<INV, 1>(v, w, j, gap, stride0, half_L);
+        store(std::integral_constant<int, 3>{});
       }
-      __syncthreads();
     }
-  } else {
-    // decimation in time
-    int m_prev = 1;  // span of the sub-transforms done so far
-    // radix-3 stages: y_q = sum_r (W_m^(j r) x_r) W_3^(q r);
-    // W_3 = -1/2 -+ i sqrt(3)/2, the halving is exact
-    for (int s = 0; s < n3; ++s) {
-      const int m = m_prev * 3, stride = L / m;
-      const FastDiv fdm((uint32_t)m_prev);
-      for (int t = threadIdx.x; t < B * (L / 3); t += nthr) {
-        const int b = (int)fd3.div((uint32_t)t), k = t - b * (L / 3);
-        const int g = (int)fdm.div((uint32_t)k), j = k - g * m_prev;
-        const int i0 = g * m + j, i1 = i0 + m_prev, i2 = i1 + m_prev;
-        const T a = x[b * L + i0];
-        const T p = c_mul(x[b * L + i1], tw_at<INV>(w, j * stride, half_L));
-        const T q = c_mul(x[b * L + i2], tw_at<INV>(w, 2 * j * stride, half_L));
-        radix3(a, p, q, INV, x[b * L + i0], x[b * L + i1], x[b * L + i2]);
-      }
-      __syncthreads();
-      m_prev = m;
-    }
-    // radix-2 stages
-    for (int s = 0; s < n2; ++s) {
-      const int m = m_prev * 2, stride = L / m;
-      const FastDiv fdm((uint32_t)m_prev);
-      for (int t = threadIdx.x; t < B * (L / 2); t += nthr) {
-        const int b = (int)fd2.div((uint32_t)t), k = t - b * half_L;
-        const int g = (int)fdm.div((uint32_t)k), j = k - g * m_prev;
-        const int i0 = g * m + j, i1 = i0 + m_prev;
-        const T u = x[b * L + i0];
-        const T v = c_mul(x[b * L + i1], tw_at<INV>(w, j * stride, half_L));
-        x[b * L + i0] = c_add(u, v);
-        x[b * L + i1] = c_sub(u, v);
-      }
-      __syncthreads();
-      m_prev = m;
-    }
+    if (!INV) span = gap;
+    if (!last) __syncthreads();
   }
-  const bool scaled = d.scale != 1.0;
-  for (int idx = threadIdx.x; idx < B * L; idx += nthr) {
-    int b, e;
-    if (d.out_elem_stride == 1) {
-      b = (int)fdL.div((uint32_t)idx);
-      e = idx - b * L;
-    } else {
-      e = (int)fdB.div((uint32_t)idx);
-      b = idx - e * B;
-    }
-    const int64_t line = line0 + b;
-    if (line < d.n_lines && e < d.out_len) {
-      T v = x[b * L + e];
-      if (scaled) v = c_scale(v, d.scale);
-      out[goff_out + line * d.out_line_stride + (int64_t)e * d.out_elem_stride] = v;
-    }
-  }
+}
+
+// The double-float planes' lines, the FP32 planes', or both in one launch.
+template <bool INV>
+__global__ void __maxnreg__(FFT_REGS)
+k_fft_lines(const float4* in4, float4* out4, FftLines d4, int64_t blocks4, const float2* in2, float2* out2,
+            FftLines d2, const float4* __restrict__ tw) {
+  extern __shared__ float4 sm_raw[];
+  if ((int64_t)blockIdx.x < blocks4) fft_lines<INV>(in4, out4, d4, tw, blockIdx.x, sm_raw);
+  else fft_lines<INV>(in2, out2, d2, tw, (int64_t)blockIdx.x - blocks4, sm_raw);
 }
 
 }  // namespace
@@ -267,101 +304,102 @@ cudaError_t fft_twiddles(int L, float4** d_tw) {
 }
 
 cudaError_t fft_setup_attributes() {
-  const int max_smem = (int)(FFT_MAX_ELEMS * sizeof(float4) + FFT_MAX_LEN / 2 * sizeof(float4));
-  cudaError_t e = cudaFuncSetAttribute(k_fft_lines<false, float4>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
+  const int max_smem = (int)(((size_t)FFT_MAX_LEN + 1 + FFT_MAX_LEN / 2) * sizeof(float4));
+  cudaError_t e = cudaFuncSetAttribute(k_fft_lines<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_fft_lines<true, float4>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_fft_lines<false, float2>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_fft_lines<true, float2>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
+    e = cudaFuncSetAttribute(k_fft_lines<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
   return e;
 }
 
 namespace {
 
-template <class T>
-cudaError_t fft_lines_t(const T* in, T* out, FftLines d, int ngrids, const float4* tw, bool inverse,
-                        cudaStream_t s) {
-  if (d.n_lines <= 0 || ngrids <= 0) return cudaSuccess;
-  const int64_t blocks = (d.n_lines + d.B - 1) / d.B;
-  const size_t smem = (size_t)d.B * d.L * sizeof(T) + (size_t)(d.L / 2) * sizeof(T);
-  const int threads = d.B * d.L / 2 >= 512 ? 512 : (d.B * d.L / 2 >= 32 ? d.B * d.L / 2 : 32);
-  dim3 grid((unsigned)blocks, (unsigned)ngrids);
-  if (inverse)
-    k_fft_lines<true, T><<<grid, threads, smem, s>>>(in, out, d, tw);
-  else
-    k_fft_lines<false, T><<<grid, threads, smem, s>>>(in, out, d, tw);
-  return cudaGetLastError();
-}
-
 // Lines per CTA for a line length L: as many as keep the CTA's lines and
-// twiddle table within a quarter of the SM's shared memory, so that up to four
+// twiddle table within a quarter of the SM's shared memory, so that several
 // CTAs share an SM and hide each other's barriers; at least one line.
 constexpr size_t FFT_CTA_BYTES = 52 * 1024;
-template <class T>
-int lines_per_cta(int L) {
-  const size_t tw = (size_t)(L / 2) * sizeof(T), line = (size_t)L * sizeof(T);
-  int B = FFT_CTA_BYTES > tw ? (int)((FFT_CTA_BYTES - tw) / line) : 0;
-  return B < 1 ? 1 : (B > 16 ? 16 : B);
+size_t cta_bytes(int L, int B, size_t elem) { return ((size_t)B * (L + 1) + L / 2) * elem; }
+int lines_per_cta(int L, size_t elem) {
+  int B = 1;
+  while (B < 16 && cta_bytes(L, B + 1, elem) <= FFT_CTA_BYTES) ++B;
+  return B;
 }
 
-template <class T>
-cudaError_t fft2d_forward_t(const T* compact, int64_t nx, int64_t ny, int64_t in_grid_stride, T* spec,
-                            const Fft2d& f, int ngrids, cudaStream_t s) {
-  // rows: compact rows [0, ny) -> spectrum rows, zero-padded to Nx
-  FftLines r{};
-  r.L = f.Nx; r.n3 = f.n3x; r.n2 = f.n2x; r.B = lines_per_cta<T>(f.Nx);
-  r.n_lines = ny; r.in_len = (int)nx; r.out_len = f.Nx;
-  r.in_line_stride = nx; r.in_elem_stride = 1; r.out_line_stride = f.Nx; r.out_elem_stride = 1;
-  r.in_grid_stride = in_grid_stride; r.out_grid_stride = (int64_t)f.Nx * f.Ny; r.scale = 1.0;
-  cudaError_t e = fft_lines_t(compact, spec, r, ngrids, f.tw_x, false, s);
-  if (e != cudaSuccess) return e;
-  // columns: all Nx, rows >= ny read as zero
-  FftLines c{};
-  c.L = f.Ny; c.n3 = f.n3y; c.n2 = f.n2y; c.B = lines_per_cta<T>(f.Ny);
-  c.n_lines = f.Nx; c.in_len = (int)ny; c.out_len = f.Ny;
-  c.in_line_stride = 1; c.in_elem_stride = f.Nx; c.out_line_stride = 1; c.out_elem_stride = f.Nx;
-  c.in_grid_stride = (int64_t)f.Nx * f.Ny; c.out_grid_stride = (int64_t)f.Nx * f.Ny; c.scale = 1.0;
-  return fft_lines_t(spec, spec, c, ngrids, f.tw_y, false, s);
+// Threads of a CTA with `smem` bytes: the SM's 24 warps over the CTAs that fit
+int cta_threads(size_t smem) {
+  const size_t fit = (size_t)228 * 1024 / (smem + 1024);
+  return fit >= 3 ? 256 : fit == 2 ? 384 : 768;
 }
 
-template <class T>
-cudaError_t fft2d_inverse_t(T* spec, const Fft2d& f, int64_t nx, int64_t ny, T* compact, int64_t out_grid_stride,
-                            int ngrids, cudaStream_t s) {
-  FftLines c{};
-  c.L = f.Ny; c.n3 = f.n3y; c.n2 = f.n2y; c.B = lines_per_cta<T>(f.Ny);
-  c.n_lines = f.Nx; c.in_len = f.Ny; c.out_len = (int)ny;
-  c.in_line_stride = 1; c.in_elem_stride = f.Nx; c.out_line_stride = 1; c.out_elem_stride = f.Nx;
-  c.in_grid_stride = (int64_t)f.Nx * f.Ny; c.out_grid_stride = (int64_t)f.Nx * f.Ny; c.scale = 1.0;
-  cudaError_t e = fft_lines_t(spec, spec, c, ngrids, f.tw_y, true, s);
-  if (e != cudaSuccess) return e;
+// One pass (rows or columns) of both plane sets: in one launch while three CTAs
+// of either kind share an SM (short lines, where launches and tails count),
+// else each with the shared memory and threads of its own.
+cudaError_t launch_lines(bool inverse, const float4* in4, float4* out4, FftLines d4, int ngrids4, const float2* in2,
+                         float2* out2, FftLines d2, int ngrids2, const float4* tw, cudaStream_t s) {
+  d4.B = lines_per_cta(d4.L, sizeof(float4));
+  d2.B = lines_per_cta(d2.L, sizeof(float2));
+  const int64_t b4 = (d4.n_lines + d4.B - 1) / d4.B * ngrids4, b2 = (d2.n_lines + d2.B - 1) / d2.B * ngrids2;
+  const size_t smem4 = cta_bytes(d4.L, d4.B, sizeof(float4)), smem2 = cta_bytes(d2.L, d2.B, sizeof(float2));
+  auto launch = [&](int64_t n4, int64_t n2, size_t smem) {
+    if (n4 + n2 <= 0) return cudaSuccess;
+    const int threads = cta_threads(smem);
+    if (inverse)
+      k_fft_lines<true><<<(unsigned)(n4 + n2), threads, smem, s>>>(in4, out4, d4, n4, in2, out2, d2, tw);
+    else
+      k_fft_lines<false><<<(unsigned)(n4 + n2), threads, smem, s>>>(in4, out4, d4, n4, in2, out2, d2, tw);
+    return cudaGetLastError();
+  };
+  const size_t both = smem4 > smem2 ? smem4 : smem2;
+  if (cta_threads(both) == 256) return launch(b4, b2, both);
+  cudaError_t e = launch(b4, 0, smem4);
+  return e == cudaSuccess ? launch(0, b2, smem2) : e;
+}
+
+FftLines row_lines(const Fft2d& f, int64_t ny) {
   FftLines r{};
-  r.L = f.Nx; r.n3 = f.n3x; r.n2 = f.n2x; r.B = lines_per_cta<T>(f.Nx);
-  r.n_lines = ny; r.in_len = f.Nx; r.out_len = (int)nx;
-  r.in_line_stride = f.Nx; r.in_elem_stride = 1; r.out_line_stride = nx; r.out_elem_stride = 1;
-  r.in_grid_stride = (int64_t)f.Nx * f.Ny; r.out_grid_stride = out_grid_stride;
-  r.scale = 1.0;
-  return fft_lines_t(spec, compact, r, ngrids, f.tw_x, true, s);
+  r.L = f.Nx; r.n3 = f.n3x; r.n2 = f.n2x;
+  r.n_lines = ny;
+  r.in_elem_stride = 1; r.out_elem_stride = 1;
+  return r;
+}
+
+FftLines col_lines(const Fft2d& f) {
+  FftLines c{};
+  c.L = f.Ny; c.n3 = f.n3y; c.n2 = f.n2y;
+  c.n_lines = f.Nx;
+  c.in_line_stride = 1; c.in_elem_stride = f.Nx; c.out_line_stride = 1; c.out_elem_stride = f.Nx;
+  c.in_grid_stride = (int64_t)f.Nx * f.Ny; c.out_grid_stride = (int64_t)f.Nx * f.Ny;
+  return c;
 }
 
 }  // namespace
 
-cudaError_t fft2d_forward(const float4* compact, int64_t nx, int64_t ny, int64_t in_grid_stride, float4* spec,
-                          const Fft2d& f, int ngrids, cudaStream_t s) {
-  return fft2d_forward_t(compact, nx, ny, in_grid_stride, spec, f, ngrids, s);
+cudaError_t fft2d_forward(const float4* compact4, float4* spec4, int ngrids4, const float2* compact2, float2* spec2,
+                          int ngrids2, int64_t nx, int64_t ny, int64_t in_grid_stride, const Fft2d& f,
+                          cudaStream_t s) {
+  // rows: compact rows [0, ny) -> spectrum rows, zero-padded to Nx
+  FftLines r = row_lines(f, ny);
+  r.in_len = (int)nx; r.out_len = f.Nx;
+  r.in_line_stride = nx; r.out_line_stride = f.Nx;
+  r.in_grid_stride = in_grid_stride; r.out_grid_stride = (int64_t)f.Nx * f.Ny;
+  cudaError_t e = launch_lines(false, compact4, spec4, r, ngrids4, compact2, spec2, r, ngrids2, f.tw_x, s);
+  if (e != cudaSuccess) return e;
+  // columns: all Nx, rows >= ny read as zero
+  FftLines c = col_lines(f);
+  c.in_len = (int)ny; c.out_len = f.Ny;
+  return launch_lines(false, spec4, spec4, c, ngrids4, spec2, spec2, c, ngrids2, f.tw_y, s);
 }
-cudaError_t fft2d_forward(const float2* compact, int64_t nx, int64_t ny, int64_t in_grid_stride, float2* spec,
-                          const Fft2d& f, int ngrids, cudaStream_t s) {
-  return fft2d_forward_t(compact, nx, ny, in_grid_stride, spec, f, ngrids, s);
-}
-cudaError_t fft2d_inverse(float4* spec, const Fft2d& f, int64_t nx, int64_t ny, float4* compact,
-                          int64_t out_grid_stride, int ngrids, cudaStream_t s) {
-  return fft2d_inverse_t(spec, f, nx, ny, compact, out_grid_stride, ngrids, s);
-}
-cudaError_t fft2d_inverse(float2* spec, const Fft2d& f, int64_t nx, int64_t ny, float2* compact,
-                          int64_t out_grid_stride, int ngrids, cudaStream_t s) {
-  return fft2d_inverse_t(spec, f, nx, ny, compact, out_grid_stride, ngrids, s);
+
+cudaError_t fft2d_inverse(float4* spec4, float4* compact4, int ngrids4, float2* spec2, float2* compact2, int ngrids2,
+                          const Fft2d& f, int64_t nx, int64_t ny, int64_t out_grid_stride, cudaStream_t s) {
+  FftLines c = col_lines(f);
+  c.in_len = f.Ny; c.out_len = (int)ny;
+  cudaError_t e = launch_lines(true, spec4, spec4, c, ngrids4, spec2, spec2, c, ngrids2, f.tw_y, s);
+  if (e != cudaSuccess) return e;
+  FftLines r = row_lines(f, ny);
+  r.in_len = f.Nx; r.out_len = (int)nx;
+  r.in_line_stride = f.Nx; r.out_line_stride = nx;
+  r.in_grid_stride = (int64_t)f.Nx * f.Ny; r.out_grid_stride = out_grid_stride;
+  return launch_lines(true, spec4, compact4, r, ngrids4, spec2, compact2, r, ngrids2, f.tw_x, s);
 }
 
 }  // namespace irs

@@ -8,9 +8,8 @@
 
 namespace irs {
 
-constexpr int FFT_MAX_ELEMS = 9216;  // double-float complex values of the largest line buffer a CTA
-                                     // may hold (144 KB; with its 72 KB twiddle table 216 KB)
-constexpr int FFT_MAX_LEN = 9216;    // longest line (3^2 2^10)
+constexpr int FFT_MAX_LEN = 9216;  // longest line (3^2 2^10): 144 KB of double-float complex values
+                                   // and a 72 KB twiddle table
 
 // One batched pass of 1-D FFTs over `n_lines` lines of length L.
 struct FftLines {
@@ -18,8 +17,7 @@ struct FftLines {
   int in_len, out_len;      // valid input elements (rest zero), outputs written
   int64_t n_lines;
   int64_t in_line_stride, in_elem_stride, out_line_stride, out_elem_stride;
-  int64_t in_grid_stride, out_grid_stride;  // between grids of a batch (gridDim.y)
-  double scale;  // applied to the outputs (1: none)
+  int64_t in_grid_stride, out_grid_stride;  // between grids of a batch
 };
 
 // A padded Nx x Ny spectrum layout with its twiddle tables.
@@ -35,19 +33,17 @@ struct Fft2d {
 int fft_good_size(int64_t n_min, int* n3, int* n2);
 cudaError_t fft_twiddles(int L, float4** d_tw);
 cudaError_t fft_setup_attributes();
-// compact [ngrids][ny][nx] -> padded spectra [ngrids][Ny][Nx], each axis in
-// the forward transform's own order (the mixed-radix digit reversal of the
-// frequency index): only pointwise products and sums of spectra made by these
-// transforms are meaningful before fft2d_inverse, which expects that order
-cudaError_t fft2d_forward(const float4* compact, int64_t nx, int64_t ny, int64_t in_grid_stride,
-                          float4* spec, const Fft2d& f, int ngrids, cudaStream_t s);
-cudaError_t fft2d_forward(const float2* compact, int64_t nx, int64_t ny, int64_t in_grid_stride,
-                          float2* spec, const Fft2d& f, int ngrids, cudaStream_t s);
+// compact [ngrids][ny][nx] -> padded spectra [ngrids][Ny][Nx], double-float planes
+// (4) and FP32 planes (2) together, each axis in the forward transform's own
+// order (the mixed-radix digit reversal of the frequency index): only pointwise
+// products and sums of spectra made by these transforms are meaningful before
+// fft2d_inverse, which expects that order
+cudaError_t fft2d_forward(const float4* compact4, float4* spec4, int ngrids4, const float2* compact2, float2* spec2,
+                          int ngrids2, int64_t nx, int64_t ny, int64_t in_grid_stride, const Fft2d& f,
+                          cudaStream_t s);
 // padded spectra (overwritten) -> compact [ngrids][ny][nx], unnormalised (the
 // 1/(Nx Ny) is the caller's)
-cudaError_t fft2d_inverse(float4* spec, const Fft2d& f, int64_t nx, int64_t ny, float4* compact,
-                          int64_t out_grid_stride, int ngrids, cudaStream_t s);
-cudaError_t fft2d_inverse(float2* spec, const Fft2d& f, int64_t nx, int64_t ny, float2* compact,
-                          int64_t out_grid_stride, int ngrids, cudaStream_t s);
+cudaError_t fft2d_inverse(float4* spec4, float4* compact4, int ngrids4, float2* spec2, float2* compact2, int ngrids2,
+                          const Fft2d& f, int64_t nx, int64_t ny, int64_t out_grid_stride, cudaStream_t s);
 
 }  // namespace irs

@@ -1903,13 +1903,13 @@ irs_status build_cells_and_far(irs_plan_t* P, const double* xy, const double* ma
     k_ip_p2m<<<(unsigned)((ncells + 127) / 128), 128, 0, s>>>(ig, S->cell_start, S->lens_pos, S->lens_m,
                                                              S->mpole_d, S->mpole_f);
     IP_TRY(cudaGetLastError());
-    IP_TRY(fft2d_forward(S->mpole_d, ig.ncx, ig.ncy, ncells, S->spec_d, S->fft, IP_PD, s));
-    IP_TRY(fft2d_forward(S->mpole_f, ig.ncx, ig.ncy, ncells, S->spec_f, S->fft, IP_P - IP_PD, s));
+    IP_TRY(fft2d_forward(S->mpole_d, S->spec_d, IP_PD, S->mpole_f, S->spec_f, IP_P - IP_PD, ig.ncx, ig.ncy, ncells,
+                         S->fft, s));
     const int64_t G = (int64_t)S->fft.Nx * S->fft.Ny;
     k_ip_m2l_freq<<<(unsigned)((G + 127) / 128), 128, 0, s>>>(G, S->spec_d, S->spec_f, S->kspec_d, S->kspec_f);
     IP_TRY(cudaGetLastError());
-    IP_TRY(fft2d_inverse(S->spec_d, S->fft, ig.ncx, ig.ncy, S->conv_d, ncells, IP_KD, s));
-    IP_TRY(fft2d_inverse(S->spec_f, S->fft, ig.ncx, ig.ncy, S->conv_f, ncells, IP_KF - IP_KD, s));
+    IP_TRY(fft2d_inverse(S->spec_d, S->conv_d, IP_KD, S->spec_f, S->conv_f, IP_KF - IP_KD, S->fft, ig.ncx, ig.ncy,
+                         ncells, s));
   }
   const int64_t nrc = (int64_t)ig.nrcx * ig.nrcy;
   if (rc1 < 0 || rc1 > nrc) rc1 = nrc;
@@ -2083,8 +2083,8 @@ irs_status interp_plan(irs_plan_t* P) {
   const int nker = ig.P + IP_KF - 1;
   k_ip_kernel_grid<<<(unsigned)((G + 255) / 256), 256>>>(f.Nx, f.Ny, ig.W, nker, IP_NKD, S->kspec_d, S->kspec_f);
   if (cudaGetLastError() != cudaSuccess) return IRS_ERR_CUDA;
-  if (fft2d_forward(S->kspec_d, f.Nx, f.Ny, G, S->kspec_d, f, IP_NKD, 0) != cudaSuccess) return IRS_ERR_CUDA;
-  if (fft2d_forward(S->kspec_f, f.Nx, f.Ny, G, S->kspec_f, f, nker, 0) != cudaSuccess) return IRS_ERR_CUDA;
+  if (fft2d_forward(S->kspec_d, S->kspec_d, IP_NKD, S->kspec_f, S->kspec_f, nker, f.Nx, f.Ny, G, f, 0) != cudaSuccess)
+    return IRS_ERR_CUDA;
   if (rect && nrc > 0) {  // the sheet's corner series, once per plan
     k_ip_sheet_table<<<(unsigned)((nrc + 127) / 128), 128>>>(g, ig, S->sheet_d, S->sheet_f, S->sheet_near, nrc);
     if (cudaGetLastError() != cudaSuccess) return IRS_ERR_CUDA;
