@@ -23,6 +23,10 @@ ROUTES = {
     "every ray its own pixel": ((0.2, 0.0, -0.2, (-1, 1, -1, 1), (700, 900), 0.25), 60, 0, {"kernel_variant": 1}),
     "shared reciprocals": ((0.3, 0.0, 0.3, (-2, 2, -2, 2), 64, 9.0), 200, 0, {"kernel_variant": 2}),
     "circle off the origin": ((0.35, 0.1, 0.25, (-1.5, 2.5, -2.7, 1.3), (61, 67), 6.0), 700, 1, {"kernel_variant": 9}),
+    # most units of these planes cannot reach the map and are left out by bound
+    "a wide border": ((0.6, 0.0, 0.1, (-0.5, 0.5, -0.4, 0.4), (40, 32), 9.0), 900, 0, {"cell_mult": 0.7}),
+    "few heavy lenses": ((0.1, 0.0, 0.1, (-1.0, 1.0, -1.0, 1.0), 60, 16.0), 5, 0, {}),
+    "over-focused": ((0.9, 0.5, 0.15, (-1.0, 1.0, -0.8, 0.8), (50, 40), 9.0), 800, 0, {"kernel_variant": 16}),
     "no lenses": ((0.2, 0.1, 0.2, (-1.5, 1.5, -1.5, 1.5), 48, 10.25), 0, 0, {"n_star": 60}),
 }
 
@@ -95,3 +99,15 @@ def test_brute_map_equals_its_rays(variant, n):
     assert np.array_equal(counts.cpu().numpy().astype(np.int64), _counts_of(pix.cpu().numpy(), shape))
     assert torch.equal(b1[:95], beta[some]) and torch.equal(p1[:95], pix[some])
     assert torch.isnan(b1[95:]).all() and (p1[95:] == -1).all()
+
+
+def test_masses_of_both_signs():
+    """Lens masses may have either sign; the bound that leaves units out takes
+    their magnitudes."""
+    torch = require_gpu()
+    args = (0.4, 0.0, 0.2, (-0.8, 0.8, -0.7, 0.7), (48, 42), 9.0)
+    po, pl = params_pair(*args, method=irs.IRS_INTERP, n_star=700)
+    xy, m = lenses_for(oracle.size(po), 700, shape="salpeter", seed=9, kappa_star=args[0])
+    m[::3] *= -1.0
+    with irs.Plan(pl) as plan:
+        _check(torch, pl, plan, *to_dev(torch, xy, m))
