@@ -2267,6 +2267,10 @@ irs_status interp_prepare(irs_plan_t* P, const double* xy, const double* mass, i
 int interp_variant(const irs_plan_t* P) { return S_(P)->ig.variant; }
 int interp_row_entries(const irs_plan_t* P) { return S_(P)->ig.nrow; }
 int interp_near_cap(const irs_plan_t* P, int64_t n) { return ip_near_cap(S_(P)->ig, n); }
+bool interp_small_ctas(const irs_plan_t* P, int64_t n) {
+  const InterpState* S = S_(P);
+  return ip_launch_shape(S->ig.variant, S->ig.nrow, ip_near_cap(S->ig, n), P->num_sms).threads == 128;
+}
 int interp_num_variants() { return IP_NVARIANT; }
 bool interp_variant_distinct(int variant) { return ip_kernel_of(variant) == variant; }
 

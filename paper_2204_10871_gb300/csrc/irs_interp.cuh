@@ -37,6 +37,8 @@ int interp_variant(const irs_plan_t* P);
 // with both)
 int interp_row_entries(const irs_plan_t* P);
 int interp_near_cap(const irs_plan_t* P, int64_t n);
+// whether a map of n lenses runs its ray pass on CTAs of 128 threads
+bool interp_small_ctas(const irs_plan_t* P, int64_t n);
 int interp_num_variants();
 // false for a variant number served by another number's kernel
 bool interp_variant_distinct(int variant);
