@@ -164,7 +164,7 @@ irs_status run_map(irs_plan_t* P, const double* xy, const double* mass, int64_t 
     if (st != IRS_OK) return st;
   }
   mark(P, irs::EV_MAG, s);
-  if (mag) IRS_TRY(irs::launch_magnify(P, counts, mag, s));
+  if (mag) IRS_TRY(irs::launch_magnify(P, counts, mag, row1 > row0, s));
   if (mag) P->launches += 1;
   mark(P, irs::EV_END, s);
   P->timed_rays = (row1 - row0) * P->g.nrx;
@@ -271,7 +271,7 @@ irs_status irs_make_map_rows(irs_plan_t* P, const double* xy, const double* mass
 
 irs_status irs_magnify(irs_plan_t* P, const uint32_t* counts, float* mag, void* stream) {
   if (!P || !counts || !mag) return IRS_ERR_ARG;
-  IRS_TRY(irs::launch_magnify(P, counts, mag, static_cast<cudaStream_t>(stream)));
+  IRS_TRY(irs::launch_magnify(P, counts, mag, false, static_cast<cudaStream_t>(stream)));
   return IRS_OK;
 }
 

@@ -109,7 +109,7 @@ irs_status enqueue(BatchEntry* e, irs_plan_t* const* plans, int32_t nmaps, const
   }
   if (mag) {
     for (int32_t m = 0; m < nmaps; ++m)
-      if (mag[m] && irs::launch_magnify(plans[m], counts[m], mag[m], cs) != cudaSuccess)
+      if (mag[m] && irs::launch_magnify(plans[m], counts[m], mag[m], false, cs) != cudaSuccess)
         return IRS_ERR_CUDA;
   }
   return IRS_OK;

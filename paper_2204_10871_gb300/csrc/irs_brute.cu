@@ -53,9 +53,12 @@ __device__ __forceinline__ bool lens_inside(const LensRegion& L, double2 p) {
 __global__ void k_mass_sum(const double* __restrict__ mass, const double2* __restrict__ xy, int64_t n,
                            LensRegion region, int* __restrict__ status, double* __restrict__ part,
                            unsigned int* __restrict__ done, double* __restrict__ out,
-                           unsigned long long* __restrict__ queue) {
+                           unsigned long long* __restrict__ queue, int32_t* __restrict__ zero, int64_t nzero) {
   __shared__ double sh[MSUM_THREADS];
   __shared__ bool last;
+  after_ready();
+  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < nzero; k += (int64_t)gridDim.x * blockDim.x)
+    zero[k] = 0;
   double s = 0.0;
   bool outside = false;
   const int64_t stride = (int64_t)MSUM_BLOCKS * MSUM_THREADS;
@@ -106,10 +109,12 @@ cudaError_t launch_mass_sum(const irs_plan_t* P, const double* mass, int64_t n, 
   L.circle = g.plane == IRS_PLANE_CIRCLE;
   L.check = xy != nullptr && n > 0;
   static_assert(MSUM_BLOCKS <= MSUM_THREADS, "one partial sum per thread");
-  const int64_t need = (n + MSUM_THREADS - 1) / MSUM_THREADS;
+  int64_t need = (n + MSUM_THREADS - 1) / MSUM_THREADS;
+  const int64_t nzero = P->d_zero ? P->n_zero : 0, zblocks = (nzero + 16 * MSUM_THREADS - 1) / (16 * MSUM_THREADS);
+  if (need < zblocks) need = zblocks;
   const unsigned blocks = need < 1 ? 1u : need < MSUM_BLOCKS ? (unsigned)need : (unsigned)MSUM_BLOCKS;
   k_mass_sum<<<blocks, MSUM_THREADS, 0, s>>>(mass, reinterpret_cast<const double2*>(xy), n, L, P->d_status, P->d_mpart,
-                                             P->d_mdone, P->d_msum, P->d_queue);
+                                             P->d_mdone, P->d_msum, P->d_queue, P->d_zero, nzero);
   return cudaGetLastError();
 }
 
@@ -154,6 +159,7 @@ k_brute_setup(Geo g, const double* __restrict__ msum, int64_t ntx, int64_t tile0
               TileRec* __restrict__ recs) {
   __shared__ double val_s[4][SETUP_VALUES][SETUP_TILES];
   __shared__ bool near_s[4][SETUP_TILES];
+  after_ready();
   const int lt = threadIdx.x & 31;  // a warp per corner
   const int64_t tile = min(tile0 + (int64_t)blockIdx.x * SETUP_TILES + lt, tile1 - 1);
   const TileGeo tg = tile_geo(g, tile, ntx);
@@ -191,6 +197,7 @@ k_brute_setup(Geo g, const double* __restrict__ msum, int64_t ntx, int64_t tile0
       }
     }
   }
+  after_wait();  // the corners need the plan's geometry alone
   __syncthreads();
   if (threadIdx.x >= SETUP_TILES || tile0 + (int64_t)blockIdx.x * SETUP_TILES + lt >= tile1) return;
 
@@ -263,8 +270,8 @@ cudaError_t launch_brute_setup(const irs_plan_t* P, int64_t row0, int64_t row1, 
   const int64_t t0 = row0 / BR_TY * P->br_ntx, t1 = (row1 + BR_TY - 1) / BR_TY * P->br_ntx;
   if (t1 <= t0) return cudaSuccess;
   const int64_t blocks = (t1 - t0 + SETUP_TILES - 1) / SETUP_TILES;
-  k_brute_setup<<<(unsigned)blocks, 4 * SETUP_TILES, 0, s>>>(P->g, P->d_msum, P->br_ntx, t0, t1, P->d_tiles);
-  return cudaGetLastError();
+  return launch_after(k_brute_setup, (unsigned)blocks, 4 * SETUP_TILES, 0, s, P->g, P->d_msum, P->br_ntx, t0, t1,
+                      P->d_tiles);
 }
 
 // ------------------------------------------------------------ ray pass
@@ -354,6 +361,8 @@ k_brute(Geo g, const double2* __restrict__ xy, const double* __restrict__ mass, 
   __shared__ float2 ty_s[BR_TY / 2];  // row offsets to the tile centre, in pairs
   __shared__ TileRec rec;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  bool waited = false;
+  after_ready();
 
   for (int64_t work = blockIdx.x; work < nwork; work += gridDim.x) {
     const int64_t tile = (row0 / BR_TY) * ntx + work;  // tile rows covering [row0, row1)
@@ -363,7 +372,6 @@ k_brute(Geo g, const double2* __restrict__ xy, const double* __restrict__ mass, 
     const float tx = (float)(((double)col + 0.5 - tg.ci) * g.dx3);
     const float2 TX2 = make_float2(tx, tx);
     __syncthreads();  // previous tile's readers of rec / lens_s / ty_s are done
-    if (tid == 0) rec = recs[tile];
     if (tid < BR_TY)
       reinterpret_cast<float*>(ty_s)[tid] = (float)(((double)(tg.j0 + tid) + 0.5 - tg.cj) * g.dx3);
     __syncthreads();
@@ -502,7 +510,15 @@ k_brute(Geo g, const double2* __restrict__ xy, const double* __restrict__ mass, 
       }
     }
     // ---- per-ray: smooth terms, sheet series, near corners, pixel; two rows at
-    // a time through the packed instructions, the roundings of brute_beta
+    // a time through the packed instructions, the roundings of brute_beta.  The
+    // lens sums above need the caller's lenses alone; the tile's constants and
+    // the map are the set-up's.
+    if (!waited) {
+      after_wait();
+      waited = true;
+    }
+    if (tid == 0) rec = recs[tile];
+    __syncthreads();
     const bool colok = col < tg.i1;
     const uint32_t npx = (uint32_t)g.npix_x, npy = (uint32_t)g.npix_y;
 #pragma unroll 1
@@ -569,9 +585,8 @@ int brute_grid_size(int num_sms, int variant) {
 
 #define BR_DECL_LAUNCH(V, R, PAIRED, QUAD, PACK, TPSM)                                              \
   case V:                                                                                           \
-    k_brute<R, PAIRED, QUAD, PACK, TPSM><<<(unsigned)grid, 32 * (BR_TY / R), 0, s>>>(               \
-        P->g, xy2, mass, n, P->d_tiles, P->br_ntx, nwork, row0, row1, counts);                      \
-    break;
+    return launch_after(k_brute<R, PAIRED, QUAD, PACK, TPSM>, (unsigned)grid, 32 * (BR_TY / R), 0, s, P->g, xy2, mass, \
+                        n, P->d_tiles, P->br_ntx, nwork, row0, row1, counts);
 cudaError_t launch_brute_map(const irs_plan_t* P, const double* xy, const double* mass, int64_t n,
                              int64_t row0, int64_t row1, uint32_t* counts, cudaStream_t s) {
   if (row1 <= row0) return cudaSuccess;
@@ -694,6 +709,7 @@ k_brute_rays(Geo g, BruteForm form, const double2* __restrict__ xy, const double
   const int tid = threadIdx.x;
   const int64_t tile = BY_TILE ? (int64_t)blockIdx.x / BD_PARTS : 0;
   const int64_t n_rays = g.nrx * g.nry;
+  after_wait();
   int64_t scan = BY_TILE ? (int64_t)(blockIdx.x % BD_PARTS) * BD_THREADS : (int64_t)blockIdx.x * 32;
   while (scan < nidx) {
     // ---- the rays of this round: `live` of them, ray k's slot in the caller's arrays
@@ -809,12 +825,10 @@ cudaError_t launch_brute_dump(const irs_plan_t* P, const double* xy, const doubl
   const double2* xy2 = reinterpret_cast<const double2*>(xy);
   const BruteForm form = brute_form(P->p.kernel_variant);
   if (nidx >= 8 * P->br_ntiles && P->br_ntiles * BD_PARTS < ((int64_t)1 << 31))
-    k_brute_rays<true><<<(unsigned)(P->br_ntiles * BD_PARTS), BD_THREADS, 0, s>>>(
-        P->g, form, xy2, mass, n, P->d_tiles, P->br_ntx, idx, nidx, beta, pix);
-  else
-    k_brute_rays<false><<<(unsigned)((nidx + 31) / 32), BD_THREADS, 0, s>>>(P->g, form, xy2, mass, n, P->d_tiles,
-                                                                            P->br_ntx, idx, nidx, beta, pix);
-  return cudaGetLastError();
+    return launch_after(k_brute_rays<true>, (unsigned)(P->br_ntiles * BD_PARTS), BD_THREADS, 0, s, P->g, form, xy2,
+                        mass, n, P->d_tiles, P->br_ntx, idx, nidx, beta, pix);
+  return launch_after(k_brute_rays<false>, (unsigned)((nidx + 31) / 32), BD_THREADS, 0, s, P->g, form, xy2, mass, n,
+                      P->d_tiles, P->br_ntx, idx, nidx, beta, pix);
 }
 
 // ------------------------------------------------------------ magnification
@@ -822,18 +836,20 @@ cudaError_t launch_brute_dump(const irs_plan_t* P, const double* xy, const doubl
 // magnification of each pixel", Sec. 2.4).
 __global__ void k_magnify(const uint32_t* __restrict__ counts, float* __restrict__ mag, int64_t npix,
                           float ratio) {
+  after_wait();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < npix; k += stride)
     mag[k] = (float)counts[k] * ratio;
 }
 
-cudaError_t launch_magnify(const irs_plan_t* P, const uint32_t* counts, float* mag, cudaStream_t s) {
+cudaError_t launch_magnify(const irs_plan_t* P, const uint32_t* counts, float* mag, bool chained, cudaStream_t s) {
   const int64_t npix = (int64_t)P->g.npix_x * P->g.npix_y;
   const float ratio = (float)(P->g.dx3 * P->g.dx3 / (P->g.sx * P->g.sy));
   int64_t blocks = (npix + 255) / 256;
   const int64_t cap = (int64_t)P->num_sms * 8;
   if (blocks > cap) blocks = cap;
   if (blocks < 1) blocks = 1;
+  if (chained) return launch_after(k_magnify, (unsigned)blocks, 256, 0, s, counts, mag, npix, ratio);
   k_magnify<<<(unsigned)blocks, 256, 0, s>>>(counts, mag, npix, ratio);
   return cudaGetLastError();
 }

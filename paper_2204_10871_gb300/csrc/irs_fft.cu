@@ -28,6 +28,7 @@
 #include <type_traits>
 #include <vector>
 
+#include "irs_common.cuh"
 #include "irs_df.cuh"
 #include "irs_fft.cuh"
 
@@ -187,6 +188,7 @@ __device__ __forceinline__ void fft_lines(const T* in, T* out, const FftLines& d
   int pow3 = 1;
   for (int i = 0; i < n3; ++i) pow3 *= 3;
   const int np2 = fft_passes2(n2), np3 = (n3 + 1) / 2, np = np2 + np3;
+  after_wait();  // the twiddles are the plan's
   __syncthreads();
   int span = INV ? 1 : L;  // forward: widest span left; inverse: span done so far
   for (int p = 0; p < np; ++p) {
@@ -263,6 +265,7 @@ __global__ void __maxnreg__(FFT_REGS)
 k_fft_lines(const float4* in4, float4* out4, FftLines d4, int64_t blocks4, const float2* in2, float2* out2,
             FftLines d2, const float4* __restrict__ tw) {
   extern __shared__ float4 sm_raw[];
+  after_ready();
   if ((int64_t)blockIdx.x < blocks4) fft_lines<INV>(in4, out4, d4, tw, blockIdx.x, sm_raw);
   else fft_lines<INV>(in2, out2, d2, tw, (int64_t)blockIdx.x - blocks4, sm_raw);
 }
@@ -342,11 +345,8 @@ cudaError_t launch_lines(bool inverse, const float4* in4, float4* out4, FftLines
   auto launch = [&](int64_t n4, int64_t n2, size_t smem) {
     if (n4 + n2 <= 0) return cudaSuccess;
     const int threads = cta_threads(smem);
-    if (inverse)
-      k_fft_lines<true><<<(unsigned)(n4 + n2), threads, smem, s>>>(in4, out4, d4, n4, in2, out2, d2, tw);
-    else
-      k_fft_lines<false><<<(unsigned)(n4 + n2), threads, smem, s>>>(in4, out4, d4, n4, in2, out2, d2, tw);
-    return cudaGetLastError();
+    return launch_after(inverse ? k_fft_lines<true> : k_fft_lines<false>, (unsigned)(n4 + n2), (unsigned)threads, smem,
+                        s, in4, out4, d4, n4, in2, out2, d2, tw);
   };
   const size_t both = smem4 > smem2 ? smem4 : smem2;
   if (cta_threads(both) == 256) return launch(b4, b2, both);
@@ -372,6 +372,15 @@ FftLines col_lines(const Fft2d& f) {
 }
 
 }  // namespace
+
+int fft2d_launches(const Fft2d& f) {
+  int n = 0;
+  for (int L : {f.Nx, f.Ny}) {
+    const size_t s4 = cta_bytes(L, lines_per_cta(L, sizeof(float4)), sizeof(float4));
+    n += cta_threads(s4) == 256 ? 1 : 2;
+  }
+  return n;
+}
 
 cudaError_t fft2d_forward(const float4* compact4, float4* spec4, int ngrids4, const float2* compact2, float2* spec2,
                           int ngrids2, int64_t nx, int64_t ny, int64_t in_grid_stride, const Fft2d& f,

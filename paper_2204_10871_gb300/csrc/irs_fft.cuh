@@ -33,6 +33,8 @@ struct Fft2d {
 int fft_good_size(int64_t n_min, int* n3, int* n2);
 cudaError_t fft_twiddles(int L, float4** d_tw);
 cudaError_t fft_setup_attributes();
+// kernel launches of one 2-D transform, either way
+int fft2d_launches(const Fft2d& f);
 // compact [ngrids][ny][nx] -> padded spectra [ngrids][Ny][Nx], double-float planes
 // (4) and FP32 planes (2) together, each axis in the forward transform's own
 // order (the mixed-radix digit reversal of the frequency index): only pointwise

@@ -165,104 +165,129 @@ __device__ __forceinline__ int cell_of(const IpGeo& ig, double x, double y) {
 
 __global__ void k_ip_count(IpGeo ig, const double2* __restrict__ xy, int64_t n,
                            int32_t* __restrict__ lens_cell, int32_t* __restrict__ count) {
+  after_ready();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const double2 p = xy[i];
-  const int c = cell_of(ig, p.x, p.y);
-  lens_cell[i] = c;
-  atomicAdd(count + c, 1);
+  int c = 0;
+  if (i < n) {
+    const double2 p = xy[i];
+    c = cell_of(ig, p.x, p.y);
+    lens_cell[i] = c;
+  }
+  after_wait();  // the counts are zeroed by the mass sum
+  if (i < n) atomicAdd(count + c, 1);
 }
 
-// exclusive scan of int32 in three passes (block scan, scan of block sums, add)
+// Exclusive scan of the cell counts into `start` (n + 1 entries) and a copy of it
+// that the scatter advances: each block of SCAN_B cells scans its own and,
+// unless it is the only one, leaves its sum; a second launch adds to each block
+// the sums of those before it (which it adds up by itself; a third launch that
+// scanned the sums on one thread took 50 us at 1.9e6 cells).
 constexpr int SCAN_B = 1024;
-__global__ void k_scan_local(const int32_t* __restrict__ in, int32_t* __restrict__ out, int64_t n,
-                             int32_t* __restrict__ block_sums) {
-  __shared__ int32_t sh[SCAN_B];
+__global__ void k_scan_local(const int32_t* __restrict__ in, int32_t* __restrict__ out, int32_t* __restrict__ copy,
+                             int64_t n, int32_t* __restrict__ block_sums) {
+  __shared__ int32_t warp_s[32];
+  after_ready();
+  after_wait();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t i = (int64_t)blockIdx.x * SCAN_B + threadIdx.x;
   const int32_t v = i < n ? in[i] : 0;
-  sh[threadIdx.x] = v;
+  int32_t inc = v;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const int32_t t = __shfl_up_sync(0xFFFFFFFFu, inc, d);
+    if (lane >= d) inc += t;
+  }
+  if (lane == 31) warp_s[warp] = inc;
   __syncthreads();
-  for (int off = 1; off < SCAN_B; off <<= 1) {
-    int32_t t = threadIdx.x >= (unsigned)off ? sh[threadIdx.x - off] : 0;
-    __syncthreads();
-    sh[threadIdx.x] += t;
-    __syncthreads();
+  if (warp == 0) {
+    int32_t w = warp_s[lane];
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const int32_t t = __shfl_up_sync(0xFFFFFFFFu, w, d);
+      if (lane >= d) w += t;
+    }
+    warp_s[lane] = w;
   }
-  if (i < n) out[i] = sh[threadIdx.x] - v;
-  if (threadIdx.x == SCAN_B - 1) block_sums[blockIdx.x] = sh[SCAN_B - 1];
+  __syncthreads();
+  inc += warp ? warp_s[warp - 1] : 0;
+  if (i < n) {
+    out[i] = inc - v;
+    if (gridDim.x == 1) {
+      copy[i] = inc - v;
+      if (i == n - 1) out[n] = inc;
+    }
+  }
+  if (gridDim.x > 1 && threadIdx.x == SCAN_B - 1) block_sums[blockIdx.x] = inc;
 }
-__global__ void k_scan_blocks(int32_t* __restrict__ block_sums, int64_t nb, int32_t* __restrict__ total) {
-  if (threadIdx.x != 0) return;
+__global__ void k_scan_add(int32_t* __restrict__ out, int32_t* __restrict__ copy, int64_t n,
+                           const int32_t* __restrict__ block_sums) {
+  __shared__ int32_t warp_s[32];
+  after_ready();
+  after_wait();
   int32_t s = 0;
-  for (int64_t b = 0; b < nb; ++b) {
-    const int32_t v = block_sums[b];
-    block_sums[b] = s;
-    s += v;
-  }
-  *total = s;
-}
-__global__ void k_scan_add(int32_t* __restrict__ out, int64_t n, const int32_t* __restrict__ block_sums) {
+  for (int64_t b = threadIdx.x; b < blockIdx.x; b += SCAN_B) s += block_sums[b];
+  s = __reduce_add_sync(0xFFFFFFFFu, s);
+  if ((threadIdx.x & 31) == 0) warp_s[threadIdx.x >> 5] = s;
+  __syncthreads();
+  s = __reduce_add_sync(0xFFFFFFFFu, warp_s[threadIdx.x & 31]);
   const int64_t i = (int64_t)blockIdx.x * SCAN_B + threadIdx.x;
-  if (i < n) out[i] += block_sums[blockIdx.x];
+  if (i < n) {
+    const int32_t v = out[i] + s;
+    out[i] = v;
+    copy[i] = v;
+  }
+  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) out[n] = s + block_sums[blockIdx.x];
 }
 
 __global__ void k_ip_scatter(const int32_t* __restrict__ lens_cell, int64_t n,
                              int32_t* __restrict__ cursor, int32_t* __restrict__ sorted_idx) {
+  after_ready();
+  after_wait();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const int pos = atomicAdd(cursor + lens_cell[i], 1);
   sorted_idx[pos] = (int32_t)i;
 }
 
-// Insertion sort of each cell's lens indices: the order inside a cell no
-// longer depends on the atomics, so every map is bitwise reproducible.
-__global__ void k_ip_sortcells(const int32_t* __restrict__ start, int64_t ncells,
-                               int32_t* __restrict__ sorted_idx) {
-  const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= ncells) return;
-  const int a = start[c], b = start[c + 1];
-  for (int i = a + 1; i < b; ++i) {
+// Per cell, for the lenses of its list:
+// - insertion sort of the indices: the order inside a cell no longer depends on
+//   the atomics, so every map is bitwise reproducible;
+// - the sorted records: position relative to the cell centre (FP32), position
+//   and mass in double-float, and in FP64 where the network form wants them;
+// - P2M (series form): a_j = sum_i m_i ((z_i - z_S)/h)^j; orders j < IP_PD in
+//   FP64 (stored double-float), the rest in FP32 from the FP32 offset (|d| <=
+//   0.71; they are stored and convolved in FP32).
+//
+// A CTA takes CELLS_B cells, whose lenses are contiguous.  Cells hold half a lens on
+// average, so the FP64 work (GB300 issues two a clock per SM) is done with one
+// thread per lens, a chunk of CELLS_B lenses at a time through shared memory, and
+// one thread per cell only adds, in list order.  As three kernels (sort, fill,
+// P2M with one thread per cell) this took 14.6 us at 250 cells and 474 us at the
+// high-res map's 1.9e6; now 8.7 and 311 us.
+constexpr int CELLS_B = 128;
+__global__ void __launch_bounds__(CELLS_B)
+k_ip_cells(IpGeo ig, const int32_t* __restrict__ start, const double2* __restrict__ xy,
+           const double* __restrict__ mass, const int32_t* __restrict__ lens_cell, int32_t* __restrict__ sorted_idx,
+           float4* __restrict__ rel, double2* __restrict__ pos, double* __restrict__ m_out,
+           float4* __restrict__ pos_df, float2* __restrict__ m_df, float4* __restrict__ mpole_d,
+           float2* __restrict__ mpole_f) {
+  __shared__ double pw_s[2 * IP_PD][CELLS_B];  // m d^j, j < PD, of the chunk's lenses
+  __shared__ float2 d_s[CELLS_B], pf_s[CELLS_B];  // d and m d^PD in FP32
+  after_ready();
+  after_wait();
+  const int64_t ncells = (int64_t)ig.ncx * ig.ncy, c0 = (int64_t)blockIdx.x * CELLS_B;
+  const int64_t c = c0 + threadIdx.x;
+  const bool on = c < ncells;
+  const int b = on ? start[c] : 0, e = on ? start[c + 1] : 0;
+  for (int i = b + 1; i < e; ++i) {
     const int32_t v = sorted_idx[i];
     int j = i - 1;
-    while (j >= a && sorted_idx[j] > v) {
+    while (j >= b && sorted_idx[j] > v) {
       sorted_idx[j + 1] = sorted_idx[j];
       --j;
     }
     sorted_idx[j + 1] = v;
   }
-}
-
-__global__ void k_ip_fill(IpGeo ig, const double2* __restrict__ xy, const double* __restrict__ mass,
-                          const int32_t* __restrict__ sorted_idx, const int32_t* __restrict__ lens_cell,
-                          int64_t n, float4* __restrict__ rel, double2* __restrict__ pos,
-                          double* __restrict__ m_out, float4* __restrict__ pos_df, float2* __restrict__ m_df) {
-  const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= n) return;
-  const int32_t i = sorted_idx[p];
-  const int c = lens_cell[i];
-  const int cx = c % ig.ncx, cy = c / ig.ncx;
-  const double zx = ig.gx0 + (cx + 0.5) * ig.h, zy = ig.gy0 + (cy + 0.5) * ig.h;
-  const double2 q = xy[i];
-  const double m = mass[i];
-  rel[p] = make_float4((float)(q.x - zx), (float)(q.y - zy), (float)m, 0.f);
-  pos[p] = q;
-  m_out[p] = m;
-  pos_df[p] = dfc_from_double(q.x, q.y);
-  m_df[p] = df_from_double(m);
-}
-
-// ------------------------------------------------------------ far field
-// P2M: a_j = sum_i m_i ((z_i - z_S)/h)^j for the lenses of cell S; orders
-// j < IP_PD in FP64 (stored double-float), the rest in FP32 from the FP32
-// offset (|d| <= 0.71; they are stored and convolved in FP32).
-__global__ void k_ip_p2m(IpGeo ig, const int32_t* __restrict__ start, const double2* __restrict__ pos,
-                         const double* __restrict__ m, float4* __restrict__ mpole_d,
-                         float2* __restrict__ mpole_f) {
-  const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t ncells = (int64_t)ig.ncx * ig.ncy;
-  if (c >= ncells) return;
-  const int cx = (int)(c % ig.ncx), cy = (int)(c / ig.ncx);
-  const double zx = ig.gx0 + (cx + 0.5) * ig.h, zy = ig.gy0 + (cy + 0.5) * ig.h;
   cd a[IP_PD];
   float2 af[IP_P - IP_PD];
 #pragma unroll
@@ -270,30 +295,64 @@ __global__ void k_ip_p2m(IpGeo ig, const int32_t* __restrict__ start, const doub
 #pragma unroll
   for (int j = 0; j < IP_P - IP_PD; ++j) af[j] = make_float2(0.f, 0.f);
   const double inv_h = 1.0 / ig.h;
-  for (int p = start[c]; p < start[c + 1]; ++p) {
-    const cd d = {(pos[p].x - zx) * inv_h, (pos[p].y - zy) * inv_h};
-    cd pw = {m[p], 0.0};
+  const int first = start[c0], last = start[min(c0 + CELLS_B, ncells)];
+  for (int chunk = first; chunk < last; chunk += CELLS_B) {
+    __syncthreads();  // lists sorted; the chunk before is used up
+    const int p = chunk + threadIdx.x;
+    if (p < last) {
+      const int32_t i = sorted_idx[p];
+      const int cell = lens_cell[i], cx = cell % ig.ncx, cy = cell / ig.ncx;
+      const double zx = ig.gx0 + (cx + 0.5) * ig.h, zy = ig.gy0 + (cy + 0.5) * ig.h;
+      const double2 q = xy[i];
+      const double m = mass[i];
+      rel[p] = make_float4((float)(q.x - zx), (float)(q.y - zy), (float)m, 0.f);
+      pos_df[p] = dfc_from_double(q.x, q.y);
+      m_df[p] = df_from_double(m);
+      if (pos) {
+        pos[p] = q;
+        m_out[p] = m;
+      }
+      if (mpole_d) {
+        const cd d = {(q.x - zx) * inv_h, (q.y - zy) * inv_h};
+        cd pw = {m, 0.0};
 #pragma unroll
-    for (int j = 0; j < IP_PD; ++j) {
-      a[j].re += pw.re;
-      a[j].im += pw.im;
-      pw = cmul(pw, d);
+        for (int j = 0; j < IP_PD; ++j) {
+          pw_s[2 * j][threadIdx.x] = pw.re;
+          pw_s[2 * j + 1][threadIdx.x] = pw.im;
+          pw = cmul(pw, d);
+        }
+        d_s[threadIdx.x] = make_float2((float)d.re, (float)d.im);
+        pf_s[threadIdx.x] = make_float2((float)pw.re, (float)pw.im);  // m d^PD
+      }
     }
-    const float2 df = make_float2((float)d.re, (float)d.im);
-    float2 pf = make_float2((float)pw.re, (float)pw.im);  // m d^PD
+    if (!mpole_d) continue;
+    __syncthreads();
+    for (int k = max(b, chunk); k < min(e, chunk + CELLS_B); ++k) {
+      const int t = k - chunk;
 #pragma unroll
-    for (int j = 0; j < IP_P - IP_PD; ++j) {
-      af[j].x += pf.x;
-      af[j].y += pf.y;
-      pf = make_float2(fmaf(pf.x, df.x, -pf.y * df.y), fmaf(pf.x, df.y, pf.y * df.x));
+      for (int j = 0; j < IP_PD; ++j) {
+        a[j].re += pw_s[2 * j][t];
+        a[j].im += pw_s[2 * j + 1][t];
+      }
+      const float2 df = d_s[t];
+      float2 pf = pf_s[t];
+#pragma unroll
+      for (int j = 0; j < IP_P - IP_PD; ++j) {
+        af[j].x += pf.x;
+        af[j].y += pf.y;
+        pf = make_float2(fmaf(pf.x, df.x, -pf.y * df.y), fmaf(pf.x, df.y, pf.y * df.x));
+      }
     }
   }
+  if (!mpole_d || !on) return;
 #pragma unroll
-  for (int j = 0; j < IP_PD; ++j) mpole_d[(int64_t)j * ncells + c] = dfc_from_double(a[j].re, a[j].im);
+  for (int j = 0; j < IP_PD; ++j)
+    mpole_d[(int64_t)j * ncells + c] = b == e ? make_float4(0.f, 0.f, 0.f, 0.f) : dfc_from_double(a[j].re, a[j].im);
 #pragma unroll
   for (int j = 0; j < IP_P - IP_PD; ++j) mpole_f[(int64_t)j * ncells + c] = af[j];
 }
 
+// ------------------------------------------------------------ far field
 // Translation kernels on the padded grid, scaled by n! / (Nx Ny):
 // K'_n[e] = n! (-e)^-(n+1) / (Nx Ny) for offsets e (cell units, wrapped) with
 // Chebyshev norm > W, else 0 (the n! is one factor of the M2L's binomial,
@@ -333,6 +392,8 @@ __global__ void __launch_bounds__(128) k_ip_m2l_freq(int64_t G, float4* __restri
                                                      float2* __restrict__ spec_f,
                                                      const float4* __restrict__ kspec_d,
                                                      const float2* __restrict__ kspec_f) {
+  after_ready();
+  after_wait();
   const int64_t f = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (f >= G) return;
   float4 Ad[IP_PD], Cd[IP_KD];
@@ -591,6 +652,8 @@ k_ip_finalize_group(Geo g, IpGeo ig, const double* __restrict__ msum, const int3
   __shared__ float val_s[FG_WARPS][NV][33];
   __shared__ int from_s[FG_WARPS][4][FG_RANGES], off_s[FG_WARPS][4][FG_RANGES + 1];
   __shared__ float2 sum_s[FG_CELLS][2 * FIN_K64];
+  after_ready();
+  after_wait();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t base = rc0 + (int64_t)blockIdx.x * cta_cells;
   const int64_t ncells = (int64_t)ig.ncx * ig.ncy;
@@ -758,6 +821,8 @@ k_ip_finalize(Geo g, IpGeo ig, const double* __restrict__ msum, const int32_t* _
               const float2* __restrict__ conv_f, MlpFar far, const double2* __restrict__ sheet_d,
               const float2* __restrict__ sheet_f, const uint8_t* __restrict__ sheet_near,
               CellRec* __restrict__ recs, float2* __restrict__ coef, int64_t rc0, int64_t rc1) {
+  after_ready();
+  after_wait();
   const int64_t rc = rc0 + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (rc >= rc1) return;
   const int cx = (int)(rc % ig.nrcx) + ig.ox, cy = (int)(rc / ig.nrcx) + ig.oy;
@@ -1622,7 +1687,9 @@ __global__ void __launch_bounds__(IP_THREADS, 3) k_ip_ray(Geo g, IpGeo ig, IpRay
   extern __shared__ __align__(16) unsigned char ip_smem[];
   __shared__ long long next_s;
   const IpSmem<Q, K2> L(ig.nrow, a.near_cap);
+  after_ready();
   ip_tables<Q, K2>(ig, L, ip_smem);
+  after_wait();
   __syncthreads();
   long long next = 0;
   for (long long work = blockIdx.x; work < a.nwork * a.parts; work = next_s) {
@@ -1681,6 +1748,7 @@ k_ip_ray_batch(const MapDesc* __restrict__ maps, int nmaps, int64_t nitems,
 // before gave each ray a whole cell's pass (all k^2 rays of it).
 template <int Q, int K2, int NPR>
 __global__ void __launch_bounds__(128) k_ip_dump(Geo g, IpGeo ig, IpRayArgs a) {
+  after_wait();
   const int64_t work = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (work >= a.nwork) return;
   const int64_t f = a.idx[work];
@@ -1847,8 +1915,7 @@ int ip_near_cap(const IpGeo& ig, int64_t n) {
 
 #define IP_DECL_LAUNCH(V, Q, K2, NPR)                                                             \
   case V:                                                                                         \
-    k_ip_ray<Q, K2, NPR><<<(unsigned)grid, sh.threads, sh.smem, s>>>(g, ig, a);                     \
-    break;
+    return launch_after(k_ip_ray<Q, K2, NPR>, (unsigned)grid, sh.threads, sh.smem, s, g, ig, a);
 // A map of few cells is cut into more work items, each a share of a cell's row
 // groups (with the cell's set-up of its own), until every CTA slot has two.
 cudaError_t launch_ip_ray(int num_sms, cudaStream_t s, const Geo& g, const IpGeo& ig, IpRayArgs a) {
@@ -1863,8 +1930,7 @@ cudaError_t launch_ip_ray(int num_sms, cudaStream_t s, const Geo& g, const IpGeo
 
 #define IP_DECL_DUMP(V, Q, K2, NPR)                                                    \
   case V:                                                                              \
-    k_ip_dump<Q, K2, NPR><<<(unsigned)((a.nwork + 127) / 128), 128, 0, s>>>(g, ig, a); \
-    break;
+    return launch_after(k_ip_dump<Q, K2, NPR>, (unsigned)((a.nwork + 127) / 128), 128, 0, s, g, ig, a);
 cudaError_t launch_ip_dump(cudaStream_t s, const Geo& g, const IpGeo& ig, const IpRayArgs& a) {
   switch (ip_kernel_of(ig.variant)) { IP_VARIANTS(IP_DECL_DUMP) default: return cudaErrorInvalidValue; }
   return cudaGetLastError();
@@ -1927,10 +1993,14 @@ void mark(irs_plan_t* P, int slot, cudaStream_t s) {
   } while (0)
 
 // kernel launches of one map, reported through irs_plan_timings
-int far_launches(int64_t n) { return (n > 0 ? 4 : 0) + 3 + 1 + 2 + 1 + 2 + 1; }  // series mode
+int far_launches(const InterpState* S, int64_t n) {  // series mode
+  const int64_t ncells = (int64_t)S->ig.ncx * S->ig.ncy;
+  return (n > 0 ? 2 : 0) + (ncells > SCAN_B ? 2 : 1) + 1 + 2 * fft2d_launches(S->fft) + 1 + 1;
+}
 
 // Cell lists and far field; the per-cell finalize covers ray cells
-// [rc0, rc1) only (rc1 < 0: all of them).
+// [rc0, rc1) only (rc1 < 0: all of them).  Follows the mass sum, which zeroes
+// the cell counts.
 irs_status build_cells_and_far(irs_plan_t* P, const double* xy, const double* mass, int64_t n,
                                cudaStream_t s, int64_t rc0 = 0, int64_t rc1 = -1) {
   InterpState* S = S_(P);
@@ -1942,39 +2012,31 @@ irs_status build_cells_and_far(irs_plan_t* P, const double* xy, const double* ma
     if (st != IRS_OK) return st;
   }
   const double2* xy2 = reinterpret_cast<const double2*>(xy);
+  const bool learned = P->p.method == IRS_MLP && mlp_trained(P);
   S->n_last = n;
-  IP_TRY(cudaMemsetAsync(S->cell_count, 0, sizeof(int32_t) * ncells, s));
-  if (n > 0) k_ip_count<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(ig, xy2, n, S->lens_cell, S->cell_count);
-  const int64_t nb = (ncells + SCAN_B - 1) / SCAN_B;
-  k_scan_local<<<(unsigned)nb, SCAN_B, 0, s>>>(S->cell_count, S->cell_start, ncells, S->scan_blocks);
-  k_scan_blocks<<<1, 32, 0, s>>>(S->scan_blocks, nb, S->cell_start + ncells);
-  k_scan_add<<<(unsigned)nb, SCAN_B, 0, s>>>(S->cell_start, ncells, S->scan_blocks);
-  IP_TRY(cudaGetLastError());
-  if (n > 0) {
-    IP_TRY(cudaMemcpyAsync(S->cell_cursor, S->cell_start, sizeof(int32_t) * ncells,
-                           cudaMemcpyDeviceToDevice, s));
-    k_ip_scatter<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(S->lens_cell, n, S->cell_cursor, S->sorted_idx);
-    k_ip_sortcells<<<(unsigned)((ncells + 255) / 256), 256, 0, s>>>(S->cell_start, ncells, S->sorted_idx);
-    k_ip_fill<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(ig, xy2, mass, S->sorted_idx, S->lens_cell, n,
-                                                         S->lens_rel, S->lens_pos, S->lens_m, S->lens_pdf,
-                                                         S->lens_mdf);
-  }
-  IP_TRY(cudaGetLastError());
+  const unsigned lens_blocks = (unsigned)((n + 255) / 256);
+  if (n > 0) IP_TRY(launch_after(k_ip_count, lens_blocks, 256, 0, s, ig, xy2, n, S->lens_cell, S->cell_count));
+  const unsigned nb = (unsigned)((ncells + SCAN_B - 1) / SCAN_B);
+  IP_TRY(launch_after(k_scan_local, nb, SCAN_B, 0, s, S->cell_count, S->cell_start, S->cell_cursor, ncells,
+                      S->scan_blocks));
+  if (nb > 1)
+    IP_TRY(launch_after(k_scan_add, nb, SCAN_B, 0, s, S->cell_start, S->cell_cursor, ncells, S->scan_blocks));
+  if (n > 0) IP_TRY(launch_after(k_ip_scatter, lens_blocks, 256, 0, s, S->lens_cell, n, S->cell_cursor, S->sorted_idx));
+  IP_TRY(launch_after(k_ip_cells, (unsigned)((ncells + CELLS_B - 1) / CELLS_B), CELLS_B, 0, s, ig, S->cell_start, xy2,
+                      mass, S->lens_cell, S->sorted_idx, S->lens_rel, learned ? S->lens_pos : nullptr, S->lens_m, S->lens_pdf, S->lens_mdf,
+                      learned ? nullptr : S->mpole_d, S->mpole_f));
   mark(P, EV_CELLS, s);
   // far field: the network (trained IRS_MLP plans) or the FFT series
   MlpFar far{};
-  if (P->p.method == IRS_MLP && mlp_trained(P)) {
+  if (learned) {
     irs_status st = mlp_prepare(P, xy, mass, n, ig.gx0, ig.gy0, ig.h, ig.nrcx, ig.nrcy, ig.ox, ig.oy, &far, s);
     if (st != IRS_OK) return st;
   } else {
-    k_ip_p2m<<<(unsigned)((ncells + 127) / 128), 128, 0, s>>>(ig, S->cell_start, S->lens_pos, S->lens_m,
-                                                             S->mpole_d, S->mpole_f);
-    IP_TRY(cudaGetLastError());
     IP_TRY(fft2d_forward(S->mpole_d, S->spec_d, IP_PD, S->mpole_f, S->spec_f, IP_P - IP_PD, ig.ncx, ig.ncy, ncells,
                          S->fft, s));
     const int64_t G = (int64_t)S->fft.Nx * S->fft.Ny;
-    k_ip_m2l_freq<<<(unsigned)((G + 127) / 128), 128, 0, s>>>(G, S->spec_d, S->spec_f, S->kspec_d, S->kspec_f);
-    IP_TRY(cudaGetLastError());
+    IP_TRY(launch_after(k_ip_m2l_freq, (unsigned)((G + 127) / 128), 128, 0, s, G, S->spec_d, S->spec_f, S->kspec_d,
+                        S->kspec_f));
     IP_TRY(fft2d_inverse(S->spec_d, S->conv_d, IP_KD, S->spec_f, S->conv_f, IP_KF - IP_KD, S->fft, ig.ncx, ig.ncy,
                          ncells, s));
   }
@@ -1988,14 +2050,15 @@ irs_status build_cells_and_far(irs_plan_t* P, const double* xy, const double* ma
       const int cta_cells = rc1 - rc0 <= 4 * FG_CELLS * (int64_t)P->num_sms ? FG_CELLS / 2 : FG_CELLS;
       const unsigned nb = (unsigned)((rc1 - rc0 + cta_cells - 1) / cta_cells);
       auto* kern = few ? k_ip_finalize_group<21> : k_ip_finalize_group<FIN_K32>;
-      kern<<<nb, 32 * FG_WARPS, 0, s>>>(P->g, ig, P->d_msum, S->cell_start, S->lens_pdf, S->lens_mdf, S->conv_d,
-                                        S->conv_f, S->sheet_d, S->sheet_f, S->sheet_near, S->recs, S->coef, rc0, rc1, cta_cells);
+      IP_TRY(launch_after(kern, nb, 32 * FG_WARPS, 0, s, P->g, ig, P->d_msum, S->cell_start, S->lens_pdf, S->lens_mdf,
+                          S->conv_d, S->conv_f, S->sheet_d, S->sheet_f, S->sheet_near, S->recs, S->coef, rc0, rc1,
+                          cta_cells));
     } else {
       const unsigned nb = (unsigned)((rc1 - rc0 + 63) / 64);
       auto* kern = few ? k_ip_finalize<21> : k_ip_finalize<FIN_K32>;
-      kern<<<nb, 64, 0, s>>>(P->g, ig, P->d_msum, S->cell_start, S->lens_pos, S->lens_m, S->lens_pdf, S->lens_mdf,
-                             S->conv_d, S->conv_f, far, S->sheet_d, S->sheet_f, S->sheet_near, S->recs, S->coef, rc0,
-                             rc1);
+      IP_TRY(launch_after(kern, nb, 64, 0, s, P->g, ig, P->d_msum, S->cell_start, S->lens_pos, S->lens_m, S->lens_pdf,
+                          S->lens_mdf, S->conv_d, S->conv_f, far, S->sheet_d, S->sheet_f, S->sheet_near, S->recs,
+                          S->coef, rc0, rc1));
     }
   }
   IP_TRY(cudaGetLastError());
@@ -2128,6 +2191,8 @@ irs_status interp_plan(irs_plan_t* P) {
   S->ws_bytes = off;
   char* b = static_cast<char*>(S->ws);
   S->cell_count = reinterpret_cast<int32_t*>(b + o_cnt);
+  P->d_zero = S->cell_count;
+  P->n_zero = ncells;
   S->cell_start = reinterpret_cast<int32_t*>(b + o_start);
   S->cell_cursor = reinterpret_cast<int32_t*>(b + o_cur);
   S->scan_blocks = reinterpret_cast<int32_t*>(b + o_sb);
@@ -2196,7 +2261,7 @@ irs_status interp_run(irs_plan_t* P, const double* xy, const double* mass, int64
   irs_status st = build_cells_and_far(P, xy, mass, n, s, rc0, rc1);
   if (st != IRS_OK) return st;
   mark(P, EV_RAY0, s);
-  P->launches += far_launches(n) - (rc1 > rc0 ? 0 : 1) + (row1 > row0 ? 1 : 0);
+  P->launches += far_launches(S, n) - (rc1 > rc0 ? 0 : 1) + (row1 > row0 ? 1 : 0);
   if (row1 > row0) {
     IpRayArgs a = ray_args(P);
     a.counts = counts;

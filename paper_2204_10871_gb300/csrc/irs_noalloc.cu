@@ -128,6 +128,6 @@ extern "C" irs_status irs_make_map_brute_noalloc(const irs_params* params, const
   if (irs::launch_brute_setup(&P, 0, P.g.nry, s) != cudaSuccess) return IRS_ERR_CUDA;
   if (irs::launch_brute_map(&P, lens_xy, mass, n, 0, P.g.nry, counts, s) != cudaSuccess)
     return IRS_ERR_CUDA;
-  if (mag && irs::launch_magnify(&P, counts, mag, s) != cudaSuccess) return IRS_ERR_CUDA;
+  if (mag && irs::launch_magnify(&P, counts, mag, true, s) != cudaSuccess) return IRS_ERR_CUDA;
   return IRS_OK;
 }
