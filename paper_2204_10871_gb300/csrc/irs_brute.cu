@@ -327,10 +327,20 @@ __device__ __forceinline__ void brute_beta(const Geo& g, const TileRec& rec, flo
 //   variant 10 (2 quads, 4 packed pairs):           MUFU  80, FP32  96 cycles
 // bounding the pair sum at 71, 77 and 83 % of the FP32 peak.  Measured on
 // the 1e5-lens band (one GB300, 2070 MHz): 59.7 % (variant 11), 62.3 %
-// (variant 0, the default), 60.6 % (variant 10): with two quads the FP32
-// pipe's longer dependent chains cost more than the MUFU cycles they save.
+// (variant 0, the default), 60.6 % (variant 10), all with four CTAs per SM and
+// two lenses an iteration: with two quads the FP32 pipe's longer dependent
+// chains cost more than the MUFU cycles they save.
+//
+// Variant 0 runs three CTAs per SM (168 registers) and eight lenses an
+// iteration: more independent chains per warp keep the MUFU busier than more
+// warps do.  The 64-row band of the 1e5-lens lattice takes 415 ms (64.7 %, 84 %
+// of the MUFU's bound); four CTAs and 2, 4 or 8 lenses took 437, 437 and 436,
+// three CTAs and 2, 4, 6, 16 or 32 lenses 432, 431, 421, 415 and 418, two CTAs
+// and 4, 8 or 16 lenses 426, 430 and 433.  CTAs of one or two warps, each with
+// its own copy of the lenses, take 452 and 447 us where this form takes 411 (128^2
+// map, 150 lenses).
 #define BR_VARIANTS(X)                                                                         \
-  X(0, 16, 0, 1, 1, 512) X(1, 16, 8, 0, 0, 512) X(2, 8, 4, 0, 0, 512) X(3, 8, 2, 0, 0, 512)      \
+  X(0, 16, 0, 1, 1, 384) X(1, 16, 8, 0, 0, 512) X(2, 8, 4, 0, 0, 512) X(3, 8, 2, 0, 0, 512)      \
   X(4, 16, 4, 0, 0, 512) X(5, 16, 2, 0, 0, 512) X(6, 16, 8, 0, 1, 512) X(7, 16, 6, 0, 1, 512)     \
   X(8, 16, 2, 0, 1, 512) X(9, 16, 4, 0, 1, 640) X(10, 16, 0, 2, 1, 512) X(11, 16, 4, 0, 1, 512)  \
   X(12, 16, 0, 3, 1, 512) X(13, 8, 0, 1, 1, 512) X(14, 16, 2, 1, 1, 512) X(15, 16, 4, 1, 1, 512)
@@ -360,13 +370,20 @@ k_brute(Geo g, const double2* __restrict__ xy, const double* __restrict__ mass, 
   __shared__ float acc_s[4][R][NT];  // x hi, x lo, y hi, y lo
   __shared__ float2 ty_s[BR_TY / 2];  // row offsets to the tile centre, in pairs
   __shared__ TileRec rec;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, lane = tid & 31;
   bool waited = false;
   after_ready();
 
   for (int64_t work = blockIdx.x; work < nwork; work += gridDim.x) {
     const int64_t tile = (row0 / BR_TY) * ntx + work;  // tile rows covering [row0, row1)
     const TileGeo tg = tile_geo(g, tile, ntx);
+    // A warp whose rows lie outside the band or the lattice sums nothing.  Which
+    // warp takes which rows varies from tile to tile: the warps of a CTA go to
+    // the SM's four schedulers in turn, and rows that the band leaves out would
+    // idle the same schedulers in every CTA (a 64-row band across two tile rows
+    // sums 64 to 80 rows instead of 128).
+    const int warp = ((tid >> 5) + (int)((uint32_t)work * 0x9E3779B1u >> 30)) & (BR_TY / R - 1);
+    const bool live = tg.j0 + warp * R < min(row1, tg.j1) && tg.j0 + (warp + 1) * R > row0;
     const double zx = g.a1 + tg.ci * g.dx3, zy = g.b1 + tg.cj * g.dx3;
     const int64_t col = tg.i0 + lane;
     const float tx = (float)(((double)col + 0.5 - tg.ci) * g.dx3);
@@ -420,8 +437,9 @@ k_brute(Geo g, const double2* __restrict__ xy, const double* __restrict__ mass, 
 #pragma unroll
       for (int q = 0; q < NPK; ++q) PAX[q] = PAY[q] = make_float2(0.f, 0.f);
       // lenses in this stage, rounded up to the unroll (padding is massless)
-      const int cnt = (int)min((int64_t)BR_LT, ((n - base) + 7) & ~(int64_t)7);
-#pragma unroll 2
+      const int cnt = live ? (int)min((int64_t)BR_LT, ((n - base) + 7) & ~(int64_t)7) : 0;
+      constexpr int UNROLL = TPSM == 384 ? 8 : 2;
+#pragma unroll UNROLL
       for (int jl = 0; jl < cnt; ++jl) {
         float4 L = lens_s[jl];
         float2 M, DX, DX2;
@@ -522,7 +540,7 @@ k_brute(Geo g, const double2* __restrict__ xy, const double* __restrict__ mass, 
     const bool colok = col < tg.i1;
     const uint32_t npx = (uint32_t)g.npix_x, npy = (uint32_t)g.npix_y;
 #pragma unroll 1
-    for (int r = 0; r < R; r += 2) {
+    for (int r = live ? 0 : R; r < R; r += 2) {
       const int64_t row = tg.j0 + warp * R + r;
       const float2 TY = ty_s[(warp * R + r) / 2], NTY = make_float2(-TY.x, -TY.y);
       float2 PR = make_float2(0.f, 0.f), PI = make_float2(0.f, 0.f);

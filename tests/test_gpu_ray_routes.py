@@ -101,6 +101,30 @@ def test_brute_map_equals_its_rays(variant, n):
     assert torch.isnan(b1[95:]).all() and (p1[95:] == -1).all()
 
 
+@pytest.mark.parametrize("variant", [0, 2, 11])
+def test_brute_bands_equal_their_rays(variant):
+    """Bands that start and end inside a tile or inside one warp's rows, down
+    to a single row, and the last, ragged tile row: warps without a row of the
+    band sum nothing."""
+    torch = require_gpu()
+    args = (0.3, 0.1, 0.25, (-2, 3, -2.5, 2.1), (37, 29), 4.0)
+    po, pl = params_pair(*args, method=irs.IRS_BRUTE, n_star=300, kernel_variant=variant)
+    xy, m = lenses_for(oracle.size(po), 300, shape="uniform", seed=5, kappa_star=args[0])
+    dxy, dm = to_dev(torch, xy, m)
+    with irs.Plan(pl) as plan:
+        nrx, nry = int(plan.info.n_rays_x), int(plan.info.n_rays_y)
+        counts, _ = plan.make_map(dxy, dm)
+        _, pix = plan.shoot_rays(dxy, dm, torch.arange(nrx * nry, device="cuda"))
+        plan.sync()
+        pix = pix.cpu().numpy()
+        for r0, r1 in ((0, 1), (15, 17), (48, 112), (63, 64), (70, 71), (nry - 1, nry), (nry - 70, nry)):
+            counts.zero_()
+            irs.irs_make_map_rows(plan.handle, dxy, dm, r0, r1, counts)
+            plan.sync()
+            want = _counts_of(pix[r0 * nrx:r1 * nrx], (pl.npix_y, pl.npix_x))
+            assert np.array_equal(counts.cpu().numpy().astype(np.int64), want), (r0, r1)
+
+
 def test_masses_of_both_signs():
     """Lens masses may have either sign; the bound that leaves units out takes
     their magnitudes."""
