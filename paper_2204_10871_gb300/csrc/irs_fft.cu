@@ -100,10 +100,16 @@ struct FastDiv {
   __device__ __forceinline__ uint32_t div(uint32_t x) const { return d > 1u ? __umulhi(x, m) : x; }
 };
 
+// Place of entry t of the twiddle table in shared memory: a gap after every 128
+// bytes.  The later stages of a pass read every 4th, 8th or 16th entry, which
+// without the gaps share one or two of the eight (sixteen) bank groups.
+template <class T> __host__ __device__ __forceinline__ int tw_place(int t) { return t + (t >> (sizeof(T) == 16 ? 3 : 4)); }
+
 // W_L^t for 0 <= t < L from the half table, conjugated for the inverse
 template <bool INV, class T>
 __device__ __forceinline__ T tw_at(const T* w, int t, int half) {
-  T v = t < half ? w[t] : c_neg(w[t - half]);
+  T v = w[tw_place<T>(t < half ? t : t - half)];
+  if (t >= half) v = c_neg(v);
   return INV ? c_conj(v) : v;
 }
 
@@ -178,13 +184,13 @@ __device__ __forceinline__ void fft_lines(const T* in, T* out, const FftLines& d
                                           int64_t block, float4* sm) {
   const int L = d.L, B = d.B, n3 = d.n3, n2 = d.n2, half_L = L / 2, LS = L + 1;
   T* x = reinterpret_cast<T*>(sm);      // [B][LS]
-  T* w = x + (size_t)B * LS;            // [L/2]
+  T* w = x + (size_t)B * LS;            // [L/2] at tw_place
   const int64_t blocks_per_grid = (d.n_lines + B - 1) / B;
   const int64_t grid = block / blocks_per_grid, line0 = (block - grid * blocks_per_grid) * B;
   in += grid * d.in_grid_stride;
   out += grid * d.out_grid_stride;
   const int nthr = blockDim.x;
-  for (int k = threadIdx.x; k < half_L; k += nthr) w[k] = tw_elem<T>(tw[k]);
+  for (int k = threadIdx.x; k < half_L; k += nthr) w[tw_place<T>(k)] = tw_elem<T>(tw[k]);
   int pow3 = 1;
   for (int i = 0; i < n3; ++i) pow3 *= 3;
   const int np2 = fft_passes2(n2), np3 = (n3 + 1) / 2, np = np2 + np3;
@@ -307,7 +313,7 @@ cudaError_t fft_twiddles(int L, float4** d_tw) {
 }
 
 cudaError_t fft_setup_attributes() {
-  const int max_smem = (int)(((size_t)FFT_MAX_LEN + 1 + FFT_MAX_LEN / 2) * sizeof(float4));
+  const int max_smem = (int)(((size_t)FFT_MAX_LEN + 1 + tw_place<float4>(FFT_MAX_LEN / 2)) * sizeof(float4));
   cudaError_t e = cudaFuncSetAttribute(k_fft_lines<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_fft_lines<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
@@ -317,15 +323,23 @@ cudaError_t fft_setup_attributes() {
 namespace {
 
 // Lines per CTA for a line length L: as many as keep the CTA's lines and
-// twiddle table within a quarter of the SM's shared memory, so that several
-// CTAs share an SM and hide each other's barriers; at least one line.
-constexpr size_t FFT_CTA_BYTES = 52 * 1024;
-size_t cta_bytes(int L, int B, size_t elem) { return ((size_t)B * (L + 1) + L / 2) * elem; }
+// twiddle table within a third of the SM's shared memory (three CTAs of 256
+// threads at 80 registers share an SM and hide each other's barriers), at
+// least one; 8 double-float or 16 FP32 columns where they fit, a 128-byte
+// segment of every row and a set of lines whose elements lie in distinct banks.
+// Fewer while a launch would not give every SM three CTAs.
+constexpr size_t FFT_CTA_BYTES = 74 * 1024;
+constexpr int64_t FFT_FILL = 3 * 152;
+size_t cta_bytes(int L, int B, size_t elem) {
+  return ((size_t)B * (L + 1) + (elem == sizeof(float4) ? tw_place<float4>(L / 2) : tw_place<float2>(L / 2))) * elem;
+}
 int lines_per_cta(int L, size_t elem) {
+  const int most = (int)(128 / elem);
   int B = 1;
-  while (B < 16 && cta_bytes(L, B + 1, elem) <= FFT_CTA_BYTES) ++B;
+  while (B < most && cta_bytes(L, B + 1, elem) <= FFT_CTA_BYTES) ++B;
   return B;
 }
+int64_t ctas(const FftLines& d, int B, int ngrids) { return (d.n_lines + B - 1) / B * ngrids; }
 
 // Threads of a CTA with `smem` bytes: the SM's 24 warps over the CTAs that fit
 int cta_threads(size_t smem) {
@@ -340,7 +354,11 @@ cudaError_t launch_lines(bool inverse, const float4* in4, float4* out4, FftLines
                          float2* out2, FftLines d2, int ngrids2, const float4* tw, cudaStream_t s) {
   d4.B = lines_per_cta(d4.L, sizeof(float4));
   d2.B = lines_per_cta(d2.L, sizeof(float2));
-  const int64_t b4 = (d4.n_lines + d4.B - 1) / d4.B * ngrids4, b2 = (d2.n_lines + d2.B - 1) / d2.B * ngrids2;
+  while (ctas(d4, d4.B, ngrids4) + ctas(d2, d2.B, ngrids2) < FFT_FILL && d4.B > 1) {
+    d4.B = (d4.B + 1) / 2;
+    d2.B = (d2.B + 1) / 2;
+  }
+  const int64_t b4 = ctas(d4, d4.B, ngrids4), b2 = ctas(d2, d2.B, ngrids2);
   const size_t smem4 = cta_bytes(d4.L, d4.B, sizeof(float4)), smem2 = cta_bytes(d2.L, d2.B, sizeof(float2));
   auto launch = [&](int64_t n4, int64_t n2, size_t smem) {
     if (n4 + n2 <= 0) return cudaSuccess;
