@@ -53,45 +53,65 @@ __device__ __forceinline__ float2 df_mul(float2 x, float2 y) {
   return make_float2(h, l);
 }
 
-// a*b + s*c*d for s = +-1: one rounding pass for a complex product's part
-__device__ __forceinline__ float2 df_dot2(float2 a, float2 b, float2 c, float2 d, float sgn) {
-  const float p1 = __fmul_rn(a.x, b.x);
-  float e1 = __fmaf_rn(a.x, b.x, -p1);
-  e1 = __fmaf_rn(a.x, b.y, e1);
-  e1 = __fmaf_rn(a.y, b.x, e1);
-  const float ch = sgn * c.x, cl = sgn * c.y;  // exact sign flips
-  const float p2 = __fmul_rn(ch, d.x);
-  float e2 = __fmaf_rn(ch, d.x, -p2);
-  e2 = __fmaf_rn(ch, d.y, e2);
-  e2 = __fmaf_rn(cl, d.x, e2);
-  float s, t, h, l;
-  df_two_sum(p1, p2, s, t);
-  t = __fadd_rn(t, __fadd_rn(e1, e2));
-  df_fast_two_sum(s, t, h, l);
-  return make_float2(h, l);
+// Complex double-float, stored as float4 (re.hi, im.hi, re.lo, im.lo): the two
+// parts' high words, and their low words, are register pairs, so that the sums
+// go through the packed FP32x2 instructions, real and imaginary part at once
+// (the same roundings in half the issue slots).  Products stay scalar, since their
+// operands cross between the parts, up to the packed sum of the two products.
+__device__ __forceinline__ float2 dfc_hi(float4 z) { return make_float2(z.x, z.y); }
+__device__ __forceinline__ float2 dfc_lo(float4 z) { return make_float2(z.z, z.w); }
+__device__ __forceinline__ float2 dfc_re(float4 z) { return make_float2(z.x, z.z); }
+__device__ __forceinline__ float2 dfc_im(float4 z) { return make_float2(z.y, z.w); }
+__device__ __forceinline__ float4 dfc_make(float2 re, float2 im) { return make_float4(re.x, im.x, re.y, im.y); }
+
+// a - b: one rounding
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
+
+// high words s + e renormalised (Fast2Sum)
+__device__ __forceinline__ float4 dfc_norm(float2 s, float2 e) {
+  const float2 h = __fadd2_rn(s, e), l = sub2(e, sub2(h, s));
+  return make_float4(h.x, h.y, l.x, l.y);
 }
 
-// Complex double-float, stored as float4 (re.hi, re.lo, im.hi, im.lo).
-__device__ __forceinline__ float2 dfc_re(float4 z) { return make_float2(z.x, z.y); }
-__device__ __forceinline__ float2 dfc_im(float4 z) { return make_float2(z.z, z.w); }
-__device__ __forceinline__ float4 dfc_make(float2 re, float2 im) { return make_float4(re.x, re.y, im.x, im.y); }
+// x + y + lo for high words x, y (TwoSum)
+__device__ __forceinline__ float4 dfc_sum(float2 x, float2 y, float2 lo) {
+  const float2 s = __fadd2_rn(x, y), bb = sub2(s, x);
+  const float2 e = __fadd2_rn(sub2(x, sub2(s, bb)), sub2(y, bb));
+  return dfc_norm(s, __fadd2_rn(e, lo));
+}
 
 __device__ __forceinline__ float4 dfc_mul(float4 a, float4 b) {
-  const float2 ar = dfc_re(a), ai = dfc_im(a), br = dfc_re(b), bi = dfc_im(b);
-  return dfc_make(df_dot2(ar, br, ai, bi, -1.0f), df_dot2(ar, bi, ai, br, 1.0f));
+  // a.re b.re - a.im b.im and a.re b.im + a.im b.re, each product as p + e
+  float2 p1, e1, p2, e2;
+  p1.x = __fmul_rn(a.x, b.x);
+  p1.y = __fmul_rn(a.x, b.y);
+  e1.x = __fmaf_rn(a.z, b.x, __fmaf_rn(a.x, b.z, __fmaf_rn(a.x, b.x, -p1.x)));
+  e1.y = __fmaf_rn(a.z, b.y, __fmaf_rn(a.x, b.w, __fmaf_rn(a.x, b.y, -p1.y)));
+  p2.x = __fmul_rn(-a.y, b.y);
+  p2.y = __fmul_rn(a.y, b.x);
+  e2.x = __fmaf_rn(-a.w, b.y, __fmaf_rn(-a.y, b.w, __fmaf_rn(-a.y, b.y, -p2.x)));
+  e2.y = __fmaf_rn(a.w, b.x, __fmaf_rn(a.y, b.z, __fmaf_rn(a.y, b.x, -p2.y)));
+  return dfc_sum(p1, p2, __fadd2_rn(e1, e2));
 }
 
 __device__ __forceinline__ float4 dfc_add(float4 a, float4 b) {
-  return dfc_make(df_add(dfc_re(a), dfc_re(b)), df_add(dfc_im(a), dfc_im(b)));
+  return dfc_sum(dfc_hi(a), dfc_hi(b), __fadd2_rn(dfc_lo(a), dfc_lo(b)));
 }
 
 __device__ __forceinline__ float4 dfc_sub(float4 a, float4 b) {
-  return dfc_make(df_sub(dfc_re(a), dfc_re(b)), df_sub(dfc_im(a), dfc_im(b)));
+  const float2 x = dfc_hi(a), y = dfc_hi(b);
+  const float2 s = sub2(x, y), bb = sub2(s, x);
+  const float2 e = sub2(sub2(x, sub2(s, bb)), __fadd2_rn(y, bb));
+  return dfc_norm(s, __fadd2_rn(e, sub2(dfc_lo(a), dfc_lo(b))));
 }
 
 // x * s for a double-float real s
 __device__ __forceinline__ float4 dfc_scale(float4 a, float2 s) {
-  return dfc_make(df_mul(dfc_re(a), s), df_mul(dfc_im(a), s));
+  const float2 p = make_float2(__fmul_rn(a.x, s.x), __fmul_rn(a.y, s.x));
+  float2 e;
+  e.x = __fmaf_rn(a.z, s.x, __fmaf_rn(a.x, s.y, __fmaf_rn(a.x, s.x, -p.x)));
+  e.y = __fmaf_rn(a.w, s.x, __fmaf_rn(a.y, s.y, __fmaf_rn(a.y, s.x, -p.y)));
+  return dfc_norm(p, e);
 }
 
 // FP64 <-> double-float
@@ -102,7 +122,7 @@ __host__ __device__ __forceinline__ float2 df_from_double(double x) {
 __host__ __device__ __forceinline__ double df_to_double(float2 x) { return (double)x.x + (double)x.y; }
 __host__ __device__ __forceinline__ float4 dfc_from_double(double re, double im) {
   const float2 r = df_from_double(re), i = df_from_double(im);
-  return make_float4(r.x, r.y, i.x, i.y);
+  return make_float4(r.x, i.x, r.y, i.y);
 }
 
 }  // namespace irs

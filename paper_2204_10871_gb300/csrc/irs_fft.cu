@@ -39,15 +39,15 @@ namespace {
 constexpr int FFT_REGS = 80;  // per thread: 24 warps per SM
 
 // Complex arithmetic of the two element types: float4 is double-float
-// (re.hi, re.lo, im.hi, im.lo), float2 is FP32 (re, im).
+// (re.hi, im.hi, re.lo, im.lo), float2 is FP32 (re, im).
 __device__ __forceinline__ float4 c_add(float4 a, float4 b) { return dfc_add(a, b); }
 __device__ __forceinline__ float4 c_sub(float4 a, float4 b) { return dfc_sub(a, b); }
 __device__ __forceinline__ float4 c_mul(float4 a, float4 b) { return dfc_mul(a, b); }
 __device__ __forceinline__ float4 c_neg(float4 a) { return make_float4(-a.x, -a.y, -a.z, -a.w); }
-__device__ __forceinline__ float4 c_conj(float4 a) { return make_float4(a.x, a.y, -a.z, -a.w); }
+__device__ __forceinline__ float4 c_conj(float4 a) { return make_float4(a.x, -a.y, a.z, -a.w); }
 __device__ __forceinline__ float4 c_half(float4 a) { return make_float4(0.5f * a.x, 0.5f * a.y, 0.5f * a.z, 0.5f * a.w); }
-__device__ __forceinline__ float2 c_add(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ float2 c_sub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
+__device__ __forceinline__ float2 c_add(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 c_sub(float2 a, float2 b) { return sub2(a, b); }
 __device__ __forceinline__ float2 c_mul(float2 a, float2 b) {
   return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
 }
@@ -62,7 +62,7 @@ template <> __device__ __forceinline__ float2 c_zero<float2>() { return make_flo
 // twiddle table entry in the element type (the table holds double-float)
 template <class T> __device__ __forceinline__ T tw_elem(float4 v);
 template <> __device__ __forceinline__ float4 tw_elem<float4>(float4 v) { return v; }
-template <> __device__ __forceinline__ float2 tw_elem<float2>(float4 v) { return make_float2(v.x, v.z); }
+template <> __device__ __forceinline__ float2 tw_elem<float2>(float4 v) { return dfc_hi(v); }
 
 // Radix-3 butterfly on a and the twiddled p, q:
 // x0 = a + t1, x1,2 = a - t1/2 -+ i s3 (p - q) with t1 = p + q and
@@ -74,10 +74,11 @@ __device__ __forceinline__ void radix3(float4 a, float4 p, float4 q, bool inv, f
   const float4 t1 = dfc_add(p, q);
   const float4 t2 = dfc_sub(a, c_half(t1));
   const float4 dd = dfc_sub(p, q);
-  const float2 u = df_mul(s3, dfc_im(dd)), v = df_mul(s3, dfc_re(dd));  // s3 Im(dd), s3 Re(dd)
+  // (s3 Im(dd), -s3 Re(dd))
+  const float4 uv = dfc_make(df_mul(s3, dfc_im(dd)), df_mul(df_neg(s3), dfc_re(dd)));
   x0 = dfc_add(a, t1);
-  x1 = dfc_make(df_add(dfc_re(t2), u), df_sub(dfc_im(t2), v));
-  x2 = dfc_make(df_sub(dfc_re(t2), u), df_add(dfc_im(t2), v));
+  x1 = dfc_add(t2, uv);
+  x2 = dfc_sub(t2, uv);
 }
 __device__ __forceinline__ void radix3(float2 a, float2 p, float2 q, bool inv, float2& x0, float2& x1,
                                        float2& x2) {

@@ -117,7 +117,7 @@ struct InterpState {
   float4* lens_rel;
   double2* lens_pos;
   double* lens_m;
-  float4* lens_pdf;  // positions as complex double-float (x.hi, x.lo, y.hi, y.lo)
+  float4* lens_pdf;  // positions as complex double-float
   float2* lens_mdf;  // masses as double-float
   // far-field convolution: complex double-float (float4, irs_df.cuh) for
   // the low orders, FP32 (float2) for the rest
@@ -405,7 +405,7 @@ __global__ void __launch_bounds__(128) k_ip_m2l_freq(int64_t G, float4* __restri
     const double sc = ((j & 1) ? -1.0 : 1.0) * ifact;
     if (j < IP_PD) {
       Ad[j] = dfc_scale(spec_d[(int64_t)j * G + f], df_from_double(sc));
-      Af[j] = make_float2(Ad[j].x, Ad[j].z);
+      Af[j] = dfc_hi(Ad[j]);
     } else {
       const float2 v = spec_f[(int64_t)(j - IP_PD) * G + f];
       Af[j] = make_float2(v.x * (float)sc, v.y * (float)sc);
@@ -436,7 +436,7 @@ __global__ void __launch_bounds__(128) k_ip_m2l_freq(int64_t G, float4* __restri
   for (int k = 0; k < IP_KF; ++k) {
     if (k > 0) kfact /= (double)k;
     if (k < IP_KD) {
-      const float4 c = dfc_add(Cd[k], make_float4(Cf[k].x, 0.f, Cf[k].y, 0.f));
+      const float4 c = dfc_add(Cd[k], make_float4(Cf[k].x, Cf[k].y, 0.f, 0.f));
       spec_d[(int64_t)k * G + f] = dfc_scale(c, df_from_double(kfact));
     } else {
       spec_f[(int64_t)(k - IP_KD) * G + f] = make_float2(Cf[k].x * (float)kfact, Cf[k].y * (float)kfact);
@@ -733,20 +733,20 @@ k_ip_finalize_group(Geo g, IpGeo ig, const double* __restrict__ msum, const int3
       const float2 m2 = next_m;
       load(t + FG_LANES);
       if (t < total) {
-        const float2 dre = df_mul(df_sub(make_float2(q4.x, q4.y), zx_df), ih_df);
-        const float2 dim = df_mul(df_sub(make_float2(q4.z, q4.w), zy_df), ih_df);
+        const float2 dre = df_mul(df_sub(dfc_re(q4), zx_df), ih_df);
+        const float2 dim = df_mul(df_sub(dfc_im(q4), zy_df), ih_df);
         const float4 inv = dfc_recip(dre, dim);
         float4 pw = dfc_scale(inv, m2);  // + m d^-(k+1)
 #pragma unroll
         for (int k = 0; k < FIN_K64; ++k) {
           val_s[warp][4 * k][lane] = pw.x;
-          val_s[warp][4 * k + 1][lane] = pw.y;
-          val_s[warp][4 * k + 2][lane] = pw.z;
+          val_s[warp][4 * k + 1][lane] = pw.z;
+          val_s[warp][4 * k + 2][lane] = pw.y;
           val_s[warp][4 * k + 3][lane] = pw.w;
           pw = dfc_mul(pw, inv);
         }
-        const float2 invf = make_float2(inv.x, inv.z);
-        float2 pf = make_float2(pw.x, pw.z);
+        const float2 invf = dfc_hi(inv);
+        float2 pf = dfc_hi(pw);
 #pragma unroll
         for (int k = 0; k < NF; ++k) {
           val_s[warp][4 * FIN_K64 + 2 * k][lane] = pf.x;
@@ -881,8 +881,8 @@ k_ip_finalize(Geo g, IpGeo ig, const double* __restrict__ msum, const int32_t* _
       pf = make_float2((float)pw.re, (float)pw.im);
     } else {  // series mode: the same terms in double-float on the FP32 pipes
       const float4 q4 = pos_df[pl];
-      const float2 dre = df_mul(df_sub(make_float2(q4.x, q4.y), zx_df), ih_df);
-      const float2 dim = df_mul(df_sub(make_float2(q4.z, q4.w), zy_df), ih_df);
+      const float2 dre = df_mul(df_sub(dfc_re(q4), zx_df), ih_df);
+      const float2 dim = df_mul(df_sub(dfc_im(q4), zy_df), ih_df);
       const float4 inv = dfc_recip(dre, dim);
       float4 pw = dfc_scale(inv, m_df[pl]);  // + m d^-(k+1)
 #pragma unroll
@@ -890,8 +890,8 @@ k_ip_finalize(Geo g, IpGeo ig, const double* __restrict__ msum, const int32_t* _
         accd[k] = dfc_add(accd[k], pw);
         pw = dfc_mul(pw, inv);
       }
-      invf = make_float2(inv.x, inv.z);
-      pf = make_float2(pw.x, pw.z);
+      invf = dfc_hi(inv);
+      pf = dfc_hi(pw);
     }
 #pragma unroll
     for (int k = 0; k < NF; ++k) {
