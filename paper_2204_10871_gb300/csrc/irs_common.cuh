@@ -35,7 +35,9 @@ struct Geo {
 // A kernel launched by launch_after may start while the kernel before it in the
 // stream still runs (programmatic stream serialisation): it calls after_wait()
 // before it touches anything that earlier work writes or still reads, and
-// kernels that another may follow call after_ready() first thing.  Both do
+// kernels that another may follow call after_ready() first thing (not the one
+// before a persistent grid that fills the SMs: its CTAs are placed best on empty
+// ones).  Both do
 // nothing after an ordinary launch.  Every thread block waits, so that a kernel
 // that has finished implies that all before it have.  The first kernel of a
 // call is launched the ordinary way: caller's buffers are complete when it

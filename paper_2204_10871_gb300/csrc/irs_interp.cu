@@ -652,7 +652,10 @@ k_ip_finalize_group(Geo g, IpGeo ig, const double* __restrict__ msum, const int3
   __shared__ float val_s[FG_WARPS][NV][33];
   __shared__ int from_s[FG_WARPS][4][FG_RANGES], off_s[FG_WARPS][4][FG_RANGES + 1];
   __shared__ float2 sum_s[FG_CELLS][2 * FIN_K64];
-  after_ready();
+  // No after_ready: the ray pass that follows is a grid of CTAs that stay, six
+  // to an SM.  Started beside this kernel's CTAs they found its shared memory
+  // in pieces and 100 of 152 SMs kept only five of them to the end (paper-mid
+  // map 12.0 ms, 11.5 this way; high-res 128.7 and 123.0; 128^2 149 and 148 us).
   after_wait();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t base = rc0 + (int64_t)blockIdx.x * cta_cells;
@@ -821,8 +824,7 @@ k_ip_finalize(Geo g, IpGeo ig, const double* __restrict__ msum, const int32_t* _
               const float2* __restrict__ conv_f, MlpFar far, const double2* __restrict__ sheet_d,
               const float2* __restrict__ sheet_f, const uint8_t* __restrict__ sheet_near,
               CellRec* __restrict__ recs, float2* __restrict__ coef, int64_t rc0, int64_t rc1) {
-  after_ready();
-  after_wait();
+  after_wait();  // no after_ready, as above
   const int64_t rc = rc0 + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (rc >= rc1) return;
   const int cx = (int)(rc % ig.nrcx) + ig.ox, cy = (int)(rc / ig.nrcx) + ig.oy;
