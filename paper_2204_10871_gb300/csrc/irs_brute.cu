@@ -18,6 +18,8 @@
 // FP32 Taylor series of the sheet's analytic part in the ray's offset t.
 #include <math.h>
 
+#include <type_traits>
+
 #include "irs_common.cuh"
 
 namespace irs {
@@ -635,7 +637,8 @@ cudaError_t launch_brute_map(const irs_plan_t* P, const double* xy, const double
 // they lie and every ray converts for itself, bound by the FP64 subtractions
 // (GB300 issues two a clock per SM).  The first is chosen from 8 rays per
 // tile on average: 5e4 rays of a 923^2 lattice with 1e4 lenses take
-// 0.91 ms by tile and 3.96 ms by ray, and took 209 ms before.
+// 0.50 ms by tile and 3.93 ms by ray, and took 209 ms before (0.76 by tile with
+// both kinds of rays in most warps).
 constexpr int BD_THREADS = 256;
 constexpr int BD_STAGES = BD_THREADS / 32;  // stages at once where every ray converts for itself
 constexpr int BD_LIST = 256;                // rays of a tile served at once
@@ -731,7 +734,7 @@ k_brute_rays(Geo g, BruteForm form, const double2* __restrict__ xy, const double
   int64_t scan = BY_TILE ? (int64_t)(blockIdx.x % BD_PARTS) * BD_THREADS : (int64_t)blockIdx.x * 32;
   while (scan < nidx) {
     // ---- the rays of this round: `live` of them, ray k's slot in the caller's arrays
-    int live;
+    int live, nplain = 32, ngrouped = 0;  // of them sharing no reciprocal, and the others
     if (BY_TILE) {
       __syncthreads();
       if (tid == 0) found_s = grouped_s = 0;
@@ -753,22 +756,30 @@ k_brute_rays(Geo g, BruteForm form, const double2* __restrict__ xy, const double
         const int have = found_s + grouped_s;  // read before the barrier: nobody adds until everyone has passed it
         const int hits = __syncthreads_count(mine);
         if (have + hits > BD_LIST) break;  // next round starts here (a scan step adds at most BD_THREADS)
-        // rays that share reciprocals from the list's end, so that few warps mix both kinds
+        // rays that share reciprocals from the list's end
         if (mine) list_s[grouped ? BD_LIST - 1 - atomicAdd(&grouped_s, 1) : atomicAdd(&found_s, 1)] = i;
         __syncthreads();
       }
-      live = found_s + grouped_s;
+      nplain = found_s;
+      ngrouped = grouped_s;
+      live = nplain + ngrouped;
       if (live == 0) continue;
     } else {
       live = (int)min((int64_t)32, nidx - scan);
     }
-    // thread (ray, stage group): rays fastest; S groups of `live` threads
+    // thread (ray, stage group): rays fastest; S groups of the rays that share
+    // no reciprocal, then S of those that do, from a warp of their own where that
+    // fits: a warp of both kinds runs both loops (8 and 19 instructions a pair)
     const int S = BY_TILE ? min(BD_STAGES, BD_THREADS / live) : BD_STAGES;
-    const int ray = BY_TILE ? tid % live : tid % 32, grp = BY_TILE ? tid / live : tid / 32;
-    const bool on = ray < live && grp < S;
+    int first = nplain * S;  // first thread of the second kind
+    if (((first + 31) & ~31) + ngrouped * S <= BD_THREADS) first = (first + 31) & ~31;
+    const bool second = tid >= first;
+    const int step = second ? ngrouped : nplain, from = second ? tid - first : tid;
+    const int grp = step > 0 ? from / step : S, ray = from - grp * step;
+    const bool on = grp < S && ray < live;
     int64_t slot = 0, f = -1;
     if (on) {
-      slot = BY_TILE ? list_s[ray < found_s ? ray : BD_LIST - live + ray] : scan + ray;
+      slot = BY_TILE ? list_s[second ? BD_LIST - ngrouped + ray : ray] : scan + ray;
       f = idx[slot];
     }
     const bool ok = f >= 0 && f < n_rays;
@@ -795,23 +806,31 @@ k_brute_rays(Geo g, BruteForm form, const double2* __restrict__ xy, const double
       float px = 0.f, py = 0.f;
       if (on && ok) {
         const int e = min((grp + 1) * BR_LT, total);
+        auto pairs = [&](auto kind) {
+          RowGroup r = q;
+          r.kind = kind;
 #pragma unroll 4
-        for (int t = grp * BR_LT; t < e; ++t) {
-          if (BY_TILE) {
-            const float4 L = lens_s[t];
-            ray_pair(tx, ty, q, L.x, L.y, L.z, px, py);
-          } else {
-            const double2 p = pos_s[t];
-            ray_pair(tx, ty, q, (float)(p.x - zx), (float)(p.y - zy), m_s[t], px, py);
+          for (int t = grp * BR_LT; t < e; ++t) {
+            if (BY_TILE) {
+              const float4 L = lens_s[t];
+              ray_pair(tx, ty, r, L.x, L.y, L.z, px, py);
+            } else {
+              const double2 p = pos_s[t];
+              ray_pair(tx, ty, r, (float)(p.x - zx), (float)(p.y - zy), m_s[t], px, py);
+            }
           }
-        }
+        };
+        if (!BY_TILE) pairs(q.kind);  // a loop per kind would convert every lens once for each
+        else if (q.kind == 0) pairs(std::integral_constant<int, 0>{});
+        else if (q.kind == 1) pairs(std::integral_constant<int, 1>{});
+        else pairs(std::integral_constant<int, 2>{});
       }
       part_s[tid] = make_float2(px, py);
       __syncthreads();
       if (on && grp == 0) {  // fold the stages in order
-        const int ns = (total + BR_LT - 1) / BR_LT, step = BY_TILE ? live : 32;
+        const int ns = (total + BR_LT - 1) / BR_LT;
         for (int k = 0; k < ns; ++k) {
-          const float2 p = part_s[ray + k * step];
+          const float2 p = part_s[tid + k * step];
           fold(axh, axl, p.x);
           fold(ayh, ayl, p.y);
         }
