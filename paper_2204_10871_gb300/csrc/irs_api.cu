@@ -150,7 +150,7 @@ irs_status run_map(irs_plan_t* P, const double* xy, const double* mass, int64_t 
   mark(P, irs::EV_START, s);
   IRS_TRY(irs::launch_mass_sum(P, mass, n, s, xy));
   if (P->p.method == IRS_BRUTE) {
-    IRS_TRY(irs::launch_brute_setup(P, row0, row1, s));
+    IRS_TRY(irs::launch_brute_setup(P, row0, row1, n, s));
     mark(P, irs::EV_PREP, s);
     mark(P, irs::EV_CELLS, s);
     mark(P, irs::EV_FIN, s);
@@ -317,7 +317,7 @@ irs_status irs_shoot_rays(irs_plan_t* P, const double* xy, const double* mass, i
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   IRS_TRY(irs::launch_mass_sum(P, mass, n, s, xy));
   if (P->p.method == IRS_BRUTE) {
-    IRS_TRY(irs::launch_brute_setup(P, 0, P->g.nry, s));
+    IRS_TRY(irs::launch_brute_setup(P, 0, P->g.nry, -1, s));
     IRS_TRY(irs::launch_brute_dump(P, xy, mass, n, ray_idx, n_idx, beta, pixel, s));
     return IRS_OK;
   }

@@ -70,7 +70,7 @@ irs_status enqueue(BatchEntry* e, irs_plan_t* const* plans, int32_t nmaps, const
     if (cudaMemsetAsync(counts[m], 0, npix * sizeof(uint32_t), s) != cudaSuccess) return IRS_ERR_CUDA;
     if (irs::launch_mass_sum(P, mass[m], n[m], s, xy[m]) != cudaSuccess) return IRS_ERR_CUDA;
     if (P->p.method == IRS_BRUTE) {
-      if (irs::launch_brute_setup(P, 0, P->g.nry, s) != cudaSuccess) return IRS_ERR_CUDA;
+      if (irs::launch_brute_setup(P, 0, P->g.nry, n[m], s) != cudaSuccess) return IRS_ERR_CUDA;
       if (irs::launch_brute_map(P, xy[m], mass[m], n[m], 0, P->g.nry, counts[m], s) != cudaSuccess)
         return IRS_ERR_CUDA;
     } else {

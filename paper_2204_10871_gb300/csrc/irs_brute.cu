@@ -157,11 +157,11 @@ constexpr int SETUP_TILES = 32;
 constexpr int SETUP_VALUES = 4 + 2 * (SHEET_TERMS - 1);  // Log w, w Log w, w^-1 ... w^-7
 
 __global__ void __launch_bounds__(4 * SETUP_TILES)
-k_brute_setup(Geo g, const double* __restrict__ msum, int64_t ntx, int64_t tile0, int64_t tile1,
+k_brute_setup(Geo g, const double* __restrict__ msum, int64_t ntx, int64_t tile0, int64_t tile1, bool early,
               TileRec* __restrict__ recs) {
   __shared__ double val_s[4][SETUP_VALUES][SETUP_TILES];
   __shared__ bool near_s[4][SETUP_TILES];
-  after_ready();
+  if (early) after_ready();
   const int lt = threadIdx.x & 31;  // a warp per corner
   const int64_t tile = min(tile0 + (int64_t)blockIdx.x * SETUP_TILES + lt, tile1 - 1);
   const TileGeo tg = tile_geo(g, tile, ntx);
@@ -268,11 +268,23 @@ k_brute_setup(Geo g, const double* __restrict__ msum, int64_t ntx, int64_t tile0
 }
 
 // Tile constants of the tile rows that cover lattice rows [row0, row1).
-cudaError_t launch_brute_setup(const irs_plan_t* P, int64_t row0, int64_t row1, cudaStream_t s) {
+//
+// The pass that follows may start beside this kernel (`early`), which hides the
+// set-up behind its lens sums: 5 to 10 % of a map of up to half a millisecond
+// (110 lenses, 4960 tiles: 305 against 325 us).  But CTAs placed around these
+// find the registers in pieces, and an SM then keeps two of k_brute's three
+// for a long time (124 lenses, 16150 tiles: 1,442 against 1,071 us; a band of
+// 1296 tiles with 14297 lenses 4.4 against 3.5 ms), and the few CTAs of chosen
+// rays crowd onto few SMs (472 rays: 254 against 88 us).  So: early for maps of
+// up to 2^20 tile-lens products (about 0.5 ms) whose set-up is at most two CTAs
+// per SM.
+constexpr int64_t EARLY_WORK = (int64_t)1 << 20, EARLY_TILES = 2 * 152 * SETUP_TILES;
+cudaError_t launch_brute_setup(const irs_plan_t* P, int64_t row0, int64_t row1, int64_t n, cudaStream_t s) {
   const int64_t t0 = row0 / BR_TY * P->br_ntx, t1 = (row1 + BR_TY - 1) / BR_TY * P->br_ntx;
   if (t1 <= t0) return cudaSuccess;
   const int64_t blocks = (t1 - t0 + SETUP_TILES - 1) / SETUP_TILES;
-  return launch_after(k_brute_setup, (unsigned)blocks, 4 * SETUP_TILES, 0, s, P->g, P->d_msum, P->br_ntx, t0, t1,
+  const bool early = n >= 0 && t1 - t0 <= EARLY_TILES && (double)n * (double)(t1 - t0) <= (double)EARLY_WORK;
+  return launch_after(k_brute_setup, (unsigned)blocks, 4 * SETUP_TILES, 0, s, P->g, P->d_msum, P->br_ntx, t0, t1, early,
                       P->d_tiles);
 }
 

@@ -218,7 +218,8 @@ constexpr int MSUM_THREADS = 256;
 // into d_status otherwise).
 cudaError_t launch_mass_sum(const irs_plan_t* P, const double* mass, int64_t n, cudaStream_t s,
                             const double* xy = nullptr);
-cudaError_t launch_brute_setup(const irs_plan_t* P, int64_t row0, int64_t row1, cudaStream_t s);
+// n: lenses of the map pass that follows, or -1 before chosen rays
+cudaError_t launch_brute_setup(const irs_plan_t* P, int64_t row0, int64_t row1, int64_t n, cudaStream_t s);
 cudaError_t launch_brute_map(const irs_plan_t* P, const double* xy, const double* mass, int64_t n,
                              int64_t row0, int64_t row1, uint32_t* counts, cudaStream_t s);
 cudaError_t launch_brute_dump(const irs_plan_t* P, const double* xy, const double* mass, int64_t n,

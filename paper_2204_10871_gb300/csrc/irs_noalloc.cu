@@ -125,7 +125,7 @@ extern "C" irs_status irs_make_map_brute_noalloc(const irs_params* params, const
   const size_t npix = (size_t)p.npix_x * p.npix_y;
   if (cudaMemsetAsync(counts, 0, npix * sizeof(uint32_t), s) != cudaSuccess) return IRS_ERR_CUDA;
   if (irs::launch_mass_sum(&P, mass, n, s) != cudaSuccess) return IRS_ERR_CUDA;
-  if (irs::launch_brute_setup(&P, 0, P.g.nry, s) != cudaSuccess) return IRS_ERR_CUDA;
+  if (irs::launch_brute_setup(&P, 0, P.g.nry, n, s) != cudaSuccess) return IRS_ERR_CUDA;
   if (irs::launch_brute_map(&P, lens_xy, mass, n, 0, P.g.nry, counts, s) != cudaSuccess)
     return IRS_ERR_CUDA;
   if (mag && irs::launch_magnify(&P, counts, mag, true, s) != cudaSuccess) return IRS_ERR_CUDA;
