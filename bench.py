@@ -7,7 +7,9 @@ unlensed pixel: 1.12e10 rays per map).
                   [--impl ours|reference]
 
 One step = one magnification map through irs_make_map (INTERP: mass sum, cell
-lists, far field, ray pass, binning, magnification).  The plain brute-force map of the
+lists, far field, ray pass, binning, magnification); its rays are those of the
+lattice.  The ray pass leaves out work units that provably send no ray onto the
+map (an exact bound, the same map bit for bit); the roofline counts the rest.  The plain brute-force map of the
 same workload costs ~1e15 pair terms (minutes), so it is timed on a band of
 lattice rows through irs_make_map_rows and reported per ray, with the same
 band made by the interpolated method as the accuracy check (per-pixel
@@ -180,14 +182,23 @@ def ip_flops_fixed(variant):
     return 8 * (IP_VARIANT_K2[variant] - 1) + IP_FLOPS_OTHER
 
 
+# Share of a map's rays that the ray pass evaluates: work units (32 columns x 8
+# rows) that provably cannot reach the map are left out.  Counted for these
+# workloads' lens fields: (workload, cell multiplier) -> share.
+IP_EVALUATED = {("paper-mid", 0.57): 0.3943, ("high-res", 0.72): 0.4749}
+
+
+def evaluated_share(name, cell_mult, landed, n_rays):
+    """The counted share, or the share of the rays that landed on the map, a
+    lower bound, for any other workload or cell size."""
+    return IP_EVALUATED.get((name.split(":")[0], round(float(cell_mult or 1.0), 2)), landed / n_rays)
+
+
 # DRAM bytes per launch of the ray pass (ncu dram__bytes_read.sum +
 # dram__bytes_write.sum), valid only for the kernel build, workload and cell
 # size they were captured on: (workload, cell multiplier, variant) -> bytes.
 # Source: profiles/k_ip_ray_paper-mid-full.md.
-IP_TRAFFIC = {("paper-mid", 0.57, 11): 106.890752e6 + 3.025408e6,
-              ("paper-mid", 0.57, 13): 107.035136e6 + 3.787776e6,
-              ("paper-mid", 0.57, 14): 106.874368e6 + 3.572224e6,
-              ("paper-mid", 0.57, 16): 106.763776e6 + 4.427264e6}
+IP_TRAFFIC = {("paper-mid", 0.57, 16): 106.676480e6 + 5.420032e6}
 
 
 def mean_near_lenses(info, xy):
@@ -350,6 +361,7 @@ def run_ours(args):
         e2e_ms = slowest_rank_ms(e2e_ms, dist, dev)
     e2e_value = (rays_per_step / (e2e_ms * 1e-3) if sharded
                  else whole_job_rays_per_s(rays_per_step, world, e2e_ms))
+    landed = int(counts.to(torch.int64).sum())
     h2d = xy.nbytes + m.nbytes
     d2h = h_counts.numel() * 4
     clocks = clk.summary()
@@ -363,7 +375,8 @@ def run_ours(args):
     if full:
         n_near = mean_near_lenses(info, xy)
         variant = int(params.kernel_variant)
-        flops_per_ray = 10.0 * n_near + ip_flops_fixed(variant)
+        share = evaluated_share(w["name"], params.cell_mult, landed, info.n_rays)
+        flops_per_ray = (10.0 * n_near + ip_flops_fixed(variant)) * share
         kname = f"k_ip_ray variant {variant} (near pair sum + level-2 Horner, FP32 pipe + MUFU)"
         key = (w["name"].split(":")[0], round(float(params.cell_mult or 1.0), 2), variant)
         if key in IP_TRAFFIC:
@@ -380,6 +393,7 @@ def run_ours(args):
                 "flops_per_ray": flops_per_ray}
     if n_near is not None:
         roofline["mean_near_lenses"] = n_near
+        roofline["evaluated_share"] = share
     if clocks.get("sm_mhz"):
         roofline["frac_at_measured_clock"] = achieved / (n_sms * 256 * clocks["sm_mhz"] * 1e6 / 1e12)
 
@@ -576,10 +590,12 @@ def high_res_record(irs, torch, lensgen, n_sms, peak_tflops, flush):
     counts = torch.zeros(shape, dtype=torch.uint32, device=dev)
     mag = torch.zeros(shape, dtype=torch.float32, device=dev)
     ms_map, ms_ray = timed_maps(irs, torch, plan, dxy, dm, counts, mag, flush)
+    landed = int(counts.to(torch.int64).sum())
     del counts, mag
     variant = int(params.kernel_variant)
     n_near = mean_near_lenses(info, xy)
-    flops = 10.0 * n_near + ip_flops_fixed(variant)
+    share = evaluated_share(w["name"], params.cell_mult, landed, info.n_rays)
+    flops = (10.0 * n_near + ip_flops_fixed(variant)) * share
     ach = flops * info.n_rays / (ms_ray * 1e-3) / 1e12
     r0 = (info.n_rays_y // 2 // 64) * 64
     brute, (rel,) = band_pair(irs, torch, w, dxy, dm, (r0, r0 + 64), [plan])
@@ -592,7 +608,7 @@ def high_res_record(irs, torch, lensgen, n_sms, peak_tflops, flush):
                          "candidates": res.candidates, "tuning_s": tune_s},
             "roofline": {"bound": "alu", "kernel": f"k_ip_ray variant {variant}", "achieved": ach,
                          "peak": peak_tflops, "unit": "TFLOP/s", "frac": ach / peak_tflops,
-                         "flops_per_ray": flops, "mean_near_lenses": n_near},
+                         "flops_per_ray": flops, "mean_near_lenses": n_near, "evaluated_share": share},
             "brute": dict(brute, roofline_frac=brute_ach / peak_tflops),
             "speedup_over_brute": value / brute["rays_per_s"],
             "map_rel_rms_vs_brute": rel, "min_rays_per_pixel": 100}
@@ -1175,7 +1191,7 @@ def run_reference(args):
 def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("--gpus", type=int, default=1)
-    ap.add_argument("--steps", type=int, default=25)
+    ap.add_argument("--steps", type=int, default=80)
     ap.add_argument("--warmup", type=int, default=3)
     ap.add_argument("--method", default="interp", choices=["interp", "brute", "mlp"])
     ap.add_argument("--impl", default="ours", choices=["ours", "reference"])

@@ -75,9 +75,8 @@ typedef struct irs_params {
   int32_t window;         /* INTERP: cells within this Chebyshev distance sum lenses directly into
                              the series; 0 = default.  MLP: the learned split's radius R_f in
                              cells; 0 = 8 */
-  int32_t kernel_variant; /* INTERP: ray-pass variant 0..16 (rays per thread, level-2 sub-cells,
-                             sub-cell terms, CTAs per SM, binning -- into the map or into a
-                             per-cell shared-memory sub-histogram --, shared reciprocals);
+  int32_t kernel_variant; /* INTERP: ray-pass variant 0..16 (level-2 sub-cells, sub-cell terms,
+                             shared reciprocals; several numbers select the same kernel);
                              irs_autotune picks one.  BRUTE: variant 0..15 (rows per thread,
                              rows sharing a reciprocal by pairs or by fours, packed FP32x2
                              rows); 0 = default.  Variants with four rows per reciprocal (0, 10,

@@ -345,9 +345,9 @@ __device__ __forceinline__ void brute_beta(const Geo& g, const TileRec& rec, flo
 // two lenses an iteration: with two quads the FP32 pipe's longer dependent
 // chains cost more than the MUFU cycles they save.
 //
-// Variant 0 runs three CTAs per SM (168 registers) and eight lenses an
+// Variant 0 runs three CTAs per SM (160 registers) and eight lenses an
 // iteration: more independent chains per warp keep the MUFU busier than more
-// warps do.  The 64-row band of the 1e5-lens lattice takes 415 ms (64.7 %, 84 %
+// warps do.  The 64-row band of the 1e5-lens lattice takes 415 ms (64 %, 83 %
 // of the MUFU's bound); four CTAs and 2, 4 or 8 lenses took 437, 437 and 436,
 // three CTAs and 2, 4, 6, 16 or 32 lenses 432, 431, 421, 415 and 418, two CTAs
 // and 4, 8 or 16 lenses 426, 430 and 433.  CTAs of one or two warps, each with

@@ -37,12 +37,11 @@ struct Geo {
 // before it touches anything that earlier work writes or still reads, and
 // kernels that another may follow call after_ready() first thing (not the one
 // before a persistent grid that fills the SMs: its CTAs are placed best on empty
-// ones).  Both do
-// nothing after an ordinary launch.  Every thread block waits, so that a kernel
+// ones).  Both do nothing after an ordinary launch.  Every thread block waits, so that a kernel
 // that has finished implies that all before it have.  The first kernel of a
 // call is launched the ordinary way: caller's buffers are complete when it
 // starts.  A map of few lenses is a chain of a dozen short kernels, whose launch
-// latencies and set-ups overlap this way (a 64^2 brute-force map: 30 us
+// latencies and set-ups overlap this way (a 64^2 brute-force map: 33 us
 // instead of 48).
 __device__ __forceinline__ void after_ready() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void after_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }

@@ -1175,14 +1175,14 @@ constexpr int IP_RC = 4;
 // the packed FP32x2 instructions (two rows share the column's dx and sigma_x),
 // which round exactly as the scalar ones.  The accumulators hold -alpha (the
 // masses are stored negated) and the level-2 Horner runs on the conjugate, so
-// no negation is issued per ray.  The pass is bound by instruction issue (0.72
-// of the slots; 52.5 instructions per ray, 62.5 before) with the MUFU next, so
+// no negation is issued per ray.  The pass is bound by instruction issue (0.69
+// of the slots, FP32 pipe 51 %, MUFU 29 %), so
 // what is the same for a row comes from a table, four rows that share a level-2
 // row read its series once, the sheet's corners sit on the general path of the
 // tail only, and a last strip of few columns takes several row groups at once
 // (a 45-ray cell: 83 % of the lanes busy instead of 70 %).  Ray pass, one
-// GB300, against the form with match-and-add binning, fixed cells per CTA and
-// one set-up chain per thread: paper-mid 20.2 ms (28.0), high-res 204 ms (275),
+// GB300, every ray evaluated, against the form with match-and-add binning, fixed
+// cells per CTA and one set-up chain per thread: paper-mid 20.2 ms (28.0), high-res 204 ms (275),
 // a 500^2 map of 1e4 lenses 0.28 ms (0.44), 128^2 with 150 lenses 0.078 (0.088).
 template <int Q, int K2, int NPR>
 __device__ __forceinline__ void ip_cell(const Geo& g, const IpGeo& ig, const IpRayArgs& a, int64_t rc,
