@@ -157,7 +157,7 @@ constexpr int SETUP_TILES = 32;
 constexpr int SETUP_VALUES = 4 + 2 * (SHEET_TERMS - 1);  // Log w, w Log w, w^-1 ... w^-7
 
 __global__ void __launch_bounds__(4 * SETUP_TILES)
-k_brute_setup(Geo g, const double* __restrict__ msum, int64_t ntx, int64_t tile0, int64_t tile1, bool early,
+k_brute_setup(Geo g, const double* msum, int64_t ntx, int64_t tile0, int64_t tile1, bool early,
               TileRec* __restrict__ recs) {
   __shared__ double val_s[4][SETUP_VALUES][SETUP_TILES];
   __shared__ bool near_s[4][SETUP_TILES];
@@ -367,7 +367,7 @@ constexpr double BR_QUAD_MAX_DIAG = 1.0e4;
 template <int R, int PAIRED, int QUAD, int PACK, int TPSM>
 __global__ void __launch_bounds__(32 * (BR_TY / R), TPSM / (32 * (BR_TY / R)))
 k_brute(Geo g, const double2* __restrict__ xy, const double* __restrict__ mass, int64_t n,
-        const TileRec* __restrict__ recs, int64_t ntx, int64_t nwork, int64_t row0, int64_t row1,
+        const TileRec* recs, int64_t ntx, int64_t nwork, int64_t row0, int64_t row1,
         uint32_t* __restrict__ counts) {
   constexpr int NT = 32 * (BR_TY / R);
   static_assert(PAIRED % 2 == 0 && (!PACK || (R - PAIRED) % 2 == 0), "rows go in pairs");
@@ -730,7 +730,7 @@ __device__ __forceinline__ void write_ray(const Geo& g, const TileRec& rec, floa
 template <bool BY_TILE>
 __global__ void __launch_bounds__(BD_THREADS)
 k_brute_rays(Geo g, BruteForm form, const double2* __restrict__ xy, const double* __restrict__ mass, int64_t n,
-             const TileRec* __restrict__ recs, int64_t ntx, const int64_t* __restrict__ idx, int64_t nidx,
+             const TileRec* recs, int64_t ntx, const int64_t* __restrict__ idx, int64_t nidx,
              double* __restrict__ beta_out, int64_t* __restrict__ pix_out) {
   // a stage's lenses: by tile as FP32 offsets (x, y, m), else as given
   __shared__ double2 pos_s[BY_TILE ? 1 : BD_STAGES * BR_LT];
@@ -883,7 +883,7 @@ cudaError_t launch_brute_dump(const irs_plan_t* P, const double* xy, const doubl
 // ------------------------------------------------------------ magnification
 // Mag_ij = N_ij * S_I / S_S with S_I = dx3^2 and S_S = s_x s_y ("Calculate the
 // magnification of each pixel", Sec. 2.4).
-__global__ void k_magnify(const uint32_t* __restrict__ counts, float* __restrict__ mag, int64_t npix,
+__global__ void k_magnify(const uint32_t* counts, float* __restrict__ mag, int64_t npix,
                           float ratio) {
   after_wait();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;

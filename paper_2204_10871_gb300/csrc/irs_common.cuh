@@ -43,6 +43,12 @@ struct Geo {
 // starts.  A map of few lenses is a chain of a dozen short kernels, whose launch
 // latencies and set-ups overlap this way (a 64^2 brute-force map: 33 us
 // instead of 48).
+//
+// A chained kernel's pointers to what an earlier kernel of the call writes are
+// plain ones.  `const __restrict__` promises data that nobody writes while the
+// kernel lives, which lets the compiler use non-coherent loads and move them
+// above the wait, and the kernel's life begins before that data is complete.  The
+// qualifier stays on the caller's inputs and the plan's tables.
 __device__ __forceinline__ void after_ready() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void after_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

@@ -183,7 +183,7 @@ __global__ void k_ip_count(IpGeo ig, const double2* __restrict__ xy, int64_t n,
 // the sums of those before it (which it adds up by itself; a third launch that
 // scanned the sums on one thread took 50 us at 1.9e6 cells).
 constexpr int SCAN_B = 1024;
-__global__ void k_scan_local(const int32_t* __restrict__ in, int32_t* __restrict__ out, int32_t* __restrict__ copy,
+__global__ void k_scan_local(const int32_t* in, int32_t* __restrict__ out, int32_t* __restrict__ copy,
                              int64_t n, int32_t* __restrict__ block_sums) {
   __shared__ int32_t warp_s[32];
   after_ready();
@@ -220,7 +220,7 @@ __global__ void k_scan_local(const int32_t* __restrict__ in, int32_t* __restrict
   if (gridDim.x > 1 && threadIdx.x == SCAN_B - 1) block_sums[blockIdx.x] = inc;
 }
 __global__ void k_scan_add(int32_t* __restrict__ out, int32_t* __restrict__ copy, int64_t n,
-                           const int32_t* __restrict__ block_sums) {
+                           const int32_t* block_sums) {
   __shared__ int32_t warp_s[32];
   after_ready();
   after_wait();
@@ -239,7 +239,7 @@ __global__ void k_scan_add(int32_t* __restrict__ out, int32_t* __restrict__ copy
   if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) out[n] = s + block_sums[blockIdx.x];
 }
 
-__global__ void k_ip_scatter(const int32_t* __restrict__ lens_cell, int64_t n,
+__global__ void k_ip_scatter(const int32_t* lens_cell, int64_t n,
                              int32_t* __restrict__ cursor, int32_t* __restrict__ sorted_idx) {
   after_ready();
   after_wait();
@@ -266,8 +266,8 @@ __global__ void k_ip_scatter(const int32_t* __restrict__ lens_cell, int64_t n,
 // high-res map's 1.9e6; now 8.7 and 311 us.
 constexpr int CELLS_B = 128;
 __global__ void __launch_bounds__(CELLS_B)
-k_ip_cells(IpGeo ig, const int32_t* __restrict__ start, const double2* __restrict__ xy,
-           const double* __restrict__ mass, const int32_t* __restrict__ lens_cell, int32_t* __restrict__ sorted_idx,
+k_ip_cells(IpGeo ig, const int32_t* start, const double2* __restrict__ xy,
+           const double* __restrict__ mass, const int32_t* lens_cell, int32_t* __restrict__ sorted_idx,
            float4* __restrict__ rel, double2* __restrict__ pos, double* __restrict__ m_out,
            float4* __restrict__ pos_df, float2* __restrict__ m_df, float4* __restrict__ mpole_d,
            float2* __restrict__ mpole_f) {
@@ -641,9 +641,8 @@ constexpr int FG_RANGES = 2 * FG_WMAX + 4;  // list ranges of a window
 
 template <int NF>
 __global__ void __launch_bounds__(32 * FG_WARPS, 6)
-k_ip_finalize_group(Geo g, IpGeo ig, const double* __restrict__ msum, const int32_t* __restrict__ start,
-                    const float4* __restrict__ pos_df, const float2* __restrict__ m_df,
-                    const float4* __restrict__ conv_d, const float2* __restrict__ conv_f,
+k_ip_finalize_group(Geo g, IpGeo ig, const double* msum, const int32_t* start, const float4* pos_df,
+                    const float2* m_df, const float4* conv_d, const float2* conv_f,
                     const double2* __restrict__ sheet_d, const float2* __restrict__ sheet_f,
                     const uint8_t* __restrict__ sheet_near, CellRec* __restrict__ recs, float2* __restrict__ coef,
                     int64_t rc0, int64_t rc1, int cta_cells) {
@@ -818,10 +817,9 @@ k_ip_finalize_group(Geo g, IpGeo ig, const double* __restrict__ msum, const int3
 // thread per cell.
 template <int NF>
 __global__ void __launch_bounds__(64)
-k_ip_finalize(Geo g, IpGeo ig, const double* __restrict__ msum, const int32_t* __restrict__ start,
-              const double2* __restrict__ pos, const double* __restrict__ m, const float4* __restrict__ pos_df,
-              const float2* __restrict__ m_df, const float4* __restrict__ conv_d,
-              const float2* __restrict__ conv_f, MlpFar far, const double2* __restrict__ sheet_d,
+k_ip_finalize(Geo g, IpGeo ig, const double* msum, const int32_t* start, const double2* pos, const double* m,
+              const float4* pos_df, const float2* m_df, const float4* conv_d, const float2* conv_f, MlpFar far,
+              const double2* __restrict__ sheet_d,
               const float2* __restrict__ sheet_f, const uint8_t* __restrict__ sheet_near,
               CellRec* __restrict__ recs, float2* __restrict__ coef, int64_t rc0, int64_t rc1) {
   after_wait();  // no after_ready, as above
