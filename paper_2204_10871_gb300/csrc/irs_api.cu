@@ -106,7 +106,6 @@ irs_status alloc_workspace(irs_plan_t* P) {
   const size_t o_mpart = take(sizeof(double) * irs::MSUM_BLOCKS);
   const size_t o_status = take(sizeof(int));
   const size_t o_queue = take(sizeof(unsigned long long));
-  const size_t o_mdone = take(sizeof(unsigned int));
   size_t o_tiles = 0;
   if (P->p.method == IRS_BRUTE) o_tiles = take(sizeof(irs::TileRec) * (size_t)P->br_ntiles);
   P->ws_bytes = off;
@@ -120,7 +119,6 @@ irs_status alloc_workspace(irs_plan_t* P) {
   P->d_mpart = reinterpret_cast<double*>(b + o_mpart);
   P->d_status = reinterpret_cast<int*>(b + o_status);
   P->d_queue = reinterpret_cast<unsigned long long*>(b + o_queue);
-  P->d_mdone = reinterpret_cast<unsigned int*>(b + o_mdone);
   P->d_tiles = P->p.method == IRS_BRUTE ? reinterpret_cast<irs::TileRec*>(b + o_tiles) : nullptr;
   if (cudaMemset(P->ws, 0, P->ws_bytes) != cudaSuccess) return IRS_ERR_CUDA;
   return IRS_OK;
@@ -146,7 +144,7 @@ irs_status run_map(irs_plan_t* P, const double* xy, const double* mass, int64_t 
   if (st != IRS_OK) return st;
   const size_t npix = (size_t)P->g.npix_x * P->g.npix_y;
   if (clear) IRS_TRY(cudaMemsetAsync(counts, 0, npix * sizeof(uint32_t), s));
-  P->launches = 1;  // mass sum
+  P->launches = irs::mass_sum_launches(n);
   mark(P, irs::EV_START, s);
   IRS_TRY(irs::launch_mass_sum(P, mass, n, s, xy));
   if (P->p.method == IRS_BRUTE) {

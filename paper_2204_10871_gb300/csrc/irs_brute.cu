@@ -47,17 +47,18 @@ __device__ __forceinline__ bool lens_inside(const LensRegion& L, double2 p) {
   return p.x >= L.x0 && p.x <= L.x1 && p.y >= L.y0 && p.y <= L.y1;
 }
 
-// One launch: the block that finishes last adds the partial sums, in block
-// order.  Blocks past the last lens would only add zeros and are not launched
-// (a map of few lenses took 8 us in a second launch of one thread that added
-// 128 of them); the stride between a thread's lenses is that of all
-// MSUM_BLOCKS either way, so the sum is the same bits.
+// The sum of up to MSUM_THREADS lenses is one block's; more blocks leave partial
+// sums that a second launch adds in block order.  (Letting the block that
+// finishes last add them saves that launch, but it needs a count of blocks that
+// is zero at the start: one that lives across calls stays wrong for good once two
+// calls on the same workspace have overlapped.)  Blocks past the last lens would
+// only add zeros and are not launched; the stride between a thread's lenses is
+// that of all MSUM_BLOCKS either way, so the sum is the same bits.
 __global__ void k_mass_sum(const double* __restrict__ mass, const double2* __restrict__ xy, int64_t n,
                            LensRegion region, int* __restrict__ status, double* __restrict__ part,
-                           unsigned int* __restrict__ done, double* __restrict__ out,
-                           unsigned long long* __restrict__ queue, int32_t* __restrict__ zero, int64_t nzero) {
+                           bool whole, double* __restrict__ out, unsigned long long* __restrict__ queue,
+                           int32_t* __restrict__ zero, int64_t nzero) {
   __shared__ double sh[MSUM_THREADS];
-  __shared__ bool last;
   after_ready();
   for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < nzero; k += (int64_t)gridDim.x * blockDim.x)
     zero[k] = 0;
@@ -75,23 +76,28 @@ __global__ void k_mass_sum(const double* __restrict__ mass, const double2* __res
     if ((int)threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
     __syncthreads();
   }
-  if (threadIdx.x == 0) {
+  if (threadIdx.x != 0) return;
+  if (!whole) {
     part[blockIdx.x] = sh[0];
-    __threadfence();
-    last = atomicAdd(done, 1u) == gridDim.x - 1;
-  }
-  __syncthreads();
-  if (!last) return;
-  __threadfence();
-  if (threadIdx.x < gridDim.x) sh[threadIdx.x] = __ldcg(part + threadIdx.x);
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (unsigned b = 0; b < gridDim.x; ++b) t += sh[b];
-    out[0] = t;
-    *done = 0u;               // for the next sum on this plan
+  } else if (blockIdx.x == 0) {  // its lenses are all there are
+    out[0] = sh[0];
     if (queue) *queue = 0ull;  // the ray pass's work counter
   }
+}
+
+__global__ void __launch_bounds__(MSUM_BLOCKS) k_mass_final(const double* part, int nblocks, double* __restrict__ out,
+                                                            unsigned long long* __restrict__ queue) {
+  __shared__ double sh[MSUM_BLOCKS];
+  after_ready();
+  after_wait();
+  if ((int)threadIdx.x < nblocks) sh[threadIdx.x] = part[threadIdx.x];
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  double t = 0.0;
+#pragma unroll 4
+  for (int b = 0; b < nblocks; ++b) t += sh[b];
+  out[0] = t;
+  if (queue) *queue = 0ull;
 }
 
 cudaError_t launch_mass_sum(const irs_plan_t* P, const double* mass, int64_t n, cudaStream_t s,
@@ -110,14 +116,16 @@ cudaError_t launch_mass_sum(const irs_plan_t* P, const double* mass, int64_t n, 
   L.r2 = (P->circle_r + tol) * (P->circle_r + tol);
   L.circle = g.plane == IRS_PLANE_CIRCLE;
   L.check = xy != nullptr && n > 0;
-  static_assert(MSUM_BLOCKS <= MSUM_THREADS, "one partial sum per thread");
-  int64_t need = (n + MSUM_THREADS - 1) / MSUM_THREADS;
+  const bool whole = mass_sum_launches(n) == 1;
+  const int64_t lens_blocks = (n + MSUM_THREADS - 1) / MSUM_THREADS;
   const int64_t nzero = P->d_zero ? P->n_zero : 0, zblocks = (nzero + 16 * MSUM_THREADS - 1) / (16 * MSUM_THREADS);
-  if (need < zblocks) need = zblocks;
-  const unsigned blocks = need < 1 ? 1u : need < MSUM_BLOCKS ? (unsigned)need : (unsigned)MSUM_BLOCKS;
-  k_mass_sum<<<blocks, MSUM_THREADS, 0, s>>>(mass, reinterpret_cast<const double2*>(xy), n, L, P->d_status, P->d_mpart,
-                                             P->d_mdone, P->d_msum, P->d_queue, P->d_zero, nzero);
-  return cudaGetLastError();
+  auto clip = [](int64_t b) { return (int)(b < 1 ? 1 : b < MSUM_BLOCKS ? b : MSUM_BLOCKS); };
+  k_mass_sum<<<(unsigned)clip(lens_blocks > zblocks ? lens_blocks : zblocks), MSUM_THREADS, 0, s>>>(
+      mass, reinterpret_cast<const double2*>(xy), n, L, P->d_status, P->d_mpart, whole, P->d_msum, P->d_queue, P->d_zero,
+      nzero);
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess || whole) return e;
+  return launch_after(k_mass_final, 1, MSUM_BLOCKS, 0, s, P->d_mpart, clip(lens_blocks), P->d_msum, P->d_queue);
 }
 
 // ------------------------------------------------------------ FP64 complex

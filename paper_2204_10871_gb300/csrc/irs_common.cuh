@@ -190,7 +190,6 @@ struct irs_plan {
   size_t ws_bytes;
   double* d_msum;          // [1] sum of masses
   double* d_mpart;         // [MSUM_BLOCKS] partial sums
-  unsigned int* d_mdone;   // blocks of the mass sum that have finished; zero between sums
   int32_t* d_zero;         // counters that the mass sum sets to zero (NULL: none)
   int64_t n_zero;
   irs::TileRec* d_tiles;   // [br_ntiles]
@@ -216,6 +215,8 @@ struct irs_plan {
 namespace irs {
 constexpr int MSUM_BLOCKS = 128;
 constexpr int MSUM_THREADS = 256;
+// kernel launches of the mass sum of n lenses
+constexpr int mass_sum_launches(int64_t n) { return n <= MSUM_THREADS ? 1 : 2; }
 
 // launchers implemented in irs_brute.cu
 // Sum of the masses into d_msum; with lens positions `xy` given (2n doubles),

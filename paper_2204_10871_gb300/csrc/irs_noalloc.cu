@@ -35,7 +35,6 @@ constexpr int64_t NOALLOC_MAX_TILES = 49152;
 constexpr size_t OFF_MSUM = 0;
 constexpr size_t OFF_MPART = 256;
 constexpr size_t OFF_STATUS = OFF_MPART + ((sizeof(double) * irs::MSUM_BLOCKS + 255) & ~(size_t)255);
-constexpr size_t OFF_MDONE = OFF_STATUS + 128;  // zero-initialised, left zero by every mass sum
 constexpr size_t OFF_TILES = OFF_STATUS + 256;
 constexpr size_t SCRATCH_BYTES = OFF_TILES + sizeof(irs::TileRec) * NOALLOC_MAX_TILES;
 
@@ -116,7 +115,6 @@ extern "C" irs_status irs_make_map_brute_noalloc(const irs_params* params, const
   P.d_mpart = reinterpret_cast<double*>(scratch + OFF_MPART);
   P.d_status = reinterpret_cast<int*>(scratch + OFF_STATUS);
   P.d_tiles = reinterpret_cast<irs::TileRec*>(scratch + OFF_TILES);
-  P.d_mdone = reinterpret_cast<unsigned int*>(scratch + OFF_MDONE);
 
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   // the partial sums and tile records are rewritten in full by every call;
