@@ -655,10 +655,10 @@ cudaError_t launch_brute_map(const irs_plan_t* P, const double* xy, const double
 // them), found by a scan over the indices, and converts each lens to the
 // tile's frame once for all of them.  Otherwise a CTA takes 32 rays wherever
 // they lie and every ray converts for itself, bound by the FP64 subtractions
-// (GB300 issues two a clock per SM).  The first is chosen from 8 rays per
-// tile on average: 5e4 rays of a 923^2 lattice with 1e4 lenses take
-// 0.50 ms by tile and 3.93 ms by ray, and took 209 ms before (0.76 by tile with
-// both kinds of rays in most warps).
+// (GB300 issues two a clock per SM).  5e4 rays of a 923^2 lattice with 1e4 lenses
+// take 0.50 ms by tile and 3.93 ms by ray, and took 209 ms before (0.76 by tile
+// with both kinds of rays in most warps).  Which is the faster depends on the
+// scan, which passes every index once per tile (rays_by_tile).
 constexpr int BD_THREADS = 256;
 constexpr int BD_STAGES = BD_THREADS / 32;  // stages at once where every ray converts for itself
 constexpr int BD_LIST = 256;                // rays of a tile served at once
@@ -876,12 +876,25 @@ static BruteForm brute_form(int variant) {
   return BruteForm{16, 0, 0};
 }
 
+// Whether chosen rays go by tile: from 8 rays per tile on average, where the
+// times below say so.  In picoseconds (one GB300, 6 to 63,000 tiles, 3 to 1e4
+// lenses, 8 to 512 rays per tile): an index scanned for a tile costs 4.4, a pair
+// by tile 0.75 and a lens converted for a tile's eight CTAs 46; a pair by ray
+// costs 7.4, and fewer than 5000 rays take as long as those.  1e6 rays of 16,000
+// tiles with 100 lenses take 72 ms by tile and 1.5 by ray, 2.6e5 rays of 4000 tiles
+// with 1e4 lenses 8.4 and 18.8.
+static bool rays_by_tile(int64_t ntiles, int64_t nidx, int64_t n) {
+  if (nidx < 8 * ntiles || ntiles * BD_PARTS >= ((int64_t)1 << 31)) return false;
+  const double T = (double)ntiles, k = (double)nidx, m = (double)n;
+  return 4.4 * T * k + m * (0.75 * k + 46.0 * T) < 7.4 * m * fmax(k, 5000.0);
+}
+
 cudaError_t launch_brute_dump(const irs_plan_t* P, const double* xy, const double* mass, int64_t n,
                               const int64_t* idx, int64_t nidx, double* beta, int64_t* pix,
                               cudaStream_t s) {
   const double2* xy2 = reinterpret_cast<const double2*>(xy);
   const BruteForm form = brute_form(P->p.kernel_variant);
-  if (nidx >= 8 * P->br_ntiles && P->br_ntiles * BD_PARTS < ((int64_t)1 << 31))
+  if (rays_by_tile(P->br_ntiles, nidx, n))
     return launch_after(k_brute_rays<true>, (unsigned)(P->br_ntiles * BD_PARTS), BD_THREADS, 0, s, P->g, form, xy2,
                         mass, n, P->d_tiles, P->br_ntx, idx, nidx, beta, pix);
   return launch_after(k_brute_rays<false>, (unsigned)((nidx + 31) / 32), BD_THREADS, 0, s, P->g, form, xy2, mass, n,
