@@ -1212,10 +1212,12 @@ __device__ __forceinline__ void ip_cell(const Geo& g, const IpGeo& ig, const IpR
   const int64_t jlo = max(j0, a.row0), jhi = min(min(j0 + k, g.nry), a.row1);
   // cell-local lattice indices: columns [0, kx), rows [ylo, yhi), of these the
   // row groups [grg0, nrg) of this part; units start on an even row so that row
-  // pairs line up with the table
+  // pairs line up with the table, and on a multiple of R where only some of a
+  // unit's pairs share a reciprocal, so that a band's rays round as the map's do
   constexpr int R = IP_R;
+  constexpr int ANCHOR = NPR > 0 && NPR < R / 2 ? R : 2;
   const int kx = (int)(min(i0 + k, g.nrx) - i0), ylo = (int)(jlo - j0), yhi = (int)(jhi - j0);
-  const int ylo2 = ylo & ~1;
+  const int ylo2 = ylo & ~(ANCHOR - 1);
   int grg0 = 0, nrg = jlo < jhi ? (yhi - ylo2 + R - 1) / R : 0;
   if (a.parts > 1) {
     const int all = nrg;
@@ -1579,7 +1581,7 @@ __device__ __forceinline__ void ip_cell(const Geo& g, const IpGeo& ig, const IpR
           for (int i = 0; i < R / 2; ++i) {
             const int ra = rl0 + 2 * i;
             NAY[i].x = ra >= ylo && ra < yhi ? NAY[i].x : fnan;
-            NAY[i].y = ra + 1 < yhi ? NAY[i].y : fnan;
+            NAY[i].y = (ANCHOR == 2 || ra + 1 >= ylo) && ra + 1 < yhi ? NAY[i].y : fnan;
           }
         }
         // tail in groups of two row pairs: level-2 series (conj, in sigma),
