@@ -453,7 +453,7 @@ __global__ void __launch_bounds__(128) k_ip_m2l_freq(int64_t G, float4* __restri
 // beta, and the two largest slopes) keep FP64.
 constexpr int FIN_K64 = 3;
 constexpr int FIN_K32 = IP_KMAX - FIN_K64;
-static_assert(IP_KD >= FIN_K64, "FP32 local planes feed only FP32 accumulators");
+static_assert(IP_KD == FIN_K64, "the M2L's double-float terms are the FP64 ones");
 
 // 1/a for complex a, |a| >~ 1e-19 (cell or theta_E units): an FP32 seed for
 // 1/|a|^2 refined by one FP64 Newton step (relative error ~1e-14), instead of
@@ -803,7 +803,6 @@ k_ip_finalize_group(Geo g, IpGeo ig, const double* msum, const int32_t* start, c
 #pragma unroll
   for (int k = 0; k < FIN_K64; ++k) {
     acc[k] = {df_to_double(sum_s[threadIdx.x][2 * k]), df_to_double(sum_s[threadIdx.x][2 * k + 1])};
-    static_assert(IP_KD == FIN_K64, "the M2L's double-float terms are the FP64 ones");
     const float4 v = conv_d[(int64_t)k * ncells + c];
     acc[k].re += df_to_double(dfc_re(v));
     acc[k].im += df_to_double(dfc_im(v));
@@ -910,15 +909,10 @@ k_ip_finalize(Geo g, IpGeo ig, const double* msum, const int32_t* start, const d
 #pragma unroll
     for (int k = 0; k < IP_KF; ++k) {
       if (k >= K) break;
-      if (k < IP_KD) {
+      if (k < FIN_K64) {
         const float4 v = conv_d[(int64_t)k * ncells + c];
-        if (k < FIN_K64) {
-          acc[k].re += df_to_double(dfc_re(v));
-          acc[k].im += df_to_double(dfc_im(v));
-        } else {
-          accf[k - FIN_K64].x += v.x + v.y;
-          accf[k - FIN_K64].y += v.z + v.w;
-        }
+        acc[k].re += df_to_double(dfc_re(v));
+        acc[k].im += df_to_double(dfc_im(v));
       } else {
         const float2 v = conv_f[(int64_t)(k - IP_KD) * ncells + c];
         accf[k - FIN_K64].x += v.x;

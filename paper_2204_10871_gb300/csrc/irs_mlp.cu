@@ -559,7 +559,6 @@ __global__ void __launch_bounds__(MLP_CTA) k_mlp_train(const float* __restrict__
   extern __shared__ __align__(16) unsigned char smem_raw[];
   MlpTrainS& S = *reinterpret_cast<MlpTrainS*>(smem_raw);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, gid = lane >> 2, tig = lane & 3;
-  after_wait();
   mlp_pack_forward(S.f, theta, freq);
 #pragma unroll 4
   for (int t = tid; t < 2 * 4 * 8 * 32 + 8 * 32; t += MLP_CTA) {
