@@ -286,12 +286,12 @@ k_brute_setup(Geo g, const double* msum, int64_t ntx, int64_t tile0, int64_t til
 // rays crowd onto few SMs (472 rays: 254 against 88 us).  So: early for maps of
 // up to 2^20 tile-lens products (about 0.5 ms) whose set-up is at most two CTAs
 // per SM.
-constexpr int64_t EARLY_WORK = (int64_t)1 << 20, EARLY_TILES = 2 * 152 * SETUP_TILES;
+constexpr int64_t EARLY_WORK = (int64_t)1 << 20;
 cudaError_t launch_brute_setup(const irs_plan_t* P, int64_t row0, int64_t row1, int64_t n, cudaStream_t s) {
   const int64_t t0 = row0 / BR_TY * P->br_ntx, t1 = (row1 + BR_TY - 1) / BR_TY * P->br_ntx;
   if (t1 <= t0) return cudaSuccess;
   const int64_t blocks = (t1 - t0 + SETUP_TILES - 1) / SETUP_TILES;
-  const bool early = n >= 0 && t1 - t0 <= EARLY_TILES && (double)n * (double)(t1 - t0) <= (double)EARLY_WORK;
+  const bool early = n >= 0 && blocks <= 2 * (int64_t)P->num_sms && (double)n * (double)(t1 - t0) <= (double)EARLY_WORK;
   return launch_after(k_brute_setup, (unsigned)blocks, 4 * SETUP_TILES, 0, s, P->g, P->d_msum, P->br_ntx, t0, t1, early,
                       P->d_tiles);
 }

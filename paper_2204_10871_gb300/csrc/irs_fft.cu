@@ -331,7 +331,6 @@ namespace {
 // segment of every row and a set of lines whose elements lie in distinct banks.
 // Fewer while a launch would not give every SM three CTAs.
 constexpr size_t FFT_CTA_BYTES = 74 * 1024;
-constexpr int64_t FFT_FILL = 3 * 152;
 size_t cta_bytes(int L, int B, size_t elem) {
   return ((size_t)B * (L + 1) + (elem == sizeof(float4) ? tw_place<float4>(L / 2) : tw_place<float2>(L / 2))) * elem;
 }
@@ -353,10 +352,10 @@ int cta_threads(size_t smem) {
 // of either kind share an SM (short lines, where launches and tails count),
 // else each with the shared memory and threads of its own.
 cudaError_t launch_lines(bool inverse, const float4* in4, float4* out4, FftLines d4, int ngrids4, const float2* in2,
-                         float2* out2, FftLines d2, int ngrids2, const float4* tw, cudaStream_t s) {
+                         float2* out2, FftLines d2, int ngrids2, const float4* tw, int num_sms, cudaStream_t s) {
   d4.B = lines_per_cta(d4.L, sizeof(float4));
   d2.B = lines_per_cta(d2.L, sizeof(float2));
-  while (ctas(d4, d4.B, ngrids4) + ctas(d2, d2.B, ngrids2) < FFT_FILL && d4.B > 1) {
+  while (ctas(d4, d4.B, ngrids4) + ctas(d2, d2.B, ngrids2) < 3 * (int64_t)num_sms && d4.B > 1) {
     d4.B = (d4.B + 1) / 2;
     d2.B = (d2.B + 1) / 2;
   }
@@ -410,25 +409,25 @@ cudaError_t fft2d_forward(const float4* compact4, float4* spec4, int ngrids4, co
   r.in_len = (int)nx; r.out_len = f.Nx;
   r.in_line_stride = nx; r.out_line_stride = f.Nx;
   r.in_grid_stride = in_grid_stride; r.out_grid_stride = (int64_t)f.Nx * f.Ny;
-  cudaError_t e = launch_lines(false, compact4, spec4, r, ngrids4, compact2, spec2, r, ngrids2, f.tw_x, s);
+  cudaError_t e = launch_lines(false, compact4, spec4, r, ngrids4, compact2, spec2, r, ngrids2, f.tw_x, f.num_sms, s);
   if (e != cudaSuccess) return e;
   // columns: all Nx, rows >= ny read as zero
   FftLines c = col_lines(f);
   c.in_len = (int)ny; c.out_len = f.Ny;
-  return launch_lines(false, spec4, spec4, c, ngrids4, spec2, spec2, c, ngrids2, f.tw_y, s);
+  return launch_lines(false, spec4, spec4, c, ngrids4, spec2, spec2, c, ngrids2, f.tw_y, f.num_sms, s);
 }
 
 cudaError_t fft2d_inverse(float4* spec4, float4* compact4, int ngrids4, float2* spec2, float2* compact2, int ngrids2,
                           const Fft2d& f, int64_t nx, int64_t ny, int64_t out_grid_stride, cudaStream_t s) {
   FftLines c = col_lines(f);
   c.in_len = f.Ny; c.out_len = (int)ny;
-  cudaError_t e = launch_lines(true, spec4, spec4, c, ngrids4, spec2, spec2, c, ngrids2, f.tw_y, s);
+  cudaError_t e = launch_lines(true, spec4, spec4, c, ngrids4, spec2, spec2, c, ngrids2, f.tw_y, f.num_sms, s);
   if (e != cudaSuccess) return e;
   FftLines r = row_lines(f, ny);
   r.in_len = f.Nx; r.out_len = (int)nx;
   r.in_line_stride = f.Nx; r.out_line_stride = nx;
   r.in_grid_stride = (int64_t)f.Nx * f.Ny; r.out_grid_stride = out_grid_stride;
-  return launch_lines(true, spec4, compact4, r, ngrids4, spec2, compact2, r, ngrids2, f.tw_x, s);
+  return launch_lines(true, spec4, compact4, r, ngrids4, spec2, compact2, r, ngrids2, f.tw_x, f.num_sms, s);
 }
 
 }  // namespace irs

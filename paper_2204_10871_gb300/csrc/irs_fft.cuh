@@ -26,6 +26,7 @@ struct Fft2d {
   int n3x, n2x, n3y, n2y;
   float4* tw_x;  // W_N^t, t < N/2, as double-float complex
   float4* tw_y;
+  int num_sms;  // of the device that runs it
 };
 
 // Smallest length 2^a 3^b >= n_min with a >= 1 and at most FFT_MAX_LEN, or -1;

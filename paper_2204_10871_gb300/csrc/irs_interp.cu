@@ -2190,6 +2190,7 @@ irs_status interp_plan(irs_plan_t* P) {
   if (ig.W < 1) ig.W = 1;
 
   Fft2d& f = S->fft;
+  f.num_sms = P->num_sms;
   // padded lengths >= 2n - 1 (linear convolution), of the form 2^a 3^b
   f.Nx = fft_good_size(2 * ncx - 1, &f.n3x, &f.n2x);
   f.Ny = fft_good_size(2 * ncy - 1, &f.n3y, &f.n2y);
