@@ -9,7 +9,8 @@ unlensed pixel: 1.12e10 rays per map).
 One step = one magnification map through irs_make_map (INTERP: mass sum, cell
 lists, far field, ray pass, binning, magnification); its rays are those of the
 lattice.  The ray pass leaves out work units that provably send no ray onto the
-map (an exact bound, the same map bit for bit); the roofline counts the rest.  The plain brute-force map of the
+map (an exact bound, the same map bit for bit); the roofline counts the rays that
+land.  The plain brute-force map of the
 same workload costs ~1e15 pair terms (minutes), so it is timed on a band of
 lattice rows through irs_make_map_rows and reported per ray, with the same
 band made by the interpolated method as the accuracy check (per-pixel
@@ -173,25 +174,15 @@ def lens_field(lensgen, box, seed, w=WORKLOAD):
 # Per-ray work of the interpolated ray pass, in flops: 10 per near pair (the
 # same pair arithmetic as the brute force), 8 per complex multiply-add of the
 # level-2 Horner (K2 - 1 of them for K2 series terms), and 20 for the smooth
-# terms, sub-cell index and pixel.
+# terms, sub-cell index and pixel.  The rays counted are those that landed on the
+# map, which the run itself counts: the pass evaluates at least these (it leaves
+# out work units that cannot reach the map), so the fraction is a lower bound.
 IP_VARIANT_K2 = [6, 7, 6, 6, 6, 6, 6, 6, 6, 8, 6, 5, 5, 5, 5, 5, 4]  # series terms K2 of ray-pass variants 0..16
 IP_FLOPS_OTHER = 20
 
 
 def ip_flops_fixed(variant):
     return 8 * (IP_VARIANT_K2[variant] - 1) + IP_FLOPS_OTHER
-
-
-# Share of a map's rays that the ray pass evaluates: work units (32 columns x 8
-# rows) that provably cannot reach the map are left out.  Counted for these
-# workloads' lens fields: (workload, cell multiplier) -> share.
-IP_EVALUATED = {("paper-mid", 0.57): 0.3943, ("high-res", 0.72): 0.4749}
-
-
-def evaluated_share(name, cell_mult, landed, n_rays):
-    """The counted share, or the share of the rays that landed on the map, a
-    lower bound, for any other workload or cell size."""
-    return IP_EVALUATED.get((name.split(":")[0], round(float(cell_mult or 1.0), 2)), landed / n_rays)
 
 
 # DRAM bytes per launch of the ray pass (ncu dram__bytes_read.sum +
@@ -375,7 +366,7 @@ def run_ours(args):
     if full:
         n_near = mean_near_lenses(info, xy)
         variant = int(params.kernel_variant)
-        share = evaluated_share(w["name"], params.cell_mult, landed, info.n_rays)
+        share = landed / info.n_rays  # work units that cannot reach the map are left out
         flops_per_ray = (10.0 * n_near + ip_flops_fixed(variant)) * share
         kname = f"k_ip_ray variant {variant} (near pair sum + level-2 Horner, FP32 pipe + MUFU)"
         key = (w["name"].split(":")[0], round(float(params.cell_mult or 1.0), 2), variant)
@@ -393,7 +384,7 @@ def run_ours(args):
                 "flops_per_ray": flops_per_ray}
     if n_near is not None:
         roofline["mean_near_lenses"] = n_near
-        roofline["evaluated_share"] = share
+        roofline["evaluated_share_at_least"] = share
     if clocks.get("sm_mhz"):
         roofline["frac_at_measured_clock"] = achieved / (n_sms * 256 * clocks["sm_mhz"] * 1e6 / 1e12)
 
@@ -594,7 +585,7 @@ def high_res_record(irs, torch, lensgen, n_sms, peak_tflops, flush):
     del counts, mag
     variant = int(params.kernel_variant)
     n_near = mean_near_lenses(info, xy)
-    share = evaluated_share(w["name"], params.cell_mult, landed, info.n_rays)
+    share = landed / info.n_rays
     flops = (10.0 * n_near + ip_flops_fixed(variant)) * share
     ach = flops * info.n_rays / (ms_ray * 1e-3) / 1e12
     r0 = (info.n_rays_y // 2 // 64) * 64
@@ -608,7 +599,7 @@ def high_res_record(irs, torch, lensgen, n_sms, peak_tflops, flush):
                          "candidates": res.candidates, "tuning_s": tune_s},
             "roofline": {"bound": "alu", "kernel": f"k_ip_ray variant {variant}", "achieved": ach,
                          "peak": peak_tflops, "unit": "TFLOP/s", "frac": ach / peak_tflops,
-                         "flops_per_ray": flops, "mean_near_lenses": n_near, "evaluated_share": share},
+                         "flops_per_ray": flops, "mean_near_lenses": n_near, "evaluated_share_at_least": share},
             "brute": dict(brute, roofline_frac=brute_ach / peak_tflops),
             "speedup_over_brute": value / brute["rays_per_s"],
             "map_rel_rms_vs_brute": rel, "min_rays_per_pixel": 100}
