@@ -54,11 +54,19 @@ irs_status st_of(cudaError_t e) {
   return e == cudaErrorMemoryAllocation ? IRS_ERR_OOM : IRS_ERR_CUDA;
 }
 
+// Interpolated maps whose ray passes go in one launch: one variant and CTA size.
+struct Group {
+  std::vector<int> maps;
+  size_t off = 0;               // of its descriptors
+  int nrow = 0, near_cap = 0;   // the largest among the maps
+  int64_t items = 0;            // work items of the launch
+  bool cut = false;             // they are shares of cells
+};
+
 // Enqueue the whole batch on the capture stream (and its side streams).
 irs_status enqueue(BatchEntry* e, irs_plan_t* const* plans, int32_t nmaps, const double* const* xy,
                    const double* const* mass, const int64_t* n, uint32_t* const* counts,
-                   float* const* mag, const std::vector<std::vector<int>>& groups,
-                   const std::vector<size_t>& group_off, size_t queue_off) {
+                   float* const* mag, const std::vector<Group>& groups, size_t queue_off) {
   cudaStream_t cs = e->cs;
   if (cudaEventRecord(e->ev[NSIDE], cs) != cudaSuccess) return IRS_ERR_CUDA;
   for (int k = 0; k < NSIDE; ++k)
@@ -88,23 +96,11 @@ irs_status enqueue(BatchEntry* e, irs_plan_t* const* plans, int32_t nmaps, const
   char* base = static_cast<char*>(e->dbuf);
   unsigned long long* queues = reinterpret_cast<unsigned long long*>(base + queue_off);
   for (size_t v = 0; v < groups.size(); ++v) {
-    const std::vector<int>& gm = groups[v];
-    if (gm.empty()) continue;
-    // item count of the group, recomputed from the plans (cheap, host side)
-    std::vector<irs_plan_t*> gp;
-    std::vector<uint32_t*> gc;
-    int nrow = 0, near_cap = 0;
-    for (int m : gm) {
-      gp.push_back(plans[m]);
-      gc.push_back(counts[m]);
-      const int r = irs::interp_row_entries(plans[m]), c = irs::interp_near_cap(plans[m], n[m]);
-      nrow = r > nrow ? r : nrow;
-      near_cap = c > near_cap ? c : near_cap;
-    }
-    std::vector<char> tmp(irs::interp_desc_bytes((int)gm.size()));
-    const int64_t items = irs::interp_fill_descs(gp.data(), gc.data(), (int)gm.size(), tmp.data());
-    irs_status st = irs::interp_batch_launch((int)v / 2, base + group_off[v], (int)gm.size(), items,
-                                             queues + v, plans[gm[0]]->num_sms, nrow, near_cap, cs);
+    const Group& gr = groups[v];
+    if (gr.maps.empty()) continue;
+    irs_status st = irs::interp_batch_launch((int)v / 2, base + gr.off, (int)gr.maps.size(), gr.items, gr.cut,
+                                             queues + v,
+                                             plans[gr.maps[0]]->num_sms, gr.nrow, gr.near_cap, cs);
     if (st != IRS_OK) return st;
   }
   if (mag) {
@@ -131,15 +127,19 @@ irs_status build_entry(BatchEntry* e, irs_plan_t* const* plans, int32_t nmaps,
   // memory is that of its largest cell: with one group per variant the maps of
   // small cells ran on the large CTAs too, 30.5 against 28.1 ms for 24 maps); descriptors + queues in one
   // buffer.  Group 2 v: variant v on CTAs of 256 threads, 2 v + 1: of 128.
-  std::vector<std::vector<int>> groups(2 * irs::interp_num_variants());
-  for (int32_t m = 0; m < nmaps; ++m)
-    if (plans[m]->p.method != IRS_BRUTE)
-      groups[2 * irs::interp_variant(plans[m]) + (irs::interp_small_ctas(plans[m], n[m]) ? 1 : 0)].push_back(m);
-  std::vector<size_t> group_off(groups.size(), 0);
+  std::vector<Group> groups(2 * irs::interp_num_variants());
+  for (int32_t m = 0; m < nmaps; ++m) {
+    if (plans[m]->p.method == IRS_BRUTE) continue;
+    Group& gr = groups[2 * irs::interp_variant(plans[m]) + (irs::interp_small_ctas(plans[m], n[m]) ? 1 : 0)];
+    const int r = irs::interp_row_entries(plans[m]), c = irs::interp_near_cap(plans[m], n[m]);
+    gr.maps.push_back(m);
+    gr.nrow = r > gr.nrow ? r : gr.nrow;
+    gr.near_cap = c > gr.near_cap ? c : gr.near_cap;
+  }
   size_t off = 0;
-  for (size_t v = 0; v < groups.size(); ++v) {
-    group_off[v] = off;
-    off += (irs::interp_desc_bytes((int)groups[v].size()) + 255) & ~(size_t)255;
+  for (Group& gr : groups) {
+    gr.off = off;
+    off += (irs::interp_desc_bytes((int)gr.maps.size()) + 255) & ~(size_t)255;
   }
   const size_t queue_off = off;
   off += sizeof(unsigned long long) * groups.size();
@@ -147,23 +147,24 @@ irs_status build_entry(BatchEntry* e, irs_plan_t* const* plans, int32_t nmaps,
     cudaGetLastError();
     return IRS_ERR_OOM;
   }
-  for (size_t v = 0; v < groups.size(); ++v) {
-    if (groups[v].empty()) continue;
+  for (Group& gr : groups) {
+    if (gr.maps.empty()) continue;
     std::vector<irs_plan_t*> gp;
     std::vector<uint32_t*> gc;
-    for (int m : groups[v]) {
+    for (int m : gr.maps) {
       gp.push_back(plans[m]);
       gc.push_back(counts[m]);
     }
-    std::vector<char> host(irs::interp_desc_bytes((int)groups[v].size()));
-    irs::interp_fill_descs(gp.data(), gc.data(), (int)groups[v].size(), host.data());
-    if (cudaMemcpy(static_cast<char*>(e->dbuf) + group_off[v], host.data(), host.size(),
-                   cudaMemcpyHostToDevice) != cudaSuccess)
+    std::vector<char> host(irs::interp_desc_bytes((int)gr.maps.size()));
+    gr.items = irs::interp_fill_descs(gp.data(), gc.data(), (int)gr.maps.size(), gr.nrow, gr.near_cap, host.data(),
+                                      &gr.cut);
+    if (cudaMemcpy(static_cast<char*>(e->dbuf) + gr.off, host.data(), host.size(), cudaMemcpyHostToDevice) !=
+        cudaSuccess)
       return IRS_ERR_CUDA;
   }
 
   if (cudaStreamBeginCapture(e->cs, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return IRS_ERR_CUDA;
-  irs_status st = enqueue(e, plans, nmaps, xy, mass, n, counts, mag, groups, group_off, queue_off);
+  irs_status st = enqueue(e, plans, nmaps, xy, mass, n, counts, mag, groups, queue_off);
   cudaGraph_t graph = nullptr;
   const cudaError_t ce = cudaStreamEndCapture(e->cs, &graph);
   if (st != IRS_OK) {

@@ -42,12 +42,14 @@ bool interp_small_ctas(const irs_plan_t* P, int64_t n);
 int interp_num_variants();
 // false for a variant number served by another number's kernel
 bool interp_variant_distinct(int variant);
-// host-side ray-pass descriptors of maps that share a kernel variant; returns
-// the total number of (map, cell) work items
+// host-side ray-pass descriptors of maps that share a launch, whose shared memory
+// is sized for nrow and near_cap (the largest among the maps); returns the total
+// number of (map, share of a cell) work items, and whether cells are cut into shares
 size_t interp_desc_bytes(int nmaps);
-int64_t interp_fill_descs(irs_plan_t* const* plans, uint32_t* const* counts, int nmaps, void* host);
+int64_t interp_fill_descs(irs_plan_t* const* plans, uint32_t* const* counts, int nmaps, int nrow, int near_cap,
+                          void* host, bool* cut);
 // one persistent launch over all maps' cells (descriptors already on the
 // device); nrow, near_cap: the largest among the maps
-irs_status interp_batch_launch(int variant, const void* dev_descs, int nmaps, int64_t nitems,
+irs_status interp_batch_launch(int variant, const void* dev_descs, int nmaps, int64_t nitems, bool cut,
                                unsigned long long* queue, int num_sms, int nrow, int near_cap, cudaStream_t s);
 }  // namespace irs
