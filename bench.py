@@ -189,7 +189,7 @@ def ip_flops_fixed(variant):
 # dram__bytes_write.sum), valid only for the kernel build, workload and cell
 # size they were captured on: (workload, cell multiplier, variant) -> bytes.
 # Source: profiles/k_ip_ray_paper-mid-full.md.
-IP_TRAFFIC = {("paper-mid", 0.57, 16): 106.676480e6 + 5.420032e6}
+IP_TRAFFIC = {("paper-mid", 0.57, 16): 106.771456e6 + 4.525568e6}
 
 
 def mean_near_lenses(info, xy):

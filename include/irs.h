@@ -136,8 +136,8 @@ irs_status irs_make_map(irs_plan_t* plan, const double* lens_xy, const double* m
  * counterpart: many maps of uneven N_*, kappa and gamma).  Each map's mass
  * sum, cell lists and far-field series (or brute-force setup and ray pass) run
  * on forked streams; the interpolated ray passes of all maps run as one
- * persistent launch per kernel variant that pulls (map, cell) items from a
- * global counter.  The sequence is captured into a CUDA graph on the first call
+ * persistent launch per kernel variant and CTA size that pulls (map, cell)
+ * items, or shares of cells where they are few, from a global counter.  The sequence is captured into a CUDA graph on the first call
  * with a given set of plans, pointers and lens counts, and later calls with the
  * same set replay the graph (the last 4 sets are kept; destroying a plan drops
  * the graphs that use it).  A plan whose lens buffers were reallocated since
@@ -192,9 +192,9 @@ irs_status irs_plan_timings(irs_plan_t* plan, irs_timings* out);
 /* Debug / parity path: the source-plane position beta (2 doubles per ray,
  * device) and pixel index (int64, -1 when outside; device; may be NULL) of
  * the lattice rays with flat indices ray_idx[k] = j * n_rays_x + i (device
- * int64).  Each ray is computed by the same kernel code and tiling that
- * irs_make_map uses for the plan's method, so the values are those that
- * were binned.  Errors: IRS_ERR_ARG, IRS_ERR_CUDA. */
+ * int64).  Each ray is computed by itself, in the operations, order and
+ * roundings of irs_make_map's ray pass for the plan's method and kernel
+ * variant, so the values are those that were binned.  Errors: IRS_ERR_ARG, IRS_ERR_CUDA. */
 irs_status irs_shoot_rays(irs_plan_t* plan, const double* lens_xy, const double* mass, int64_t n,
                           const int64_t* ray_idx, int64_t n_idx, double* beta, int64_t* pixel,
                           void* stream);
@@ -303,7 +303,8 @@ irs_status irs_mlp_forward(irs_plan_t* plan, const float* x, int64_t n, float* y
  * device before any stream capture and outside latency-critical loops; later
  * calls allocate nothing.  Lens positions are not checked against the lens
  * region (there is no plan to report a device-side error to).  All calls share
- * the array: calls whose work overlaps on the GPU race.  Errors: IRS_ERR_ARG,
+ * the array: calls whose work overlaps on the GPU race, and only those maps are
+ * spoilt.  Errors: IRS_ERR_ARG,
  * IRS_ERR_DEGENERATE, IRS_ERR_OVERFLOW, IRS_ERR_UNSUPPORTED (method other than
  * IRS_BRUTE), IRS_ERR_CUDA. */
 irs_status irs_make_map_brute_noalloc(const irs_params* params, const double* lens_xy,
@@ -313,8 +314,8 @@ irs_status irs_make_map_brute_noalloc(const irs_params* params, const double* le
 /* Wait for `stream` and return the first error a kernel of this plan raised
  * since the last sync (IRS_OK if none), clearing it: IRS_ERR_ARG for a lens
  * outside the plan's lens region, IRS_ERR_OVERFLOW when the 3 x 3 block of
- * level-1 cells around some cell held more than the 1024 lenses the
- * interpolated ray pass keeps in shared memory (that cell's near sum used the
+ * level-1 cells around some cell held more than 1024 lenses, the most that
+ * the interpolated ray pass sums directly (that cell's near sum used the
  * first 1024; the map is not valid).  The plan stays usable. */
 irs_status irs_plan_sync(irs_plan_t* plan, void* stream);
 

@@ -3,8 +3,9 @@
 // Maps with uneven lens counts, kappa and gamma are prepared on NSIDE forked
 // capture streams (each map's mass sum, cell lists and far-field series, or
 // the brute-force tile setup and ray pass), joined, and their interpolated ray
-// passes run as ONE persistent launch per kernel variant whose CTAs pull
-// (map, cell) items from a global counter.  The whole sequence is captured once
+// passes run as ONE persistent launch per kernel variant and CTA size whose CTAs
+// pull (map, cell) items -- (map, share of a cell) where cells are few -- from a
+// global counter.  The whole sequence is captured once
 // per distinct (plans, buffers) set and replayed from the instantiated graph.
 #include <string.h>
 

@@ -41,7 +41,7 @@ struct Geo {
 // that has finished implies that all before it have.  The first kernel of a
 // call is launched the ordinary way: caller's buffers are complete when it
 // starts.  A map of few lenses is a chain of a dozen short kernels, whose launch
-// latencies and set-ups overlap this way (a 64^2 brute-force map: 33 us
+// latencies and set-ups overlap this way (a 64^2 brute-force map: 32 us
 // instead of 48).
 //
 // A chained kernel's pointers to what an earlier kernel of the call writes are

@@ -4,7 +4,7 @@
 // FP32 (float2 elements).
 //
 // A CTA takes B lines of length L = 3^n3 2^n2 (B as large as keeps it within
-// 52 KB of shared memory, at least one) with a twiddle table W_L^t (t < L/2;
+// 74 KB of shared memory, at least one, fewer in small launches) with a twiddle table W_L^t (t < L/2;
 // W_L^(t + L/2) = -W_L^t) beside them, and runs the butterfly stages in passes:
 // up to three radix-2 or two radix-3 stages of a line's element group in
 // registers, then an exchange through shared memory; the first pass reads

@@ -1,6 +1,6 @@
 // irs_fft.cuh -- complex FFTs of length 2^a 3^b (a >= 1) in shared memory
-// (irs_fft.cu), in double-float arithmetic on float4 values (re.hi, re.lo,
-// im.hi, im.lo; irs_df.cuh) or in FP32 on float2 values (re, im).
+// (irs_fft.cu), in double-float arithmetic on float4 values (re.hi, im.hi,
+// re.lo, im.lo; irs_df.cuh) or in FP32 on float2 values (re, im).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -9,7 +9,7 @@
 namespace irs {
 
 constexpr int FFT_MAX_LEN = 9216;  // longest line (3^2 2^10): 144 KB of double-float complex values
-                                   // and a 72 KB twiddle table
+                                   // and an 81 KB twiddle table
 
 // One batched pass of 1-D FFTs over `n_lines` lines of length L.
 struct FftLines {

@@ -1052,8 +1052,8 @@ constexpr int IP_HIST = IP_HS * IP_BOX_H;
 
 // Dynamic shared memory of the ray pass: the level-2 series as conj duplicated
 // (c.re, c.re, -c.im, -c.im), the histogram, the level-1 series scaled for the
-// re-centring with its scale factors, the row table, and the near lenses.
-// size come first, so that the addresses of the hot ones are constants.
+// re-centring with its scale factors, the row table, and the near lenses.  Tables
+// of fixed size come first, so that the addresses of the hot ones are constants.
 struct __align__(16) IpRowPair {  // one entry per pair of cell rows (2l, 2l + 1)
   float4 sg;      // (sigma_y, sigma_y', -sigma_y, -sigma_y'), sigma_y = (l + 1/2) Q/k - v - 1/2
   float4 ty;      // (tau_y h, tau_y' h, y0, y0'), y0 = by_lo + lambda_2 tau_y h: the row's share of beta_2
@@ -1946,7 +1946,7 @@ IpShape ip_launch_shape(int variant, int nrow, int near_cap, int num_sms) {
 }
 
 // Lenses of a 3x3 block kept in shared memory: the mean of n lenses over the
-// cell grid and six deviations; fuller blocks read theirs from memory.
+// cell grid and six deviations; fuller blocks take theirs through it in turns.
 int ip_near_cap(const IpGeo& ig, int64_t n) {
   const double mean = 9.0 * (double)n / ((double)ig.ncx * (double)ig.ncy);
   double cap = mean + 6.0 * sqrt(mean) + 8.0;
